@@ -83,7 +83,9 @@ typedef struct dj_graph_info {
  *              Ids are 0-based in [0, n); 0 <= w < DJ_INF.
  *   directed   0: G[u][v] = G[v][u] = w;  1 (the paper's -w): G[u][v] = w only
  * The diagonal is 0, missing entries DJ_INF, a repeated pair keeps its minimum
- * weight, self-loops are ignored.  On success *out owns the device matrix until
+ * weight, self-loops are ignored.  The list is checked by the device as it
+ * reads it (on the host where there is no device); a bad list's first bad edge
+ * is named in dj_last_error().  On success *out owns the device matrix until
  * dj_graph_free.  Synchronous with respect to the host (the edge arrays may be
  * reused on return); the device work is ordered on `stream`.
  * Errors: DJ_EINVAL (bad id/weight/n/m, NULL pointer), DJ_EOVERFLOW

@@ -50,6 +50,7 @@ int get_ctx(DevCtx** out) {
     int cl = 0;
     cudaDeviceGetAttribute(&cl, cudaDevAttrClusterLaunch, dev);
     c.cluster_launch = cl;
+    cudaDeviceGetAttribute(&c.pageable, cudaDevAttrPageableMemoryAccess, dev);
     e = cudaMalloc(&c.words, 64 * sizeof(uint32_t));
     if (e != cudaSuccess) return cuda_error(e, "cudaMalloc(device words)");
     e = cudaMemset(c.words, 0, 64 * sizeof(uint32_t));

@@ -94,6 +94,7 @@ struct DevCtx {
   int max_smem_optin = 0;
   int coop = 0;
   int cluster_launch = 0;
+  int pageable = 0;  // the device reads pageable host memory coherently
   uint32_t* words = nullptr;  // device: [0] error bits, [1] phases of the last single solve
   std::vector<StreamWs> ws;   // per-stream workspaces of the grid engine (see stream_workspace)
   std::vector<FnSetup> fns;   // see prepare_function

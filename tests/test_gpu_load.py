@@ -1,0 +1,51 @@
+"""Building the matrix from an edge list read by the device itself: every size around the scatter's
+grid, arrays at odd offsets, and the first bad edge named whatever its place in the list."""
+import numpy as np
+import pytest
+
+import graphgen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dj():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2504_03667_gb300 import dj as _dj
+    torch.cuda.set_device(0)
+    return _dj
+
+
+@pytest.mark.parametrize("m", [0, 1, 3, 255, 256, 1023, 1025, 40000])
+@pytest.mark.parametrize("directed", [False, True])
+def test_matrix_matches_the_fill_rules(dj, orc, m, directed):
+    n = 61
+    e = graphgen.random_edges(n, m + 1, 0, 9, seed=500 + m, directed=directed)
+    src, dst, w = e.src[1:], e.dst[1:], e.w[1:]  # one entry off the arrays' alignment
+    G = dj.dj_load_edges(n, src, dst, w, directed)
+    assert np.array_equal(dj.dj_graph_download(G), orc.build_matrix(n, src, dst, w, directed))
+    G.free()
+
+
+@pytest.mark.parametrize("at", [0, 1, 1024, 77777, 99999])
+def test_first_bad_edge_is_named(dj, at):
+    n, m = 500, 100000
+    e = graphgen.random_edges(n, m, 1, 9, seed=9, directed=True)
+    for what, value, word in (("src", n, "node id"), ("dst", -1, "node id"), ("w", -5, "weight"), ("w", 2**31 - 1, "weight")):
+        a = {"src": e.src.copy(), "dst": e.dst.copy(), "w": e.w.copy()}
+        a[what][at] = value
+        a["w"][min(m - 1, at + 5000)] = -1  # a later one
+        with pytest.raises(dj.DjError) as ei:
+            dj.dj_load_edges(n, a["src"], a["dst"], a["w"], True)
+        assert ei.value.status == dj.DJ_EINVAL
+        assert f"edge {at} " in str(ei.value) and word in str(ei.value)
+    w = e.w.copy()
+    w[at] = (2**31 - 1) // (n - 1) + 1
+    if e.src[at] != e.dst[at]:
+        with pytest.raises(dj.DjError) as ei:
+            dj.dj_load_edges(n, e.src, e.dst, w, True)
+        assert ei.value.status == dj.DJ_EOVERFLOW
