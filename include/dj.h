@@ -65,7 +65,7 @@ typedef struct dj_graph_info {
   const int32_t* matrix; /* device pointer: n rows x pitch int32, row-major; columns >= n hold DJ_INF */
   const int32_t* minout; /* device pointer: n int32, min finite off-diagonal weight of row u (DJ_INF if none) */
   const int32_t* minin;  /* device pointer: n int32, min finite off-diagonal weight of column v (DJ_INF if none) */
-  uint64_t bytes;        /* device bytes owned by the graph */
+  uint64_t bytes;        /* device bytes owned by the graph (the light-edge index included) */
   uint64_t entries;      /* finite off-diagonal matrix entries (directed edges; twice the undirected ones) */
   int32_t format;        /* DJ_FORMAT_DENSE (matrix) or DJ_FORMAT_CSR (compressed rows, matrix NULL) */
   int32_t reserved;
@@ -97,9 +97,9 @@ int dj_load_edges(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, 
  * names that matrix's n^2 memory as the limit for sparse graphs, Section IV
  * and Conclusion).  Arguments, validation and fill rules as dj_load_edges
  * (repeats keep their smallest weight, self-loops are dropped, undirected
- * graphs store both directions); the edges are sorted on the host and the
- * device holds n + 1 64-bit row offsets, the targets and the weights
- * (8 bytes per directed edge) plus the row and column minima.  dj_sssp and
+ * graphs store both directions); the rows are sorted on the host and the
+ * device holds n + 1 64-bit row offsets and the edges, target and weight in
+ * one word (4 bytes per directed edge), plus the row and column minima.  dj_sssp and
  * dj_sssp_ex solve it with the same phase logic and give the same dist and
  * pred as on the dense matrix; dj_graph_download / upload, dj_sssp_noalloc,
  * dj_sssp_lc, batches and serving need the matrix and return
@@ -146,9 +146,20 @@ int dj_graph_free(dj_graph* g);
                            visit order in one fused relaxation pass (same dist and pred) */
 #define DJ_MODE_PLAIN 2 /* literal Algorithm 1: one argmin + one row relaxation per step */
 
-#define DJ_ENGINE_AUTO 0     /* grid for n >= 4096, or n >= 2560 with at least n^2/4 finite entries */
+#define DJ_ENGINE_AUTO 0     /* the light engine (below) where it applies; else grid for n >= 4096, or
+                                n >= 2560 with at least n^2/4 finite entries, and cluster below */
 #define DJ_ENGINE_GRID 1    /* one cooperative persistent kernel over every SM; column slices per CTA */
 #define DJ_ENGINE_CLUSTER 2 /* one thread-block cluster; state in distributed shared memory */
+
+/* The light engine.  A loaded graph keeps, beside its matrix, each row's up to
+ * 64 lightest edges and the smallest weight not among them (256 bytes a node,
+ * rebuilt by dj_graph_upload).  A solve relaxes those; then dist[u] + (u's
+ * smallest unlisted weight) > max dist proves that no unlisted edge matters,
+ * and rows that fail the test are relaxed whole from the matrix, so dist and
+ * pred are Algorithm 1's on every graph.  Taken by DJ_ENGINE_AUTO in phase
+ * mode when every weight is >= 1, every other option below is left at its
+ * default, and a trial solve at load needed at most n/16 whole rows; also for
+ * graphs in compressed rows. */
 
 typedef struct dj_solve_opts {
   int32_t mode;           /* DJ_MODE_* */
@@ -384,7 +395,8 @@ int dj_tune_lookup(int32_t n, uint64_t entries, int32_t num_sms, int32_t* engine
 typedef struct dj_server dj_server;
 
 typedef struct dj_serve_opts {
-  uint64_t hbm_budget;   /* bytes of device memory the server may hold (graphs + result pool) */
+  uint64_t hbm_budget;   /* bytes of device memory the server may hold (graphs without their
+                            light-edge index + result pool) */
   int32_t max_slots;     /* requests in flight on the device at most (<= 4096) */
   int32_t cluster_size;  /* CTAs per solve cluster, 0 = auto */
   int32_t threads;       /* 0 = auto */

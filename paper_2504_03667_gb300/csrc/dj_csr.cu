@@ -3,14 +3,16 @@
 // The paper stores every graph as a dense adjacency matrix and concludes that
 // its n^2 memory is what limits sparse graphs (Section IV, Conclusion).  A
 // graph loaded with dj_load_edges_csr keeps only its edges (row offsets,
-// columns, weights: 8 bytes per directed edge), and dj_sssp runs it on a
+// packed edges: 4 bytes per directed edge), and dj_sssp runs it on a
 // cooperative kernel that keeps the grid engine's phase logic -- per-CTA
 // column slices, one exchange of partials and candidates per phase, the OUT
 // and IN settle bounds, lexicographic keys -- and replaces the row streaming:
 // each CTA takes every G-th settled candidate and pushes its row's edges as
 // 64-bit keys (candidate << 32) | tie word into a global per-node key array
 // with atomicMin; after a second grid barrier the owners commit their slices
-// from it exactly as the row-split phases of the dense engine do.
+// from it exactly as the row-split phases of the dense engine do.  That kernel serves plain mode,
+// zero weights and callers that choose a settle bound; every other solve takes the light engine
+// (dj_light_grid.cu), whose keys need no settle bounds and whose phases cost one barrier, not two.
 #include <algorithm>
 #include <string>
 #include <vector>
@@ -23,8 +25,7 @@ namespace dj {
 
 struct CsrParams {
   const int64_t* row_ptr;  // n + 1
-  const int32_t* col;      // nnz
-  const int32_t* wt;       // nnz
+  const uint32_t* edge;    // nnz packed (weight << bits_u) | target
   const int32_t* minout;   // n
   const int32_t* minin;    // n
   int32_t* dist_out;
@@ -94,9 +95,10 @@ __global__ void __launch_bounds__(kCsrThreads, 1) k_sssp_csr(const CsrParams p) 
   if (!p.plain) {  // the first step settles only the source: apply its edges that land in this slice
     const int64_t e0 = p.row_ptr[p.source], e1 = p.row_ptr[p.source + 1];
     for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-      const int v = __ldg(p.col + e);
+      const uint32_t x = __ldg(p.edge + e);
+      const int v = static_cast<int>(x & ((1u << p.bits_u) - 1u));
       if (v >= s.c0 && v < s.c0 + s.sw) {
-        s.dist[v - s.c0] = static_cast<uint32_t>(__ldg(p.wt + e));
+        s.dist[v - s.c0] = x >> p.bits_u;
         s.pred[v - s.c0] = p.source;
         s.pdist[v - s.c0] = 0u;
       }
@@ -190,9 +192,9 @@ __global__ void __launch_bounds__(kCsrThreads, 1) k_sssp_csr(const CsrParams p) 
       const uint32_t du = D.m + (tb >> p.bits_u);
       const int64_t e0 = p.row_ptr[u], e1 = p.row_ptr[u + 1];
       for (int64_t e = e0 + lane; e < e1; e += 32) {
-        const int v = __ldg(p.col + e);
-        const unsigned long long kk =
-            (static_cast<unsigned long long>(du + static_cast<uint32_t>(__ldg(p.wt + e))) << 32) | tb;
+        const uint32_t x = __ldg(p.edge + e);
+        const uint32_t v = x & umask;
+        const unsigned long long kk = (static_cast<unsigned long long>(du + (x >> p.bits_u)) << 32) | tb;
         if (kk < *reinterpret_cast<volatile unsigned long long*>(gk + v)) atomicMin(gk + v, kk);
       }
     }
@@ -225,13 +227,8 @@ extern "C" int dj_load_edges_csr(int32_t n, int64_t m, const int32_t* src, const
   if (n < 1) return set_error(DJ_EINVAL, "n must be >= 1");
   if (m < 0) return set_error(DJ_EINVAL, "m must be >= 0");
   if (m > 0 && (!src || !dst || !w)) return set_error(DJ_EINVAL, "edge arrays are NULL");
-  // validation and the kept (u, v, w) triples, both directions for undirected graphs
-  struct Edge {
-    uint64_t key;  // (u << 32) | v
-    int32_t w;
-  };
-  std::vector<Edge> es;
-  es.reserve(static_cast<size_t>(directed ? m : 2 * m));
+  // validation; edges per row, both directions for undirected graphs
+  std::vector<int64_t> row_ptr(static_cast<size_t>(n) + 1, 0);
   int64_t wmax = 0;
   for (int64_t e = 0; e < m; ++e) {
     const int32_t u = src[e], v = dst[e], x = w[e];
@@ -241,31 +238,64 @@ extern "C" int dj_load_edges_csr(int32_t n, int64_t m, const int32_t* src, const
       return set_error(DJ_EINVAL, "edge " + std::to_string(e) + " has a weight outside [0, INT32_MAX)");
     if (u == v) continue;  // self-loops never shorten a path
     if (x > wmax) wmax = x;
-    es.push_back({(static_cast<uint64_t>(u) << 32) | static_cast<uint32_t>(v), x});
-    if (!directed) es.push_back({(static_cast<uint64_t>(v) << 32) | static_cast<uint32_t>(u), x});
+    ++row_ptr[static_cast<size_t>(u) + 1];
+    if (!directed) ++row_ptr[static_cast<size_t>(v) + 1];
   }
   if (n > 1 && static_cast<int64_t>(n - 1) * wmax >= static_cast<int64_t>(DJ_INF))
     return set_error(DJ_EOVERFLOW, "(n-1) * max weight >= INT32_MAX: path lengths could overflow int32");
-  // sort by (u, v, w); a repeated pair keeps its smallest weight
-  std::sort(es.begin(), es.end(), [](const Edge& a, const Edge& b) { return a.key != b.key ? a.key < b.key : a.w < b.w; });
-  std::vector<int64_t> row_ptr(static_cast<size_t>(n) + 1, 0);
-  std::vector<int32_t> col, wt;
-  col.reserve(es.size());
-  wt.reserve(es.size());
+  for (int32_t u = 0; u < n; ++u) row_ptr[static_cast<size_t>(u) + 1] += row_ptr[u];
+  // the rows' edges as (target, weight), bucketed by row
+  std::vector<uint64_t> es(static_cast<size_t>(row_ptr[n]));
+  std::vector<int64_t> at(row_ptr.begin(), row_ptr.end() - 1);
+  for (int64_t e = 0; e < m; ++e) {
+    const int32_t u = src[e], v = dst[e], x = w[e];
+    if (u == v) continue;
+    es[static_cast<size_t>(at[u]++)] = (static_cast<uint64_t>(v) << 32) | static_cast<uint32_t>(x);
+    if (!directed) es[static_cast<size_t>(at[v]++)] = (static_cast<uint64_t>(u) << 32) | static_cast<uint32_t>(x);
+  }
+  // row by row: a repeated target keeps its smallest weight; then packed edges ascending by
+  // (weight, target).  The overflow rule above leaves every weight 32 - bits(n) bits.
+  const uint32_t bits_u = host_bits_for(static_cast<uint32_t>(n));
+  std::vector<uint32_t> edge;
+  edge.reserve(es.size());
   std::vector<int32_t> minout(static_cast<size_t>(n), DJ_INF), minin(static_cast<size_t>(n), DJ_INF);
   int32_t wmin = DJ_INF;
-  for (size_t i = 0; i < es.size(); ++i) {
-    if (i > 0 && es[i].key == es[i - 1].key) continue;
-    const int32_t u = static_cast<int32_t>(es[i].key >> 32), v = static_cast<int32_t>(es[i].key & 0xFFFFFFFFu);
-    col.push_back(v);
-    wt.push_back(es[i].w);
-    ++row_ptr[static_cast<size_t>(u) + 1];
-    minout[u] = std::min(minout[u], es[i].w);
-    minin[v] = std::min(minin[v], es[i].w);
-    wmin = std::min(wmin, es[i].w);
+  double sum_last = 0, sum_cnt = 0;  // for the mean spacing of the rows' (lightest kLightCap) weights
+  auto sort = [](auto first, auto last) {
+    if (last - first > 48) {
+      std::sort(first, last);
+      return;
+    }
+    for (auto i = first; i != last; ++i) {  // most rows are short
+      const auto x = *i;
+      auto j = i;
+      for (; j != first && x < *(j - 1); --j) *j = *(j - 1);
+      *j = x;
+    }
+  };
+  int64_t r0 = 0;
+  for (int32_t u = 0; u < n; ++u) {
+    const int64_t r1 = row_ptr[static_cast<size_t>(u) + 1];
+    sort(es.begin() + r0, es.begin() + r1);
+    const size_t p0 = edge.size();
+    for (int64_t i = r0; i < r1; ++i) {
+      if (i > r0 && (es[i] >> 32) == (es[i - 1] >> 32)) continue;
+      const uint32_t v = static_cast<uint32_t>(es[i] >> 32), x = static_cast<uint32_t>(es[i]);
+      edge.push_back((x << bits_u) | v);
+      minin[v] = std::min(minin[v], static_cast<int32_t>(x));
+    }
+    r0 = r1;
+    row_ptr[static_cast<size_t>(u) + 1] = static_cast<int64_t>(edge.size());
+    const size_t len = edge.size() - p0;
+    if (len == 0) continue;
+    sort(edge.begin() + static_cast<int64_t>(p0), edge.end());
+    minout[u] = static_cast<int32_t>(edge[p0] >> bits_u);
+    wmin = std::min(wmin, minout[u]);
+    const size_t c = std::min<size_t>(len, kLightCap);
+    sum_last += edge[p0 + c - 1] >> bits_u;
+    sum_cnt += static_cast<double>(c);
   }
-  for (int32_t u = 0; u < n; ++u) row_ptr[static_cast<size_t>(u) + 1] += row_ptr[u];
-  const int64_t nnz = static_cast<int64_t>(col.size());
+  const int64_t nnz = static_cast<int64_t>(edge.size());
 
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
@@ -280,22 +310,24 @@ extern "C" int dj_load_edges_csr(int32_t n, int64_t m, const int32_t* src, const
   g->entries = static_cast<uint64_t>(nnz);
   g->nnz = nnz;
   const size_t rp_bytes = (static_cast<size_t>(n) + 1) * sizeof(int64_t);
-  const size_t e_bytes = static_cast<size_t>(std::max<int64_t>(nnz, 1)) * sizeof(int32_t);
+  const size_t e_bytes = static_cast<size_t>(std::max<int64_t>(nnz, 1)) * sizeof(uint32_t);
   const size_t m_bytes = 2 * static_cast<size_t>(n) * sizeof(int32_t);
-  if (cudaMalloc(&g->row_ptr, rp_bytes) != cudaSuccess || cudaMalloc(&g->col, e_bytes) != cudaSuccess ||
-      cudaMalloc(&g->wt, e_bytes) != cudaSuccess || cudaMalloc(&g->minout, m_bytes) != cudaSuccess) {
+  if (cudaMalloc(&g->row_ptr, rp_bytes) != cudaSuccess || cudaMalloc(&g->edge, e_bytes) != cudaSuccess ||
+      cudaMalloc(&g->block, m_bytes) != cudaSuccess) {
     cudaGetLastError();
     dj_graph_free(g);
     return set_error(DJ_ENOMEM, "cudaMalloc of the compressed-row arrays failed");
   }
+  g->minout = static_cast<int32_t*>(g->block);
   g->minin = g->minout + n;
-  g->bytes = rp_bytes + 2 * e_bytes + m_bytes;
+  g->bytes = rp_bytes + e_bytes + m_bytes;
+  g->light_ok = wmin >= 1;
+  g->light_spacing = sum_cnt > 0 ? static_cast<float>(sum_last / sum_cnt) : 0.f;
+  while (g->light_gshift > 2 && (nnz >> (g->light_gshift - 1)) < n) --g->light_gshift;  // lanes per row: about its edges
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   cudaError_t e = cudaMemcpyAsync(g->row_ptr, row_ptr.data(), rp_bytes, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && nnz > 0)
-    e = cudaMemcpyAsync(g->col, col.data(), static_cast<size_t>(nnz) * 4, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && nnz > 0)
-    e = cudaMemcpyAsync(g->wt, wt.data(), static_cast<size_t>(nnz) * 4, cudaMemcpyHostToDevice, st);
+    e = cudaMemcpyAsync(g->edge, edge.data(), static_cast<size_t>(nnz) * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(g->minout, minout.data(), static_cast<size_t>(n) * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
@@ -345,8 +377,7 @@ int launch_csr(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, 
   cudaMemsetAsync(ws, 0, ctl_bytes, st);
   CsrParams p;
   p.row_ptr = g->row_ptr;
-  p.col = g->col;
-  p.wt = g->wt;
+  p.edge = g->edge;
   p.minout = g->minout;
   p.minin = g->minin;
   p.dist_out = dist;

@@ -16,6 +16,7 @@ struct dj_graph {
   int32_t device = 0;
   int32_t wmin = DJ_INF;  // smallest finite off-diagonal weight
   int32_t wmax = 0;       // largest finite off-diagonal weight
+  void* block = nullptr;      // the allocation the next pointers (and the index) lie in
   int32_t* W = nullptr;       // n x pitch, row-major
   int32_t* minout = nullptr;  // n row minima (then the n column minima, same allocation)
   int32_t* minin = nullptr;   // n column minima
@@ -31,13 +32,20 @@ struct dj_graph {
   // matrix is symmetric (undirected graph)
   uint2* outlist = nullptr;
   uint32_t* outrest = nullptr;
+  // the light-edge index (dj_light.cuh): kLightStats words of statistics, the rows' hmin (light_pad(n)
+  // words), then n x kLightCap packed edges; nullptr if the graph keeps none
+  uint32_t* light = nullptr;
+  uint64_t light_bytes = 0;
+  bool light_ok = false;      // solves take the light engine unless the caller chose another
+  float light_deg = 0.f;      // dense: edges per row
+  float light_spacing = 0.f;  // compressed rows: mean spacing of a row's lightest weights
+  int32_t light_gshift = 5;   // compressed rows: log2 of the lanes that share a row
   uint64_t bytes = 0;
   uint64_t entries = 0;       // finite off-diagonal matrix entries (directed edges)
   int32_t format = DJ_FORMAT_DENSE;  // DJ_FORMAT_CSR: no matrix, the arrays below
   int64_t nnz = 0;
   int64_t* row_ptr = nullptr;  // n + 1 edge offsets
-  int32_t* col = nullptr;      // nnz targets, sorted within a row
-  int32_t* wt = nullptr;       // nnz weights
+  uint32_t* edge = nullptr;    // nnz packed edges (weight << bits(n)) | target, ascending within a row
   // set by dj_graph_upload: the next solve waits for the kernels before it on its stream
   // before it reads the matrix (solves otherwise read the graph while the previous kernel ends)
   int32_t upload_pending = 0;
@@ -50,6 +58,24 @@ struct dj_graph {
 namespace dj {
 
 constexpr int kInLists = 4;  // in-edges listed per column for the dynamic IN bound
+
+// The light-edge index (dj_light.cuh).
+constexpr int kLightCap = 64;    // edges listed per row
+constexpr int kLightStats = 64;  // leading words: [0] ~(smallest hmin), [1] rows relaxed whole by the trial solve,
+                                 // [2..3] sum of the rows' largest listed weights, [4..5] of their listed edges,
+                                 // [6] most edges listed in a row, [8..11] ~(finite min), finite max, finite entries
+                                 // (at load), [12..14] the edge list's check (k_scatter)
+inline
+#ifdef __CUDACC__
+    __host__ __device__
+#endif
+    int32_t
+    light_pad(int32_t n) {
+  return (n + 63) / 64 * 64;
+}
+inline size_t light_index_bytes(int32_t n) {
+  return (static_cast<size_t>(kLightStats) + light_pad(n) + static_cast<size_t>(n) * kLightCap) * 4;
+}
 
 // Descriptor of one solve for the cluster engine (64 bytes).
 struct SolveDesc {
@@ -229,6 +255,9 @@ int lockstep_tiles(dj_graph* g, const LockstepPlan& plan, cudaStream_t st, const
 // allow_in = 0 keeps to the OUT bound (DJ_SETTLE_OUT).
 int run_lockstep(const dj_graph* g, const LockstepPlan& plan, const int32_t* tiled, const LsSource* src_dev,
                  uint8_t* ws, uint32_t* words, int64_t timeout_ns, int allow_in, cudaStream_t st);
+// One solve over every SM (a graph with an index, or in compressed rows).
+int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
+                      uint32_t* heavy, cudaStream_t st);
 int cluster_max_clusters(int32_t max_pitch, const ClusterLaunch& cl, int* clusters);
 bool cluster_config_ok(int32_t max_pitch, const ClusterLaunch& cl);
 

@@ -11,10 +11,12 @@
 // padded to a multiple of 32 int32 (128 bytes) with INF, the device analogue
 // of the paper's INF padding of Section III-B.
 #include <algorithm>
+#include <cstring>
 #include <string>
 
 #include "dj_common.cuh"
 #include "dj_internal.h"
+#include "dj_light.cuh"
 
 namespace dj {
 
@@ -124,102 +126,200 @@ __global__ void k_rowmin(const int32_t* __restrict__ W, int64_t pitch, int32_t n
   }
 }
 
-// Upload from pinned host memory (device-accessible through unified addressing):
-// each warp copies one row at a time from `src` (row stride ld) into the
-// graph's row and takes the row's minimum finite off-diagonal entry on the
-// way, so the matrix crosses the host link once and is not read again for
-// its row minima.  With `vec` (ld a multiple of 4, src 16-byte aligned) the
-// row moves in 16-byte pieces, four in flight per lane, and its last n mod 4
-// entries one by one.  Padding columns are left as they are (INF).  With
-// `ties` (a symmetric matrix, whose column v is row v and whose minin is
-// minout) the warp also lists column u's tie sources as k_tiesrc would: the
-// entries of row u other than the diagonal equal to its minimum, up to cap of
-// them, and their count.
+// One warp per row: the row's light-edge list (dj_light.cuh) and, from it, what the other engines
+// keep of a row: minout[u], with `ties` (a symmetric matrix, whose column u is row u and whose minin is
+// minout) column u's tie sources as k_tiesrc lists them, and the statistics of the index.
 constexpr int kTieSourceCap = 32;
-__global__ void k_upload_rows(const int32_t* __restrict__ src, int64_t ld, int32_t* __restrict__ W, int64_t pitch,
-                              int32_t n, int32_t* __restrict__ minout, int vec, int ties,
-                              int32_t* __restrict__ tsrc, int32_t* __restrict__ tcnt, int32_t cap) {
+struct LightOut {
+  uint32_t* light;  // the index (stats, hmin, edges)
+  int32_t* minout;
+  int32_t* tsrc;  // nullptr: not symmetric
+  int32_t* tcnt;
+  int32_t cap;
+  uint32_t bits_u;
+  int32_t n;
+  float deg;      // edges per row and largest weight if known (deg 0: not; wmax 0: word 14 of the index),
+  uint32_t wmax;  // for each warp's first threshold
+};
+struct LightSums {
+  unsigned long long last = 0, cnt = 0;
+  uint32_t hmin = 0xFFFFFFFFu, most = 0;
+};
+
+// The first threshold of light_select, in the middle of its window of counts: as if the weights were
+// uniform up to the largest (of the edge list: word 14), with deg edges per row.  A warp has only a few
+// rows, so a bad guess costs scans: 8192 rows of 4096 edges took 265 us from 0 and take 98 us, against
+// 125 us for the row minima and tie sources this pass replaces.
+__device__ __forceinline__ uint32_t first_threshold(const LightOut& o) {
+  const float want = 2.25f * kLightCap, wmax = static_cast<float>(o.wmax ? o.wmax : o.light[14]);
+  return static_cast<uint32_t>(fminf(2.0e9f, o.deg <= want ? (o.deg > 0.f ? wmax : 0.f) : wmax * want / o.deg));
+}
+
+template <class Scan>
+__device__ __forceinline__ void light_row(const LightOut& o, const Scan& scan, uint32_t u, uint32_t* buf,
+                                          uint32_t& thr, LightSums& sums) {
+  const int lane = threadIdx.x & 31;
+  uint32_t* hmin = o.light + kLightStats;
+  uint32_t* edge = hmin + light_pad(o.n) + static_cast<size_t>(u) * kLightCap;
+  const LightRow r = light_select(scan, u, o.bits_u, buf, edge, thr);
+  if (lane == 0) {
+    o.minout[u] = static_cast<int32_t>(r.first);
+    if (o.tsrc) o.minout[o.n + u] = static_cast<int32_t>(r.first);  // minin: the same
+    hmin[u] = r.hmin;
+    // a list that misses some edges of the smallest weight counts as too many to list
+    if (o.tsrc) o.tcnt[u] = r.first >= kInf ? 0 : static_cast<int32_t>(r.hmin > r.first ? r.ties : max(r.ties, o.cap + 1u));
+  }
+  if (o.tsrc && lane < o.cap && static_cast<uint32_t>(lane) < r.ties)
+    o.tsrc[static_cast<int64_t>(u) * o.cap + lane] = static_cast<int32_t>(edge[lane] & ((1u << o.bits_u) - 1u));
+  sums.last += r.last;
+  sums.cnt += r.cnt;
+  sums.hmin = min(sums.hmin, r.hmin);
+  sums.most = max(sums.most, r.cnt);
+}
+
+__device__ __forceinline__ void light_sums_out(const LightOut& o, const LightSums& s) {
+  if ((threadIdx.x & 31) != 0) return;
+  if (s.hmin < kInf) atomicMax(o.light, ~s.hmin);
+  atomicAdd(reinterpret_cast<unsigned long long*>(o.light + 2), s.last);
+  atomicAdd(reinterpret_cast<unsigned long long*>(o.light + 4), s.cnt);
+  atomicMax(o.light + 6, s.most);
+}
+
+// The rows of the resident matrix; with `stats` also the finite min / max and the number of finite
+// entries (the index's words 8..11).
+__global__ void __launch_bounds__(256) k_light_rows(const int32_t* __restrict__ W, int64_t pitch, const LightOut o,
+                                                    bool stats) {
+  __shared__ uint32_t s_buf[8][kLightBuf];
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-  for (int64_t u = warp; u < n; u += nwarps) {
-    const int32_t* s = src + u * ld;
-    int32_t* d = W + u * pitch;
-    uint32_t mn = kInf;
-    auto take = [&](int64_t c, int32_t x) {
-      if (c != u && static_cast<uint32_t>(x) < kInf) mn = min(mn, static_cast<uint32_t>(x));
-    };
-    int64_t done = 0;
-    if (vec) {
-      const int64_t nq = n / 4;
-      const int4* s4 = reinterpret_cast<const int4*>(s);
-      int4* d4 = reinterpret_cast<int4*>(d);
+  const int64_t nq = pitch / 4;
+  uint32_t thr = first_threshold(o), gmin = kInf, gmax = 0;
+  unsigned long long cnt = 0;
+  LightSums sums;
+  for (int64_t u = warp; u < o.n; u += nwarps) {
+    const int32_t* row = W + u * pitch;
+    uint32_t mx = 0, c = 0;
+    auto scan = [&](const auto& f, int pass) {
       for (int64_t q0 = 0; q0 < nq; q0 += 4 * 32) {
         int4 x[4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
           const int64_t q = q0 + 32 * r + lane;
-          x[r] = q < nq ? s4[q] : make_int4(0, 0, 0, 0);
+          x[r] = q < nq ? __ldg(reinterpret_cast<const int4*>(row) + q)
+                        : make_int4(int(kInf), int(kInf), int(kInf), int(kInf));
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const uint32_t c0 = static_cast<uint32_t>(4 * (q0 + 32 * r + lane));
+          if (pass == 0 && stats) {
+            const uint32_t w4[4] = {static_cast<uint32_t>(x[r].x), static_cast<uint32_t>(x[r].y),
+                                    static_cast<uint32_t>(x[r].z), static_cast<uint32_t>(x[r].w)};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (w4[k] < kInf && c0 + k != u) {
+                mx = max(mx, w4[k]);
+                ++c;
+              }
+          }
+          f(c0, x[r]);
+        }
+      }
+    };
+    light_row(o, scan, static_cast<uint32_t>(u), s_buf[threadIdx.x >> 5], thr, sums);
+    if (lane == 0) gmin = min(gmin, static_cast<uint32_t>(o.minout[u]));
+    gmax = max(gmax, mx);
+    cnt += c;
+  }
+  light_sums_out(o, sums);
+  if (stats) {
+    for (int k = 16; k > 0; k >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, k);
+    gmax = __reduce_max_sync(0xffffffffu, gmax);
+    if (lane == 0) {
+      atomicMax(o.light + 8, ~gmin);
+      atomicMax(o.light + 9, gmax);
+      atomicAdd(reinterpret_cast<unsigned long long*>(o.light + 10), cnt);
+    }
+  }
+}
+
+// Upload from pinned host memory (device-accessible through unified addressing): each warp copies one
+// row at a time from `src` (row stride ld) into the graph's row and selects its light edges on the
+// way (k_light_rows), so the matrix crosses the host link once and is not read from HBM again.  With
+// `vec` (ld a multiple of 4, src 16-byte aligned) the row moves in 16-byte pieces, four in flight per
+// lane; otherwise it is copied entry by entry and selected from the copy.  Padding columns are left
+// as they are (INF).
+__global__ void __launch_bounds__(256) k_upload_rows(const int32_t* __restrict__ src, int64_t ld,
+                                                     int32_t* __restrict__ W, int64_t pitch, const LightOut o,
+                                                     int vec) {
+  __shared__ uint32_t s_buf[8][kLightBuf];
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
+  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
+  const int4 none = make_int4(int(kInf), int(kInf), int(kInf), int(kInf));
+  uint32_t thr = first_threshold(o);
+  LightSums sums;
+  for (int64_t u = warp; u < o.n; u += nwarps) {
+    const int32_t* s = src + u * ld;
+    int32_t* d = W + u * pitch;
+    if (!vec) {
+      for (int64_t c = lane; c < o.n; c += 32) d[c] = s[c];
+      __syncwarp();  // the row as every lane wrote it
+    }
+    auto scan = [&](const auto& f, int pass) {
+      const bool copy = vec && pass == 0;
+      const int4* from = reinterpret_cast<const int4*>(copy ? s : d);
+      const int64_t nq = copy ? o.n / 4 : pitch / 4;
+      for (int64_t q0 = 0; q0 < nq; q0 += 4 * 32) {
+        int4 x[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int64_t q = q0 + 32 * r + lane;
+          x[r] = q < nq ? from[q] : none;
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
           const int64_t q = q0 + 32 * r + lane;
-          if (q < nq) {
-            d4[q] = x[r];
-            take(4 * q, x[r].x);
-            take(4 * q + 1, x[r].y);
-            take(4 * q + 2, x[r].z);
-            take(4 * q + 3, x[r].w);
-          }
+          if (copy && q < nq) reinterpret_cast<int4*>(d)[q] = x[r];
+          f(static_cast<uint32_t>(4 * q), x[r]);
         }
       }
-      done = 4 * nq;
-    }
-    for (int64_t c = done + lane; c < n; c += 32) {
-      const int32_t x = s[c];
-      d[c] = x;
-      take(c, x);
-    }
-    mn = warp_min_u32(mn);
-    if (lane == 0) minout[u] = static_cast<int32_t>(mn);
-    if (ties) {
-      __syncwarp();  // the row as every lane wrote it (now in L2)
-      int32_t cnt = 0;
-      const uint32_t lt = (1u << lane) - 1u;
-      auto one = [&](int64_t c, int32_t x) {  // every lane calls it together
-        const bool hit = c < n && c != u && static_cast<uint32_t>(x) == mn;
-        const uint32_t bal = __ballot_sync(0xffffffffu, hit);
-        if (hit) {
-          const int32_t pos = cnt + __popc(bal & lt);
-          if (pos < cap) tsrc[u * cap + pos] = static_cast<int32_t>(c);
+      if (copy) {
+        const int64_t c0 = 4 * nq;  // the last n mod 4 entries
+        int4 x = none;
+        if (lane == 0) {
+          if (c0 < o.n) d[c0] = x.x = s[c0];
+          if (c0 + 1 < o.n) d[c0 + 1] = x.y = s[c0 + 1];
+          if (c0 + 2 < o.n) d[c0 + 2] = x.z = s[c0 + 2];
         }
-        cnt += __popc(bal);
-      };
-      if (mn < kInf) {
-        // the row's (device, pitch-aligned) 16-byte pieces, 4 per lane in flight; the list order
-        // is fixed by the loop but immaterial to its users
-        const int64_t nq = (n + 3) / 4;  // pieces covering the row (the last may hold padding: INF)
-        const int4* d4 = reinterpret_cast<const int4*>(d);
-        for (int64_t q0 = 0; q0 < nq; q0 += 4 * 32) {
-          int4 x[4];
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const int64_t q = q0 + 32 * r + lane;
-            x[r] = q < nq ? d4[q] : make_int4(int(kInf), int(kInf), int(kInf), int(kInf));
-          }
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const int64_t c = 4 * (q0 + 32 * r + lane);
-            one(c, x[r].x);
-            one(c + 1, x[r].y);
-            one(c + 2, x[r].z);
-            one(c + 3, x[r].w);
-          }
-        }
+        if (c0 < o.n) f(static_cast<uint32_t>(c0 + 4 * lane), x);
+        __syncwarp();  // later scans read the row as every lane wrote it
       }
-      if (lane == 0) tcnt[u] = cnt;
-    }
+    };
+    light_row(o, scan, static_cast<uint32_t>(u), s_buf[threadIdx.x >> 5], thr, sums);
   }
+  light_sums_out(o, sums);
+}
+
+// The rows' kInLists smallest weights with their columns (what k_outlist gives), from the index: a
+// thread per row.  A row whose index list is shorter than that and misses edges lists nothing, which
+// keeps the static minimum as its bound.
+__global__ void k_index_lists(const uint32_t* __restrict__ light, int32_t n, uint32_t bits_u,
+                              uint2* __restrict__ outlist, uint32_t* __restrict__ outrest) {
+  const int64_t u = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (u >= n) return;
+  const uint32_t* hmin = light + kLightStats;
+  const uint32_t* edge = hmin + light_pad(n) + u * kLightCap;
+  uint32_t e[kInLists + 1];
+#pragma unroll
+  for (int i = 0; i <= kInLists; ++i) e[i] = edge[i];
+  const bool missing = hmin[u] < kInf;
+  const bool use = !missing || e[kInLists - 1] != kNoEdge;
+#pragma unroll
+  for (int i = 0; i < kInLists; ++i)
+    outlist[u * kInLists + i] =
+        use && e[i] != kNoEdge ? make_uint2(e[i] >> bits_u, e[i] & ((1u << bits_u) - 1u)) : make_uint2(kInf, 0xFFFFFFFFu);
+  outrest[u] = use && (e[kInLists] != kNoEdge || missing) ? e[kInLists - 1] >> bits_u : kInf;
 }
 
 // minin[v] = min finite W[u][v], u != v.  A block covers 256 columns x kColRows
@@ -385,63 +485,78 @@ static int grid_for(int64_t work, int threads = 256) {
   return static_cast<int>(std::min<int64_t>(std::max<int64_t>(b, 1), 152 * 32));
 }
 
+// One allocation for the matrix, the minima, the tie sources and the light-edge index (a cudaMalloc
+// each cost as much as building a small graph).
 static int alloc_graph(int32_t n, int directed, dj_graph** out) {
   auto* g = new dj_graph();
   g->n = n;
   g->pitch = (n + 31) / 32 * 32;
   g->directed = directed ? 1 : 0;
   cudaGetDevice(&g->device);
+  auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
   const size_t mbytes = static_cast<size_t>(n) * g->pitch * sizeof(int32_t);
-  cudaError_t e = cudaMalloc(&g->W, mbytes);
-  if (e != cudaSuccess) {
+  const size_t min_bytes = 2 * static_cast<size_t>(n) * sizeof(int32_t);
+  const size_t tie_bytes = static_cast<size_t>(n) * (kTieSourceCap + 1) * sizeof(int32_t);
+  const size_t base = up(mbytes) + up(min_bytes) + up(tie_bytes);
+  g->light_bytes = light_index_bytes(n);
+  if (cudaMalloc(&g->block, base + g->light_bytes) != cudaSuccess) {
     cudaGetLastError();
-    delete g;
-    return set_error(DJ_ENOMEM, "cudaMalloc of the adjacency matrix failed (" + std::to_string(mbytes) + " bytes)");
+    g->light_bytes = 0;  // no room for the index: the graph is solved from the matrix alone
+    if (cudaMalloc(&g->block, base) != cudaSuccess) {
+      cudaGetLastError();
+      delete g;
+      return set_error(DJ_ENOMEM, "cudaMalloc of the adjacency matrix failed (" + std::to_string(mbytes) + " bytes)");
+    }
   }
-  e = cudaMalloc(&g->minout, 2 * static_cast<size_t>(n) * sizeof(int32_t));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(g->W);
-    delete g;
-    return set_error(DJ_ENOMEM, "cudaMalloc of the row / column minima failed");
-  }
+  auto* p = static_cast<uint8_t*>(g->block);
+  g->W = reinterpret_cast<int32_t*>(p);
+  g->minout = reinterpret_cast<int32_t*>(p + up(mbytes));
   g->minin = g->minout + n;
+  g->tsrc = reinterpret_cast<int32_t*>(p + up(mbytes) + up(min_bytes));
   g->tcap = kTieSourceCap;
-  e = cudaMalloc(&g->tsrc, static_cast<size_t>(n) * (kTieSourceCap + 1) * sizeof(int32_t));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(g->W);
-    cudaFree(g->minout);
-    delete g;
-    return set_error(DJ_ENOMEM, "cudaMalloc of the tie sources failed");
-  }
   g->tcnt = g->tsrc + static_cast<size_t>(n) * kTieSourceCap;
-  g->bytes = mbytes + static_cast<size_t>(n) * (kTieSourceCap + 3) * sizeof(int32_t);
+  if (g->light_bytes) g->light = reinterpret_cast<uint32_t*>(p + base);
+  g->bytes = mbytes + min_bytes + tie_bytes + g->light_bytes;
   *out = g;
   return DJ_OK;
 }
 
 static void launch_inlists(dj_graph* g, cudaStream_t st) {
+  if (g->light) {
+    k_index_lists<<<static_cast<unsigned>((g->n + 255) / 256), 256, 0, st>>>(
+        g->light, g->n, host_bits_for(static_cast<uint32_t>(g->n)), g->outlist, g->outrest);
+    if (g->outlist == g->inlist) return;  // symmetric: a node's in-edges are its out-edges
+    k_inlist<<<static_cast<unsigned>((g->n + 127) / 128), 128, 0, st>>>(g->W, g->pitch, g->n, g->inlist, g->inrest);
+    return;
+  }
   k_inlist<<<static_cast<unsigned>((g->n + 127) / 128), 128, 0, st>>>(g->W, g->pitch, g->n, g->inlist, g->inrest);
   if (g->outlist != g->inlist)
     k_outlist<<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(g->W, g->pitch, g->n, g->outlist, g->outrest);
 }
 
-// Column minima (a copy of the row minima for undirected graphs, else
-// k_colmin), then the columns' tie sources (and in-lists, where the graph keeps them).
-// Row minima (unless `have_rows`: the upload kernel took them, and on a symmetric matrix the tie
-// sources too), column minima, tie sources and, for graphs that keep them, the in- and out-lists.
+static LightOut light_out(const dj_graph* g) {
+  return LightOut{g->light, g->minout, g->directed ? nullptr : g->tsrc, g->tcnt, g->tcap,
+                  host_bits_for(static_cast<uint32_t>(g->n)), g->n, g->light_deg,
+                  static_cast<uint32_t>(g->wmax)};
+}
+
+// Row minima (with the index, on a symmetric matrix the tie sources too; unless `have_rows`: the upload kernel took
+// them), column minima, tie sources and, for graphs that keep them, the in- and out-lists.
 static void launch_minima(dj_graph* g, uint32_t* stats, cudaStream_t st, bool have_rows = false) {
-  if (!have_rows)
+  const bool rows_done = have_rows || g->light;
+  if (!have_rows && g->light) {
+    k_light_rows<<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(g->W, g->pitch, light_out(g), stats != nullptr);
+  } else if (!have_rows) {
     k_rowmin<<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(g->W, g->pitch, g->n, g->minout, stats);
-  if (!g->directed) {
-    cudaMemcpyAsync(g->minin, g->minout, static_cast<size_t>(g->n) * sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
-  } else {
-    k_fill_i32<<<grid_for(g->n), 256, 0, st>>>(g->minin, g->n, static_cast<int32_t>(kInf));
-    dim3 grid(static_cast<unsigned>((g->n + 255) / 256), static_cast<unsigned>((g->n + kColRows - 1) / kColRows));
-    k_colmin<<<grid, 256, 0, st>>>(g->W, g->pitch, g->n, g->minin);
   }
-  if (!(have_rows && !g->directed)) {
+  if (!(rows_done && !g->directed)) {  // symmetric: the rows gave minin and the tie sources
+    if (!g->directed) {
+      cudaMemcpyAsync(g->minin, g->minout, static_cast<size_t>(g->n) * sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
+    } else {
+      k_fill_i32<<<grid_for(g->n), 256, 0, st>>>(g->minin, g->n, static_cast<int32_t>(kInf));
+      dim3 grid(static_cast<unsigned>((g->n + 255) / 256), static_cast<unsigned>((g->n + kColRows - 1) / kColRows));
+      k_colmin<<<grid, 256, 0, st>>>(g->W, g->pitch, g->n, g->minin);
+    }
     cudaMemsetAsync(g->tcnt, 0, static_cast<size_t>(g->n) * sizeof(int32_t), st);
     dim3 tgrid(static_cast<unsigned>((g->n + 255) / 256), static_cast<unsigned>((g->n + kColRows - 1) / kColRows));
     k_tiesrc<<<tgrid, 256, 0, st>>>(g->W, g->pitch, g->n, g->minin, g->tsrc, g->tcnt, g->tcap);
@@ -449,24 +564,46 @@ static void launch_minima(dj_graph* g, uint32_t* stats, cudaStream_t st, bool ha
   if (g->inlist) launch_inlists(g, st);
 }
 
-// Row and column minima + global weight range, then the overflow rule (n-1) * wmax < INT32_MAX.
-static int finish_graph(dj_graph* g, cudaStream_t st) {
-  uint32_t* stats = nullptr;
-  cudaError_t e = cudaMallocAsync(&stats, 4 * sizeof(uint32_t), st);
-  if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync(stats)");
-  uint32_t init[4] = {kInf, 0, 0, 0};
-  cudaMemcpyAsync(stats, init, sizeof(init), cudaMemcpyHostToDevice, st);
+// Row and column minima, index, global weight range, then the overflow rule (n-1) * wmax < INT32_MAX.
+// The index's leading words are zero before, but for the edge list's check (words 12..14), whose
+// verdict *list gets (nullptr: there was no list).
+//
+// Whether solves take the light engine is judged here: at once if every row's list is complete, else
+// if a trial solve relaxes at most a sixteenth of the rows whole (graphs of nearly equal weights, or
+// whose distances are long against what the lists reach, need far more of the matrix, and the other
+// engines stream it better).  The trial is one more kernel in front of the only wait.
+static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
+  uint32_t* stats = g->light ? g->light + 8 : nullptr;
+  uint32_t idx[16] = {0};
+  cudaError_t e = cudaSuccess;
+  if (!g->light) {
+    e = cudaMallocAsync(&stats, 4 * sizeof(uint32_t), st);
+    if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync(stats)");
+    uint32_t init[4] = {kInf, 0, 0, 0};
+    cudaMemcpyAsync(stats, init, sizeof(init), cudaMemcpyHostToDevice, st);
+  }
   launch_minima(g, stats, st);
-  uint32_t res[4];
-  cudaMemcpyAsync(res, stats, sizeof(res), cudaMemcpyDeviceToHost, st);
-  cudaFreeAsync(stats, st);
+  bool tried = false;
+  if (g->light) {
+    dj_solve_opts o;
+    dj_solve_opts_init(&o);
+    tried = launch_light_grid(g, g->n / 2, nullptr, nullptr, o, g->light + 1, st) == DJ_OK;
+    clear_error();  // it cannot run here: the other engines
+    cudaMemcpyAsync(idx, g->light, sizeof(idx), cudaMemcpyDeviceToHost, st);
+  } else {
+    cudaMemcpyAsync(idx + 8, stats, 4 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
+    cudaFreeAsync(stats, st);
+  }
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_error(e, "building the row minima");
-  g->wmin = static_cast<int32_t>(res[0]);
-  g->wmax = static_cast<int32_t>(res[1]);
-  g->entries = static_cast<uint64_t>(res[2]) | (static_cast<uint64_t>(res[3]) << 32);
+  if (list && g->light) std::memcpy(list, idx + 12, 3 * sizeof(uint32_t));
+  g->wmin = static_cast<int32_t>(g->light ? ~idx[8] : idx[8]);
+  g->wmax = static_cast<int32_t>(idx[9]);
+  g->entries = static_cast<uint64_t>(idx[10]) | (static_cast<uint64_t>(idx[11]) << 32);
+  g->light_deg = static_cast<float>(static_cast<double>(g->entries) / g->n);
   if (g->n > 1 && static_cast<int64_t>(g->n - 1) * g->wmax >= static_cast<int64_t>(DJ_INF))
     return set_error(DJ_EOVERFLOW, "(n-1) * max weight >= INT32_MAX: path lengths could overflow int32");
+  g->light_ok = tried && g->wmin >= 1 && (~idx[0] >= kInf || idx[1] <= static_cast<uint32_t>(g->n) / 16);
   // graphs that are not dense keep in-lists for the grid engine's dynamic IN bound
   const uint64_t nn = static_cast<uint64_t>(g->n) * static_cast<uint64_t>(g->n);
   if (g->entries * 32 < nn && g->wmin >= 1 && !g->inlist) {
@@ -528,6 +665,7 @@ extern "C" int dj_load_edges(int32_t n, int64_t m, const int32_t* src, const int
   DevCtx* ctx = nullptr;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   dj_graph* g = nullptr;
+  uint32_t res[3] = {0, 0, 0};
   int rc = get_ctx(&ctx);
   if (rc == DJ_OK) rc = alloc_graph(n, directed, &g);
   if (rc != DJ_OK) {
@@ -535,16 +673,20 @@ extern "C" int dj_load_edges(int32_t n, int64_t m, const int32_t* src, const int
     if (int lrc = list_status(n, m, src, dst, w)) return lrc;
     return set_error(rc, why);
   }
+  // the list's check words lie in the index (read with its statistics), or without one in the tie
+  // sources' place, which is filled later
+  uint32_t* check = g->light ? g->light + 12 : reinterpret_cast<uint32_t*>(g->tsrc);
+  if (g->light) cudaMemsetAsync(g->light, 0, kLightStats * sizeof(uint32_t), st);
+  g->light_deg = static_cast<float>(static_cast<double>(directed ? m : 2 * m) / n);
   k_fill<<<grid_for(static_cast<int64_t>(n) * g->pitch / 4), 256, 0, st>>>(g->W, g->pitch, n);
   if (m > 0) {
-    // the check words lie in the tie sources' place, which is filled later
-    uint32_t* check = reinterpret_cast<uint32_t*>(g->tsrc);
-    cudaError_t e = cudaMemsetAsync(check, 0, 16, st);
+    cudaError_t e = cudaSuccess;
+    if (!g->light) e = cudaMemsetAsync(check, 0, 16, st);
     if (e == cudaSuccess && ctx->pageable) {
       // the device reads the caller's arrays over the host link itself (coherent host memory): one pass,
-      // no staging copies, no host loop.  Loading 67 M edges (805 MB) into n = 16384: 5.6-6.1 ms, against
-      // 86 ms with a host check and pageable copies, most of it the host's two walks over the list;
-      // 2.5 M edges into n = 4099: 0.60 against 3.67 ms; 1491 edges: 0.33 either way.
+      // no staging copies, no host loop, no wait of its own.  Loading 67 M edges (805 MB) into n = 16384:
+      // 5.4 ms, against 86 ms with a host check and pageable copies, most of it the host's two walks over
+      // the list; 2.5 M edges into n = 4099: 0.45 against 3.6 ms; 1491 edges into n = 100: 0.07 against 0.31.
       k_scatter<<<grid_for((m + kScatterEdges - 1) / kScatterEdges), 256, 0, st>>>(g->W, g->pitch, n, src, dst, w, m, 0,
                                                                                    directed, check);
     } else if (e == cudaSuccess) {
@@ -563,19 +705,23 @@ extern "C" int dj_load_edges(int32_t n, int64_t m, const int32_t* src, const int
       }
       if (stage) cudaFreeAsync(stage, st);
     }
-    uint32_t res[4] = {0, 0, 0, 0};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(res, check, sizeof(res), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the edge arrays are the caller's again
-    if (e != cudaSuccess) {
-      rc = cuda_error(e, "scattering edges");
-    } else if (const uint64_t bad = static_cast<uint64_t>(res[0]) | (static_cast<uint64_t>(res[1]) << 32)) {
-      rc = edge_status(static_cast<int64_t>(~bad), n, src, dst, w);
-      if (rc == DJ_OK) rc = set_error(DJ_EINVAL, "the edge list changed while it was read");
-    } else {
-      rc = weight_status(n, res[2]);
+    if (e == cudaSuccess && !g->light) {
+      e = cudaMemcpyAsync(res, check, 3 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
+    if (e != cudaSuccess) rc = cuda_error(e, "scattering edges");
   }
-  if (rc == DJ_OK) rc = finish_graph(g, st);
+  // a bad list's first bad edge is reported before anything the built matrix shows
+  const int frc = rc == DJ_OK ? finish_graph(g, st, res) : rc;  // the edge arrays are the caller's again
+  const std::string fwhy = dj_last_error();
+  if (const uint64_t bad = static_cast<uint64_t>(res[0]) | (static_cast<uint64_t>(res[1]) << 32)) {
+    rc = edge_status(static_cast<int64_t>(~bad), n, src, dst, w);
+    if (rc == DJ_OK) rc = set_error(DJ_EINVAL, "the edge list changed while it was read");
+  } else if (frc != DJ_OK) {
+    rc = set_error(frc, fwhy);
+  } else {
+    rc = weight_status(n, res[2]);
+  }
   if (rc != DJ_OK) {
     const std::string why = dj_last_error();
     dj_graph_free(g);
@@ -631,7 +777,8 @@ extern "C" int dj_load_dense(int32_t n, const int32_t* W, int64_t ld, int w_on_d
     dj_graph_free(g);
     return rc;
   }
-  if (int rc = finish_graph(g, st)) {
+  if (g->light) cudaMemsetAsync(g->light, 0, kLightStats * sizeof(uint32_t), st);
+  if (int rc = finish_graph(g, st, nullptr)) {
     dj_graph_free(g);
     return rc;
   }
@@ -649,12 +796,13 @@ extern "C" int dj_graph_upload(dj_graph* g, const int32_t* W, int64_t ld, uint64
   cudaPointerAttributes pa;
   const cudaError_t pe = cudaPointerGetAttributes(&pa, W);
   if (pe != cudaSuccess) cudaGetLastError();  // clear that query's own status only
-  const bool zero_copy = pe == cudaSuccess && pa.type == cudaMemoryTypeHost && pa.devicePointer != nullptr;
+  const bool zero_copy =
+      g->light && pe == cudaSuccess && pa.type == cudaMemoryTypeHost && pa.devicePointer != nullptr;
   if (zero_copy) {
     const int32_t* src = static_cast<const int32_t*>(pa.devicePointer);
     const int vec = (ld % 4 == 0 && reinterpret_cast<uintptr_t>(src) % 16 == 0) ? 1 : 0;
-    k_upload_rows<<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(
-        src, ld, g->W, g->pitch, g->n, g->minout, vec, g->directed ? 0 : 1, g->tsrc, g->tcnt, g->tcap);
+    cudaMemsetAsync(g->light, 0, 12 * sizeof(uint32_t), st);
+    k_upload_rows<<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(src, ld, g->W, g->pitch, light_out(g), vec);
     e = cudaGetLastError();
   } else if (ld == g->n && g->n == g->pitch) {  // no padding columns on either side: one contiguous copy
     e = cudaMemcpyAsync(g->W, W, static_cast<size_t>(g->n) * g->pitch * sizeof(int32_t), cudaMemcpyHostToDevice, st);
@@ -706,13 +854,10 @@ extern "C" int dj_graph_get_info(const dj_graph* g, dj_graph_info* info) {
 extern "C" int dj_graph_free(dj_graph* g) {
   clear_error();
   if (!g) return DJ_OK;
-  cudaFree(g->W);
-  cudaFree(g->minout);  // minin shares this allocation
-  cudaFree(g->tsrc);    // tcnt shares this allocation
+  cudaFree(g->block);   // dense: matrix, minima, tie sources and index; compressed rows: the minima
   cudaFree(g->inlist);  // inrest shares this allocation
   cudaFree(g->row_ptr);
-  cudaFree(g->col);
-  cudaFree(g->wt);
+  cudaFree(g->edge);
   cudaFree(g->tiled);
   delete g;
   return DJ_OK;

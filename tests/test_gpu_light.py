@@ -1,0 +1,133 @@
+"""The light engine (the default on graphs of positive weights) against the oracle: sizes at the
+edges of its lists, slices and key words, rows whose lists are complete, cut or empty, nodes nothing
+leads to, and sources for which the lists do not suffice and rows are relaxed whole."""
+import numpy as np
+import pytest
+
+import graphgen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dj():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2504_03667_gb300 import dj as _dj
+    torch.cuda.set_device(0)
+    return _dj
+
+
+def check(dj, orc, e, sources, what):
+    import torch
+    W = orc.build_matrix(e.n, e.src, e.dst, e.w, e.directed)
+    graphs = [dj.dj_load_edges(e.n, e.src, e.dst, e.w, e.directed),
+              dj.dj_load_edges_csr(e.n, e.src, e.dst, e.w, e.directed)]
+    k = len(sources)
+    D = torch.full((2 * k, e.n), -5, dtype=torch.int32, device="cuda")
+    P = torch.full((2 * k, e.n), -5, dtype=torch.int32, device="cuda")
+    for j, g in enumerate(graphs):
+        for i, s in enumerate(sources):
+            dj.dj_sssp(g, s, D[j * k + i], P[j * k + i])
+    dj.dj_sync()
+    B = torch.full((2, k, e.n), -5, dtype=torch.int32, device="cuda")
+    dj.dj_sssp_batch([graphs[0]] * k, sources, list(B[0]), list(B[1]))
+    dj.dj_sync()
+    for i, s in enumerate(sources):
+        ref = orc.dijkstra(W, s)
+        got = [("dense", D[i], P[i]), ("compressed rows", D[k + i], P[k + i]), ("batch", B[0, i], B[1, i])]
+        for form, d, p in got:
+            assert np.array_equal(d.cpu().numpy(), ref[0]), f"{what}, {form}, s={s}: dist"
+            assert np.array_equal(p.cpu().numpy(), ref[1]), f"{what}, {form}, s={s}: pred"
+    for g in graphs:
+        g.free()
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 63, 64, 65, 66, 130, 1000, 2047, 2049, 4095, 4097])
+def test_sizes(dj, orc, n):
+    for wlo, whi, deg, directed in ((1, 3, 4, True), (1, 1000, 70, False), (1, 1, 9, False), (7, 9, 200, True)):
+        m = min(n * deg, max(n * (n - 1), 1))
+        e = graphgen.random_edges(n, m, wlo, whi, seed=7 * n + deg, directed=directed)
+        check(dj, orc, e, sorted({0, n // 2, n - 1}), f"n={n} w in [{wlo}, {whi}] deg {deg}")
+
+
+def far_source(n, p, seed):
+    """A dense directed graph where nothing leads to nodes 0 and n/2, and node 1 is near n/2 but far
+    from 0: from n/2 the lists suffice, from 0 every row's unlisted edges stay below the largest
+    distance, so every row is relaxed whole."""
+    b = graphgen.bernoulli(n, p, 1, 1000, seed)
+    h = n // 2
+    src, dst, w = np.concatenate([b.src, b.dst]), np.concatenate([b.dst, b.src]), np.concatenate([b.w, b.w])
+    keep = (dst != 0) & (dst != h) & (dst != 1)
+    src = np.concatenate([src[keep], [h, 0]]).astype(np.int32)
+    dst = np.concatenate([dst[keep], [1, 1]]).astype(np.int32)
+    w = np.concatenate([w[keep], [1, 3000]]).astype(np.int32)
+    return graphgen.EdgeList(n, src, dst, w, True)
+
+
+@pytest.mark.parametrize("n", [700, 3001, 4500])
+def test_rows_relaxed_whole(dj, orc, n):
+    check(dj, orc, far_source(n, 0.4, n), [0, 1, n // 2], f"far source n={n}")
+
+
+def test_lists_cut_in_ties(dj, orc):
+    """Rows with more edges of one weight than the list or its buffer holds, next to light ones."""
+    rng = np.random.default_rng(3)
+    n = 1500
+    src = np.repeat(np.arange(n, dtype=np.int32), 600)
+    dst = rng.integers(0, n, src.shape[0]).astype(np.int32)
+    w = np.where(rng.random(src.shape[0]) < 0.02, rng.integers(1, 5, src.shape[0]), 40).astype(np.int32)
+    check(dj, orc, graphgen.EdgeList(n, src, dst, w, True), [0, 77, n - 1], "weights 1..4 and many 40s")
+    check(dj, orc, graphgen.EdgeList(n, src, dst, w, False), [5], "the same undirected")
+
+
+def test_hub_rows(dj, orc):
+    """Stars: one row much longer than the others (taken by a whole block in compressed rows)."""
+    n = 9001
+    rng = np.random.default_rng(4)
+    hub = np.zeros(n - 1, dtype=np.int32)
+    rim = np.arange(1, n, dtype=np.int32)
+    ring = np.stack([rim, np.roll(rim, 1)])
+    src = np.concatenate([hub, ring[0]])
+    dst = np.concatenate([rim, ring[1]])
+    w = np.concatenate([rng.integers(500, 900, n - 1), rng.integers(1, 4, n - 1)]).astype(np.int32)
+    check(dj, orc, graphgen.EdgeList(n, src, dst, w, False), [0, 1, 4500], "hub and ring")
+
+
+def test_upload_rebuilds_the_index(dj, orc):
+    """After an upload the same handle (and a captured solve) answers for the new matrix, from aligned
+    and unaligned pinned buffers and from pageable memory."""
+    import torch
+    for n in (203, 4500):
+        a = graphgen.bernoulli(n, 0.3, 1, 1000, 1)
+        b = graphgen.bernoulli(n, 0.05, 1, 9, 2)
+        Wb = orc.build_matrix(n, b.src, b.dst, b.w, False)
+        ref = orc.dijkstra(Wb, 5)
+        pinned = torch.from_numpy(Wb).pin_memory()
+        padded = torch.empty((n, n + 3), dtype=torch.int32).pin_memory()
+        padded[:, 1:n + 1] = pinned
+        d = torch.empty(n, dtype=torch.int32, device="cuda")
+        p = torch.empty_like(d)
+        for what, src in (("pinned", pinned), ("offset", padded[:, 1:n + 1]), ("pageable", Wb)):
+            G = dj.dj_load_edges(n, a.src, a.dst, a.w, False)
+            st = torch.cuda.Stream()
+            dj.dj_sssp(G, 5, d, p, st)
+            dj.dj_sync(st)
+            cg = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(cg, stream=st):
+                dj.dj_sssp(G, 5, d, p, st)
+            dj.dj_graph_upload(G, src, st)
+            d.fill_(-5)
+            torch.cuda.synchronize()
+            dj.dj_sssp(G, 5, d, p, st)
+            dj.dj_sync(st)
+            assert np.array_equal(d.cpu().numpy(), ref[0]) and np.array_equal(p.cpu().numpy(), ref[1]), (n, what)
+            d.fill_(-5)
+            cg.replay()
+            torch.cuda.synchronize()
+            assert np.array_equal(d.cpu().numpy(), ref[0]) and np.array_equal(p.cpu().numpy(), ref[1]), (n, what, "replay")
+            del cg
+            G.free()
