@@ -307,8 +307,8 @@ int dj_sssp_noalloc(const dj_graph* g, int32_t source, int32_t* dist, int32_t* p
 int dj_sssp_lc(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, uint64_t stream);
 
 /* ------------------------------------------------------------------ batched solves */
-/* k solves (graph[i], sources[i]) in one persistent launch: one thread-block
- * cluster per solve at a time, solves pulled from a device queue (largest n
+/* k solves (graph[i], sources[i]) in one persistent launch: one CTA (light
+ * engine) or one thread-block cluster per solve at a time, solves pulled from a device queue (largest n
  * first), graphs of different n allowed, rows shared by concurrent solves of
  * one graph reused through L2; or, for solves of one graph whose shape the
  * autotuner found faster that way, the lockstep engine
@@ -331,7 +331,11 @@ typedef struct dj_batch_opts {
   int32_t reserved[5];
 } dj_batch_opts;
 
-#define DJ_BATCH_ENGINE_AUTO 0     /* the tuned engine for this graph shape if there is one, else clusters */
+#define DJ_BATCH_ENGINE_AUTO 0     /* lockstep if the tuned entry for this graph shape says so; else, where
+                                      every graph takes the light engine (see dj_sssp), every option is at
+                                      its default and n is at most about 22000, one CTA per solve with the
+                                      light engine (reported as the cluster engine); else clusters, of the
+                                      tuned size if there is one */
 #define DJ_BATCH_ENGINE_CLUSTER 1  /* one thread-block cluster per solve, solves pulled from a device queue */
 #define DJ_BATCH_ENGINE_LOCKSTEP 2 /* every solve of ONE graph advances phase by phase together over every
                                       SM, so a row a phase needs is read once for all the sources that
@@ -364,9 +368,10 @@ int dj_batch_create(const dj_graph* const* graphs, const int32_t* sources, int32
 int dj_batch_launch(dj_batch* b, uint64_t stream);
 int dj_batch_free(dj_batch* b); /* caller synchronises first */
 
-/* Autotuner: times every supported cluster size (2, 4, 8, 16) and, for
- * solves of one graph, the lockstep engine, on the device, and keeps the
- * fastest for the batch and in the process-wide table keyed by (n bucket =
+/* Autotuner: times every supported cluster size (2, 4, 8, 16), for solves
+ * of one graph the lockstep engine, and the light engine where the batch takes
+ * it, on the device, and keeps the fastest for the batch.  The fastest of the
+ * others goes into the process-wide table keyed by (n bucket =
  * floor(log2 n), density bucket = floor(log2(n^2 / finite entries)) capped at
  * 20, SM count), which later batches of one graph consult.  When the
  * environment variable DJ_TUNE_FILE names a file, the table is read from it on

@@ -321,6 +321,10 @@ struct dj_batch {
   ClusterLaunch cl;
   ClusterPlan plan;
   bool tuned = false;
+  // light engine (one CTA per solve)
+  bool light = false;     // launches run the light engine
+  bool light_ok = false;  // it can run this batch (and the caller left the choice open)
+  LightPlan lp;
   // lockstep engine (every solve on one graph)
   dj_graph* graph = nullptr;   // the shared graph, or nullptr
   bool lockstep = false;       // launches run the lockstep engine
@@ -514,7 +518,15 @@ static int batch_descs(const dj_graph* const* graphs, const int32_t* sources, in
                        int32_t* const* pred, int plain, int device, std::vector<SolveDesc>* h, int32_t* max_n,
                        int32_t* max_pitch);
 
+// Whether every solve's graph takes the light engine and its keys fit one CTA.
+static bool light_batch_ok(const dj_graph* const* graphs, int32_t k, int32_t max_n) {
+  for (int32_t i = 0; i < k; ++i)
+    if (!graphs[i]->light_ok) return false;
+  return k > 0 && light_cta_fits(max_n);
+}
+
 // The one graph every solve of the batch uses, or nullptr.
+
 static dj_graph* shared_graph(const dj_graph* const* graphs, int32_t k) {
   if (k < 1) return nullptr;
   for (int32_t i = 1; i < k; ++i)
@@ -638,6 +650,15 @@ extern "C" int dj_batch_create(const dj_graph* const* graphs, const int32_t* sou
     if (rc != DJ_OK) clear_error();
   }
   b->lockstep = want_ls && b->ls_ok;
+  // the light engine where the caller left engine, cluster shape and bounds to the library
+  b->light_ok = o.engine == DJ_BATCH_ENGINE_AUTO && o.mode != DJ_MODE_PLAIN && o.cluster_size == 0 && o.clusters == 0 &&
+                o.threads == 0 && o.settle == DJ_SETTLE_AUTO && o.copies == DJ_COPIES_AUTO &&
+                light_batch_ok(graphs, k, max_n);
+  if (b->light_ok && plan_light(max_n, k, kJobsBatch, &b->lp) != DJ_OK) {
+    clear_error();
+    b->light_ok = false;
+  }
+  b->light = b->light_ok && !b->lockstep;
   *out = b;
   return DJ_OK;
 }
@@ -651,6 +672,7 @@ static int launch_batch(dj_batch* b, cudaStream_t st) {
     if (int rc = lockstep_tiles(b->graph, b->ls, st, &tiled)) return rc;
     return run_lockstep(b->graph, b->ls, tiled, b->ls_src, b->ls_ws, ctx->words, 0, b->ls_use_in, st);
   }
+  if (b->light) return run_light_batch(b->lp, b->descs, b->k, b->queue, false, st);
   return run_cluster(b->plan, b->descs, b->k, b->queue, st, false);
 }
 
@@ -702,6 +724,7 @@ extern "C" int dj_batch_autotune(dj_batch* b, uint64_t stream, int32_t* cluster_
   ClusterLaunch best_cl = b->cl;
   const ClusterLaunch saved = b->cl;
   b->lockstep = false;
+  b->light = false;
   for (int c : {2, 4, 8, 16}) {
     ClusterLaunch cl = saved;
     cl.cluster_size = c;
@@ -735,11 +758,24 @@ extern "C" int dj_batch_autotune(dj_batch* b, uint64_t stream, int32_t* cluster_
     }
     b->lockstep = false;
   }
+  bool best_light = false;
+  float light_ms = 0.f;
+  if (b->light_ok) {  // and the light engine, which this batch keeps if it is the fastest
+    b->light = true;
+    if (time_it(&light_ms)) {
+      best_light = light_ms < best;
+    } else {
+      clear_error();
+      cudaGetLastError();
+    }
+    b->light = false;
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   b->cl = best_cl;
   if (int rc = plan_cluster(b->max_pitch, b->cl, b->k, &b->plan)) return rc;
-  b->lockstep = best_engine == DJ_BATCH_ENGINE_LOCKSTEP;
+  b->light = best_light;
+  b->lockstep = best_engine == DJ_BATCH_ENGINE_LOCKSTEP && !best_light;
   b->tuned = true;
   if (b->graph) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -752,7 +788,7 @@ extern "C" int dj_batch_autotune(dj_batch* b, uint64_t stream, int32_t* cluster_
   }
   if (cluster_size) *cluster_size = best_engine == DJ_BATCH_ENGINE_LOCKSTEP ? 0 : best_cl.cluster_size;
   if (threads) *threads = best_engine == DJ_BATCH_ENGINE_LOCKSTEP ? 512 : best_cl.threads;
-  if (best_ms) *best_ms = best;
+  if (best_ms) *best_ms = best_light ? light_ms : best;
   if (best >= 1e29f) return set_error(DJ_EUNSUPPORTED, "no batch configuration could run");
   return DJ_OK;
 }
@@ -811,6 +847,10 @@ extern "C" int dj_sssp_batch(const dj_graph* const* graphs, const int32_t* sourc
     return rc;
   }
   clear_error();
+  LightPlan lp;
+  const bool light = !(have_tune && tv.engine == DJ_BATCH_ENGINE_LOCKSTEP) && light_batch_ok(graphs, k, max_n) &&
+                     plan_light(max_n, k, kJobsBatch, &lp) == DJ_OK;
+  clear_error();
   // stream-ordered table: allocated, filled, used and freed in stream order
   uint8_t* ws = nullptr;
   const size_t tbytes = static_cast<size_t>(k) * sizeof(SolveDesc);
@@ -824,6 +864,11 @@ extern "C" int dj_sssp_batch(const dj_graph* const* graphs, const int32_t* sourc
   ClusterLaunch cl;
   cl.cluster_size = heuristic_cluster_size(max_pitch);
   if (have_tune && tv.engine == DJ_BATCH_ENGINE_CLUSTER) cl.cluster_size = tv.cluster_size;
+  if (light) {
+    int rc = run_light_batch(lp, reinterpret_cast<SolveDesc*>(ws), k, reinterpret_cast<uint32_t*>(ws + tbytes), true, st);
+    cudaFreeAsync(ws, st);
+    return rc;
+  }
   int rc = launch_cluster(reinterpret_cast<SolveDesc*>(ws), k, max_n, max_pitch,
                           reinterpret_cast<uint32_t*>(ws + tbytes), cl, st);
   cudaFreeAsync(ws, st);

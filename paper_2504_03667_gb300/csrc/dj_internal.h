@@ -77,7 +77,7 @@ inline size_t light_index_bytes(int32_t n) {
   return (static_cast<size_t>(kLightStats) + light_pad(n) + static_cast<size_t>(n) * kLightCap) * 4;
 }
 
-// Descriptor of one solve for the cluster engine (64 bytes).
+// Descriptor of one solve for the cluster and light engines (80 bytes).
 struct SolveDesc {
   const int32_t* W;
   const int32_t* minout;
@@ -90,8 +90,10 @@ struct SolveDesc {
   uint32_t span;
   int32_t plain;
   int32_t use_in;  // settle by the IN bound too (every off-diagonal weight >= 1); minin = minout + n
+  const uint32_t* light;  // light engine: the graph's index
+  int64_t reserved;
 };
-static_assert(sizeof(SolveDesc) == 64, "descriptor layout");
+static_assert(sizeof(SolveDesc) == 80, "descriptor layout");
 
 // A workspace kept for one stream: solves enqueued on the same stream run one
 // after another, so they can share it without any per-solve allocation.
@@ -255,6 +257,21 @@ int lockstep_tiles(dj_graph* g, const LockstepPlan& plan, cudaStream_t st, const
 // allow_in = 0 keeps to the OUT bound (DJ_SETTLE_OUT).
 int run_lockstep(const dj_graph* g, const LockstepPlan& plan, const int32_t* tiled, const LsSource* src_dev,
                  uint8_t* ws, uint32_t* words, int64_t timeout_ns, int allow_in, cudaStream_t st);
+// Light engine (dj_light_cta.cu, dj_light_grid.cu): solves on the light-edge index, or on compressed rows.
+struct LightPlan {
+  void* fn = nullptr;
+  int ctas = 0, threads = 0, npad = 0;
+  size_t smem = 0;
+};
+bool light_cta_fits(int32_t n);  // one CTA's shared memory holds the keys of n nodes
+int plan_light(int32_t max_n, int32_t k, int kind, LightPlan* plan);
+// as run_cluster, run_cluster_single and run_serve_kernel; heavy: optional device word counting the rows
+// relaxed whole
+int run_light_batch(const LightPlan& plan, const SolveDesc* descs_dev, int32_t k, uint32_t* queue, bool zero_queue,
+                    cudaStream_t st);
+int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, uint32_t* heavy, bool early,
+                     cudaStream_t st);
+int run_light_serve(const LightPlan& plan, const ServeRing& r, cudaStream_t st);
 // One solve over every SM (a graph with an index, or in compressed rows).
 int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
                       uint32_t* heavy, cudaStream_t st);
