@@ -158,8 +158,10 @@ int dj_graph_free(dj_graph* g);
  * and rows that fail the test are relaxed whole from the matrix, so dist and
  * pred are Algorithm 1's on every graph.  Taken by DJ_ENGINE_AUTO in phase
  * mode when every weight is >= 1, every other option below is left at its
- * default, and a trial solve at load needed at most n/16 whole rows; also for
- * graphs in compressed rows. */
+ * default, and a trial solve at load needed next to no whole row; also for
+ * graphs in compressed rows.  After dj_graph_upload a graph's solves take the
+ * other engines (the new matrix has not been tried); solves captured into a
+ * CUDA graph before stay valid. */
 
 typedef struct dj_solve_opts {
   int32_t mode;           /* DJ_MODE_* */
@@ -333,7 +335,7 @@ typedef struct dj_batch_opts {
 
 #define DJ_BATCH_ENGINE_AUTO 0     /* lockstep if the tuned entry for this graph shape says so; else, where
                                       every graph takes the light engine (see dj_sssp), every option is at
-                                      its default and n is at most about 22000, one CTA per solve with the
+                                      its default and n is at most about 26000, one CTA per solve with the
                                       light engine (reported as the cluster engine); else clusters, of the
                                       tuned size if there is one */
 #define DJ_BATCH_ENGINE_CLUSTER 1  /* one thread-block cluster per solve, solves pulled from a device queue */

@@ -223,15 +223,31 @@ static int solve_cluster_single(const dj_graph* g, int32_t source, int32_t* dist
   return run_cluster_single(plan, d, ctx->words + 1, o.trace, o.trace ? o.trace_cap : 0, early, st);
 }
 
-// Dense graphs below this size stay with the cluster engine (and the grid engine where it was better).
-static constexpr int32_t kLightGridMinN = 2560;
-
 // The light engine's place: the caller left every choice of engine, bound and path to the library,
 // and the graph's index pays (judge_index; compressed rows of weights >= 1).
 static bool light_auto(const dj_graph* g, const dj_solve_opts& o) {
-  return g->light_ok && (g->format == DJ_FORMAT_CSR || g->n >= kLightGridMinN) && o.mode != DJ_MODE_PLAIN && o.engine == DJ_ENGINE_AUTO && o.settle == DJ_SETTLE_AUTO &&
+  return g->light_ok && o.mode != DJ_MODE_PLAIN && o.engine == DJ_ENGINE_AUTO && o.settle == DJ_SETTLE_AUTO &&
          o.cluster_size == 0 && o.threads == 0 && o.ctas_per_sm == 0 && o.unroll == 0 && o.live == 0 &&
          o.rowsplit == 0 && o.rowpush == 0 && o.trace == nullptr;
+}
+
+// Dense graphs below this size take the light engine's CTA form: back-to-back solves overlap there, one
+// per SM, and small ones are faster alone too (n = 1024: 10 us each and 43 us alone, grid form 49 and 58;
+// n = 5003, p = 0.3: 13.8 and 98, grid form 49.6 and 59; n = 16384: 35 and 255, grid form 37 and 46).
+static constexpr int32_t kLightGridMinN = 6144;
+
+static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
+                       cudaStream_t st) {
+  if (!g->light_cta || g->n >= kLightGridMinN || !light_cta_fits(g->n))
+    return launch_light_grid(g, source, dist, pred, o, nullptr, st);
+  DevCtx* ctx = nullptr;
+  if (int rc = get_ctx(&ctx)) return rc;
+  LightPlan plan;
+  if (int rc = plan_light(g->n, 1, kJobsSingle, &plan)) return rc;
+  // right after an upload the solve waits for the kernels before it before reading the graph
+  const bool early = g->upload_pending == 0;
+  const_cast<dj_graph*>(g)->upload_pending = 0;
+  return run_light_single(plan, make_desc(g, source, dist, pred, 0), ctx->words + 1, nullptr, early, st);
 }
 
 extern "C" int dj_sssp_ex(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts* opts,
@@ -248,7 +264,7 @@ extern "C" int dj_sssp_ex(const dj_graph* g, int32_t source, int32_t* dist, int3
   if (o.rowsplit < -1) return set_error(DJ_EINVAL, "rowsplit must be -1, 0 or a candidate count");
   if (o.rowpush < -1) return set_error(DJ_EINVAL, "rowpush must be -1, 0 or a candidate count");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (light_auto(g, o)) return launch_light_grid(g, source, dist, pred, o, nullptr, st);
+  if (light_auto(g, o)) return solve_light(g, source, dist, pred, o, st);
   if (g->format == DJ_FORMAT_CSR) return launch_csr(g, source, dist, pred, o, st);
   int engine = o.engine;
   if (engine == DJ_ENGINE_AUTO) engine = auto_grid(g) ? DJ_ENGINE_GRID : DJ_ENGINE_CLUSTER;
@@ -325,6 +341,7 @@ struct dj_batch {
   bool light = false;     // launches run the light engine
   bool light_ok = false;  // it can run this batch (and the caller left the choice open)
   LightPlan lp;
+  std::vector<const dj_graph*> light_graphs;  // its graphs (an upload takes a graph off the light engine)
   // lockstep engine (every solve on one graph)
   dj_graph* graph = nullptr;   // the shared graph, or nullptr
   bool lockstep = false;       // launches run the lockstep engine
@@ -521,7 +538,7 @@ static int batch_descs(const dj_graph* const* graphs, const int32_t* sources, in
 // Whether every solve's graph takes the light engine and its keys fit one CTA.
 static bool light_batch_ok(const dj_graph* const* graphs, int32_t k, int32_t max_n) {
   for (int32_t i = 0; i < k; ++i)
-    if (!graphs[i]->light_ok) return false;
+    if (!graphs[i]->light_cta) return false;
   return k > 0 && light_cta_fits(max_n);
 }
 
@@ -659,6 +676,11 @@ extern "C" int dj_batch_create(const dj_graph* const* graphs, const int32_t* sou
     b->light_ok = false;
   }
   b->light = b->light_ok && !b->lockstep;
+  if (b->light_ok) {
+    b->light_graphs.assign(graphs, graphs + k);
+    std::sort(b->light_graphs.begin(), b->light_graphs.end());
+    b->light_graphs.erase(std::unique(b->light_graphs.begin(), b->light_graphs.end()), b->light_graphs.end());
+  }
   *out = b;
   return DJ_OK;
 }
@@ -672,7 +694,11 @@ static int launch_batch(dj_batch* b, cudaStream_t st) {
     if (int rc = lockstep_tiles(b->graph, b->ls, st, &tiled)) return rc;
     return run_lockstep(b->graph, b->ls, tiled, b->ls_src, b->ls_ws, ctx->words, 0, b->ls_use_in, st);
   }
-  if (b->light) return run_light_batch(b->lp, b->descs, b->k, b->queue, false, st);
+  if (b->light) {
+    bool still = true;
+    for (const dj_graph* g : b->light_graphs) still = still && g->light_cta;
+    if (still) return run_light_batch(b->lp, b->descs, b->k, b->queue, false, st);
+  }
   return run_cluster(b->plan, b->descs, b->k, b->queue, st, false);
 }
 

@@ -37,6 +37,7 @@ struct dj_graph {
   uint32_t* light = nullptr;
   uint64_t light_bytes = 0;
   bool light_ok = false;      // solves take the light engine unless the caller chose another
+  bool light_cta = false;     // its CTA form too: hardly any source needs whole rows (slow in one CTA)
   float light_deg = 0.f;      // dense: edges per row
   float light_spacing = 0.f;  // compressed rows: mean spacing of a row's lightest weights
   int32_t light_gshift = 5;   // compressed rows: log2 of the lanes that share a row
@@ -64,7 +65,9 @@ constexpr int kLightCap = 64;    // edges listed per row
 constexpr int kLightStats = 64;  // leading words: [0] ~(smallest hmin), [1] rows relaxed whole by the trial solve,
                                  // [2..3] sum of the rows' largest listed weights, [4..5] of their listed edges,
                                  // [6] most edges listed in a row, [8..11] ~(finite min), finite max, finite entries
-                                 // (at load), [12..14] the edge list's check (k_scatter)
+                                 // (at load), [12..14] the edge list's check (k_scatter),
+                                 // [15] kLightGuess
+constexpr int kLightGuess = 15;  // a little above the trial solve's largest dist (0: unknown)
 inline
 #ifdef __CUDACC__
     __host__ __device__

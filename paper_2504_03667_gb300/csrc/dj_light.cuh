@@ -35,6 +35,9 @@ __device__ __forceinline__ uint64_t light_key(uint32_t du, uint32_t w, uint32_t 
   return (static_cast<uint64_t>(du + w) << 32) | ((weight_field(bits_u) - w) << bits_u) | u;
 }
 
+// The low word of the key that u makes from its listed edge e.
+__device__ __forceinline__ uint32_t light_tie(uint32_t e, uint32_t u, uint32_t umask) { return (~e & ~umask) | u; }
+
 // What a solve takes from the index's statistics: its phase window (c times the mean spacing of a
 // row's listed weights) and log2 of the lanes that share a row (about the longest list's length).
 __device__ __forceinline__ void light_window(const uint32_t* light, float c, uint32_t* delta, int* gshift) {
@@ -44,6 +47,13 @@ __device__ __forceinline__ void light_window(const uint32_t* light, float c, uin
   const float cnt = static_cast<float>((static_cast<uint64_t>(b.y) << 32) | b.x);
   *delta = static_cast<uint32_t>(fminf(1.0e9f, cnt > 0.f ? c * last / cnt : 0.f));
   *gshift = b.z <= 8 ? 3 : b.z <= 16 ? 4 : 5;
+}
+
+__device__ __forceinline__ uint32_t light_delta(const uint32_t* light, float c) {
+  uint32_t delta;
+  int unused;
+  light_window(light, c, &delta, &unused);
+  return delta;
 }
 
 // Per-warp selection of a row's lightest edges.  scan(f, pass) must call f(c0, x) for every group of

@@ -1,4 +1,4 @@
-// Light engine, CTA form: one CTA per solve with the keys in shared memory (n up to about 22000),
+// Light engine, CTA form: one CTA per solve with its state in shared memory (n up to about 26000),
 // for batches and small single solves on graphs whose every weight is >= 1.  The algorithm is the
 // grid form's (dj_light_grid.cu) without any communication between CTAs.
 #include <algorithm>
@@ -13,39 +13,162 @@ namespace dj {
 
 namespace {
 constexpr uint32_t kNone = 0xFFFFFFFFu;
-constexpr int kLightRows = 4;  // rows in flight per lane group
-// delta in units of the listed weights' mean spacing (narrower than the grid form's: a phase costs
-// little here)
-constexpr float kCtaDelta = 1.0f;
+// delta in units of the listed weights' mean spacing: 19 phases instead of 25 with 1, and 4 % more rows
+constexpr float kCtaDelta = 3.0f;
+constexpr int kLoads = 2;      // 16-byte loads in flight per lane (4: 395 against 298 us for the batch below)
+constexpr int kWarpRows = 64;  // a warp's waiting rows: 31 left over and 32 of the next word
 }  // namespace
 
 struct LightCtaParams {
   uint32_t* heavy;  // optional: rows relaxed whole are counted here
-  int32_t npad;     // key slots (largest graph of the launch, rounded up to 64)
+  int32_t npad;     // node slots (largest graph of the launch, rounded up to 64)
 };
 
-// Offer w's key to v in shared memory; a shorter dist makes v dirty and lowers lmin.
-__device__ __forceinline__ void light_offer(unsigned long long* keys, uint32_t* dirty, uint32_t v, uint64_t key,
-                                            uint32_t& lmin) {
-  if (key < keys[v]) {
-    const uint64_t old = atomicMin(keys + v, static_cast<unsigned long long>(key));
-    const uint32_t c = static_cast<uint32_t>(key >> 32);
-    if (c < static_cast<uint32_t>(old >> 32)) {
-      atomicOr(dirty + (v >> 5), 1u << (v & 31u));
-      lmin = min(lmin, c);
-    }
-  }
+// Shared memory of a solve (dynamic).  A word of 32 nodes has a mask of dirty ones and a lower bound on
+// their dists.
+struct LightCta {
+  uint32_t* dist;   // kNone: not reached
+  uint32_t* tie;    // low word of the key (dj_light.cuh) of the best offer, found last
+  uint32_t* dirty;
+  uint32_t* wmin;
+  uint32_t* whole;  // rows relaxed whole
+};
+
+// Shared words that other warps change meanwhile are read through this.
+__device__ __forceinline__ uint32_t word_now(const uint32_t* p) { return *const_cast<const volatile uint32_t*>(p); }
+
+// An offer of dist c to v; a shorter one makes v dirty.  32-bit shared atomics cost what a load costs
+// (2.5 cycles a warp, against 9.4 for a 64-bit compare-and-swap and 4.6 for a 64-bit load), so dists are
+// settled alone and the ties, which need them final anyway, in one pass at the end.
+__device__ __forceinline__ void light_won(const LightCta& s, uint32_t v, uint32_t c, uint32_t& lmin) {
+  atomicOr(s.dirty + (v >> 5), 1u << (v & 31u));
+  atomicMin(s.wmin + (v >> 5), c);
+  lmin = min(lmin, c);
 }
 
-template <int THREADS, class Jobs>
-__global__ void __launch_bounds__(THREADS) k_light_cta(const LightCtaParams p, const Jobs jobs) {
+// Relax (with kTies: take the ties of) the listed edges of a warp's rows: get(i) is row i, i < count, as
+// (u, dist[u]) or, where there is nothing to do, (u, kNone).  Four lanes share a row and take four edges
+// each with one 16-byte load, so a warp's load covers 16 edges of 8 rows in 8 pieces of 64 bytes, and
+// 8 kLoads rows are in flight.  Edges whose offer exceeds B are dropped; a row goes on to its next 16
+// edges only if the heaviest of these was of use.  (A lane per edge, 16 lanes per row, took three times the
+// instructions per edge; a lane per row read 32 lines with every load and was bound by the L1.)
+template <bool kTies, class Get>
+__device__ __forceinline__ void light_rows(const LightCta& s, const Get& get, int count, int most, uint32_t B,
+                                           uint32_t bits_u, const uint32_t* __restrict__ edge, uint32_t& lmin) {
+  const int lane = static_cast<int>(threadIdx.x) & 31, sub = lane & 3;
+  const uint32_t umask = (1u << bits_u) - 1u;
+  constexpr int R = kLoads;
+  for (int i0 = 0; i0 < count; i0 += 8 * R) {
+    uint32_t u[R], du[R];
+    bool on[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = i0 + 8 * r + (lane >> 2);
+      const uint2 x = get(min(i, count - 1));
+      u[r] = x.x;
+      du[r] = x.y;
+      on[r] = i < count && x.y != kNone;
+    }
+    for (int k0 = 0; k0 < most; k0 += 16) {
+      uint4 x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        x[r] = on[r] ? __ldg(reinterpret_cast<const uint4*>(edge + u[r] * kLightCap + k0) + sub)
+                     : make_uint4(kNoEdge, kNoEdge, kNoEdge, kNoEdge);
+      uint32_t more = 0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const uint32_t e[4] = {x[r].x, x[r].y, x[r].z, x[r].w};
+        uint32_t old[4];
+        bool use = false;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t c = du[r] + (e[q] >> bits_u), v = e[q] & umask;
+          use = e[q] != kNoEdge && c <= B;
+          if (kTies)
+            old[q] = use ? s.dist[v] : 0u;
+          else
+            old[q] = use ? atomicMin(s.dist + v, c) : 0u;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t c = du[r] + (e[q] >> bits_u), v = e[q] & umask;
+          if (kTies) {
+            if (old[q] == c && e[q] != kNoEdge) atomicMin(s.tie + v, light_tie(e[q], u[r], umask));
+          } else if (c < old[q]) {
+            light_won(s, v, c, lmin);
+          }
+        }
+        const uint32_t bal = __ballot_sync(0xffffffffu, use);  // the last of the lane's four edges
+        on[r] = (bal >> (lane | 3)) & 1u;
+        more |= bal & 0x88888888u;
+      }
+      if (more == 0) break;
+    }
+  }
+  __syncwarp();
+}
+
+// The same for row u of dist du from the matrix (one warp).
+template <bool kTies>
+__device__ __forceinline__ void light_whole_row(const LightCta& s, const SolveDesc& d, uint32_t u, uint32_t du,
+                                                uint32_t D, uint32_t& lmin) {
+  const int lane = static_cast<int>(threadIdx.x) & 31;
+  const int nv = static_cast<int>(d.pitch / 4);
+  const int32_t* row = d.W + static_cast<int64_t>(u) * d.pitch;
+  constexpr int R = 4;
+  for (int g0 = lane; g0 < nv; g0 += 32 * R) {
+    int4 x[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      x[r] = g0 + 32 * r < nv ? ld_stream16(row + 4 * (g0 + 32 * r))
+                              : make_int4(int(kInf), int(kInf), int(kInf), int(kInf));
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const uint32_t w4[4] = {static_cast<uint32_t>(x[r].x), static_cast<uint32_t>(x[r].y),
+                              static_cast<uint32_t>(x[r].z), static_cast<uint32_t>(x[r].w)};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t v = 4 * (g0 + 32 * r) + q, c = du + w4[q];
+        if (w4[q] >= kInf || c > D || v == u) continue;
+        if (kTies) {
+          if (s.dist[v] == c) atomicMin(s.tie + v, static_cast<uint32_t>(light_key(du, w4[q], u, d.bits_u)));
+        } else {
+          const uint32_t old = atomicMin(s.dist + v, c);
+          if (c < old) light_won(s, v, c, lmin);
+        }
+      }
+    }
+  }
+  __syncwarp();
+}
+
+// One phase has one block-wide barrier.  Each warp owns every (THREADS / 32)-th word of 32 nodes: it
+// takes the dirty nodes of its words whose dist lies in the window, gathers them in its own list and
+// relaxes their rows 32 at a time, while other warps may already make more of them dirty -- those go
+// along if their word is still to come, else in a later phase.
+//
+// Rows are first relaxed up to a bound B on the offers: a little above the largest dist of the graph's
+// trial solve (word 15 of the index), which holds for most sources.  When nothing is dirty the true
+// largest dist D is taken; if it is above B every row is relaxed once more up to D.  Dropping offers
+// above the largest dist leaves 13 of the 64 listed edges per row for n = 8192, p = 0.05; waiting for D
+// to be known first left 37.
+template <int THREADS, int PER_SM, class Jobs>
+__global__ void __launch_bounds__(THREADS, PER_SM)
+    k_light_cta(const LightCtaParams p, const Jobs jobs) {
   extern __shared__ __align__(16) uint8_t smem[];
-  __shared__ uint32_t s_job, s_cnt, s_m[2], s_D;
-  unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem);
-  uint16_t* list = reinterpret_cast<uint16_t*>(smem + static_cast<size_t>(p.npad) * 8);
-  uint32_t* dirty = reinterpret_cast<uint32_t*>(smem + static_cast<size_t>(p.npad) * 10);
-  uint32_t* hdone = dirty + p.npad / 32;
-  const int tid = static_cast<int>(threadIdx.x), lane = tid & 31;
+  __shared__ uint2 s_rows[THREADS / 32][kWarpRows];
+  __shared__ uint32_t s_job, s_bound, s_m[3];
+  LightCta s;
+  s.dist = reinterpret_cast<uint32_t*>(smem);
+  s.tie = s.dist + p.npad;
+  s.dirty = s.tie + p.npad;
+  s.wmin = s.dirty + p.npad / 32;
+  s.whole = s.wmin + p.npad / 32;
+  constexpr int NW = THREADS / 32;
+  const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
+  const uint32_t lt = (1u << lane) - 1u;
+  uint2* rows = s_rows[warp];
   pdl_launch_dependents();
 
   for (uint32_t iter = 0;; ++iter) {
@@ -65,163 +188,186 @@ __global__ void __launch_bounds__(THREADS) k_light_cta(const LightCtaParams p, c
     const uint32_t* hmin = d.light + kLightStats;
     const uint32_t* edge = hmin + light_pad(n);
     const uint32_t hmin_min = ~__ldg(d.light);  // >= INF: every row's list is complete
-    uint32_t delta;
-    int gshift;
-    light_window(d.light, kCtaDelta, &delta, &gshift);
-    const int gl = tid & ((1 << gshift) - 1), gid = tid >> gshift, ng = THREADS >> gshift, gsz = 1 << gshift;
+    const int most = static_cast<int>(__ldg(d.light + 6));  // edges in the longest list
+    const uint32_t guess = __ldg(d.light + kLightGuess);
+    const uint32_t delta = light_delta(d.light, kCtaDelta);
+    uint32_t B = hmin_min < kInf && guess > 0 ? guess : kNone;
 
-    for (int v = tid; v < n; v += THREADS) keys[v] = ~0ull;
-    for (int i = tid; i < nwords; i += THREADS) {
-      dirty[i] = 0;
-      hdone[i] = 0;
+    for (int wi = warp; wi < nwords; wi += NW) {
+      const int v = 32 * wi + lane;
+      s.dist[v] = v == d.source ? 0u : kNone;
+      s.tie[v] = kNone;
+      if (lane == 0) {
+        const bool src = wi == (d.source >> 5);
+        s.whole[wi] = 0;
+        s.dirty[wi] = src ? 1u << (d.source & 31) : 0u;
+        s.wmin[wi] = src ? 0u : kNone;
+      }
     }
-    __syncthreads();
     if (tid == 0) {
-      keys[d.source] = 0;
-      dirty[d.source >> 5] = 1u << (d.source & 31);
       s_m[0] = 0;
-      s_cnt = 0;
-      s_D = 0;
+      s_m[1] = kNone;
     }
     __syncthreads();
-    uint32_t phase = 0;
-    uint32_t D = kNone;
-    for (;;) {
-      const uint32_t m = s_m[phase & 1];
+    uint32_t phase = 0, cur = 0;  // cur = phase % 3: the slot of this phase's m, the smallest dirty dist
+    int raised = 0;
+    for (;; ++phase) {
+      const uint32_t m = s_m[cur];
+      const uint32_t nxt = cur == 2 ? 0 : cur + 1;
+      if (tid == 0) s_m[nxt == 2 ? 0 : nxt + 1] = kNone;  // the slot after the next: everyone has read it a phase ago
       uint32_t lmin = kNone;
+      int cnt = 0;  // rows waiting in this warp's list
+      auto relax = [&](int have) {
+        __syncwarp();
+        light_rows<false>(s, [rows](int i) { return rows[i]; }, have, most, B, bits_u, edge, lmin);
+      };
+      auto add = [&](uint32_t take, int wi, uint32_t dv) {  // the nodes `take` of word wi, dv: this lane's dist
+        if ((take >> lane) & 1u) rows[cnt + __popc(take & lt)] = make_uint2(static_cast<uint32_t>(32 * wi + lane), dv);
+        cnt += __popc(take);
+        if (cnt >= 32) {
+          relax(32);
+          cnt -= 32;
+          if (lane < cnt) rows[lane] = rows[32 + lane];
+        }
+        __syncwarp();
+      };
       if (m != kNone) {
-        // the dirty nodes within the window, into list (a warp per word of 32 nodes, a lane per node)
         const uint32_t T = m + delta;
-        for (int wi = tid >> 5; wi < nwords; wi += THREADS / 32) {
-          const uint32_t bits = dirty[wi];
-          if (bits == 0) continue;
-          const int v = 32 * wi + lane;
-          const bool on = (bits >> lane) & 1u;
-          const uint32_t dv = on ? static_cast<uint32_t>(keys[v] >> 32) : kNone;
-          const bool take = on && dv <= T;
-          if (on && !take) lmin = min(lmin, dv);
-          const uint32_t bal = __ballot_sync(0xffffffffu, take);
-          if (bal == 0) continue;
-          uint32_t pos = 0;
-          if (lane == 0) {
-            pos = atomicAdd(&s_cnt, static_cast<uint32_t>(__popc(bal)));
-            dirty[wi] = bits & ~bal;
-          }
-          pos = __shfl_sync(0xffffffffu, pos, 0);
-          if (take) list[pos + __popc(bal & ((1u << lane) - 1u))] = static_cast<uint16_t>(v);
-        }
-        // D: no offer beyond the largest dist can matter (complete lists are short: not worth it)
-        if (hmin_min < kInf) {
-          uint32_t mx = 0;
-          for (int v = tid; v < n; v += THREADS) {
-            const uint32_t dv = static_cast<uint32_t>(keys[v] >> 32);
-            if (dv < kInf)
-              mx = max(mx, dv);
-            else if (static_cast<uint32_t>(__ldg(d.minout + n + v)) < kInf)
-              mx = kNone;  // not reached yet, and something leads to it
-          }
-          mx = __reduce_max_sync(0xffffffffu, mx);
-          if (lane == 0) atomicMax(&s_D, mx);
-        }
-        if (tid == 0) s_m[(phase + 1) & 1] = kNone;
-        __syncthreads();
-        const int cnt = static_cast<int>(s_cnt);
-        if (hmin_min < kInf) D = s_D;
-        for (int i0 = gid; i0 < cnt; i0 += ng * kLightRows) {
-          uint32_t u[kLightRows], du[kLightRows];
-          const uint32_t* row[kLightRows];
-          bool on[kLightRows];
+        for (int base = 0; base < nwords; base += 32 * NW) {
+          const int mine = base + warp + NW * lane;  // a word per lane; needed words are taken 4 at a time
+          const uint32_t wm = mine < nwords ? word_now(s.wmin + mine) : kNone;
+          const bool need = wm != kNone && wm <= T;
+          if (!need) lmin = min(lmin, wm);
+          uint32_t todo = __ballot_sync(0xffffffffu, need);
+          while (todo) {
+            constexpr int kWords = 4;
+            int wi[kWords];
 #pragma unroll
-          for (int r = 0; r < kLightRows; ++r) {
-            const int i = i0 + r * ng;
-            on[r] = i < cnt;
-            u[r] = on[r] ? list[i] : 0u;
-            row[r] = edge + static_cast<size_t>(u[r]) * kLightCap;
-          }
-#pragma unroll
-          for (int r = 0; r < kLightRows; ++r) du[r] = static_cast<uint32_t>(keys[u[r]] >> 32);
-          for (int k = gl; k < kLightCap; k += gsz) {
-            uint32_t e[kLightRows];
-#pragma unroll
-            for (int r = 0; r < kLightRows; ++r) e[r] = on[r] ? __ldg(row[r] + k) : kNoEdge;
-            bool any = false;
-#pragma unroll
-            for (int r = 0; r < kLightRows; ++r) {
-              const uint32_t w = e[r] >> bits_u;
-              on[r] = e[r] != kNoEdge && du[r] + w <= D;  // sorted: what follows is heavier
-              any |= on[r];
-              if (on[r]) light_offer(keys, dirty, e[r] & umask, light_key(du[r], w, u[r], bits_u), lmin);
+            for (int j = 0; j < kWords; ++j) {
+              wi[j] = todo ? base + warp + NW * (__ffs(todo) - 1) : -1;
+              todo &= todo - 1;
             }
-            if (!any) break;
+            // the masks go before the dists are read: a dist lowered before is seen here, one lowered
+            // later sets its bit again
+            uint32_t bits = 0;
+#pragma unroll
+            for (int j = 0; j < kWords; ++j)
+              if (lane == j && wi[j] >= 0) {
+                atomicExch(s.wmin + wi[j], kNone);
+                bits = atomicExch(s.dirty + wi[j], 0u);
+              }
+            __syncwarp();
+            uint32_t dv[kWords];
+#pragma unroll
+            for (int j = 0; j < kWords; ++j) dv[j] = wi[j] >= 0 ? word_now(s.dist + 32 * wi[j] + lane) : kNone;
+#pragma unroll
+            for (int j = 0; j < kWords; ++j) {
+              if (wi[j] < 0) break;
+              const uint32_t b = __shfl_sync(0xffffffffu, bits, j);
+              const uint32_t take = __ballot_sync(0xffffffffu, ((b >> lane) & 1u) && dv[j] <= T);
+              const uint32_t keep = b & ~take;
+              if (keep) {
+                const uint32_t low = warp_min_u32((keep >> lane) & 1u ? dv[j] : kNone);
+                lmin = min(lmin, low);
+                if (lane == 0) {
+                  atomicOr(s.dirty + wi[j], keep);
+                  atomicMin(s.wmin + wi[j], low);
+                }
+              }
+              add(take, wi[j], dv[j]);
+            }
           }
         }
+        if (cnt > 0) relax(cnt);
       } else {
-        // nothing is dirty: the index proves the answer, or some rows are relaxed whole
-        if (hmin_min > D || hmin_min >= kInf) break;
-        if (tid == 0) {
-          s_cnt = 0;
-          s_job = kNone;  // here: the smallest dist + hmin of the pending rows
-          s_m[(phase + 1) & 1] = kNone;
-        }
+        // nothing is dirty; with complete lists (B is kNone then) that is all
+        if (hmin_min >= kInf) break;
+        if (tid == 0) s_bound = 0;
         __syncthreads();
-        uint32_t hb = kNone;
+        uint32_t D = 0;
         for (int v = tid; v < n; v += THREADS) {
-          const uint32_t dv = static_cast<uint32_t>(keys[v] >> 32);
-          if (dv >= kInf || ((hdone[v >> 5] >> (v & 31)) & 1u)) continue;
-          const uint32_t x = dv + __ldg(hmin + v);
-          if (x <= D && x < kInf) hb = min(hb, x);
+          const uint32_t dv = word_now(s.dist + v);
+          if (dv < kInf)
+            D = max(D, dv);
+          else if (static_cast<uint32_t>(__ldg(d.minout + n + v)) < kInf)
+            D = kNone;  // not reached yet, and something leads to it
         }
-        hb = warp_min_u32(hb);
-        if (lane == 0 && hb != kNone) atomicMin(&s_job, hb);
+        D = __reduce_max_sync(0xffffffffu, D);
+        if (lane == 0) atomicMax(&s_bound, D);
         __syncthreads();
-        hb = s_job;
-        if (hb == kNone) break;
-        for (int v = tid; v < n; v += THREADS) {
-          const uint32_t dv = static_cast<uint32_t>(keys[v] >> 32);
-          if (dv >= hb || ((hdone[v >> 5] >> (v & 31)) & 1u)) continue;
-          const uint32_t x = dv + __ldg(hmin + v);
-          if (x > D || x >= kInf) continue;
-          list[atomicAdd(&s_cnt, 1u)] = static_cast<uint16_t>(v);
-          atomicOr(hdone + (v >> 5), 1u << (v & 31));
-        }
-        __syncthreads();
-        const int cnt = static_cast<int>(s_cnt);
-        if (p.heavy && tid == 0) atomicAdd(p.heavy, static_cast<uint32_t>(cnt));
-        const int nv = static_cast<int>(d.pitch / 4);
-        for (int i = 0; i < cnt; ++i) {
-          const uint32_t u = list[i];
-          const uint32_t du = static_cast<uint32_t>(keys[u] >> 32);
-          const int4* row = reinterpret_cast<const int4*>(d.W + static_cast<int64_t>(u) * d.pitch);
-          for (int g = tid; g < nv; g += THREADS) {
-            const int4 x = __ldg(row + g);
-            const uint32_t w4[4] = {static_cast<uint32_t>(x.x), static_cast<uint32_t>(x.y), static_cast<uint32_t>(x.z),
-                                    static_cast<uint32_t>(x.w)};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const uint32_t v = 4 * g + q;
-              if (w4[q] < kInf && du + w4[q] <= D && v != u)
-                light_offer(keys, dirty, v, light_key(du, w4[q], u, bits_u), lmin);
+        D = s_bound;
+        if (D > B) {  // the bound was too low: every row once more, up to D or, with nodes unreached, a higher guess
+          B = D != kNone ? D : ++raised < 4 ? B + B / 4 + 1 : kNone;
+          for (int wi = warp; wi < nwords; wi += NW) {
+            const uint32_t dv = word_now(s.dist + 32 * wi + lane);
+            add(__ballot_sync(0xffffffffu, dv < kInf), wi, dv);
+          }
+          if (cnt > 0) relax(cnt);
+        } else {
+          // the index proves the answer, or some rows are relaxed whole, a warp per row
+          if (hmin_min > D) break;
+          B = D;
+          __syncthreads();  // everyone has read s_bound
+          if (tid == 0) s_bound = kNone;  // the smallest dist + hmin of the pending rows
+          __syncthreads();
+          uint32_t hb = kNone;
+          for (int wi = warp; wi < nwords; wi += NW) {
+            const int v = 32 * wi + lane;
+            const uint32_t dv = word_now(s.dist + v);
+            if (dv >= kInf || ((s.whole[wi] >> lane) & 1u)) continue;
+            const uint32_t x = dv + __ldg(hmin + v);
+            if (x <= D && x < kInf) hb = min(hb, x);
+          }
+          hb = warp_min_u32(hb);
+          if (lane == 0 && hb != kNone) atomicMin(&s_bound, hb);
+          __syncthreads();
+          hb = s_bound;
+          if (hb == kNone) break;
+          for (int wi = warp; wi < nwords; wi += NW) {
+            const int v = 32 * wi + lane;
+            const uint32_t dv = word_now(s.dist + v);
+            bool go = dv < hb && !((s.whole[wi] >> lane) & 1u);  // final, whatever others offer meanwhile
+            if (go) {
+              const uint32_t x = dv + __ldg(hmin + v);
+              go = x <= D && x < kInf;
+            }
+            uint32_t todo = __ballot_sync(0xffffffffu, go);
+            __syncwarp();
+            if (lane == 0) {
+              s.whole[wi] |= todo;
+              if (p.heavy && todo) atomicAdd(p.heavy, static_cast<uint32_t>(__popc(todo)));
+            }
+            for (; todo; todo &= todo - 1) {
+              const int i = __ffs(todo) - 1;
+              light_whole_row<false>(s, d, 32 * wi + i, __shfl_sync(0xffffffffu, dv, i), D, lmin);
             }
           }
         }
       }
       lmin = warp_min_u32(lmin);
-      if (lane == 0 && lmin != kNone) atomicMin(&s_m[(phase + 1) & 1], lmin);
+      if (lane == 0 && lmin != kNone) atomicMin(&s_m[nxt], lmin);
       __syncthreads();
-      if (tid == 0) {  // for the next phase's scan; ordered before it by the barrier below
-        s_cnt = 0;
-        s_D = 0;
-      }
-      __syncthreads();
-      ++phase;
+      cur = nxt;
     }
+    // the dists are final: the best offer of each node's dist.  Only listed edges, and rows relaxed
+    // whole, can make one.
+    for (int wi = warp; wi < nwords; wi += NW) {
+      uint32_t unused = 0;
+      const uint32_t dv = s.dist[32 * wi + lane];
+      light_rows<true>(
+          s, [wi, dv](int i) { return make_uint2(32 * wi + i, __shfl_sync(0xffffffffu, dv, i)); }, 32, most, B, bits_u,
+          edge, unused);
+      for (uint32_t todo = s.whole[wi]; todo; todo &= todo - 1) {
+        const int i = __ffs(todo) - 1;
+        light_whole_row<true>(s, d, 32 * wi + i, __shfl_sync(0xffffffffu, dv, i), B, unused);
+      }
+    }
+    __syncthreads();
     jobs.before_write();  // results reach memory in stream order
     for (int v = tid; v < n; v += THREADS) {
-      const uint64_t k = keys[v];
-      const uint32_t dv = static_cast<uint32_t>(k >> 32);
-      const bool reached = dv < kInf;
-      d.dist[v] = static_cast<int32_t>(reached ? dv : kInf);
-      d.pred[v] = reached && v != d.source ? static_cast<int32_t>(static_cast<uint32_t>(k) & umask) : -1;
+      const uint32_t dv = s.dist[v];
+      d.dist[v] = static_cast<int32_t>(dv == kNone ? kInf : dv);
+      d.pred[v] = dv == kNone || v == d.source ? -1 : static_cast<int32_t>(s.tie[v] & umask);
     }
     __syncthreads();
     if (tid == 0) {
@@ -240,17 +386,11 @@ namespace dj {
 namespace {
 
 
-int light_smem_nodes(int32_t n) { return light_pad(n); }
-size_t light_cta_smem(int32_t n) {
-  const size_t np = static_cast<size_t>(light_smem_nodes(n));
-  return np * 10 + np / 32 * 8;
-}
+constexpr size_t kLightCtaStatic = 10 * 1024;  // static shared memory (512 threads: 8.1 KB) and the system's
 
-template <int THREADS>
-void* light_cta_kernel(int kind) {
-  if (kind == kJobsServe) return reinterpret_cast<void*>(&k_light_cta<THREADS, ServeJobs>);
-  if (kind == kJobsSingle) return reinterpret_cast<void*>(&k_light_cta<THREADS, SingleJob>);
-  return reinterpret_cast<void*>(&k_light_cta<THREADS, BatchJobs>);
+size_t light_cta_smem(int32_t n) {
+  const size_t np = static_cast<size_t>(light_pad(n));
+  return np * 8 + np / 32 * 12;
 }
 
 }  // namespace
@@ -258,27 +398,29 @@ void* light_cta_kernel(int kind) {
 bool light_cta_fits(int32_t n) {
   DevCtx* ctx = nullptr;
   if (get_ctx(&ctx) != DJ_OK) return false;
-  return light_cta_smem(n) + 1024 <= static_cast<size_t>(ctx->max_smem_optin);
+  return light_cta_smem(n) + kLightCtaStatic <= static_cast<size_t>(ctx->max_smem_optin);
 }
 
+// CTAs of 512 threads, one per SM; two per SM in batches with more solves than SMs where shared memory
+// allows (256 sources of n = 8192: 298 us, 354 with one; 48 graphs, which have an SM each, 112 with the
+// registers of one, 129 with those of two).  The server's persistent CTAs have 256 threads, one per SM:
+// other kernels must find room beside them for as long as the server runs (two CTAs of 512 threads fill
+// every register of an SM, and a caller's own kernels waited until the server left).
 int plan_light(int32_t max_n, int32_t k, int kind, LightPlan* plan) {
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   plan->smem = light_cta_smem(max_n);
-  plan->npad = light_smem_nodes(max_n);
-  // two or more CTAs per SM where shared memory allows, else one large one
-  const bool large = plan->smem > static_cast<size_t>(ctx->max_smem_optin) / 2 - 2048;
-  plan->threads = large || (kind == kJobsSingle && max_n >= 2048) ? 1024 : 512;
-  plan->fn = plan->threads == 1024 ? light_cta_kernel<1024>(kind) : light_cta_kernel<512>(kind);
+  plan->npad = light_pad(max_n);
+  plan->threads = kind == kJobsServe ? 256 : 512;
+  const bool two = kind == kJobsBatch && k > ctx->num_sms &&
+                   2 * (plan->smem + kLightCtaStatic) <= static_cast<size_t>(ctx->max_smem_optin);
+  plan->fn = kind == kJobsServe    ? reinterpret_cast<void*>(&k_light_cta<256, 1, ServeJobs>)
+             : kind == kJobsSingle ? reinterpret_cast<void*>(&k_light_cta<512, 1, SingleJob>)
+             : two                 ? reinterpret_cast<void*>(&k_light_cta<512, 2, BatchJobs>)
+                                   : reinterpret_cast<void*>(&k_light_cta<512, 1, BatchJobs>);
   if (int rc = prepare_function(ctx, plan->fn, plan->smem, false)) return rc;
-  plan->ctas = 1;
-  if (kind != kJobsSingle) {
-    int occ = 0;
-    if (int rc = function_occupancy(ctx, plan->fn, plan->threads, plan->smem, &occ)) return rc;
-    if (occ < 1) return set_error(DJ_EUNSUPPORTED, "light engine cannot be resident");
-    plan->ctas = ctx->num_sms * occ;
-    if (kind == kJobsBatch) plan->ctas = std::max(1, std::min(plan->ctas, static_cast<int>(k)));
-  }
+  plan->ctas = kind == kJobsSingle ? 1 : ctx->num_sms * (two ? 2 : 1);
+  if (kind == kJobsBatch) plan->ctas = std::max(1, std::min(plan->ctas, static_cast<int>(k)));
   return DJ_OK;
 }
 

@@ -6,9 +6,11 @@
 // phases: the nodes whose dist changed since their row was last relaxed are dirty; a phase relaxes
 // the dirty nodes of dist <= m + delta (m: the smallest dirty dist, delta: a few times the mean
 // spacing of a row's listed weights, so a row has a few edges that stay inside the window).  A row is
-// read up to the first edge whose offer exceeds D, the largest dist of any node (all ones until every
-// node something leads to is reached).  When nothing is dirty, the index's test (hmin) either proves
-// the answer complete or names the rows to relax whole from the matrix:
+// read up to the first edge whose offer exceeds a bound: D, the largest dist of any node (all ones until
+// every node something leads to is reached), or the guess of D that the graph's trial solve left, if
+// that is less.  When nothing is dirty and D is above the guess, the guess is raised and every row
+// relaxed once more.  Then the index's test (hmin) either proves the answer complete or names the rows to
+// relax whole from the matrix:
 //   pending = { u : dist[u] + hmin[u] <= D, not yet relaxed whole }, and
 //   those with dist[u] < min over pending of (dist + hmin) are final -- a shorter path would use an
 //   unlisted edge of a pending row -- so each row is read from the matrix at most once.
@@ -45,6 +47,7 @@ struct LightGridParams {
   unsigned long long* gkey;   // n keys
   uint32_t* words;            // per-device words: [0] error bits, [1] phases
   uint32_t* heavy;            // optional: rows relaxed whole are counted here
+  uint32_t* guess;            // trial: the index's kLightGuess
   int64_t pitch;
   int64_t timeout_ns;
   int32_t n;
@@ -171,10 +174,14 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
   const uint32_t bits_u = p.bits_u, umask = (1u << bits_u) - 1u;
   const uint32_t* hmin = CSR ? nullptr : p.light + kLightStats;
   const uint32_t hmin_min = CSR ? kInf : ~__ldg(p.light);
+  const uint32_t most = CSR ? 0u : __ldg(p.light + 6);  // edges in the longest list
   uint32_t delta = p.delta;
   int gshift = p.gshift;
   if (!CSR) light_window(p.light, kGridDelta, &delta, &gshift);
   if (!CSR && p.trial && hmin_min >= kInf) return;
+  // offers above the guessed largest dist are dropped at first (see below); the trial makes the guess
+  uint32_t guess = CSR || p.trial || hmin_min >= kInf ? kNone : __ldg(p.light + kLightGuess);
+  if (guess == 0) guess = kNone;
   for (int j = tid; j < sw; j += T0) {
     const int v = c0 + j;
     p.gkey[v] = v == p.source ? 0ull : ~0ull;
@@ -211,12 +218,18 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
   const int gsz = 1 << gshift;
   const int gl = tid & (gsz - 1), gid = tid >> gshift, ng = T0 >> gshift;
   const uint32_t longrow = CSR ? static_cast<uint32_t>(gsz) * 16u : kNone;
+  const int last = (tid & 31) | (gsz - 1);  // last lane of this lane's group; lasts: of every group
+  const uint32_t lasts = gshift == 2 ? 0x88888888u : gshift == 3 ? 0x80808080u : gshift == 4 ? 0x80008000u : 0x80000000u;
   uint32_t phases = 0;
+  bool again = false;  // this phase relaxes every reached row, whatever its dist
+  int raised = 0;
   for (;;) {
     lmin = kNone;
     uint32_t dmax = 0;
     if (m != kNone) {
-      const uint32_t T = m + delta;
+      const uint32_t T = again ? kNone : m + delta;
+      const uint32_t B = min(D, guess);
+      again = false;
       for (int j = tid; j < sw; j += T0) {
         const uint32_t d = static_cast<uint32_t>(__ldcg(p.gkey + c0 + j) >> 32);
         if (d < kInf)
@@ -237,40 +250,40 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
       }
       __syncthreads();
       const int cnt = static_cast<int>(sh.cnt);
-      for (int i0 = gid; i0 < cnt; i0 += ng * kLightRows) {
+      for (int i0 = 0; i0 < cnt; i0 += ng * kLightRows) {
         uint32_t u[kLightRows], du[kLightRows], len[kLightRows];
         const uint32_t* row[kLightRows];
         bool on[kLightRows];
 #pragma unroll
         for (int r = 0; r < kLightRows; ++r) {
-          const int i = i0 + r * ng;
+          const int i = i0 + r * ng + gid;
           on[r] = i < cnt;
           const uint2 x = on[r] ? list[i] : make_uint2(0u, 0u);
           u[r] = static_cast<uint32_t>(c0) + x.x;
           du[r] = x.y;
           row[r] = CSR ? p.edge + start[x.x] : p.edge + static_cast<size_t>(u[r]) * kLightCap;
-          len[r] = CSR ? aux[x.x] : static_cast<uint32_t>(kLightCap);
+          len[r] = CSR ? aux[x.x] : most;
         }
         for (uint32_t k = gl;; k += gsz) {
-          uint32_t e[kLightRows];
+          uint32_t e[kLightRows], more = 0;
           uint64_t old[kLightRows];
-          bool any = false;
+          bool use[kLightRows];
+#pragma unroll
+          for (int r = 0; r < kLightRows; ++r) e[r] = on[r] && k < len[r] ? __ldg(row[r] + k) : kNoEdge;
 #pragma unroll
           for (int r = 0; r < kLightRows; ++r) {
-            on[r] = on[r] && k < len[r];
-            e[r] = on[r] ? __ldg(row[r] + k) : kNoEdge;
+            use[r] = e[r] != kNoEdge && du[r] + (e[r] >> bits_u) <= B;
+            old[r] = use[r] ? __ldcg(p.gkey + (e[r] & umask)) : 0ull;
+            // sorted: a row goes on only if it has more and its group's last lane still had a use for its edge
+            const uint32_t bal = __ballot_sync(0xffffffffu, use[r] && k - gl + gsz < len[r]);
+            on[r] = (bal >> last) & 1u;
+            more |= bal & lasts;
           }
-#pragma unroll
-          for (int r = 0; r < kLightRows; ++r) {
-            on[r] = e[r] != kNoEdge && du[r] + (e[r] >> bits_u) <= D;  // sorted: what follows is heavier
-            any |= on[r];
-            old[r] = on[r] ? __ldcg(p.gkey + (e[r] & umask)) : 0ull;
-          }
-          if (!any) break;
 #pragma unroll
           for (int r = 0; r < kLightRows; ++r)
-            if (on[r])
+            if (use[r])
               light_offer_global(p.gkey, e[r] & umask, light_key(du[r], e[r] >> bits_u, u[r], bits_u), old[r], lmin);
+          if (more == 0) break;
         }
       }
       if (CSR) {  // long rows: the whole block takes one after another
@@ -281,7 +294,7 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
           const uint32_t* row = p.edge + start[x.x];
           for (uint32_t k = tid; k < aux[x.x]; k += T0) {
             const uint32_t e = __ldg(row + k);
-            if (x.y + (e >> bits_u) > D) break;
+            if (x.y + (e >> bits_u) > B) break;
             light_offer_global(p.gkey, e & umask, light_key(x.y, e >> bits_u, u, bits_u), __ldcg(p.gkey + (e & umask)),
                                lmin);
           }
@@ -291,8 +304,18 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
       ++phases;
       continue;
     }
-    // nothing is dirty anywhere: the index proves the answer, or some rows are relaxed whole
-    if (CSR || hmin_min > D || hmin_min >= kInf) break;
+    // nothing is dirty anywhere; with complete lists (no bound was set) that is all
+    if (CSR || hmin_min >= kInf) break;
+    if (D > guess) {  // the bound was too low: every row once more, up to D or, with nodes unreached, a higher guess
+      guess = D != kNone ? D : ++raised < 4 ? guess + guess / 4 + 1 : kNone;
+      for (int j = tid; j < sw; j += T0)
+        if (rdist[j] < kInf) rdist[j] = kNone;
+      again = true;
+      m = 0;
+      continue;
+    }
+    // the index proves the answer, or some rows are relaxed whole
+    if (hmin_min > D) break;
     const uint32_t Dx = D;
     uint32_t hb = kNone;
     for (int j = tid; j < sw; j += T0) {
@@ -302,6 +325,7 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
     }
     if (!light_barrier(p, sh, nbar++, hb, 0u, &m, &D)) return;
     hb = m;
+    D = Dx;
     if (hb == kNone) break;
     for (int j = tid; j < sw; j += T0) {
       if ((flags[j] & 2) || rdist[j] >= hb || rdist[j] + aux[j] > Dx || rdist[j] + aux[j] >= kInf) continue;
@@ -346,7 +370,12 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
     p.dist_out[c0 + j] = static_cast<int32_t>(reached ? d : kInf);
     p.pred_out[c0 + j] = reached && c0 + j != p.source ? static_cast<int32_t>(static_cast<uint32_t>(k) & umask) : -1;
   }
-  if (b == 0 && tid == 0 && !p.trial) p.words[1] = phases;
+  if (b == 0 && tid == 0) {
+    if (!p.trial)
+      p.words[1] = phases;
+    else if (D < kInf)
+      p.guess[0] = D + D / 8 + 1;
+  }
 }
 
 template <bool CSR>
@@ -415,6 +444,7 @@ int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t*
   p.gkey = reinterpret_cast<unsigned long long*>(ws + ctl_bytes);
   p.words = ctx->words;
   p.heavy = heavy;
+  p.guess = csr ? nullptr : g->light + kLightGuess;
   p.pitch = g->pitch;
   p.timeout_ns = o.timeout_ns > 0 ? o.timeout_ns : 2000000000LL;
   p.n = g->n;

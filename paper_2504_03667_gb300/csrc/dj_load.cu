@@ -568,10 +568,8 @@ static void launch_minima(dj_graph* g, uint32_t* stats, cudaStream_t st, bool ha
 // The index's leading words are zero before, but for the edge list's check (words 12..14), whose
 // verdict *list gets (nullptr: there was no list).
 //
-// Whether solves take the light engine is judged here: at once if every row's list is complete, else
-// if a trial solve relaxes at most a sixteenth of the rows whole (graphs of nearly equal weights, or
-// whose distances are long against what the lists reach, need far more of the matrix, and the other
-// engines stream it better).  The trial is one more kernel in front of the only wait.
+// Whether solves take the light engine is judged here, by a trial solve: one more kernel in front of
+// the only wait.
 static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   uint32_t* stats = g->light ? g->light + 8 : nullptr;
   uint32_t idx[16] = {0};
@@ -603,7 +601,15 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   g->light_deg = static_cast<float>(static_cast<double>(g->entries) / g->n);
   if (g->n > 1 && static_cast<int64_t>(g->n - 1) * g->wmax >= static_cast<int64_t>(DJ_INF))
     return set_error(DJ_EOVERFLOW, "(n-1) * max weight >= INT32_MAX: path lengths could overflow int32");
-  g->light_ok = tried && g->wmin >= 1 && (~idx[0] >= kInf || idx[1] <= static_cast<uint32_t>(g->n) / 16);
+  // Taken at once if every row's list is complete, else if a trial solve relaxed next to no row whole:
+  // where many are needed (nearly equal weights, distances long against what the lists reach) the other
+  // engines stream the matrix better (n = 8192, p = 0.5, weights 1..10: 410 rows whole, 112 us; grid
+  // engine 37).  One CTA relaxes whole rows slowly (4500 of them in 7 ms, the grid form in 0.2), so its
+  // form is for complete lists, or symmetric matrices without one in the trial: no source's largest
+  // dist is then more than twice the trial's, while a directed graph's may be by any factor.
+  const bool complete = ~idx[0] >= kInf;
+  g->light_ok = tried && g->wmin >= 1 && (complete || idx[1] <= 4);
+  g->light_cta = g->light_ok && (complete || (!g->directed && idx[1] == 0));
   // graphs that are not dense keep in-lists for the grid engine's dynamic IN bound
   const uint64_t nn = static_cast<uint64_t>(g->n) * static_cast<uint64_t>(g->n);
   if (g->entries * 32 < nn && g->wmin >= 1 && !g->inlist) {
@@ -813,6 +819,9 @@ extern "C" int dj_graph_upload(dj_graph* g, const int32_t* W, int64_t ld, uint64
   }
   if (e != cudaSuccess) return cuda_error(e, "host-to-device matrix copy (upload)");
   g->upload_pending = 1;
+  // The index follows the matrix (a captured solve may be replayed on it), but it was judged for the
+  // loaded one: nothing tells here, without a wait, whether the new one suits it.
+  g->light_ok = g->light_cta = false;
   launch_minima(g, nullptr, st, zero_copy);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_error(e, "row minima");

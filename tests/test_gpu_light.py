@@ -101,9 +101,9 @@ def test_upload_rebuilds_the_index(dj, orc):
     """After an upload the same handle (and a captured solve) answers for the new matrix, from aligned
     and unaligned pinned buffers and from pageable memory."""
     import torch
-    for n in (203, 4500):
+    for n in (203, 4500, 6200):  # the last beyond the CTA form
         a = graphgen.bernoulli(n, 0.3, 1, 1000, 1)
-        b = graphgen.bernoulli(n, 0.05, 1, 9, 2)
+        b = graphgen.bernoulli(n, 0.4, 1, 2, 2)  # the replayed solves need whole rows on it
         Wb = orc.build_matrix(n, b.src, b.dst, b.w, False)
         ref = orc.dijkstra(Wb, 5)
         pinned = torch.from_numpy(Wb).pin_memory()
