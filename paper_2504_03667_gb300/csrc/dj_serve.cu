@@ -86,6 +86,9 @@ struct dj_server {
   std::vector<PoolBuf> pool;
   int32_t plan_pitch = 0;
   ClusterPlan plan;
+  LightPlan lplan;
+  bool light = false;        // the persistent kernel is the light engine's (every graph takes it and fits)
+  size_t planned_graphs = 0;
   bool plan_valid = false;
   // statistics
   std::vector<double> lat_us;
@@ -106,10 +109,26 @@ int stop_kernel(dj_server* s) {
 }
 
 int ensure_plan(dj_server* s) {
-  int32_t pitch = 32;
-  for (auto* g : s->graphs) pitch = std::max(pitch, g->pitch);
-  if (s->plan_valid && pitch <= s->plan_pitch) return DJ_OK;
+  if (s->plan_valid && s->planned_graphs == s->graphs.size()) return DJ_OK;  // (no request without a graph)
+  int32_t pitch = 32, n = 1;
+  bool light = s->opts.cluster_size == 0 && s->opts.clusters == 0;
+  for (auto* g : s->graphs) {
+    pitch = std::max(pitch, g->pitch);
+    n = std::max(n, g->n);
+    light = light && g->light_cta;
+  }
+  light = light && light_cta_fits(n);
+  s->planned_graphs = s->graphs.size();
+  if (s->plan_valid && pitch <= s->plan_pitch && light == s->light) return DJ_OK;
   if (int rc = stop_kernel(s)) return rc;
+  s->plan_valid = false;  // until the new plan is made
+  s->light = light;
+  if (light) {
+    if (int rc = plan_light(n, 0, kJobsServe, &s->lplan)) return rc;
+    s->plan_pitch = pitch;
+    s->plan_valid = true;
+    return DJ_OK;
+  }
   ClusterLaunch cl;
   cl.cluster_size = s->opts.cluster_size > 0 ? s->opts.cluster_size : heuristic_cluster(pitch);
   cl.clusters = s->opts.clusters;
@@ -137,7 +156,7 @@ int ensure_kernel(dj_server* s) {
   r.head = s->head_d;
   r.cap_mask = s->cap - 1;
   r.idle_ns = s->opts.idle_timeout_ns > 0 ? s->opts.idle_timeout_ns : 200000000LL;
-  if (int rc = run_serve_kernel(s->plan, r, s->stream)) return rc;
+  if (int rc = s->light ? run_light_serve(s->lplan, r, s->stream) : run_serve_kernel(s->plan, r, s->stream)) return rc;
   cudaError_t e = cudaEventRecord(s->kernel_end, s->stream);
   if (e != cudaSuccess) return cuda_error(e, "cudaEventRecord");
   s->kernel_live = true;
@@ -208,6 +227,13 @@ int submit(dj_server* s, int32_t gid, int32_t source, int32_t* dist, int32_t* pr
     s->pool[pool].busy = true;
     dist = s->pool[pool].ptr;
     pred = s->pool[pool].ptr + g->n;
+  }
+  // a graph added since the running kernel was planned, or taken off the light engine by an upload, may
+  // need another plan: before the kernel can see the request
+  if (s->light && !g->light_cta) s->planned_graphs = 0;
+  if (int rc = ensure_plan(s)) {
+    if (pool >= 0) s->pool[pool].busy = false;
+    return rc;
   }
   const uint64_t tk = s->next_ticket;
   const uint32_t slot = static_cast<uint32_t>(tk & (s->cap - 1));

@@ -1,6 +1,8 @@
 """The light engine (the default on graphs of positive weights) against the oracle: sizes at the
 edges of its lists, slices and key words, rows whose lists are complete, cut or empty, nodes nothing
 leads to, and sources for which the lists do not suffice and rows are relaxed whole."""
+import time
+
 import numpy as np
 import pytest
 
@@ -131,3 +133,38 @@ def test_upload_rebuilds_the_index(dj, orc):
             assert np.array_equal(d.cpu().numpy(), ref[0]) and np.array_equal(p.cpu().numpy(), ref[1]), (n, what, "replay")
             del cg
             G.free()
+
+
+def test_server_replans(dj, orc):
+    """A running server takes a larger graph, then one the light engine does not take, then an upload:
+    every request is answered for the graph as it is."""
+    import torch
+    small, large = graphgen.bernoulli(150, 0.3, 1, 1000, 5), graphgen.bernoulli(3000, 0.05, 1, 1000, 6)
+    narrow = graphgen.bernoulli(900, 0.5, 1, 2, 7)
+    g = [dj.dj_load_edges(e.n, e.src, e.dst, e.w, False) for e in (small, large, narrow)]
+    W = [orc.build_matrix(e.n, e.src, e.dst, e.w, False) for e in (small, large, narrow)]
+    srv = dj.dj_serve_create(dj.make_serve_opts(max_slots=8, idle_timeout_ns=300_000_000))
+
+    def ask(gid, k, s):
+        t = dj.dj_serve_submit(srv, gid, s)
+        assert t is not None
+        dj.dj_serve_wait(srv, t)
+        got, ref = dj.dj_serve_result(srv, t, W[k].shape[0]), orc.dijkstra(W[k], s)
+        assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1]), (k, s)
+
+    ids = []
+    for k in range(3):  # each added while the kernel planned for the earlier ones is running
+        ids.append(dj.dj_serve_add_graph(srv, g[k]))
+        for j in range(k + 1):
+            ask(ids[j], j, 7 * j + 3)
+    srv.destroy()
+    srv = dj.dj_serve_create(dj.make_serve_opts(max_slots=8, idle_timeout_ns=300_000_000))
+    gid = dj.dj_serve_add_graph(srv, g[1])
+    ask(gid, 1, 11)
+    W[1] = orc.build_matrix(3000, large.src, large.dst, (large.w % 3 + 1).astype(np.int32), False)
+    dj.dj_graph_upload(g[1], torch.from_numpy(W[1]).pin_memory(), torch.cuda.Stream())
+    time.sleep(0.05)  # the upload is done; the server still runs
+    ask(gid, 1, 12)
+    srv.destroy()
+    for x in g:
+        x.free()
