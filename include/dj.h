@@ -156,7 +156,9 @@ int dj_graph_free(dj_graph* g);
  * rebuilt by dj_graph_upload).  A solve relaxes those; then dist[u] + (u's
  * smallest unlisted weight) > max dist proves that no unlisted edge matters,
  * and rows that fail the test are relaxed whole from the matrix, so dist and
- * pred are Algorithm 1's on every graph.  Taken by DJ_ENGINE_AUTO in phase
+ * pred are Algorithm 1's on every graph.  One solve runs on one CTA, on one
+ * cluster or on every SM, by size and by whether anything is ahead of it on
+ * its stream (dj_sssp).  Taken by DJ_ENGINE_AUTO in phase
  * mode when every weight is >= 1, every other option below is left at its
  * default, and a trial solve at load needed next to no whole row; also for
  * graphs in compressed rows.  After dj_graph_upload a graph's solves take the
@@ -228,7 +230,10 @@ void dj_solve_opts_init(dj_solve_opts* opts);
 
 /* One solve of Algorithm 1 from `source` on graph g.
  *   dist, pred  DEVICE pointers to n int32 each (caller-owned), written by the kernel.
- * Asynchronous on `stream`: one kernel launch.  The grid engine keeps a small
+ * Asynchronous on `stream`: one kernel launch.  Large solves on an idle stream
+ * use every SM; small ones, and those behind other work on their stream, a CTA
+ * or a cluster each, so that back-to-back solves run side by side (same
+ * results).  The grid engine keeps a small
  * workspace per (device, stream) -- about 32 bytes per matrix column plus 16 *
  * pitch bytes with the row split, at least 1 MiB -- created on the first solve
  * on that stream (a cudaMalloc) and grown, after synchronising the stream,

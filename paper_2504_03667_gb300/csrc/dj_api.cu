@@ -231,23 +231,54 @@ static bool light_auto(const dj_graph* g, const dj_solve_opts& o) {
          o.rowsplit == 0 && o.rowpush == 0 && o.trace == nullptr;
 }
 
-// Dense graphs below this size take the light engine's CTA form: back-to-back solves overlap there, one
-// per SM, and small ones are faster alone too (n = 1024: 10 us each and 43 us alone, grid form 49 and 58;
-// n = 5003, p = 0.3: 13.8 and 98, grid form 49.6 and 59; n = 16384: 35 and 255, grid form 37 and 46).
-static constexpr int32_t kLightGridMinN = 6144;
+// Which form of the light engine a single solve takes (GB300; us each back to back, and alone):
+//                                    CTA          cluster       grid
+//   n = 200, 6 edges per node         9 /  30       9 /  37      40 /  49
+//   n = 1024, p = 0.1                 9 /  43       9 /  45      49 /  58
+//   n = 5003, p = 0.3                12 /  98       9 /  61      49 /  59
+//   n = 16384, p = 0.5               35 / 255      16 / 117      31 /  41
+//   n = 32768, 8 edges per node                    20 / 142      81 /  91
+// CTA and cluster solves leave most SMs to the next solves on the stream, which then run side by side;
+// the grid form gives one solve every SM.  So a large solve takes the grid form only when nothing is
+// ahead of it on its stream (someone is waiting for this one), and so it does when one CTA or cluster
+// would be slow with the whole rows its graph may need.
+static constexpr int32_t kLightClusterMinN = 2048;
+static constexpr int32_t kLightIdleGridMinN = 6144;
+static constexpr int32_t kLightIdleGridMinNComplete = 16384;  // compressed rows: fewer offers per phase
+static constexpr uint32_t kLightClusterMaxRow = 512;          // longer compressed rows: the grid form shares them out
+
+static bool stream_idle(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (cap != cudaStreamCaptureStatusNone) return false;
+  const cudaError_t e = cudaStreamQuery(st);
+  if (e != cudaSuccess && e != cudaErrorNotReady) cudaGetLastError();  // the launch reports it
+  return e == cudaSuccess;
+}
 
 static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
                        cudaStream_t st) {
-  if (!g->light_cta || g->n >= kLightGridMinN || !light_cta_fits(g->n))
+  const bool csr = g->format == DJ_FORMAT_CSR;
+  const int C = g->n < 1024 ? 4 : g->n < 4096 ? 8 : 16;
+  const bool cta = !csr && g->light_cta && g->n < kLightClusterMinN && light_cta_fits(g->n);
+  const bool cluster = !cta && (csr ? g->light_longest <= kLightClusterMaxRow : g->light_cta) &&
+                       light_cluster_fits(g->n, C, csr);
+  if (!cta && (!cluster || o.debug_skip_cta >= 0 ||
+               (g->n >= (csr ? kLightIdleGridMinNComplete : kLightIdleGridMinN) && stream_idle(st))))
     return launch_light_grid(g, source, dist, pred, o, nullptr, st);
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
-  LightPlan plan;
-  if (int rc = plan_light(g->n, 1, kJobsSingle, &plan)) return rc;
+  const SolveDesc d = make_desc(g, source, dist, pred, 0);
   // right after an upload the solve waits for the kernels before it before reading the graph
   const bool early = g->upload_pending == 0;
   const_cast<dj_graph*>(g)->upload_pending = 0;
-  return run_light_single(plan, make_desc(g, source, dist, pred, 0), ctx->words + 1, nullptr, early, st);
+  if (cluster) return run_light_cluster(g, C, d, ctx->words + 1, early, st);
+  LightPlan plan;
+  if (int rc = plan_light(g->n, 1, kJobsSingle, &plan)) return rc;
+  return run_light_single(plan, d, ctx->words + 1, nullptr, early, st);
 }
 
 extern "C" int dj_sssp_ex(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts* opts,

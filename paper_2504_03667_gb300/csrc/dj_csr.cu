@@ -274,6 +274,7 @@ extern "C" int dj_load_edges_csr(int32_t n, int64_t m, const int32_t* src, const
     }
   };
   int64_t r0 = 0;
+  size_t longest = 0;
   for (int32_t u = 0; u < n; ++u) {
     const int64_t r1 = row_ptr[static_cast<size_t>(u) + 1];
     sort(es.begin() + r0, es.begin() + r1);
@@ -287,6 +288,7 @@ extern "C" int dj_load_edges_csr(int32_t n, int64_t m, const int32_t* src, const
     r0 = r1;
     row_ptr[static_cast<size_t>(u) + 1] = static_cast<int64_t>(edge.size());
     const size_t len = edge.size() - p0;
+    longest = std::max(longest, len);
     if (len == 0) continue;
     sort(edge.begin() + static_cast<int64_t>(p0), edge.end());
     minout[u] = static_cast<int32_t>(edge[p0] >> bits_u);
@@ -322,6 +324,7 @@ extern "C" int dj_load_edges_csr(int32_t n, int64_t m, const int32_t* src, const
   g->minin = g->minout + n;
   g->bytes = rp_bytes + e_bytes + m_bytes;
   g->light_ok = wmin >= 1;
+  g->light_longest = static_cast<uint32_t>(std::min<size_t>(longest, 0xFFFFFFFFu));
   g->light_spacing = sum_cnt > 0 ? static_cast<float>(sum_last / sum_cnt) : 0.f;
   while (g->light_gshift > 2 && (nnz >> (g->light_gshift - 1)) < n) --g->light_gshift;  // lanes per row: about its edges
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

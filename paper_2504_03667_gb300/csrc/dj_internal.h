@@ -40,6 +40,7 @@ struct dj_graph {
   bool light_cta = false;     // its CTA form too: hardly any source needs whole rows (slow in one CTA)
   float light_deg = 0.f;      // dense: edges per row
   float light_spacing = 0.f;  // compressed rows: mean spacing of a row's lightest weights
+  uint32_t light_longest = 0; // compressed rows: edges of the longest row
   int32_t light_gshift = 5;   // compressed rows: log2 of the lanes that share a row
   uint64_t bytes = 0;
   uint64_t entries = 0;       // finite off-diagonal matrix entries (directed edges)
@@ -275,6 +276,10 @@ int run_light_batch(const LightPlan& plan, const SolveDesc* descs_dev, int32_t k
 int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, uint32_t* heavy, bool early,
                      cudaStream_t st);
 int run_light_serve(const LightPlan& plan, const ServeRing& r, cudaStream_t st);
+// One solve on one cluster of C CTAs (a power of two up to 16), as run_light_single.
+bool light_cluster_fits(int32_t n, int C, bool csr);
+int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t* phases_out, bool early,
+                      cudaStream_t st);
 // One solve over every SM (a graph with an index, or in compressed rows).
 int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
                       uint32_t* heavy, cudaStream_t st);

@@ -158,4 +158,120 @@ __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, u
   return r;
 }
 
+// ------------------------------------------------------------------ relaxing rows from shared memory
+
+constexpr uint32_t kNone = 0xFFFFFFFFu;  // no dist, no bound
+constexpr int kWarpRows = 64;            // a warp's waiting rows: 31 left over and 32 of the next word
+
+// Shared words that other warps change meanwhile are read through this.
+__device__ __forceinline__ uint32_t word_now(const uint32_t* p) { return *const_cast<const volatile uint32_t*>(p); }
+
+// The rows of the index: up to `most` edges each, padded.
+struct LightListEdges {
+  const uint32_t* __restrict__ edge;
+  uint32_t most;
+  __device__ __forceinline__ uint4 load(uint32_t u, uint32_t k0, int sub) const {
+    return __ldg(reinterpret_cast<const uint4*>(edge + static_cast<size_t>(u) * kLightCap + k0) + sub);
+  }
+};
+
+// Relax (with kTies: take the ties of) the listed edges of a warp's rows: get(i) is row i, i < count, as
+// (u, dist[u]) or, where there is nothing to do, (u, kNone).  Four lanes share a row and take four edges
+// each with one 16-byte load, so a warp's load covers 16 edges of 8 rows in 8 pieces of 64 bytes, and
+// 16 rows are in flight.  Edges whose offer exceeds B are dropped; a row goes on to its next 16
+// edges only if the heaviest of these was of use.  (A lane per edge, 16 lanes per row, took three times the
+// instructions per edge; a lane per row read 32 lines with every load and was bound by the L1.)
+template <bool kTies, class Store, class Edges, class Get>
+__device__ __forceinline__ void light_rows(const Store& s, const Edges& edges, const Get& get, int count, uint32_t B,
+                                           uint32_t bits_u, uint32_t& lmin) {
+  const int lane = static_cast<int>(threadIdx.x) & 31, sub = lane & 3;
+  const uint32_t umask = (1u << bits_u) - 1u;
+  constexpr int R = 2;  // 16-byte loads in flight per lane (4: 395 against 298 us for the batch)
+  for (int i0 = 0; i0 < count; i0 += 8 * R) {
+    uint32_t u[R], du[R];
+    bool on[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int i = i0 + 8 * r + (lane >> 2);
+      const uint2 x = get(min(i, count - 1));
+      u[r] = x.x;
+      du[r] = x.y;
+      on[r] = i < count && x.y != kNone;
+    }
+    for (uint32_t k0 = 0; k0 < edges.most; k0 += 16) {  // most bounds every row
+      uint4 x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        x[r] = on[r] ? edges.load(u[r], k0, sub) : make_uint4(kNoEdge, kNoEdge, kNoEdge, kNoEdge);
+      uint32_t more = 0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const uint32_t e[4] = {x[r].x, x[r].y, x[r].z, x[r].w};
+        uint32_t old[4];
+        bool use = false;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t c = du[r] + (e[q] >> bits_u), v = e[q] & umask;
+          use = e[q] != kNoEdge && c <= B;
+          if (kTies)
+            old[q] = use ? s.dist_of(v) : 0u;
+          else
+            old[q] = use ? s.offer(v, c) : 0u;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t c = du[r] + (e[q] >> bits_u), v = e[q] & umask;
+          if (kTies) {
+            if (old[q] == c && e[q] != kNoEdge) s.tie_min(v, light_tie(e[q], u[r], umask));
+          } else if (c < old[q]) {
+            s.won(v, c);
+            lmin = min(lmin, c);
+          }
+        }
+        const uint32_t bal = __ballot_sync(0xffffffffu, use);  // the last of the lane's four edges
+        on[r] = (bal >> (lane | 3)) & 1u;
+        more |= bal & 0x88888888u;
+      }
+      if (more == 0) break;
+    }
+  }
+  __syncwarp();
+}
+
+// The same for row u of dist du from the matrix (one warp).
+template <bool kTies, class Store>
+__device__ __forceinline__ void light_whole_row(const Store& s, const SolveDesc& d, uint32_t u, uint32_t du,
+                                                uint32_t D, uint32_t& lmin) {
+  const int lane = static_cast<int>(threadIdx.x) & 31;
+  const int nv = static_cast<int>(d.pitch / 4);
+  const int32_t* row = d.W + static_cast<int64_t>(u) * d.pitch;
+  constexpr int R = 4;
+  for (int g0 = lane; g0 < nv; g0 += 32 * R) {
+    int4 x[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      x[r] = g0 + 32 * r < nv ? ld_stream16(row + 4 * (g0 + 32 * r))
+                              : make_int4(int(kInf), int(kInf), int(kInf), int(kInf));
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const uint32_t w4[4] = {static_cast<uint32_t>(x[r].x), static_cast<uint32_t>(x[r].y),
+                              static_cast<uint32_t>(x[r].z), static_cast<uint32_t>(x[r].w)};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t v = 4 * (g0 + 32 * r) + q, c = du + w4[q];
+        if (w4[q] >= kInf || c > D || v == u) continue;
+        if (kTies) {
+          if (s.dist_of(v) == c) s.tie_min(v, static_cast<uint32_t>(light_key(du, w4[q], u, d.bits_u)));
+        } else {
+          if (c < s.offer(v, c)) {
+            s.won(v, c);
+            lmin = min(lmin, c);
+          }
+        }
+      }
+    }
+  }
+  __syncwarp();
+}
+
 }  // namespace dj

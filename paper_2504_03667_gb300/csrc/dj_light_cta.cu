@@ -12,11 +12,8 @@
 namespace dj {
 
 namespace {
-constexpr uint32_t kNone = 0xFFFFFFFFu;
 // delta in units of the listed weights' mean spacing: 19 phases instead of 25 with 1, and 4 % more rows
 constexpr float kCtaDelta = 3.0f;
-constexpr int kLoads = 2;      // 16-byte loads in flight per lane (4: 395 against 298 us for the batch below)
-constexpr int kWarpRows = 64;  // a warp's waiting rows: 31 left over and 32 of the next word
 }  // namespace
 
 struct LightCtaParams {
@@ -32,116 +29,18 @@ struct LightCta {
   uint32_t* dirty;
   uint32_t* wmin;
   uint32_t* whole;  // rows relaxed whole
+
+  // An offer of dist c to v (light_rows); a shorter one makes v dirty.  32-bit shared atomics cost what a
+  // load costs (2.5 cycles a warp, against 9.4 for a 64-bit compare-and-swap and 4.6 for a 64-bit load),
+  // so dists are settled alone and the ties, which need them final anyway, in one pass at the end.
+  __device__ __forceinline__ uint32_t offer(uint32_t v, uint32_t c) const { return atomicMin(dist + v, c); }
+  __device__ __forceinline__ void won(uint32_t v, uint32_t c) const {
+    atomicOr(dirty + (v >> 5), 1u << (v & 31u));
+    atomicMin(wmin + (v >> 5), c);
+  }
+  __device__ __forceinline__ uint32_t dist_of(uint32_t v) const { return dist[v]; }
+  __device__ __forceinline__ void tie_min(uint32_t v, uint32_t t) const { atomicMin(tie + v, t); }
 };
-
-// Shared words that other warps change meanwhile are read through this.
-__device__ __forceinline__ uint32_t word_now(const uint32_t* p) { return *const_cast<const volatile uint32_t*>(p); }
-
-// An offer of dist c to v; a shorter one makes v dirty.  32-bit shared atomics cost what a load costs
-// (2.5 cycles a warp, against 9.4 for a 64-bit compare-and-swap and 4.6 for a 64-bit load), so dists are
-// settled alone and the ties, which need them final anyway, in one pass at the end.
-__device__ __forceinline__ void light_won(const LightCta& s, uint32_t v, uint32_t c, uint32_t& lmin) {
-  atomicOr(s.dirty + (v >> 5), 1u << (v & 31u));
-  atomicMin(s.wmin + (v >> 5), c);
-  lmin = min(lmin, c);
-}
-
-// Relax (with kTies: take the ties of) the listed edges of a warp's rows: get(i) is row i, i < count, as
-// (u, dist[u]) or, where there is nothing to do, (u, kNone).  Four lanes share a row and take four edges
-// each with one 16-byte load, so a warp's load covers 16 edges of 8 rows in 8 pieces of 64 bytes, and
-// 8 kLoads rows are in flight.  Edges whose offer exceeds B are dropped; a row goes on to its next 16
-// edges only if the heaviest of these was of use.  (A lane per edge, 16 lanes per row, took three times the
-// instructions per edge; a lane per row read 32 lines with every load and was bound by the L1.)
-template <bool kTies, class Get>
-__device__ __forceinline__ void light_rows(const LightCta& s, const Get& get, int count, int most, uint32_t B,
-                                           uint32_t bits_u, const uint32_t* __restrict__ edge, uint32_t& lmin) {
-  const int lane = static_cast<int>(threadIdx.x) & 31, sub = lane & 3;
-  const uint32_t umask = (1u << bits_u) - 1u;
-  constexpr int R = kLoads;
-  for (int i0 = 0; i0 < count; i0 += 8 * R) {
-    uint32_t u[R], du[R];
-    bool on[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int i = i0 + 8 * r + (lane >> 2);
-      const uint2 x = get(min(i, count - 1));
-      u[r] = x.x;
-      du[r] = x.y;
-      on[r] = i < count && x.y != kNone;
-    }
-    for (int k0 = 0; k0 < most; k0 += 16) {
-      uint4 x[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        x[r] = on[r] ? __ldg(reinterpret_cast<const uint4*>(edge + u[r] * kLightCap + k0) + sub)
-                     : make_uint4(kNoEdge, kNoEdge, kNoEdge, kNoEdge);
-      uint32_t more = 0;
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const uint32_t e[4] = {x[r].x, x[r].y, x[r].z, x[r].w};
-        uint32_t old[4];
-        bool use = false;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint32_t c = du[r] + (e[q] >> bits_u), v = e[q] & umask;
-          use = e[q] != kNoEdge && c <= B;
-          if (kTies)
-            old[q] = use ? s.dist[v] : 0u;
-          else
-            old[q] = use ? atomicMin(s.dist + v, c) : 0u;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint32_t c = du[r] + (e[q] >> bits_u), v = e[q] & umask;
-          if (kTies) {
-            if (old[q] == c && e[q] != kNoEdge) atomicMin(s.tie + v, light_tie(e[q], u[r], umask));
-          } else if (c < old[q]) {
-            light_won(s, v, c, lmin);
-          }
-        }
-        const uint32_t bal = __ballot_sync(0xffffffffu, use);  // the last of the lane's four edges
-        on[r] = (bal >> (lane | 3)) & 1u;
-        more |= bal & 0x88888888u;
-      }
-      if (more == 0) break;
-    }
-  }
-  __syncwarp();
-}
-
-// The same for row u of dist du from the matrix (one warp).
-template <bool kTies>
-__device__ __forceinline__ void light_whole_row(const LightCta& s, const SolveDesc& d, uint32_t u, uint32_t du,
-                                                uint32_t D, uint32_t& lmin) {
-  const int lane = static_cast<int>(threadIdx.x) & 31;
-  const int nv = static_cast<int>(d.pitch / 4);
-  const int32_t* row = d.W + static_cast<int64_t>(u) * d.pitch;
-  constexpr int R = 4;
-  for (int g0 = lane; g0 < nv; g0 += 32 * R) {
-    int4 x[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-      x[r] = g0 + 32 * r < nv ? ld_stream16(row + 4 * (g0 + 32 * r))
-                              : make_int4(int(kInf), int(kInf), int(kInf), int(kInf));
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const uint32_t w4[4] = {static_cast<uint32_t>(x[r].x), static_cast<uint32_t>(x[r].y),
-                              static_cast<uint32_t>(x[r].z), static_cast<uint32_t>(x[r].w)};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t v = 4 * (g0 + 32 * r) + q, c = du + w4[q];
-        if (w4[q] >= kInf || c > D || v == u) continue;
-        if (kTies) {
-          if (s.dist[v] == c) atomicMin(s.tie + v, static_cast<uint32_t>(light_key(du, w4[q], u, d.bits_u)));
-        } else {
-          const uint32_t old = atomicMin(s.dist + v, c);
-          if (c < old) light_won(s, v, c, lmin);
-        }
-      }
-    }
-  }
-  __syncwarp();
-}
 
 // One phase has one block-wide barrier.  Each warp owns every (THREADS / 32)-th word of 32 nodes: it
 // takes the dirty nodes of its words whose dist lies in the window, gathers them in its own list and
@@ -186,9 +85,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
     const int n = d.n, nwords = (n + 31) / 32;
     const uint32_t bits_u = d.bits_u, umask = (1u << bits_u) - 1u;
     const uint32_t* hmin = d.light + kLightStats;
-    const uint32_t* edge = hmin + light_pad(n);
     const uint32_t hmin_min = ~__ldg(d.light);  // >= INF: every row's list is complete
-    const int most = static_cast<int>(__ldg(d.light + 6));  // edges in the longest list
+    const LightListEdges edges{hmin + light_pad(n), __ldg(d.light + 6)};
     const uint32_t guess = __ldg(d.light + kLightGuess);
     const uint32_t delta = light_delta(d.light, kCtaDelta);
     uint32_t B = hmin_min < kInf && guess > 0 ? guess : kNone;
@@ -219,7 +117,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
       int cnt = 0;  // rows waiting in this warp's list
       auto relax = [&](int have) {
         __syncwarp();
-        light_rows<false>(s, [rows](int i) { return rows[i]; }, have, most, B, bits_u, edge, lmin);
+        light_rows<false>(s, edges, [rows](int i) { return rows[i]; }, have, B, bits_u, lmin);
       };
       auto add = [&](uint32_t take, int wi, uint32_t dv) {  // the nodes `take` of word wi, dv: this lane's dist
         if ((take >> lane) & 1u) rows[cnt + __popc(take & lt)] = make_uint2(static_cast<uint32_t>(32 * wi + lane), dv);
@@ -355,8 +253,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
       uint32_t unused = 0;
       const uint32_t dv = s.dist[32 * wi + lane];
       light_rows<true>(
-          s, [wi, dv](int i) { return make_uint2(32 * wi + i, __shfl_sync(0xffffffffu, dv, i)); }, 32, most, B, bits_u,
-          edge, unused);
+          s, edges, [wi, dv](int i) { return make_uint2(32 * wi + i, __shfl_sync(0xffffffffu, dv, i)); }, 32, B,
+          bits_u, unused);
       for (uint32_t todo = s.whole[wi]; todo; todo &= todo - 1) {
         const int i = __ffs(todo) - 1;
         light_whole_row<true>(s, d, 32 * wi + i, __shfl_sync(0xffffffffu, dv, i), B, unused);

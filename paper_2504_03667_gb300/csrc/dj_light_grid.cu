@@ -27,12 +27,11 @@
 namespace dj {
 
 namespace {
-constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr int kLightGridThreads = 512;
 constexpr int kLightRows = 4;  // rows in flight per lane group
 // delta in units of the listed weights' mean spacing: a wider window means fewer phases and more
-// rows relaxed twice.
-constexpr float kGridDelta = 3.0f;
+// rows relaxed twice (directed n = 32768, 8 edges per node: 90 us with 3, 81 with 8).
+constexpr float kGridDelta = 8.0f;
 }  // namespace
 
 struct LightGridParams {

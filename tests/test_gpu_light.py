@@ -70,6 +70,48 @@ def far_source(n, p, seed):
     return graphgen.EdgeList(n, src, dst, w, True)
 
 
+@pytest.mark.parametrize("n", [2048, 6143, 6145, 8200])
+def test_forms_agree(dj, orc, n):
+    """A solve on an idle stream and solves behind one another on a stream may take different forms
+    (one cluster, every SM); all are Algorithm 1's, into one buffer pair and into their own."""
+    import torch
+    for e in (graphgen.bernoulli(n, 0.2, 1, 1000, n), graphgen.outdeg(n, 5, 1, 500, n + 1)):
+        W = orc.build_matrix(e.n, e.src, e.dst, e.w, e.directed)
+        srcs = [int(x) for x in graphgen.sources(n, 6, 3)]
+        refs = [orc.dijkstra(W, s) for s in srcs]
+        for load in (dj.dj_load_edges, dj.dj_load_edges_csr):
+            g = load(e.n, e.src, e.dst, e.w, e.directed)
+            st = torch.cuda.Stream()
+            D = torch.full((6, n), -5, dtype=torch.int32, device="cuda")
+            P = torch.full((6, n), -5, dtype=torch.int32, device="cuda")
+            torch.cuda.synchronize()
+            for i, s in enumerate(srcs):  # back to back
+                dj.dj_sssp(g, s, D[i], P[i], st)
+            dj.dj_sync(st)
+            for i in range(6):
+                assert np.array_equal(D[i].cpu().numpy(), refs[i][0]) and np.array_equal(P[i].cpu().numpy(), refs[i][1]), i
+            for i, s in enumerate(srcs):  # each alone
+                dj.dj_sssp(g, s, D[0], P[0], st)
+                dj.dj_sync(st)
+                assert np.array_equal(D[0].cpu().numpy(), refs[i][0]) and np.array_equal(P[0].cpu().numpy(), refs[i][1]), i
+            for s in srcs:  # one buffer pair: the last solve wins
+                dj.dj_sssp(g, s, D[0], P[0], st)
+            dj.dj_sync(st)
+            assert np.array_equal(D[0].cpu().numpy(), refs[5][0]) and np.array_equal(P[0].cpu().numpy(), refs[5][1])
+            cg = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(cg, stream=st):
+                for i, s in enumerate(srcs):
+                    dj.dj_sssp(g, s, D[i], P[i], st)
+            D.fill_(-5)
+            torch.cuda.synchronize()
+            cg.replay()
+            torch.cuda.synchronize()
+            for i in range(6):
+                assert np.array_equal(D[i].cpu().numpy(), refs[i][0]) and np.array_equal(P[i].cpu().numpy(), refs[i][1]), i
+            del cg
+            g.free()
+
+
 @pytest.mark.parametrize("n", [700, 3001, 4500])
 def test_rows_relaxed_whole(dj, orc, n):
     check(dj, orc, far_source(n, 0.4, n), [0, 1, n // 2], f"far source n={n}")
