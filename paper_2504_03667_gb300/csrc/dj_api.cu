@@ -266,6 +266,9 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   const bool cta = !csr && g->light_cta && g->n < kLightClusterMinN && light_cta_fits(g->n);
   const bool cluster = !cta && (csr ? g->light_longest <= kLightClusterMaxRow : g->light_cta) &&
                        light_cluster_fits(g->n, C, csr);
+  if (cluster) {  // whichever form this call takes: a later one may be captured
+    if (int rc = prepare_light_cluster(csr, C)) return rc;
+  }
   if (!cta && (!cluster || o.debug_skip_cta >= 0 ||
                (g->n >= (csr ? kLightIdleGridMinNComplete : kLightIdleGridMinN) && stream_idle(st))))
     return launch_light_grid(g, source, dist, pred, o, nullptr, st);

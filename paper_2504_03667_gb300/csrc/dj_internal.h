@@ -68,7 +68,7 @@ constexpr int kLightStats = 64;  // leading words: [0] ~(smallest hmin), [1] row
                                  // [6] most edges listed in a row, [8..11] ~(finite min), finite max, finite entries
                                  // (at load), [12..14] the edge list's check (k_scatter),
                                  // [15] kLightGuess
-constexpr int kLightGuess = 15;  // a little above the trial solve's largest dist (0: unknown)
+constexpr int kLightGuess = 15;  // 1 + the trial solve's largest dist (0: unknown)
 inline
 #ifdef __CUDACC__
     __host__ __device__
@@ -278,6 +278,7 @@ int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases
 int run_light_serve(const LightPlan& plan, const ServeRing& r, cudaStream_t st);
 // One solve on one cluster of C CTAs (a power of two up to 16), as run_light_single.
 bool light_cluster_fits(int32_t n, int C, bool csr);
+int prepare_light_cluster(bool csr, int C);  // its launch attributes, before a capture may need them
 int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t* phases_out, bool early,
                       cudaStream_t st);
 // One solve over every SM (a graph with an index, or in compressed rows).

@@ -18,6 +18,7 @@ struct BatchJobs {
   }
   __device__ SolveDesc desc(uint32_t job) const { return descs[job]; }
   __device__ void complete(uint32_t, uint32_t) const {}
+  static constexpr uint32_t kGuessPart = 3;  // light engine: the margin of its bound (light_guess)
   static constexpr bool kTrace = false;
   __device__ bool early() const { return true; }  // launched the ordinary way: nothing to wait for
   __device__ void before_write() const {}
@@ -56,6 +57,7 @@ struct SingleJob {
   __device__ void complete(uint32_t, uint32_t phases) const {
     if (phases_out) *phases_out = phases;
   }
+  static constexpr uint32_t kGuessPart = 8;
   static constexpr bool kTrace = true;  // the per-phase timeline is compiled into this kernel only
   __device__ bool early() const { return early_ok != 0; }
   __device__ void before_write() const { pdl_wait(); }
@@ -107,6 +109,7 @@ struct ServeJobs {
     __threadfence_system();
     st_release_sys(done + (job & cap_mask), job + 1);
   }
+  static constexpr uint32_t kGuessPart = 8;
   static constexpr bool kTrace = false;
   __device__ bool early() const { return true; }
   __device__ void before_write() const {}

@@ -26,6 +26,7 @@
 
 namespace dj {
 
+constexpr uint32_t kNone = 0xFFFFFFFFu;    // no dist, no bound
 constexpr uint32_t kNoEdge = 0xFFFFFFFFu;  // an unused slot of a row's list (no edge packs to all ones)
 
 __device__ __forceinline__ uint32_t weight_field(uint32_t bits_u) { return 0xFFFFFFFFu >> bits_u; }
@@ -54,6 +55,13 @@ __device__ __forceinline__ uint32_t light_delta(const uint32_t* light, float c) 
   int unused;
   light_window(light, c, &delta, &unused);
   return delta;
+}
+
+// A guess of the largest dist, from the trial solve's (word kLightGuess): that and 1 / part of it more,
+// no guess without one.
+__device__ __forceinline__ uint32_t light_guess(const uint32_t* light, uint32_t part) {
+  const uint32_t x = __ldg(light + kLightGuess);
+  return x == 0 ? kNone : x - 1 + max(1u, (x - 1) / part);
 }
 
 // Per-warp selection of a row's lightest edges.  scan(f, pass) must call f(c0, x) for every group of
@@ -160,7 +168,6 @@ __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, u
 
 // ------------------------------------------------------------------ relaxing rows from shared memory
 
-constexpr uint32_t kNone = 0xFFFFFFFFu;  // no dist, no bound
 constexpr int kWarpRows = 64;            // a warp's waiting rows: 31 left over and 32 of the next word
 
 // Shared words that other warps change meanwhile are read through this.

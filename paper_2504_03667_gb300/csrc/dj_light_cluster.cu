@@ -121,10 +121,9 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
   const uint32_t bits_u = d.bits_u, umask = (1u << bits_u) - 1u;
   const uint32_t* hmin = CSR ? nullptr : d.light + kLightStats;
   const uint32_t hmin_min = CSR ? kInf : ~__ldg(d.light);  // >= INF: every row's list is complete
-  const uint32_t guess = CSR ? 0u : __ldg(d.light + kLightGuess);
   const uint32_t most = CSR ? kNone : __ldg(d.light + 6);  // edges in the longest list
   const uint32_t delta = CSR ? p.delta : light_delta(d.light, kClDelta);
-  uint32_t B = hmin_min < kInf && guess > 0 ? guess : kNone;
+  uint32_t B = hmin_min < kInf ? light_guess(d.light, 8) : kNone;
   auto global_word = [&](int lw) { return (lw << p.cshift) + static_cast<int>(rank); };
 
   for (int lw = warp; lw < LW; lw += kClWarps) {
@@ -319,6 +318,13 @@ bool light_cluster_fits(int32_t n, int C, bool csr) {
   DevCtx* ctx = nullptr;
   if (get_ctx(&ctx) != DJ_OK) return false;
   return ctx->cluster_launch && light_cluster_smem(n, C, csr) + 10 * 1024 <= static_cast<size_t>(ctx->max_smem_optin);
+}
+
+int prepare_light_cluster(bool csr, int C) {
+  DevCtx* ctx = nullptr;
+  if (int rc = get_ctx(&ctx)) return rc;
+  return prepare_function(ctx, csr ? reinterpret_cast<void*>(&k_light_cluster<true>) : reinterpret_cast<void*>(&k_light_cluster<false>),
+                          0, C > 8);
 }
 
 int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t* phases_out, bool early,

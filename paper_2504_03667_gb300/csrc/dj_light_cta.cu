@@ -47,8 +47,8 @@ struct LightCta {
 // relaxes their rows 32 at a time, while other warps may already make more of them dirty -- those go
 // along if their word is still to come, else in a later phase.
 //
-// Rows are first relaxed up to a bound B on the offers: a little above the largest dist of the graph's
-// trial solve (word 15 of the index), which holds for most sources.  When nothing is dirty the true
+// Rows are first relaxed up to a bound B on the offers: somewhat above the largest dist of the graph's
+// trial solve (light_guess), which holds for most sources.  When nothing is dirty the true
 // largest dist D is taken; if it is above B every row is relaxed once more up to D.  Dropping offers
 // above the largest dist leaves 13 of the 64 listed edges per row for n = 8192, p = 0.05; waiting for D
 // to be known first left 37.
@@ -87,9 +87,10 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
     const uint32_t* hmin = d.light + kLightStats;
     const uint32_t hmin_min = ~__ldg(d.light);  // >= INF: every row's list is complete
     const LightListEdges edges{hmin + light_pad(n), __ldg(d.light + 6)};
-    const uint32_t guess = __ldg(d.light + kLightGuess);
     const uint32_t delta = light_delta(d.light, kCtaDelta);
-    uint32_t B = hmin_min < kInf && guess > 0 ? guess : kNone;
+    // a wide margin in batches: one takes as long as its slowest solve, one whose bound was too low (256 sources of
+    // n = 8192: 296 us with an eighth, 285 with a quarter, 261 with 3/8)
+    uint32_t B = hmin_min < kInf ? light_guess(d.light, Jobs::kGuessPart) : kNone;
 
     for (int wi = warp; wi < nwords; wi += NW) {
       const int v = 32 * wi + lane;
@@ -301,18 +302,19 @@ bool light_cta_fits(int32_t n) {
 
 // CTAs of 512 threads, one per SM; two per SM in batches with more solves than SMs where shared memory
 // allows (256 sources of n = 8192: 298 us, 354 with one; 48 graphs, which have an SM each, 112 with the
-// registers of one, 129 with those of two).  The server's persistent CTAs have 256 threads, one per SM:
+// registers of one, 129 with those of two).  The server's persistent CTAs have 192 threads, one per SM:
 // other kernels must find room beside them for as long as the server runs (two CTAs of 512 threads fill
-// every register of an SM, and a caller's own kernels waited until the server left).
+// every register of an SM, and a caller's own kernels waited until the server left).  Its rate is the
+// host's (1500 waiting requests: 3.4 ms with 192 threads, 3.3 with 256, 3.1 with 512).
 int plan_light(int32_t max_n, int32_t k, int kind, LightPlan* plan) {
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   plan->smem = light_cta_smem(max_n);
   plan->npad = light_pad(max_n);
-  plan->threads = kind == kJobsServe ? 256 : 512;
+  plan->threads = kind == kJobsServe ? 192 : 512;
   const bool two = kind == kJobsBatch && k > ctx->num_sms &&
                    2 * (plan->smem + kLightCtaStatic) <= static_cast<size_t>(ctx->max_smem_optin);
-  plan->fn = kind == kJobsServe    ? reinterpret_cast<void*>(&k_light_cta<256, 1, ServeJobs>)
+  plan->fn = kind == kJobsServe    ? reinterpret_cast<void*>(&k_light_cta<192, 1, ServeJobs>)
              : kind == kJobsSingle ? reinterpret_cast<void*>(&k_light_cta<512, 1, SingleJob>)
              : two                 ? reinterpret_cast<void*>(&k_light_cta<512, 2, BatchJobs>)
                                    : reinterpret_cast<void*>(&k_light_cta<512, 1, BatchJobs>);

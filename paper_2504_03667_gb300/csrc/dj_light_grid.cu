@@ -179,8 +179,7 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
   if (!CSR) light_window(p.light, kGridDelta, &delta, &gshift);
   if (!CSR && p.trial && hmin_min >= kInf) return;
   // offers above the guessed largest dist are dropped at first (see below); the trial makes the guess
-  uint32_t guess = CSR || p.trial || hmin_min >= kInf ? kNone : __ldg(p.light + kLightGuess);
-  if (guess == 0) guess = kNone;
+  uint32_t guess = CSR || p.trial || hmin_min >= kInf ? kNone : light_guess(p.light, 8);
   for (int j = tid; j < sw; j += T0) {
     const int v = c0 + j;
     p.gkey[v] = v == p.source ? 0ull : ~0ull;
@@ -373,7 +372,7 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
     if (!p.trial)
       p.words[1] = phases;
     else if (D < kInf)
-      p.guess[0] = D + D / 8 + 1;
+      p.guess[0] = D + 1;
   }
 }
 
