@@ -245,27 +245,25 @@ __device__ __forceinline__ void light_rows(const Store& s, const Edges& edges, c
   __syncwarp();
 }
 
-// The same for row u of dist du from the matrix (one warp).
+// The same for a piece of row u, of dist du, from the matrix: 16-byte groups [g0, g1) (one warp).
 template <bool kTies, class Store>
-__device__ __forceinline__ void light_whole_row(const Store& s, const SolveDesc& d, uint32_t u, uint32_t du,
-                                                uint32_t D, uint32_t& lmin) {
+__device__ __forceinline__ void light_matrix_row(const Store& s, const SolveDesc& d, uint32_t u, uint32_t du, int g0,
+                                                 int g1, uint32_t D, uint32_t& lmin) {
   const int lane = static_cast<int>(threadIdx.x) & 31;
-  const int nv = static_cast<int>(d.pitch / 4);
   const int32_t* row = d.W + static_cast<int64_t>(u) * d.pitch;
   constexpr int R = 4;
-  for (int g0 = lane; g0 < nv; g0 += 32 * R) {
+  for (int g = g0 + lane; g < g1; g += 32 * R) {
     int4 x[R];
 #pragma unroll
     for (int r = 0; r < R; ++r)
-      x[r] = g0 + 32 * r < nv ? ld_stream16(row + 4 * (g0 + 32 * r))
-                              : make_int4(int(kInf), int(kInf), int(kInf), int(kInf));
+      x[r] = g + 32 * r < g1 ? ld_stream16(row + 4 * (g + 32 * r)) : make_int4(int(kInf), int(kInf), int(kInf), int(kInf));
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const uint32_t w4[4] = {static_cast<uint32_t>(x[r].x), static_cast<uint32_t>(x[r].y),
                               static_cast<uint32_t>(x[r].z), static_cast<uint32_t>(x[r].w)};
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const uint32_t v = 4 * (g0 + 32 * r) + q, c = du + w4[q];
+        const uint32_t v = 4 * (g + 32 * r) + q, c = du + w4[q];
         if (w4[q] >= kInf || c > D || v == u) continue;
         if (kTies) {
           if (s.dist_of(v) == c) s.tie_min(v, static_cast<uint32_t>(light_key(du, w4[q], u, d.bits_u)));
@@ -279,6 +277,34 @@ __device__ __forceinline__ void light_whole_row(const Store& s, const SolveDesc&
     }
   }
   __syncwarp();
+}
+
+// Rows relaxed whole are cut into pieces of this many 16-byte groups, which the CTA's warps take in turn
+// (one warp per row of 16384 columns took 32 us a row).
+constexpr int kRowPiece = 256;
+template <class Store>
+__device__ __forceinline__ void light_whole_rows(const Store& s, const SolveDesc& d, const uint2* list, int count,
+                                                 uint32_t D, uint32_t& lmin) {
+  const int nv = static_cast<int>(d.pitch / 4), pieces = (nv + kRowPiece - 1) / kRowPiece;
+  for (int it = static_cast<int>(threadIdx.x >> 5); it < count * pieces; it += static_cast<int>(blockDim.x >> 5)) {
+    const uint2 x = list[it / pieces];
+    const int g0 = (it % pieces) * kRowPiece;
+    light_matrix_row<false>(s, d, x.x, x.y, g0, min(nv, g0 + kRowPiece), D, lmin);
+  }
+}
+// Their ties: row(word, bit) is the row of a bit of whole[word] with its dist.
+template <class Store, class Row>
+__device__ __forceinline__ void light_whole_ties(const Store& s, const SolveDesc& d, const uint32_t* whole, int words,
+                                                 const Row& row, uint32_t B) {
+  const int nv = static_cast<int>(d.pitch / 4);
+  uint32_t unused = 0;
+  for (int w = 0; w < words; ++w)
+    for (uint32_t todo = whole[w]; todo; todo &= todo - 1) {
+      const uint2 x = row(w, __ffs(todo) - 1);
+      for (int g0 = static_cast<int>(threadIdx.x >> 5) * kRowPiece; g0 < nv;
+           g0 += static_cast<int>(blockDim.x >> 5) * kRowPiece)
+        light_matrix_row<true>(s, d, x.x, x.y, g0, min(nv, g0 + kRowPiece), B, unused);
+    }
 }
 
 }  // namespace dj

@@ -100,7 +100,7 @@ template <bool CSR>
 __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClusterParams p) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ uint2 s_rows[kClWarps][kWarpRows];
-  __shared__ uint32_t s_m[3], s_D, s_bound;
+  __shared__ uint32_t s_m[3], s_D, s_bound, s_cnt, s_end;
   const uint32_t rank = cluster_rank(), C = 1u << p.cshift;
   const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
   const uint32_t lt = (1u << lane) - 1u;
@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
   };
   uint32_t phase = 0, cur = 0;  // cur = phase % 3: the slot of this phase's m, the smallest dirty dist
   int raised = 0;
+  bool any_whole = false;
   for (;; ++phase) {
     const uint32_t m = s_m[cur];  // every rank has the same
     const uint32_t nxt = cur == 2 ? 0 : cur + 1;
@@ -219,6 +220,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
       if (tid == 0) {
         s_D = 0;
         s_bound = kNone;
+        s_cnt = 0;
+        s_end = kClWarps * kWarpRows;
       }
       cluster_sync_all();
       uint32_t D = 0;
@@ -246,34 +249,38 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
         // the index proves the answer, or some rows are relaxed whole, a warp per row
         if (hmin_min > D) break;
         B = D;
-        uint32_t hb = kNone;  // the smallest dist + hmin of the pending rows
-        for (int lw = warp; lw < LW; lw += kClWarps) {
-          const uint32_t dv = dist[32 * lw + lane];
-          if (dv == kNone || ((whole[lw] >> lane) & 1u)) continue;
+        auto pending = [&](int lw, uint32_t dv) {  // dist + hmin of this lane's node if its row is pending
+          if (dv == kNone || ((whole[lw] >> lane) & 1u)) return kNone;
           const uint32_t x = dv + __ldg(hmin + 32 * global_word(lw) + lane);
-          if (x <= D && x < kInf) hb = min(hb, x);
-        }
+          return x <= D && x < kInf ? x : kNone;
+        };
+        uint32_t hb = kNone;  // the smallest dist + hmin of the pending rows
+        for (int lw = warp; lw < LW; lw += kClWarps) hb = min(hb, pending(lw, dist[32 * lw + lane]));
         hb = warp_min_u32(hb);
         if (lane < static_cast<int>(C) && hb != kNone) LightClusterStore::red_min(s.at(smem_u32(&s_bound), lane, 0), hb);
         __syncwarp();
         cluster_sync_all();
         hb = s_bound;
         if (hb == kNone) break;
+        // those below it are final: relaxed whole, as many as the list holds now
         for (int lw = warp; lw < LW; lw += kClWarps) {
-          const uint32_t dv = word_now(dist + 32 * lw + lane);
-          bool go = dv < hb && !((whole[lw] >> lane) & 1u);  // final, whatever others offer meanwhile
-          if (go) {
-            const uint32_t x = dv + __ldg(hmin + 32 * global_word(lw) + lane);
-            go = x <= D && x < kInf;
+          const uint32_t dv = dist[32 * lw + lane];
+          const bool go = dv < hb && pending(lw, dv) != kNone;
+          const uint32_t todo = __ballot_sync(0xffffffffu, go);
+          if (todo == 0) continue;
+          uint32_t pos = 0;
+          if (lane == 0) pos = atomicAdd(&s_cnt, static_cast<uint32_t>(__popc(todo)));
+          pos = __shfl_sync(0xffffffffu, pos, 0);
+          if (pos + __popc(todo) > kClWarps * kWarpRows) {
+            if (lane == 0) atomicMin(&s_end, pos);
+            continue;
           }
-          uint32_t todo = __ballot_sync(0xffffffffu, go);
-          __syncwarp();
+          if (go) s_rows[0][pos + __popc(todo & lt)] = make_uint2(static_cast<uint32_t>(32 * global_word(lw) + lane), dv);
           if (lane == 0) whole[lw] |= todo;
-          for (; todo; todo &= todo - 1) {
-            const int i = __ffs(todo) - 1;
-            light_whole_row<false>(s, d, 32 * global_word(lw) + i, __shfl_sync(0xffffffffu, dv, i), D, lmin);
-          }
         }
+        cluster_sync_all();  // the lists are complete, and every rank has taken its own before dists change
+        any_whole = true;
+        light_whole_rows(s, d, s_rows[0], static_cast<int>(min(s_cnt, s_end)), D, lmin);
       }
     }
     lmin = warp_min_u32(lmin);
@@ -289,12 +296,11 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
     const int v0 = 32 * global_word(lw);
     const uint32_t dv = dist[32 * lw + lane];
     run_rows(std::true_type{}, [v0, dv](int i) { return make_uint2(v0 + i, __shfl_sync(0xffffffffu, dv, i)); }, 32, unused);
-    if (!CSR)
-      for (uint32_t todo = whole[lw]; todo; todo &= todo - 1) {
-        const int i = __ffs(todo) - 1;
-        light_whole_row<true>(s, d, v0 + i, __shfl_sync(0xffffffffu, dv, i), B, unused);
-      }
   }
+  if (any_whole)
+    light_whole_ties(
+        s, d, whole, LW,
+        [&](int lw, int i) { return make_uint2(static_cast<uint32_t>(32 * global_word(lw) + i), dist[32 * lw + i]); }, B);
   cluster_sync_all();  // every offer has arrived; nobody touches another CTA's memory from here on
   pdl_wait();          // results reach memory in stream order
   for (int lw = warp; lw < LW; lw += kClWarps) {

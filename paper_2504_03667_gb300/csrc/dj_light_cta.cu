@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
     k_light_cta(const LightCtaParams p, const Jobs jobs) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ uint2 s_rows[THREADS / 32][kWarpRows];
-  __shared__ uint32_t s_job, s_bound, s_m[3];
+  __shared__ uint32_t s_job, s_bound, s_cnt, s_end, s_m[3];
   LightCta s;
   s.dist = reinterpret_cast<uint32_t*>(smem);
   s.tie = s.dist + p.npad;
@@ -110,6 +110,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
     __syncthreads();
     uint32_t phase = 0, cur = 0;  // cur = phase % 3: the slot of this phase's m, the smallest dirty dist
     int raised = 0;
+    bool any_whole = false;
     for (;; ++phase) {
       const uint32_t m = s_m[cur];
       const uint32_t nxt = cur == 2 ? 0 : cur + 1;
@@ -207,40 +208,45 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
           if (hmin_min > D) break;
           B = D;
           __syncthreads();  // everyone has read s_bound
-          if (tid == 0) s_bound = kNone;  // the smallest dist + hmin of the pending rows
-          __syncthreads();
-          uint32_t hb = kNone;
-          for (int wi = warp; wi < nwords; wi += NW) {
-            const int v = 32 * wi + lane;
-            const uint32_t dv = word_now(s.dist + v);
-            if (dv >= kInf || ((s.whole[wi] >> lane) & 1u)) continue;
-            const uint32_t x = dv + __ldg(hmin + v);
-            if (x <= D && x < kInf) hb = min(hb, x);
+          if (tid == 0) {
+            s_bound = kNone;  // the smallest dist + hmin of the pending rows
+            s_cnt = 0;
+            s_end = NW * kWarpRows;
           }
+          __syncthreads();
+          auto pending = [&](int wi, uint32_t dv) {  // dist + hmin of this lane's node if its row is pending
+            if (dv == kNone || ((s.whole[wi] >> lane) & 1u)) return kNone;
+            const uint32_t x = dv + __ldg(hmin + 32 * wi + lane);
+            return x <= D && x < kInf ? x : kNone;
+          };
+          uint32_t hb = kNone;
+          for (int wi = warp; wi < nwords; wi += NW) hb = min(hb, pending(wi, s.dist[32 * wi + lane]));
           hb = warp_min_u32(hb);
           if (lane == 0 && hb != kNone) atomicMin(&s_bound, hb);
           __syncthreads();
           hb = s_bound;
           if (hb == kNone) break;
+          // those below it are final: relaxed whole, as many as the list holds now
           for (int wi = warp; wi < nwords; wi += NW) {
-            const int v = 32 * wi + lane;
-            const uint32_t dv = word_now(s.dist + v);
-            bool go = dv < hb && !((s.whole[wi] >> lane) & 1u);  // final, whatever others offer meanwhile
-            if (go) {
-              const uint32_t x = dv + __ldg(hmin + v);
-              go = x <= D && x < kInf;
+            const uint32_t dv = s.dist[32 * wi + lane];
+            const bool go = dv < hb && pending(wi, dv) != kNone;
+            const uint32_t todo = __ballot_sync(0xffffffffu, go);
+            if (todo == 0) continue;
+            uint32_t pos = 0;
+            if (lane == 0) pos = atomicAdd(&s_cnt, static_cast<uint32_t>(__popc(todo)));
+            pos = __shfl_sync(0xffffffffu, pos, 0);
+            if (pos + __popc(todo) > NW * kWarpRows) {
+              if (lane == 0) atomicMin(&s_end, pos);
+              continue;
             }
-            uint32_t todo = __ballot_sync(0xffffffffu, go);
-            __syncwarp();
-            if (lane == 0) {
-              s.whole[wi] |= todo;
-              if (p.heavy && todo) atomicAdd(p.heavy, static_cast<uint32_t>(__popc(todo)));
-            }
-            for (; todo; todo &= todo - 1) {
-              const int i = __ffs(todo) - 1;
-              light_whole_row<false>(s, d, 32 * wi + i, __shfl_sync(0xffffffffu, dv, i), D, lmin);
-            }
+            if (go) s_rows[0][pos + __popc(todo & lt)] = make_uint2(static_cast<uint32_t>(32 * wi + lane), dv);
+            if (lane == 0) s.whole[wi] |= todo;
           }
+          __syncthreads();
+          any_whole = true;
+          const int count = static_cast<int>(min(s_cnt, s_end));
+          if (p.heavy && tid == 0) atomicAdd(p.heavy, static_cast<uint32_t>(count));
+          light_whole_rows(s, d, s_rows[0], count, D, lmin);
         }
       }
       lmin = warp_min_u32(lmin);
@@ -256,11 +262,11 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
       light_rows<true>(
           s, edges, [wi, dv](int i) { return make_uint2(32 * wi + i, __shfl_sync(0xffffffffu, dv, i)); }, 32, B,
           bits_u, unused);
-      for (uint32_t todo = s.whole[wi]; todo; todo &= todo - 1) {
-        const int i = __ffs(todo) - 1;
-        light_whole_row<true>(s, d, 32 * wi + i, __shfl_sync(0xffffffffu, dv, i), B, unused);
-      }
     }
+    if (any_whole)
+      light_whole_ties(
+          s, d, s.whole, nwords,
+          [&s](int w, int i) { return make_uint2(static_cast<uint32_t>(32 * w + i), s.dist[32 * w + i]); }, B);
     __syncthreads();
     jobs.before_write();  // results reach memory in stream order
     for (int v = tid; v < n; v += THREADS) {

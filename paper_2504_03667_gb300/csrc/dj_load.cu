@@ -604,12 +604,12 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   // Taken at once if every row's list is complete, else if a trial solve relaxed next to no row whole:
   // where many are needed (nearly equal weights, distances long against what the lists reach) the other
   // engines stream the matrix better (n = 8192, p = 0.5, weights 1..10: 410 rows whole, 112 us; grid
-  // engine 37).  One CTA relaxes whole rows slowly (4500 of them in 7 ms, the grid form in 0.2), so its
-  // form is for complete lists, or symmetric matrices without one in the trial: no source's largest
-  // dist is then more than twice the trial's, while a directed graph's may be by any factor.
+  // engine 37).  One CTA or cluster relaxes many whole rows slowly (4500 in 7 ms, the grid form in 0.2),
+  // so these forms are for complete lists and symmetric matrices: no source's largest dist is then more
+  // than twice the trial's, while a directed graph's may be by any factor.
   const bool complete = ~idx[0] >= kInf;
   g->light_ok = tried && g->wmin >= 1 && (complete || idx[1] <= 4);
-  g->light_cta = g->light_ok && (complete || (!g->directed && idx[1] == 0));
+  g->light_cta = g->light_ok && (complete || !g->directed);
   // graphs that are not dense keep in-lists for the grid engine's dynamic IN bound
   const uint64_t nn = static_cast<uint64_t>(g->n) * static_cast<uint64_t>(g->n);
   if (g->entries * 32 < nn && g->wmin >= 1 && !g->inlist) {
