@@ -278,7 +278,12 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   // right after an upload the solve waits for the kernels before it before reading the graph
   const bool early = g->upload_pending == 0;
   const_cast<dj_graph*>(g)->upload_pending = 0;
-  if (cluster) return run_light_cluster(g, C, d, ctx->words + 1, early, st);
+  if (cluster) {
+    const int rc = run_light_cluster(g, C, d, ctx->words + 1, early, st);
+    if (rc != DJ_ECUDA) return rc;
+    clear_error();  // no such cluster here
+    return launch_light_grid(g, source, dist, pred, o, nullptr, st);
+  }
   LightPlan plan;
   if (int rc = plan_light(g->n, 1, kJobsSingle, &plan)) return rc;
   return run_light_single(plan, d, ctx->words + 1, nullptr, early, st);

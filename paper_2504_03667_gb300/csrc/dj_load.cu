@@ -75,17 +75,32 @@ __global__ void __launch_bounds__(256) k_scatter(int32_t* __restrict__ W, int64_
   if ((threadIdx.x & 31) == 0 && wmax > 0) atomicMax(check + 2, static_cast<uint32_t>(wmax));
 }
 
-// Copy a dense matrix with row stride ld into the padded layout, checking every
-// entry lies in [0, INF]; bad entries set flags[0].
-__global__ void k_copy_dense(int32_t* __restrict__ W, int64_t pitch, const int32_t* __restrict__ A, int64_t ld,
-                             int32_t n, uint32_t* flags) {
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < static_cast<int64_t>(n) * n;
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t r = i / n, c = i - r * n;
-    const int32_t x = A[r * ld + c];
-    if (x < 0 && flags) atomicOr(flags, 1u);
-    W[r * pitch + c] = x;
+// Copy a dense matrix with row stride ld into the padded layout (padding columns INF), checking every
+// entry lies in [0, INF]; bad entries set flags[0].  A block per row at a time, in 16-byte pieces where A
+// allows them (vec): n = 16384 (1 GiB read, 1 GiB written) was bound by a 64-bit division per entry.
+__global__ void __launch_bounds__(256) k_copy_dense(int32_t* __restrict__ W, int64_t pitch, const int32_t* __restrict__ A,
+                                                    int64_t ld, int32_t n, int vec, uint32_t* flags) {
+  uint32_t sign = 0;  // the entries' top bits
+  for (int64_t r = blockIdx.x; r < n; r += gridDim.x) {
+    const int32_t* a = A + r * ld;
+    int32_t* d = W + r * pitch;
+    int c0 = 0;
+    if (vec) {
+      const int nq = n / 4;
+      for (int q = threadIdx.x; q < nq; q += 256) {
+        const int4 x = reinterpret_cast<const int4*>(a)[q];
+        sign |= static_cast<uint32_t>(x.x | x.y | x.z | x.w);
+        reinterpret_cast<int4*>(d)[q] = x;
+      }
+      c0 = 4 * nq;
+    }
+    for (int c = c0 + static_cast<int>(threadIdx.x); c < pitch; c += 256) {
+      const int32_t x = c < n ? a[c] : static_cast<int32_t>(kInf);
+      sign |= static_cast<uint32_t>(x);
+      d[c] = x;
+    }
   }
+  if (sign >> 31) atomicOr(flags, 1u);
 }
 
 // One warp per row: minout[u] = min finite W[u][v], v != u; plus the global
@@ -150,9 +165,27 @@ struct LightSums {
 // uniform up to the largest (of the edge list: word 14), with deg edges per row.  A warp has only a few
 // rows, so a bad guess costs scans: 8192 rows of 4096 edges took 265 us from 0 and take 98 us, against
 // 125 us for the row minima and tie sources this pass replaces.
-__device__ __forceinline__ uint32_t first_threshold(const LightOut& o) {
-  const float want = 2.25f * kLightCap, wmax = static_cast<float>(o.wmax ? o.wmax : o.light[14]);
-  return static_cast<uint32_t>(fminf(2.0e9f, o.deg <= want ? (o.deg > 0.f ? wmax : 0.f) : wmax * want / o.deg));
+// Where deg is not known (a matrix was loaded), the warp takes both from the first columns of its first row.
+__device__ __forceinline__ uint32_t first_threshold(const LightOut& o, const int32_t* row = nullptr) {
+  float deg = o.deg, wmax = static_cast<float>(o.wmax ? o.wmax : o.light[14]);
+  if (deg == 0.f && row) {
+    const int c1 = min(o.n, 1024);
+    float sum = 0.f;
+    uint32_t cnt = 0;
+    for (int c = static_cast<int>(threadIdx.x) & 31; c < c1; c += 32) {
+      const uint32_t w = static_cast<uint32_t>(row[c]);
+      if (w > 0 && w < kInf) {
+        sum += static_cast<float>(w);
+        ++cnt;
+      }
+    }
+    for (int k = 16; k > 0; k >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, k);
+    cnt = warp_sum_u32(cnt);
+    deg = static_cast<float>(cnt) / static_cast<float>(c1) * static_cast<float>(o.n);
+    wmax = cnt ? 2.f * sum / static_cast<float>(cnt) : 2.0e9f;
+  }
+  const float want = 2.25f * kLightCap;
+  return static_cast<uint32_t>(fminf(2.0e9f, deg <= want ? wmax : wmax * want / deg));
 }
 
 template <class Scan>
@@ -194,7 +227,7 @@ __global__ void __launch_bounds__(256) k_light_rows(const int32_t* __restrict__ 
   const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
   const int64_t nq = pitch / 4;
-  uint32_t thr = first_threshold(o), gmin = kInf, gmax = 0;
+  uint32_t thr = first_threshold(o, warp < o.n ? W + warp * pitch : nullptr), gmin = kInf, gmax = 0;
   unsigned long long cnt = 0;
   LightSums sums;
   for (int64_t u = warp; u < o.n; u += nwarps) {
@@ -468,12 +501,12 @@ __global__ void k_pad_cols(int32_t* __restrict__ W, int64_t pitch, int32_t n) {
 }
 
 // flags[0] |= 1 if any of the n x n entries is negative.
-__global__ void k_check_nonneg(const int32_t* __restrict__ W, int64_t pitch, int32_t n, uint32_t* flags) {
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < static_cast<int64_t>(n) * n;
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t r = i / n;
-    if (W[r * pitch + (i - r * n)] < 0) atomicOr(flags, 1u);
-  }
+__global__ void __launch_bounds__(256) k_check_nonneg(const int32_t* __restrict__ W, int64_t pitch, int32_t n,
+                                                      uint32_t* flags) {
+  uint32_t sign = 0;
+  for (int64_t r = blockIdx.x; r < n; r += gridDim.x)
+    for (int c = threadIdx.x; c < n; c += 256) sign |= static_cast<uint32_t>(W[r * pitch + c]);
+  if (sign >> 31) atomicOr(flags, 1u);
 }
 
 }  // namespace dj
@@ -737,28 +770,23 @@ extern "C" int dj_load_edges(int32_t n, int64_t m, const int32_t* src, const int
   return DJ_OK;
 }
 
-static int copy_dense_in(dj_graph* g, const int32_t* W, int64_t ld, int w_on_device, bool check, cudaStream_t st) {
+static int copy_dense_in(dj_graph* g, const int32_t* W, int64_t ld, int w_on_device, cudaStream_t st) {
   const int32_t n = g->n;
   uint32_t* flags = nullptr;
-  cudaError_t e;
-  if (check) {
-    e = cudaMallocAsync(&flags, sizeof(uint32_t), st);
-    if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync(flags)");
-    cudaMemsetAsync(flags, 0, sizeof(uint32_t), st);
-  }
+  cudaError_t e = cudaMallocAsync(&flags, sizeof(uint32_t), st);
+  if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync(flags)");
+  cudaMemsetAsync(flags, 0, sizeof(uint32_t), st);
   if (w_on_device) {
-    k_copy_dense<<<grid_for(static_cast<int64_t>(n) * n), 256, 0, st>>>(g->W, g->pitch, W, ld, n,
-                                                                         flags ? flags : nullptr);
+    const int vec = ld % 4 == 0 && reinterpret_cast<uintptr_t>(W) % 16 == 0;
+    k_copy_dense<<<std::min(n, 152 * 16), 256, 0, st>>>(g->W, g->pitch, W, ld, n, vec, flags);
   } else {
     e = cudaMemcpy2DAsync(g->W, static_cast<size_t>(g->pitch) * sizeof(int32_t), W,
                           static_cast<size_t>(ld) * sizeof(int32_t), static_cast<size_t>(n) * sizeof(int32_t),
                           static_cast<size_t>(n), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_error(e, "cudaMemcpy2DAsync(host matrix)");
-    if (check) k_check_nonneg<<<grid_for(static_cast<int64_t>(n) * n), 256, 0, st>>>(g->W, g->pitch, n, flags);
+    k_check_nonneg<<<std::min(n, 152 * 16), 256, 0, st>>>(g->W, g->pitch, n, flags);
+    if (g->pitch > n) k_pad_cols<<<grid_for(static_cast<int64_t>(g->pitch - n) * n), 256, 0, st>>>(g->W, g->pitch, n);
   }
-  if (g->pitch > n)
-    k_pad_cols<<<grid_for(static_cast<int64_t>(g->pitch - n) * n), 256, 0, st>>>(g->W, g->pitch, n);
-  if (!check) return DJ_OK;
   uint32_t bad = 0;
   cudaMemcpyAsync(&bad, flags, sizeof(bad), cudaMemcpyDeviceToHost, st);
   cudaFreeAsync(flags, st);
@@ -779,7 +807,7 @@ extern "C" int dj_load_dense(int32_t n, const int32_t* W, int64_t ld, int w_on_d
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   dj_graph* g = nullptr;
   if (int rc = alloc_graph(n, 1, &g)) return rc;
-  if (int rc = copy_dense_in(g, W, ld, w_on_device, true, st)) {
+  if (int rc = copy_dense_in(g, W, ld, w_on_device, st)) {
     dj_graph_free(g);
     return rc;
   }

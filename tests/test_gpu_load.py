@@ -49,3 +49,34 @@ def test_first_bad_edge_is_named(dj, at):
         with pytest.raises(dj.DjError) as ei:
             dj.dj_load_edges(n, e.src, e.dst, w, True)
         assert ei.value.status == dj.DJ_EOVERFLOW
+
+
+@pytest.mark.parametrize("n", [1, 3, 31, 33, 130, 517])
+def test_dense_matrix_from_aligned_and_odd_places(dj, orc, n):
+    """A device matrix at any alignment, and a host one, give the same graph; a negative entry anywhere
+    is refused."""
+    import torch
+    e = graphgen.random_edges(n, 9 * n, 1, 50, seed=n, directed=True)
+    W = orc.build_matrix(n, e.src, e.dst, e.w, True)
+    room = torch.full((n * n + 8,), -9, dtype=torch.int32, device="cuda")
+    for c in (0, 1, 4):
+        A = room[c:c + n * n].view(n, n)
+        A.copy_(torch.from_numpy(W))
+        G = dj.dj_load_dense(A)
+        assert np.array_equal(dj.dj_graph_download(G), W)
+        d = torch.empty(n, dtype=torch.int32, device="cuda")
+        p = torch.empty_like(d)
+        dj.dj_sssp(G, n // 2, d, p)
+        dj.dj_sync()
+        ref = orc.dijkstra(W, n // 2)
+        assert np.array_equal(d.cpu().numpy(), ref[0]) and np.array_equal(p.cpu().numpy(), ref[1])
+        G.free()
+        for r, k in ((0, n - 1), (n - 1, 0)):
+            A[r, k] = -1
+            with pytest.raises(dj.DjError):
+                dj.dj_load_dense(A)
+            A[r, k] = int(W[r, k])
+        room.fill_(-9)
+    G = dj.dj_load_dense(W)
+    assert np.array_equal(dj.dj_graph_download(G), W)
+    G.free()
