@@ -269,6 +269,10 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   if (cluster) {  // whichever form this call takes: a later one may be captured
     if (int rc = prepare_light_cluster(csr, C)) return rc;
   }
+  // Longer lists have ten times the edges to offer, which every SM takes faster than one CTA or cluster, at
+  // any size: 6001 nodes alone 127 us on a cluster, 52 here (the streaming grid engine: 78), 1500 nodes
+  // 82 and 44 (94); behind other solves the forms that run side by side stay (15 us a solve against 50).
+  if (g->light_wide && stream_idle(st)) return launch_light_grid(g, source, dist, pred, o, nullptr, st);
   if (!cta && (!cluster || o.debug_skip_cta >= 0 ||
                (g->n >= (csr ? kLightIdleGridMinNComplete : kLightIdleGridMinN) && stream_idle(st))))
     return launch_light_grid(g, source, dist, pred, o, nullptr, st);

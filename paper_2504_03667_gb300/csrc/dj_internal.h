@@ -33,11 +33,12 @@ struct dj_graph {
   uint2* outlist = nullptr;
   uint32_t* outrest = nullptr;
   // the light-edge index (dj_light.cuh): kLightStats words of statistics, the rows' hmin (light_pad(n)
-  // words), then n x kLightCap packed edges; nullptr if the graph keeps none
+  // words), n x kLightCap packed edges, then room for as many more; nullptr if the graph keeps none
   uint32_t* light = nullptr;
   uint64_t light_bytes = 0;
   bool light_ok = false;      // solves take the light engine unless the caller chose another
   bool light_cta = false;     // its CTA form too: hardly any source needs whole rows (slow in one CTA)
+  bool light_wide = false;    // the lists are kLightWide long
   float light_deg = 0.f;      // dense: edges per row
   float light_spacing = 0.f;  // compressed rows: mean spacing of a row's lightest weights
   uint32_t light_longest = 0; // compressed rows: edges of the longest row
@@ -63,6 +64,7 @@ constexpr int kInLists = 4;  // in-edges listed per column for the dynamic IN bo
 
 // The light-edge index (dj_light.cuh).
 constexpr int kLightCap = 64;    // edges listed per row
+constexpr int kLightWide = 128;  // ... where so many are needed and do; those beyond kLightCap lie apart
 constexpr int kLightStats = 64;  // leading words: [0] ~(smallest hmin), [1] rows relaxed whole by the trial solve,
                                  // [2..3] sum of the rows' largest listed weights, [4..5] of their listed edges,
                                  // [6] most edges listed in a row, [8..11] ~(finite min), finite max, finite entries
@@ -78,7 +80,7 @@ inline
   return (n + 63) / 64 * 64;
 }
 inline size_t light_index_bytes(int32_t n) {
-  return (static_cast<size_t>(kLightStats) + light_pad(n) + static_cast<size_t>(n) * kLightCap) * 4;
+  return (static_cast<size_t>(kLightStats) + light_pad(n) + static_cast<size_t>(n) * kLightWide) * 4;
 }
 
 // Descriptor of one solve for the cluster and light engines (80 bytes).

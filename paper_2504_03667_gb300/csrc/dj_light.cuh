@@ -5,8 +5,8 @@
 // path length - dist[u]) can still change anything.  On a random graph of n nodes whose rows list
 // their K lightest edges up to weight h, the largest distance is about 2 ln(n) / K of h (the
 // flooding time of a graph with K / h edges per node and unit of weight), far below h for K = 64.
-// So every graph keeps, beside its matrix, each row's up to kLightCap lightest edges and the
-// smallest weight it does not list (hmin).  A solve runs on the listed edges, and then
+// So every graph keeps, beside its matrix, each row's up to kLightCap lightest edges (kLightWide, if the
+// first are too few and these are enough) and the smallest weight it does not list (hmin).  A solve runs on the listed edges, and then
 //   dist[u] + hmin[u] > max over v of dist[v]   for every u
 // proves that no unlisted entry can improve or tie any node: the answer is exact.  The rows that
 // fail the test are relaxed whole from the matrix (see dj_light.cu), so the answer is exact on
@@ -69,11 +69,11 @@ __device__ __forceinline__ uint32_t light_guess(const uint32_t* light, uint32_t 
 // group, and columns beyond n, pass INF).  `thr` is the warp's weight threshold, carried from row to
 // row: rows of one graph look alike, so one scan is the rule.
 //   A scan puts the edges of weight <= thr into buf (kLightBuf words of shared memory) and takes
-//   their count and the smallest weight above thr.  Too few (below kLightCap, and more exist) or too
+//   their count and the smallest weight above thr.  Too few (below Cap, and more exist) or too
 //   many (above kLightBuf): thr moves and the row (in L2 by now) is scanned again; thr is bracketed
 //   by [lo, hi], which shrinks with every scan.
-// Then the kLightCap smallest packed words (weight, column) go out in ascending order: an entry's
-// place is the number of smaller ones.
+// Then the Cap smallest packed words (weight, column) go out in ascending order, from the kLightCap-th on
+// at edge2: an entry's place is the number of smaller ones.
 constexpr int kLightBuf = 384;
 
 struct LightRow {
@@ -84,9 +84,9 @@ struct LightRow {
   uint32_t last;   // largest weight listed (0: none)
 };
 
-template <class Scan>
+template <int Cap, class Scan>
 __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, uint32_t bits_u, uint32_t* buf,
-                                                 uint32_t* edge, uint32_t& thr) {
+                                                 uint32_t* edge, uint32_t* edge2, uint32_t& thr) {
   const int lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
   const uint32_t wcap = min(weight_field(bits_u), kInf - 1u);  // weights beyond it are never listed
@@ -128,7 +128,7 @@ __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, u
       }
       hi = t - 1;
       thr = hi > lo ? lo + (hi - lo) / 2 : hi;
-    } else if (cnt < static_cast<uint32_t>(kLightCap) && rest < kInf && t < hi) {  // too few, and more exist
+    } else if (cnt < static_cast<uint32_t>(Cap) && rest < kInf && t < hi) {  // too few, and more exist
       lo = t + 1;
       // the next weight at least; fast growth while there is no upper bracket
       thr = min(hi, max(hi == wcap ? 2 * t + 1 : lo + (hi - lo) / 2, rest));
@@ -148,8 +148,11 @@ __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, u
     const uint32_t e = buf[i];
     uint32_t rank = 0;
     for (uint32_t j = 0; j < cnt; ++j) rank += buf[j] < e ? 1u : 0u;
-    if (rank < static_cast<uint32_t>(kLightCap)) {
-      edge[rank] = e;
+    if (rank < static_cast<uint32_t>(Cap)) {
+      if (Cap == kLightCap || rank < static_cast<uint32_t>(kLightCap))
+        edge[rank] = e;
+      else
+        edge2[rank - kLightCap] = e;
       ties += (e >> bits_u) == r.first ? 1u : 0u;
       last = max(last, e >> bits_u);
     } else {
@@ -159,9 +162,12 @@ __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, u
   beyond = warp_min_u32(beyond);
   r.ties = warp_sum_u32(ties);
   r.last = __reduce_max_sync(0xffffffffu, last);
-  r.cnt = min(cnt, static_cast<uint32_t>(kLightCap));
+  r.cnt = min(cnt, static_cast<uint32_t>(Cap));
   r.hmin = min(rest, beyond == kNoEdge ? kInf : beyond >> bits_u);
   for (uint32_t i = r.cnt + lane; i < static_cast<uint32_t>(kLightCap); i += 32) edge[i] = kNoEdge;
+  if (Cap > kLightCap)
+    for (uint32_t i = max(r.cnt, static_cast<uint32_t>(kLightCap)) + lane; i < static_cast<uint32_t>(Cap); i += 32)
+      edge2[i - kLightCap] = kNoEdge;
   __syncwarp();  // buf is rewritten by the next row
   return r;
 }
@@ -173,9 +179,15 @@ constexpr int kWarpRows = 64;            // a warp's waiting rows: 31 left over 
 // Shared words that other warps change meanwhile are read through this.
 __device__ __forceinline__ uint32_t word_now(const uint32_t* p) { return *const_cast<const volatile uint32_t*>(p); }
 
+// Where a row's edges beyond the first kLightCap lie, counted from where they would follow these (so that
+// the first keep their 256 bytes a row, which is all that most graphs use).
+__device__ __forceinline__ size_t light_apart(int32_t n) { return (static_cast<size_t>(n) - 1) * kLightCap; }
+
 // The rows of the index: up to `most` edges each, padded.
 struct LightListEdges {
+  static constexpr bool kApart = true;
   const uint32_t* __restrict__ edge;
+  int32_t n;
   uint32_t most;
   __device__ __forceinline__ uint4 load(uint32_t u, uint32_t k0, int sub) const {
     return __ldg(reinterpret_cast<const uint4*>(edge + static_cast<size_t>(u) * kLightCap + k0) + sub);
@@ -205,11 +217,12 @@ __device__ __forceinline__ void light_rows(const Store& s, const Edges& edges, c
       du[r] = x.y;
       on[r] = i < count && x.y != kNone;
     }
+    uint32_t part = 0;  // where the listed edges beyond kLightCap lie, counted in rows (light_apart)
     for (uint32_t k0 = 0; k0 < edges.most; k0 += 16) {  // most bounds every row
       uint4 x[R];
 #pragma unroll
       for (int r = 0; r < R; ++r)
-        x[r] = on[r] ? edges.load(u[r], k0, sub) : make_uint4(kNoEdge, kNoEdge, kNoEdge, kNoEdge);
+        x[r] = on[r] ? edges.load(u[r] + part, k0, sub) : make_uint4(kNoEdge, kNoEdge, kNoEdge, kNoEdge);
       uint32_t more = 0;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -240,6 +253,7 @@ __device__ __forceinline__ void light_rows(const Store& s, const Edges& edges, c
         more |= bal & 0x88888888u;
       }
       if (more == 0) break;
+      if (Edges::kApart && k0 == static_cast<uint32_t>(kLightCap) - 16u) part = edges.n - 1;
     }
   }
   __syncwarp();

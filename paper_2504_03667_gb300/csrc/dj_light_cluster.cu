@@ -80,6 +80,8 @@ struct LightClusterStore {
 
 // Compressed rows: row u of this CTA starts at start[] and has len[] edges (slots as the store's).
 struct LightCsrEdges {
+  static constexpr bool kApart = false;
+  static constexpr int32_t n = 0;
   const uint32_t* __restrict__ edge;
   const int64_t* start;  // shared
   const uint32_t* len;   // shared
@@ -150,7 +152,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
     if constexpr (CSR)
       light_rows<decltype(ties)::value>(s, LightCsrEdges{p.edge, start, len, p.cshift, most}, get, count, B, bits_u, lmin);
     else
-      light_rows<decltype(ties)::value>(s, LightListEdges{hmin + light_pad(n), most}, get, count, B, bits_u, lmin);
+      light_rows<decltype(ties)::value>(s, LightListEdges{hmin + light_pad(n), n, most}, get, count, B, bits_u, lmin);
   };
   uint32_t phase = 0, cur = 0;  // cur = phase % 3: the slot of this phase's m, the smallest dirty dist
   int raised = 0;

@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
     const uint32_t bits_u = d.bits_u, umask = (1u << bits_u) - 1u;
     const uint32_t* hmin = d.light + kLightStats;
     const uint32_t hmin_min = ~__ldg(d.light);  // >= INF: every row's list is complete
-    const LightListEdges edges{hmin + light_pad(n), __ldg(d.light + 6)};
+    const LightListEdges edges{hmin + light_pad(n), n, __ldg(d.light + 6)};
     const uint32_t delta = light_delta(d.light, kCtaDelta);
     // a wide margin in batches: one takes as long as its slowest solve, one whose bound was too low (256 sources of
     // n = 8192: 296 us with an eighth, 285 with a quarter, 261 with 3/8)

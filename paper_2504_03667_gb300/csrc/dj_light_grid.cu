@@ -198,9 +198,9 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
   uint32_t lmin = kNone;
   {
     const int64_t s0 = CSR ? p.row_ptr[p.source] : static_cast<int64_t>(p.source) * kLightCap;
-    const int64_t len = CSR ? p.row_ptr[p.source + 1] - s0 : kLightCap;
+    const int64_t len = CSR ? p.row_ptr[p.source + 1] - s0 : most;
     for (int64_t i = tid; i < len; i += T0) {
-      const uint32_t e = __ldg(p.edge + s0 + i);
+      const uint32_t e = __ldg(p.edge + s0 + i + (!CSR && i >= kLightCap ? light_apart(p.n) : 0));
       if (e == kNoEdge) break;
       const uint32_t v = e & umask;
       if (v - static_cast<uint32_t>(c0) >= static_cast<uint32_t>(sw) || static_cast<int>(v) == p.source) continue;
@@ -267,7 +267,10 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
           uint64_t old[kLightRows];
           bool use[kLightRows];
 #pragma unroll
-          for (int r = 0; r < kLightRows; ++r) e[r] = on[r] && k < len[r] ? __ldg(row[r] + k) : kNoEdge;
+          for (int r = 0; r < kLightRows; ++r) {
+            if (!CSR && k - gl == kLightCap) row[r] += light_apart(p.n);
+            e[r] = on[r] && k < len[r] ? __ldg(row[r] + k) : kNoEdge;
+          }
 #pragma unroll
           for (int r = 0; r < kLightRows; ++r) {
             use[r] = e[r] != kNoEdge && du[r] + (e[r] >> bits_u) <= B;

@@ -166,7 +166,7 @@ struct LightSums {
 // rows, so a bad guess costs scans: 8192 rows of 4096 edges took 265 us from 0 and take 98 us, against
 // 125 us for the row minima and tie sources this pass replaces.
 // Where deg is not known (a matrix was loaded), the warp takes both from the first columns of its first row.
-__device__ __forceinline__ uint32_t first_threshold(const LightOut& o, const int32_t* row = nullptr) {
+__device__ __forceinline__ uint32_t first_threshold(const LightOut& o, const int32_t* row, float most) {
   float deg = o.deg, wmax = static_cast<float>(o.wmax ? o.wmax : o.light[14]);
   if (deg == 0.f && row) {
     const int c1 = min(o.n, 1024);
@@ -184,17 +184,17 @@ __device__ __forceinline__ uint32_t first_threshold(const LightOut& o, const int
     deg = static_cast<float>(cnt) / static_cast<float>(c1) * static_cast<float>(o.n);
     wmax = cnt ? 2.f * sum / static_cast<float>(cnt) : 2.0e9f;
   }
-  const float want = 2.25f * kLightCap;
+  const float want = 2.25f * most;
   return static_cast<uint32_t>(fminf(2.0e9f, deg <= want ? wmax : wmax * want / deg));
 }
 
-template <class Scan>
+template <int Cap, class Scan>
 __device__ __forceinline__ void light_row(const LightOut& o, const Scan& scan, uint32_t u, uint32_t* buf,
                                           uint32_t& thr, LightSums& sums) {
   const int lane = threadIdx.x & 31;
   uint32_t* hmin = o.light + kLightStats;
   uint32_t* edge = hmin + light_pad(o.n) + static_cast<size_t>(u) * kLightCap;
-  const LightRow r = light_select(scan, u, o.bits_u, buf, edge, thr);
+  const LightRow r = light_select<Cap>(scan, u, o.bits_u, buf, edge, edge + kLightCap + light_apart(o.n), thr);
   if (lane == 0) {
     o.minout[u] = static_cast<int32_t>(r.first);
     if (o.tsrc) o.minout[o.n + u] = static_cast<int32_t>(r.first);  // minin: the same
@@ -220,6 +220,7 @@ __device__ __forceinline__ void light_sums_out(const LightOut& o, const LightSum
 
 // The rows of the resident matrix; with `stats` also the finite min / max and the number of finite
 // entries (the index's words 8..11).
+template <int Cap>
 __global__ void __launch_bounds__(256) k_light_rows(const int32_t* __restrict__ W, int64_t pitch, const LightOut o,
                                                     bool stats) {
   __shared__ uint32_t s_buf[8][kLightBuf];
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(256) k_light_rows(const int32_t* __restrict__ 
   const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
   const int64_t nq = pitch / 4;
-  uint32_t thr = first_threshold(o, warp < o.n ? W + warp * pitch : nullptr), gmin = kInf, gmax = 0;
+  uint32_t thr = first_threshold(o, warp < o.n ? W + warp * pitch : nullptr, Cap), gmin = kInf, gmax = 0;
   unsigned long long cnt = 0;
   LightSums sums;
   for (int64_t u = warp; u < o.n; u += nwarps) {
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(256) k_light_rows(const int32_t* __restrict__ 
         }
       }
     };
-    light_row(o, scan, static_cast<uint32_t>(u), s_buf[threadIdx.x >> 5], thr, sums);
+    light_row<Cap>(o, scan, static_cast<uint32_t>(u), s_buf[threadIdx.x >> 5], thr, sums);
     if (lane == 0) gmin = min(gmin, static_cast<uint32_t>(o.minout[u]));
     gmax = max(gmax, mx);
     cnt += c;
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(256) k_upload_rows(const int32_t* __restrict__
   const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
   const int4 none = make_int4(int(kInf), int(kInf), int(kInf), int(kInf));
-  uint32_t thr = first_threshold(o);
+  uint32_t thr = first_threshold(o, nullptr, kLightCap);
   LightSums sums;
   for (int64_t u = warp; u < o.n; u += nwarps) {
     const int32_t* s = src + u * ld;
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(256) k_upload_rows(const int32_t* __restrict__
         __syncwarp();  // later scans read the row as every lane wrote it
       }
     };
-    light_row(o, scan, static_cast<uint32_t>(u), s_buf[threadIdx.x >> 5], thr, sums);
+    light_row<kLightCap>(o, scan, static_cast<uint32_t>(u), s_buf[threadIdx.x >> 5], thr, sums);
   }
   light_sums_out(o, sums);
 }
@@ -595,7 +596,7 @@ static LightOut light_out(const dj_graph* g) {
 static void launch_minima(dj_graph* g, uint32_t* stats, cudaStream_t st, bool have_rows = false) {
   const bool rows_done = have_rows || g->light;
   if (!have_rows && g->light) {
-    k_light_rows<<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(g->W, g->pitch, light_out(g), stats != nullptr);
+    k_light_rows<kLightCap><<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(g->W, g->pitch, light_out(g), stats != nullptr);
   } else if (!have_rows) {
     k_rowmin<<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(g->W, g->pitch, g->n, g->minout, stats);
   }
@@ -619,7 +620,27 @@ static void launch_minima(dj_graph* g, uint32_t* stats, cudaStream_t st, bool ha
 // verdict *list gets (nullptr: there was no list).
 //
 // Whether solves take the light engine is judged here, by a trial solve: one more kernel in front of
-// the only wait.
+// the wait, the only one unless longer lists are worth a try.
+static bool launch_trial(dj_graph* g, uint32_t* idx, cudaStream_t st) {
+  dj_solve_opts o;
+  dj_solve_opts_init(&o);
+  const bool tried = launch_light_grid(g, g->n / 2, nullptr, nullptr, o, g->light + 1, st) == DJ_OK;
+  clear_error();  // it cannot run here: the other engines
+  cudaMemcpyAsync(idx, g->light, 16 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
+  return tried;
+}
+
+// Whether lists of kLightWide edges would hold every edge that matters: the source's row needs the most of
+// them, those of weight up to the largest dist (the trial's).  Their number is estimated from the lists, and as
+// if the weights were uniform between the smallest and the largest, whichever is more.
+static bool wide_suffices(const dj_graph* g, const uint32_t* idx) {
+  if (idx[kLightGuess] == 0) return false;
+  const double D = idx[kLightGuess] - 1.0;
+  const double last = idx[2] + 4294967296.0 * idx[3], cnt = idx[4] + 4294967296.0 * idx[5];
+  const double uniform = g->light_deg * (D - g->wmin + 1.0) / (static_cast<double>(g->wmax) - g->wmin + 1.0);
+  return std::max(last > 0 ? cnt / last * D : 0.0, uniform) <= 1.1 * kLightWide;
+}
+
 static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   uint32_t* stats = g->light ? g->light + 8 : nullptr;
   uint32_t idx[16] = {0};
@@ -633,11 +654,7 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   launch_minima(g, stats, st);
   bool tried = false;
   if (g->light) {
-    dj_solve_opts o;
-    dj_solve_opts_init(&o);
-    tried = launch_light_grid(g, g->n / 2, nullptr, nullptr, o, g->light + 1, st) == DJ_OK;
-    clear_error();  // it cannot run here: the other engines
-    cudaMemcpyAsync(idx, g->light, sizeof(idx), cudaMemcpyDeviceToHost, st);
+    tried = launch_trial(g, idx, st);
   } else {
     cudaMemcpyAsync(idx + 8, stats, 4 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
     cudaFreeAsync(stats, st);
@@ -657,6 +674,19 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   // engine 37).  One CTA or cluster relaxes many whole rows slowly (4500 in 7 ms, the grid form in 0.2),
   // so these forms are for complete lists and symmetric matrices: no source's largest dist is then more
   // than twice the trial's, while a directed graph's may be by any factor.
+  // Lists of kLightWide edges are built instead (one more pass and trial) where these look enough: n = 6001,
+  // p = 0.05, weights 1..10 needs 288 rows whole with 64 edges listed, none with 128, and takes 14.6 us a
+  // solve (the streaming grid engine 51) for a load of 0.54 ms instead of 0.45 (before the index: 1.64).
+  if (tried && g->wmin >= 1 && ~idx[0] < kInf && idx[1] > 4 && wide_suffices(g, idx)) {
+    cudaMemsetAsync(g->light, 0, 8 * sizeof(uint32_t), st);
+    cudaMemsetAsync(g->light + kLightGuess, 0, sizeof(uint32_t), st);
+    k_light_rows<kLightWide><<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(g->W, g->pitch, light_out(g),
+                                                                                        false);
+    tried = launch_trial(g, idx, st);
+    e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_error(e, "building the longer lists");
+    g->light_wide = true;
+  }
   const bool complete = ~idx[0] >= kInf;
   g->light_ok = tried && g->wmin >= 1 && (complete || idx[1] <= 4);
   g->light_cta = g->light_ok && (complete || !g->directed);
@@ -866,7 +896,7 @@ extern "C" int dj_graph_upload(dj_graph* g, const int32_t* W, int64_t ld, uint64
   g->upload_pending = 1;
   // The index follows the matrix (a captured solve may be replayed on it), but it was judged for the
   // loaded one: nothing tells here, without a wait, whether the new one suits it.
-  g->light_ok = g->light_cta = false;
+  g->light_ok = g->light_cta = g->light_wide = false;
   launch_minima(g, nullptr, st, zero_copy);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_error(e, "row minima");

@@ -128,6 +128,39 @@ def test_lists_cut_in_ties(dj, orc):
     check(dj, orc, graphgen.EdgeList(n, src, dst, w, False), [5], "the same undirected")
 
 
+@pytest.mark.parametrize("n", [130, 400, 1500, 3001, 6143, 6145])
+def test_longer_lists(dj, orc, n):
+    """About 30 edges per row and unit of weight: lists of 64 edges are too short for most sources, lists of
+    128 long enough; then an upload takes the same handle (and a captured solve) back to lists of 64."""
+    import torch
+    p = min(300 / n, 0.9)
+    whi = max(2, round(p * n / 30))
+    for directed in (False, True):
+        e = (graphgen.random_edges(n, 30 * whi * n, 1, whi, seed=n, directed=True) if directed
+             else graphgen.bernoulli(n, p, 1, whi, n))
+        check(dj, orc, e, sorted({0, n // 3, n // 2, n - 1}), f"n={n} directed={directed}")
+    a, b = graphgen.bernoulli(n, p, 1, whi, n + 1), graphgen.bernoulli(n, p / 2, 1, 40, n + 2)
+    st = torch.cuda.Stream()
+    d = torch.empty(n, dtype=torch.int32, device="cuda")
+    q = torch.empty_like(d)
+    G = dj.dj_load_edges(n, a.src, a.dst, a.w, False)
+    dj.dj_sssp(G, 5, d, q, st)
+    dj.dj_sync(st)
+    cg = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(cg, stream=st):
+        dj.dj_sssp(G, 5, d, q, st)
+    W = orc.build_matrix(n, b.src, b.dst, b.w, False)
+    ref = orc.dijkstra(W, 5)
+    dj.dj_graph_upload(G, W, st)
+    d.fill_(-5)
+    torch.cuda.synchronize()
+    cg.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(d.cpu().numpy(), ref[0]) and np.array_equal(q.cpu().numpy(), ref[1])
+    del cg
+    G.free()
+
+
 def test_hub_rows(dj, orc):
     """Stars: one row much longer than the others (taken by a whole block in compressed rows)."""
     n = 9001
