@@ -152,8 +152,8 @@ int dj_graph_free(dj_graph* g);
 #define DJ_ENGINE_CLUSTER 2 /* one thread-block cluster; state in distributed shared memory */
 
 /* The light engine.  A loaded graph keeps, beside its matrix, each row's up to
- * 64 lightest edges and the smallest weight not among them (256 bytes a node,
- * rebuilt by dj_graph_upload).  A solve relaxes those; then dist[u] + (u's
+ * 64 lightest edges, or 128 where 64 are too few and these enough, and the
+ * smallest weight not among them (516 bytes a node; dj_graph_upload rebuilds 64).  A solve relaxes those; then dist[u] + (u's
  * smallest unlisted weight) > max dist proves that no unlisted edge matters,
  * and rows that fail the test are relaxed whole from the matrix, so dist and
  * pred are Algorithm 1's on every graph.  One solve runs on one CTA, on one

@@ -615,12 +615,7 @@ static void launch_minima(dj_graph* g, uint32_t* stats, cudaStream_t st, bool ha
   if (g->inlist) launch_inlists(g, st);
 }
 
-// Row and column minima, index, global weight range, then the overflow rule (n-1) * wmax < INT32_MAX.
-// The index's leading words are zero before, but for the edge list's check (words 12..14), whose
-// verdict *list gets (nullptr: there was no list).
-//
-// Whether solves take the light engine is judged here, by a trial solve: one more kernel in front of
-// the wait, the only one unless longer lists are worth a try.
+// The trial solve on the index, and the index's leading words on their way to the host.
 static bool launch_trial(dj_graph* g, uint32_t* idx, cudaStream_t st) {
   dj_solve_opts o;
   dj_solve_opts_init(&o);
@@ -641,6 +636,12 @@ static bool wide_suffices(const dj_graph* g, const uint32_t* idx) {
   return std::max(last > 0 ? cnt / last * D : 0.0, uniform) <= 1.1 * kLightWide;
 }
 
+// Row and column minima, index, global weight range, then the overflow rule (n-1) * wmax < INT32_MAX.
+// The index's leading words are zero before, but for the edge list's check (words 12..14), whose
+// verdict *list gets (nullptr: there was no list).
+//
+// Whether solves take the light engine is judged here, by a trial solve: one more kernel in front of
+// the wait, the only one unless longer lists are worth a try.
 static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   uint32_t* stats = g->light ? g->light + 8 : nullptr;
   uint32_t idx[16] = {0};
