@@ -22,7 +22,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["dj_load.cu", "dj_solve.cu", "dj_api.cu", "dj_serve.cu", "dj_lc.cu", "dj_csr.cu", "dj_lockstep.cu",
            "dj_light_grid.cu", "dj_light_cta.cu", "dj_light_cluster.cu"]
 HEADERS = ["dj_common.cuh", "dj_core.cuh", "dj_internal.h", "dj_noalloc_size.h", "dj_jobs.cuh",
-           "dj_light.cuh"]
+           "dj_light.cuh", "dj_light_rules.h"]
 
 
 def _nvcc() -> str:

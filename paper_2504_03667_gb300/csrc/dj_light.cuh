@@ -23,10 +23,11 @@
 
 #include "dj_common.cuh"
 #include "dj_internal.h"
+#include "dj_light_rules.h"
 
 namespace dj {
 
-constexpr uint32_t kNone = 0xFFFFFFFFu;    // no dist, no bound
+constexpr uint32_t kNone = kRuleNone;      // no dist, no bound
 constexpr uint32_t kNoEdge = 0xFFFFFFFFu;  // an unused slot of a row's list (no edge packs to all ones)
 
 __device__ __forceinline__ uint32_t weight_field(uint32_t bits_u) { return 0xFFFFFFFFu >> bits_u; }

@@ -253,8 +253,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
         B = D;
         auto pending = [&](int lw, uint32_t dv) {  // dist + hmin of this lane's node if its row is pending
           if (dv == kNone || ((whole[lw] >> lane) & 1u)) return kNone;
-          const uint32_t x = dv + __ldg(hmin + 32 * global_word(lw) + lane);
-          return x <= D && x < kInf ? x : kNone;
+          return light_pending(dv, __ldg(hmin + 32 * global_word(lw) + lane), D);
         };
         uint32_t hb = kNone;  // the smallest dist + hmin of the pending rows
         for (int lw = warp; lw < LW; lw += kClWarps) hb = min(hb, pending(lw, dist[32 * lw + lane]));
@@ -264,10 +263,10 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
         cluster_sync_all();
         hb = s_bound;
         if (hb == kNone) break;
-        // those below it are final: relaxed whole, as many as the list holds now
+        // those up to it are final: relaxed whole, as many as the list holds now
         for (int lw = warp; lw < LW; lw += kClWarps) {
           const uint32_t dv = dist[32 * lw + lane];
-          const bool go = dv < hb && pending(lw, dv) != kNone;
+          const bool go = light_final(dv, hb) && pending(lw, dv) != kNone;
           const uint32_t todo = __ballot_sync(0xffffffffu, go);
           if (todo == 0) continue;
           uint32_t pos = 0;

@@ -216,8 +216,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
           __syncthreads();
           auto pending = [&](int wi, uint32_t dv) {  // dist + hmin of this lane's node if its row is pending
             if (dv == kNone || ((s.whole[wi] >> lane) & 1u)) return kNone;
-            const uint32_t x = dv + __ldg(hmin + 32 * wi + lane);
-            return x <= D && x < kInf ? x : kNone;
+            return light_pending(dv, __ldg(hmin + 32 * wi + lane), D);
           };
           uint32_t hb = kNone;
           for (int wi = warp; wi < nwords; wi += NW) hb = min(hb, pending(wi, s.dist[32 * wi + lane]));
@@ -226,10 +225,10 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
           __syncthreads();
           hb = s_bound;
           if (hb == kNone) break;
-          // those below it are final: relaxed whole, as many as the list holds now
+          // those up to it are final: relaxed whole, as many as the list holds now
           for (int wi = warp; wi < nwords; wi += NW) {
             const uint32_t dv = s.dist[32 * wi + lane];
-            const bool go = dv < hb && pending(wi, dv) != kNone;
+            const bool go = light_final(dv, hb) && pending(wi, dv) != kNone;
             const uint32_t todo = __ballot_sync(0xffffffffu, go);
             if (todo == 0) continue;
             uint32_t pos = 0;

@@ -12,8 +12,9 @@
 // relaxed once more.  Then the index's test (hmin) either proves the answer complete or names the rows to
 // relax whole from the matrix:
 //   pending = { u : dist[u] + hmin[u] <= D, not yet relaxed whole }, and
-//   those with dist[u] < min over pending of (dist + hmin) are final -- a shorter path would use an
-//   unlisted edge of a pending row -- so each row is read from the matrix at most once.
+//   those with dist[u] <= min over pending of (dist + hmin) are final -- a shorter path would use an
+//   unlisted edge of a pending row -- so each row is read from the matrix at most once, and every round
+//   takes at least the row that gives the minimum.
 //
 // What bounds it: latency.  A phase is one grid barrier (which also carries m and D) and a chain of
 // three L2 round trips (own keys, edges, targets' keys) around a few hundred KB of list reads.
@@ -56,7 +57,7 @@ struct LightGridParams {
   uint32_t delta;     // compressed rows (dense graphs: from the index's statistics, light_window)
   int32_t gshift;     // the same: log2 of the lanes that share a row
   int32_t skip_cta;
-  int32_t trial;      // nothing is written; a graph whose lists are all complete needs none
+  int32_t trial;      // nothing is written (light_needs_trial)
 };
 
 // Control words: an abort flag and an exit counter at the grid engine's places, and three barrier
@@ -177,7 +178,8 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
   uint32_t delta = p.delta;
   int gshift = p.gshift;
   if (!CSR) light_window(p.light, kGridDelta, &delta, &gshift);
-  if (!CSR && p.trial && hmin_min >= kInf) return;
+  // a trial is of use to graphs whose solves may take this engine: some list cut, no weight of 0
+  if (!CSR && p.trial && !light_needs_trial(hmin_min, ~__ldg(p.light + 8))) return;
   // offers above the guessed largest dist are dropped at first (see below); the trial makes the guess
   uint32_t guess = CSR || p.trial || hmin_min >= kInf ? kNone : light_guess(p.light, 8);
   for (int j = tid; j < sw; j += T0) {
@@ -321,15 +323,15 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
     uint32_t hb = kNone;
     for (int j = tid; j < sw; j += T0) {
       if ((flags[j] & 2) || rdist[j] >= kInf) continue;  // rdist is the dist of every reached node now
-      const uint32_t x = rdist[j] + aux[j];
-      if (x <= Dx && x < kInf) hb = min(hb, x);
+      hb = min(hb, light_pending(rdist[j], aux[j], Dx));
     }
     if (!light_barrier(p, sh, nbar++, hb, 0u, &m, &D)) return;
     hb = m;
     D = Dx;
     if (hb == kNone) break;
     for (int j = tid; j < sw; j += T0) {
-      if ((flags[j] & 2) || rdist[j] >= hb || rdist[j] + aux[j] > Dx || rdist[j] + aux[j] >= kInf) continue;
+      if ((flags[j] & 2) || rdist[j] >= kInf || !light_final(rdist[j], hb) || light_pending(rdist[j], aux[j], Dx) == kNone)
+        continue;
       list[atomicAdd(&sh.cnt, 1u)] = make_uint2(static_cast<uint32_t>(j), rdist[j]);
       flags[j] |= 2;
     }

@@ -1,0 +1,36 @@
+// The rules by which the light engine takes rows, in plain C++ for host and device, so that a host-only
+// test can run them.
+#pragma once
+
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define DJ_RULE __host__ __device__ __forceinline__
+#else
+#define DJ_RULE inline
+#endif
+
+namespace dj {
+
+constexpr uint32_t kRuleInf = 0x7FFFFFFFu;   // the paper's infinity
+constexpr uint32_t kRuleNone = 0xFFFFFFFFu;  // no dist
+
+// What a reached row's unlisted edges offer at least, if that can still matter to a solve whose largest
+// dist is D; kRuleNone otherwise.
+DJ_RULE uint32_t light_pending(uint32_t dist, uint32_t hmin, uint32_t D) {
+  if (dist == kRuleNone) return kRuleNone;
+  const uint32_t x = dist + hmin;  // both below 2^31
+  return x <= D && x < kRuleInf ? x : kRuleNone;
+}
+
+// Whether a pending row is relaxed whole now, hb being the least of what the pending rows offer: a path
+// shorter than dist would have to use an unlisted edge of a pending row, which offers no less than hb.
+// So dist <= hb is final, and the row that gives hb is always among those taken, even with unlisted edges
+// of weight 0 (dist < hb took none then, and the solve never ended).
+DJ_RULE bool light_final(uint32_t dist, uint32_t hb) { return dist <= hb; }
+
+// Whether a graph's trial solve is run: some list is cut, and no weight is 0 (its solves take the other
+// engines then, and its lists may hold nothing but a few of a row's edges of weight 0).
+DJ_RULE bool light_needs_trial(uint32_t hmin_min, uint32_t wmin) { return hmin_min < kRuleInf && wmin > 0; }
+
+}  // namespace dj

@@ -243,3 +243,39 @@ def test_server_replans(dj, orc):
     srv.destroy()
     for x in g:
         x.free()
+
+
+@pytest.mark.parametrize("n,p,whi", [(80, 1.0, 0), (700, 1.0, 0), (700, 0.5, 3), (2049, 0.5, 2), (4097, 0.3, 1)])
+def test_many_weights_of_zero(dj, orc, n, p, whi):
+    """Rows with more edges of weight 0 than a list holds: loaded, solved and batched as any graph."""
+    b = graphgen.bernoulli(n, p, 0, whi, n)
+    check(dj, orc, b, [0, n // 2], f"n={n} w in [0, {whi}]")
+    e = graphgen.EdgeList(n, np.concatenate([b.src, b.dst]), np.concatenate([b.dst, b.src]),
+                          np.concatenate([b.w, np.maximum(b.w, 1)]), True)
+    check(dj, orc, e, [n - 1], f"n={n} w in [0, {whi}] directed")
+
+
+@pytest.mark.parametrize("n,directed", [(400, False), (3001, False), (4500, True)])
+def test_captured_solve_ends_on_weights_of_zero(dj, orc, n, directed):
+    """A solve captured on positive weights and replayed on a matrix of many zeros ends, with Algorithm 1's dist."""
+    import torch
+    a = graphgen.bernoulli(n, 0.3, 1, 1000, n)
+    b = graphgen.bernoulli(n, 0.6, 0, 2, n + 1)
+    W = orc.build_matrix(n, b.src, b.dst, b.w, False)
+    st = torch.cuda.Stream()
+    d = torch.empty(n, dtype=torch.int32, device="cuda")
+    q = torch.empty_like(d)
+    both = [np.concatenate(x) for x in ((a.src, a.dst), (a.dst, a.src), (a.w, a.w))]
+    G = dj.dj_load_edges(n, *both, True) if directed else dj.dj_load_edges(n, a.src, a.dst, a.w, False)
+    dj.dj_sssp(G, 5, d, q, st)
+    dj.dj_sync(st)
+    cg = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(cg, stream=st):
+        dj.dj_sssp(G, 5, d, q, st)
+    dj.dj_graph_upload(G, W, st)
+    torch.cuda.synchronize()
+    cg.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(d.cpu().numpy(), orc.dijkstra(W, 5)[0])
+    del cg
+    G.free()

@@ -1,0 +1,95 @@
+"""The light engine's rules as the library compiles them (dj_light_rules.h), run on the CPU: the stage that
+relaxes rows whole ends on every matrix, whatever its rows leave unlisted, and keeps the answer."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from test_light_model import INF, build_index
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2504_03667_gb300", "csrc")
+NONE = 2**32 - 1
+
+PROG = r"""
+#include "dj_light_rules.h"
+extern "C" {
+unsigned pending(unsigned dist, unsigned hmin, unsigned D) { return dj::light_pending(dist, hmin, D); }
+int is_final(unsigned dist, unsigned hb) { return dj::light_final(dist, hb); }
+int needs_trial(unsigned hmin_min, unsigned wmin) { return dj::light_needs_trial(hmin_min, wmin); }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        pytest.skip("no host C++ compiler")
+    d = tmp_path_factory.mktemp("rules")
+    src, lib = d / "rules.cpp", d / "librules.so"
+    src.write_text(PROG)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-fPIC", "-shared", "-I", CSRC, str(src), "-o", str(lib)], check=True)
+    lib = ctypes.CDLL(str(lib))
+    for f, args in ((lib.pending, 3), (lib.is_final, 2), (lib.needs_trial, 2)):
+        f.argtypes = [ctypes.c_uint32] * args
+    lib.pending.restype = ctypes.c_uint32
+    return lib
+
+
+def solve(W, s, rows, hmin, rules):
+    """dist by the listed edges and whole rows; at most one round of whole rows per node."""
+    n, b = W.shape[0], 1
+    while (1 << b) < n:
+        b += 1
+    dist = [NONE] * n
+    dist[s] = 0
+    whole = set()
+    has_in = [any(W[u, v] < INF for u in range(n) if u != v) for v in range(n)]
+    for rounds in range(n + 2):
+        dirty = list(range(n))
+        while dirty:  # settle on the listed edges
+            u = dirty.pop()
+            if dist[u] == NONE:
+                continue
+            for e in rows[u]:
+                v, c = e & ((1 << b) - 1), dist[u] + (e >> b)
+                if c < dist[v]:
+                    dist[v] = c
+                    dirty.append(v)
+        D = max(dist[v] if dist[v] != NONE else (NONE if has_in[v] else 0) for v in range(n))
+        pend = {u: rules.pending(dist[u], hmin[u], D) for u in range(n) if u not in whole}
+        hb = min([x for x in pend.values()] + [NONE])
+        if hb == NONE:
+            return [d if d != NONE else INF for d in dist]
+        for u in [u for u, x in pend.items() if x != NONE and rules.is_final(dist[u], hb)]:
+            whole.add(u)
+            for v in np.flatnonzero(W[u] < INF):
+                if v != u:
+                    dist[v] = min(dist[v], dist[u] + int(W[u, v]))
+    raise AssertionError(f"no end after {rounds} rounds of whole rows")
+
+
+@pytest.mark.parametrize("wlo,whi", [(0, 0), (0, 1), (0, 3), (1, 1), (1, 4)])
+@pytest.mark.parametrize("directed", [False, True])
+def test_whole_rows_end(orc, rules, wlo, whi, directed):
+    for n, p, cap in ((80, 1.0, 64), (40, 0.8, 3), (33, 0.5, 1), (70, 0.9, 8)):
+        rng = np.random.default_rng(n + whi)
+        k = rng.random((n, n)) < p
+        k = np.triu(k, 1) if not directed else k & ~np.eye(n, dtype=bool)
+        src, dst = (x.astype(np.int32) for x in np.nonzero(k))
+        w = rng.integers(wlo, whi + 1, src.size).astype(np.int32)
+        W = orc.build_matrix(n, src, dst, w, directed)
+        for partial in (True, False):
+            rows, hmin = build_index(W, cap, partial)
+            for s in (0, n - 1):
+                assert solve(W, s, rows, hmin, rules) == list(orc.dijkstra(W, s)[0]), (n, cap, partial, s)
+
+
+def test_trial_is_for_graphs_that_may_take_the_engine(rules):
+    assert rules.needs_trial(5, 1) == 1
+    assert rules.needs_trial(INF, 1) == 0  # every list complete
+    assert rules.needs_trial(5, 0) == 0 and rules.needs_trial(0, 0) == 0  # weights of 0
