@@ -874,6 +874,10 @@ extern "C" int dj_graph_upload(dj_graph* g, const int32_t* W, int64_t ld, uint64
   if (!g || !W || ld < g->n) return set_error(DJ_EINVAL, "need g, W != NULL and ld >= n");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   cudaError_t e;
+  // The index is rebuilt below whichever way the matrix comes: its statistics start anew, above all the
+  // length of the longest list, which captured solves read (past it lie edges of the old matrix).  The
+  // trial's largest dist (kLightGuess) stays: it only bounds offers at first.
+  if (g->light) cudaMemsetAsync(g->light, 0, 12 * sizeof(uint32_t), st);
   // pinned host memory the device can address: one kernel copies the rows and takes their minima
   cudaPointerAttributes pa;
   const cudaError_t pe = cudaPointerGetAttributes(&pa, W);
@@ -883,7 +887,6 @@ extern "C" int dj_graph_upload(dj_graph* g, const int32_t* W, int64_t ld, uint64
   if (zero_copy) {
     const int32_t* src = static_cast<const int32_t*>(pa.devicePointer);
     const int vec = (ld % 4 == 0 && reinterpret_cast<uintptr_t>(src) % 16 == 0) ? 1 : 0;
-    cudaMemsetAsync(g->light, 0, 12 * sizeof(uint32_t), st);
     k_upload_rows<<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(src, ld, g->W, g->pitch, light_out(g), vec);
     e = cudaGetLastError();
   } else if (ld == g->n && g->n == g->pitch) {  // no padding columns on either side: one contiguous copy

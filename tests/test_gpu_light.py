@@ -279,3 +279,50 @@ def test_captured_solve_ends_on_weights_of_zero(dj, orc, n, directed):
     assert np.array_equal(d.cpu().numpy(), orc.dijkstra(W, 5)[0])
     del cg
     G.free()
+
+
+@pytest.mark.parametrize("n", [1500, 3001, 6001])
+def test_longer_lists_end_with_an_upload(dj, orc, n):
+    """A solve and a batch captured on lists of 128 edges, replayed on another matrix of the same kind: its
+    lists are cut at 64, where many rows would go on, and what lay behind them is the old matrix's."""
+    import torch
+    p = 300 / n
+    a, b = graphgen.bernoulli(n, p, 1, 10, n + 1), graphgen.bernoulli(n, p, 1, 10, n + 2)
+    W = orc.build_matrix(n, b.src, b.dst, b.w, False)
+    srcs = [5, n // 2, n - 1]
+    refs = [orc.dijkstra(W, s) for s in srcs]
+    pinned = torch.from_numpy(W).pin_memory()
+    padded = torch.empty((n, n + 3), dtype=torch.int32).pin_memory()
+    padded[:, 1:n + 1] = pinned
+    for what, src in (("pageable", W), ("pinned", pinned), ("offset", padded[:, 1:n + 1])):
+        st = torch.cuda.Stream()
+        D = torch.empty((2, 3, n), dtype=torch.int32, device="cuda")
+        P = torch.empty_like(D)
+        G = dj.dj_load_edges(n, a.src, a.dst, a.w, False)
+        batch = dj.dj_batch_create([G] * 3, srcs, list(D[1]), list(P[1]))
+
+        def solve():
+            for i, s in enumerate(srcs):
+                dj.dj_sssp(G, s, D[0, i], P[0, i], st)
+            dj.dj_batch_launch(batch, st)
+
+        solve()
+        dj.dj_sync(st)
+        cg = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(cg, stream=st):
+            solve()
+        dj.dj_graph_upload(G, src, st)
+        for how, again in (("replay", cg.replay), ("new calls", solve)):
+            torch.cuda.synchronize()
+            D.fill_(-5)
+            P.fill_(-5)
+            torch.cuda.synchronize()
+            again()
+            torch.cuda.synchronize()
+            for j, form in enumerate(("single", "batch")):
+                for i in range(3):
+                    assert np.array_equal(D[j, i].cpu().numpy(), refs[i][0]), (what, how, form, i)
+                    assert np.array_equal(P[j, i].cpu().numpy(), refs[i][1]), (what, how, form, i)
+        del cg
+        batch.free()
+        G.free()
