@@ -1,5 +1,5 @@
-// The rules by which the light engine takes rows, in plain C++ for host and device, so that a host-only
-// test can run them.
+// The rules by which the light engine takes rows and graphs are loaded, in plain C++ (some for host and
+// device), so that a host-only test can run them.
 #pragma once
 
 #include <cstdint>
@@ -32,5 +32,10 @@ DJ_RULE bool light_final(uint32_t dist, uint32_t hb) { return dist <= hb; }
 // Whether a graph's trial solve is run: some list is cut, and no weight is 0 (its solves take the other
 // engines then, and its lists may hold nothing but a few of a row's edges of weight 0).
 DJ_RULE bool light_needs_trial(uint32_t hmin_min, uint32_t wmin) { return hmin_min < kRuleInf && wmin > 0; }
+
+// Whether the device may read the caller's edge arrays in place: 4-byte loads fault on other addresses.
+inline bool edges_in_place(const void* src, const void* dst, const void* w) {
+  return ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(w)) & 3u) == 0;
+}
 
 }  // namespace dj

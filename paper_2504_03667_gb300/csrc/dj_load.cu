@@ -17,6 +17,7 @@
 #include "dj_common.cuh"
 #include "dj_internal.h"
 #include "dj_light.cuh"
+#include "dj_light_rules.h"
 
 namespace dj {
 
@@ -769,11 +770,12 @@ extern "C" int dj_load_edges(int32_t n, int64_t m, const int32_t* src, const int
   if (m > 0) {
     cudaError_t e = cudaSuccess;
     if (!g->light) e = cudaMemsetAsync(check, 0, 16, st);
-    if (e == cudaSuccess && ctx->pageable) {
+    if (e == cudaSuccess && ctx->pageable && edges_in_place(src, dst, w)) {
       // the device reads the caller's arrays over the host link itself (coherent host memory): one pass,
       // no staging copies, no host loop, no wait of its own.  Loading 67 M edges (805 MB) into n = 16384:
       // 5.4 ms, against 86 ms with a host check and pageable copies, most of it the host's two walks over
       // the list; 2.5 M edges into n = 4099: 0.45 against 3.6 ms; 1491 edges into n = 100: 0.07 against 0.31.
+      // Arrays that are not 4-byte aligned go through the copies below, which take any address.
       k_scatter<<<grid_for((m + kScatterEdges - 1) / kScatterEdges), 256, 0, st>>>(g->W, g->pitch, n, src, dst, w, m, 0,
                                                                                    directed, check);
     } else if (e == cudaSuccess) {

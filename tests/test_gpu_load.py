@@ -80,3 +80,30 @@ def test_dense_matrix_from_aligned_and_odd_places(dj, orc, n):
     G = dj.dj_load_dense(W)
     assert np.array_equal(dj.dj_graph_download(G), W)
     G.free()
+
+
+@pytest.mark.parametrize("off", [1, 2, 3])
+def test_arrays_at_odd_byte_addresses(dj, orc, off):
+    """Edge arrays that are not 4-byte aligned (views into a byte buffer) load like any others."""
+    n, m = 300, 20000
+    e = graphgen.random_edges(n, m, 1, 90, seed=off, directed=True)
+
+    def odd(a):
+        buf = bytearray(4 * a.size + 4)
+        x = np.frombuffer(buf, np.int32, a.size, off)
+        x[:] = a
+        assert x.ctypes.data % 4 == off % 4
+        return x
+
+    for load in (dj.dj_load_edges, dj.dj_load_edges_csr):
+        for odd_src, odd_dst, odd_w in ((1, 1, 1), (1, 0, 0), (0, 1, 0), (0, 0, 1)):
+            s, t, w = (odd(a) if o else a for o, a in ((odd_src, e.src), (odd_dst, e.dst), (odd_w, e.w)))
+            G = load(n, s, t, w, True)
+            if load is dj.dj_load_edges:
+                assert np.array_equal(dj.dj_graph_download(G), orc.build_matrix(n, e.src, e.dst, e.w, True))
+            G.free()
+            bad = e.w.copy()
+            bad[m - 3] = -7
+            with pytest.raises(dj.DjError) as ei:
+                load(n, s, t, odd(bad), True)
+            assert f"edge {m - 3} " in str(ei.value) and "weight" in str(ei.value)

@@ -15,10 +15,12 @@ CSRC = os.path.join(ROOT, "paper_2504_03667_gb300", "csrc")
 NONE = 2**32 - 1
 
 PROG = r"""
+#include <cstddef>
 #include "dj_light_rules.h"
 extern "C" {
 unsigned pending(unsigned dist, unsigned hmin, unsigned D) { return dj::light_pending(dist, hmin, D); }
 int is_final(unsigned dist, unsigned hb) { return dj::light_final(dist, hb); }
+int in_place(size_t a, size_t b, size_t c) { return dj::edges_in_place((void*)a, (void*)b, (void*)c); }
 int needs_trial(unsigned hmin_min, unsigned wmin) { return dj::light_needs_trial(hmin_min, wmin); }
 }
 """
@@ -36,6 +38,7 @@ def rules(tmp_path_factory):
     lib = ctypes.CDLL(str(lib))
     for f, args in ((lib.pending, 3), (lib.is_final, 2), (lib.needs_trial, 2)):
         f.argtypes = [ctypes.c_uint32] * args
+    lib.in_place.argtypes = [ctypes.c_size_t] * 3
     lib.pending.restype = ctypes.c_uint32
     return lib
 
@@ -93,3 +96,11 @@ def test_trial_is_for_graphs_that_may_take_the_engine(rules):
     assert rules.needs_trial(5, 1) == 1
     assert rules.needs_trial(INF, 1) == 0  # every list complete
     assert rules.needs_trial(5, 0) == 0 and rules.needs_trial(0, 0) == 0  # weights of 0
+
+
+def test_unaligned_edge_arrays_are_not_read_in_place(rules):
+    for a in range(4096, 4104):
+        for place in range(3):
+            at = [8192, 12288, 16384]
+            at[place] = a
+            assert rules.in_place(*at) == (a % 4 == 0), at
