@@ -33,9 +33,10 @@ DJ_RULE bool light_final(uint32_t dist, uint32_t hb) { return dist <= hb; }
 // engines then, and its lists may hold nothing but a few of a row's edges of weight 0).
 DJ_RULE bool light_needs_trial(uint32_t hmin_min, uint32_t wmin) { return hmin_min < kRuleInf && wmin > 0; }
 
-// Whether the device may read the caller's edge arrays in place: 4-byte loads fault on other addresses.
+// Whether the device may read a caller's host array in place: 4-byte loads fault on other addresses.
+inline bool in_place(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
 inline bool edges_in_place(const void* src, const void* dst, const void* w) {
-  return ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(w)) & 3u) == 0;
+  return in_place(src) && in_place(dst) && in_place(w);
 }
 
 }  // namespace dj

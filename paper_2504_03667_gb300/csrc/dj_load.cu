@@ -884,8 +884,8 @@ extern "C" int dj_graph_upload(dj_graph* g, const int32_t* W, int64_t ld, uint64
   cudaPointerAttributes pa;
   const cudaError_t pe = cudaPointerGetAttributes(&pa, W);
   if (pe != cudaSuccess) cudaGetLastError();  // clear that query's own status only
-  const bool zero_copy =
-      g->light && pe == cudaSuccess && pa.type == cudaMemoryTypeHost && pa.devicePointer != nullptr;
+  const bool zero_copy = g->light && pe == cudaSuccess && pa.type == cudaMemoryTypeHost &&
+                         pa.devicePointer != nullptr && in_place(pa.devicePointer);  // else the copies: any address
   if (zero_copy) {
     const int32_t* src = static_cast<const int32_t*>(pa.devicePointer);
     const int vec = (ld % 4 == 0 && reinterpret_cast<uintptr_t>(src) % 16 == 0) ? 1 : 0;

@@ -107,3 +107,23 @@ def test_arrays_at_odd_byte_addresses(dj, orc, off):
             with pytest.raises(dj.DjError) as ei:
                 load(n, s, t, odd(bad), True)
             assert f"edge {m - 3} " in str(ei.value) and "weight" in str(ei.value)
+
+
+@pytest.mark.parametrize("n", [33, 64, 300])
+def test_upload_from_an_odd_byte_address(dj, orc, n):
+    """A matrix in pinned memory that is not 4-byte aligned uploads like any other."""
+    import torch
+    e = graphgen.random_edges(n, 9 * n, 1, 90, seed=n, directed=True)
+    W = orc.build_matrix(n, e.src, e.dst, e.w, True)
+    ref = orc.dijkstra(W, n // 2)
+    pinned = torch.zeros(4 * n * n + 4, dtype=torch.uint8).pin_memory()
+    for off in (1, 2, 3):
+        A = np.frombuffer(pinned.numpy(), np.int32, n * n, off).reshape(n, n)
+        A[:] = W
+        assert A.ctypes.data % 4 == off
+        G = dj.dj_load_edges(n, e.src, e.dst, np.ones(9 * n, np.int32), True)
+        dj.dj_graph_upload(G, A)
+        got = dj.dj_sssp_host(G, n // 2)
+        assert np.array_equal(dj.dj_graph_download(G), W)
+        assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+        G.free()

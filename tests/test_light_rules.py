@@ -21,6 +21,7 @@ extern "C" {
 unsigned pending(unsigned dist, unsigned hmin, unsigned D) { return dj::light_pending(dist, hmin, D); }
 int is_final(unsigned dist, unsigned hb) { return dj::light_final(dist, hb); }
 int in_place(size_t a, size_t b, size_t c) { return dj::edges_in_place((void*)a, (void*)b, (void*)c); }
+int upload_in_place(size_t a) { return dj::in_place((void*)a); }
 int needs_trial(unsigned hmin_min, unsigned wmin) { return dj::light_needs_trial(hmin_min, wmin); }
 }
 """
@@ -38,6 +39,7 @@ def rules(tmp_path_factory):
     lib = ctypes.CDLL(str(lib))
     for f, args in ((lib.pending, 3), (lib.is_final, 2), (lib.needs_trial, 2)):
         f.argtypes = [ctypes.c_uint32] * args
+    lib.upload_in_place.argtypes = [ctypes.c_size_t]
     lib.in_place.argtypes = [ctypes.c_size_t] * 3
     lib.pending.restype = ctypes.c_uint32
     return lib
@@ -104,3 +106,7 @@ def test_unaligned_edge_arrays_are_not_read_in_place(rules):
             at = [8192, 12288, 16384]
             at[place] = a
             assert rules.in_place(*at) == (a % 4 == 0), at
+
+
+def test_unaligned_matrix_is_not_read_in_place(rules):
+    assert [rules.upload_in_place(4096 + i) for i in range(5)] == [1, 0, 0, 0, 1]
