@@ -272,10 +272,10 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   // Longer lists have ten times the edges to offer, which every SM takes faster than one CTA or cluster, at
   // any size: 6001 nodes alone 127 us on a cluster, 52 here (the streaming grid engine: 78), 1500 nodes
   // 82 and 44 (94); behind other solves the forms that run side by side stay (15 us a solve against 50).
-  if (g->light_wide && stream_idle(st)) return launch_light_grid(g, source, dist, pred, o, nullptr, st);
+  if (g->light_wide && stream_idle(st)) return launch_light_grid(g, source, dist, pred, o, st);
   if (!cta && (!cluster || o.debug_skip_cta >= 0 ||
                (g->n >= (csr ? kLightIdleGridMinNComplete : kLightIdleGridMinN) && stream_idle(st))))
-    return launch_light_grid(g, source, dist, pred, o, nullptr, st);
+    return launch_light_grid(g, source, dist, pred, o, st);
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   const SolveDesc d = make_desc(g, source, dist, pred, 0);
@@ -286,11 +286,11 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
     const int rc = run_light_cluster(g, C, d, ctx->words + 1, early, st);
     if (rc != DJ_ECUDA) return rc;
     clear_error();  // no such cluster here
-    return launch_light_grid(g, source, dist, pred, o, nullptr, st);
+    return launch_light_grid(g, source, dist, pred, o, st);
   }
   LightPlan plan;
   if (int rc = plan_light(g->n, 1, kJobsSingle, &plan)) return rc;
-  return run_light_single(plan, d, ctx->words + 1, nullptr, early, st);
+  return run_light_single(plan, d, ctx->words + 1, early, st);
 }
 
 extern "C" int dj_sssp_ex(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts* opts,

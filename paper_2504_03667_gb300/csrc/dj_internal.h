@@ -67,10 +67,15 @@ constexpr int kLightCap = 64;    // edges listed per row
 constexpr int kLightWide = 128;  // ... where so many are needed and do; those beyond kLightCap lie apart
 constexpr int kLightStats = 64;  // leading words: [0] ~(smallest hmin), [1] rows relaxed whole by the trial solve,
                                  // [2..3] sum of the rows' largest listed weights, [4..5] of their listed edges,
-                                 // [6] most edges listed in a row, [8..11] ~(finite min), finite max, finite entries
+                                 // [6] most edges listed in a row, [7] the first trial's source
+                                 // (light_trial_word), [8..11] ~(finite min), finite max, finite entries
                                  // (at load), [12..14] the edge list's check (k_scatter),
-                                 // [15] kLightGuess
+                                 // [15] kLightGuess, [16..17] the trials' farthest node (dist, node),
+                                 // [24..] rows relaxed whole by each further trial
 constexpr int kLightGuess = 15;  // 1 + the trial solve's largest dist (0: unknown)
+constexpr int kLightFar = 16;
+constexpr int kLightMore = 24;
+constexpr int kMoreTrials = 16;  // from the farthest node and fifteen places (without the CTA form: fewer)
 inline
 #ifdef __CUDACC__
     __host__ __device__
@@ -212,6 +217,7 @@ struct ClusterPlan {
 constexpr int kJobsBatch = 0;
 constexpr int kJobsServe = 1;
 constexpr int kJobsSingle = 2;
+constexpr int kJobsTrial = 3;  // light engine: trial solves
 int plan_cluster(int32_t max_pitch, const ClusterLaunch& cl, int32_t k, ClusterPlan* plan, int kind = kJobsBatch);
 // queue: two device words (next solve, exit count), zero when the launch starts; with
 // zero_queue the launch zeroes them first, otherwise the previous launch left them zero
@@ -271,12 +277,13 @@ struct LightPlan {
 };
 bool light_cta_fits(int32_t n);  // one CTA's shared memory holds the keys of n nodes
 int plan_light(int32_t max_n, int32_t k, int kind, LightPlan* plan);
-// as run_cluster, run_cluster_single and run_serve_kernel; heavy: optional device word counting the rows
-// relaxed whole
+// as run_cluster, run_cluster_single and run_serve_kernel
 int run_light_batch(const LightPlan& plan, const SolveDesc* descs_dev, int32_t k, uint32_t* queue, bool zero_queue,
                     cudaStream_t st);
-int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, uint32_t* heavy, bool early,
-                     cudaStream_t st);
+int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, bool early, cudaStream_t st);
+// kMoreTrials trial solves of one graph side by side (LightTrialJobs): words [kLightMore..] count the rows
+// that each relaxed whole, up to the first count above kTrialRows.
+int run_light_trials(const LightPlan& plan, const SolveDesc& d, uint32_t* light, cudaStream_t st);
 int run_light_serve(const LightPlan& plan, const ServeRing& r, cudaStream_t st);
 // One solve on one cluster of C CTAs (a power of two up to 16), as run_light_single.
 bool light_cluster_fits(int32_t n, int C, bool csr);
@@ -285,7 +292,12 @@ int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t*
                       cudaStream_t st);
 // One solve over every SM (a graph with an index, or in compressed rows).
 int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
-                      uint32_t* heavy, cudaStream_t st);
+                      cudaStream_t st);
+// A trial solve, which writes nothing but the index's words.  From the source that the rows' words name
+// (kTrialFirst: it leaves kLightGuess), from the farthest node of the trials so far (kTrialFar), or from a
+// given one; those stop once more than kTrialRows rows were relaxed whole, counted in *heavy.
+constexpr int32_t kTrialFirst = -1, kTrialFar = -2;
+int launch_light_trial(const dj_graph* g, int32_t source, uint32_t* heavy, cudaStream_t st);
 int cluster_max_clusters(int32_t max_pitch, const ClusterLaunch& cl, int* clusters);
 bool cluster_config_ok(int32_t max_pitch, const ClusterLaunch& cl);
 

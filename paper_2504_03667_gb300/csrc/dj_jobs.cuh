@@ -19,6 +19,7 @@ struct BatchJobs {
   __device__ SolveDesc desc(uint32_t job) const { return descs[job]; }
   __device__ void complete(uint32_t, uint32_t) const {}
   static constexpr uint32_t kGuessPart = 3;  // light engine: the margin of its bound (light_guess)
+  static constexpr bool kTrial = false;      // light engine: nothing is written, whole rows are counted
   static constexpr bool kTrace = false;
   __device__ bool early() const { return true; }  // launched the ordinary way: nothing to wait for
   __device__ void before_write() const {}
@@ -58,6 +59,7 @@ struct SingleJob {
     if (phases_out) *phases_out = phases;
   }
   static constexpr uint32_t kGuessPart = 8;
+  static constexpr bool kTrial = false;
   static constexpr bool kTrace = true;  // the per-phase timeline is compiled into this kernel only
   __device__ bool early() const { return early_ok != 0; }
   __device__ void before_write() const { pdl_wait(); }
@@ -110,8 +112,34 @@ struct ServeJobs {
     st_release_sys(done + (job & cap_mask), job + 1);
   }
   static constexpr uint32_t kGuessPart = 8;
+  static constexpr bool kTrial = false;
   static constexpr bool kTrace = false;
   __device__ bool early() const { return true; }
+  __device__ void before_write() const {}
+  __device__ void leave(uint32_t) const {}
+};
+
+// Light engine: a CTA each for kMoreTrials trial solves of one graph, the first from the farthest node of
+// the trial before, the others from places spread over the ids.
+struct LightTrialJobs {
+  SolveDesc d;  // without outputs
+  uint32_t* light;
+  __device__ bool fetch(uint32_t* job, uint32_t iter) const {
+    *job = blockIdx.x;
+    return iter == 0;
+  }
+  __device__ SolveDesc desc(uint32_t job) const {
+    SolveDesc x = d;
+    x.source = job == 0 ? static_cast<int32_t>(__ldcg(light + kLightFar))
+                        : static_cast<int32_t>(static_cast<int64_t>(d.n) * (2 * job - 1) / (2 * kMoreTrials - 2));
+    return x;
+  }
+  __device__ void complete(uint32_t, uint32_t) const {}
+  __device__ uint32_t* whole(uint32_t job) const { return light + kLightMore + job; }
+  static constexpr uint32_t kGuessPart = 8;
+  static constexpr bool kTrial = true;
+  static constexpr bool kTrace = false;
+  __device__ bool early() const { return true; }  // launched the ordinary way: nothing to wait for
   __device__ void before_write() const {}
   __device__ void leave(uint32_t) const {}
 };

@@ -17,7 +17,6 @@ constexpr float kCtaDelta = 3.0f;
 }  // namespace
 
 struct LightCtaParams {
-  uint32_t* heavy;  // optional: rows relaxed whole are counted here
   int32_t npad;     // node slots (largest graph of the launch, rounded up to 64)
 };
 
@@ -111,6 +110,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
     uint32_t phase = 0, cur = 0;  // cur = phase % 3: the slot of this phase's m, the smallest dirty dist
     int raised = 0;
     bool any_whole = false;
+    uint32_t nwhole = 0;  // trial: rows relaxed whole
     for (;; ++phase) {
       const uint32_t m = s_m[cur];
       const uint32_t nxt = cur == 2 ? 0 : cur + 1;
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
           __syncthreads();
           any_whole = true;
           const int count = static_cast<int>(min(s_cnt, s_end));
-          if (p.heavy && tid == 0) atomicAdd(p.heavy, static_cast<uint32_t>(count));
+          if (Jobs::kTrial && (nwhole += static_cast<uint32_t>(count)) > kTrialRows) break;  // it has its answer
           light_whole_rows(s, d, s_rows[0], count, D, lmin);
         }
       }
@@ -252,6 +252,10 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
       if (lane == 0 && lmin != kNone) atomicMin(&s_m[nxt], lmin);
       __syncthreads();
       cur = nxt;
+    }
+    if constexpr (Jobs::kTrial) {
+      if (tid == 0) *jobs.whole(job) = nwhole;
+      continue;
     }
     // the dists are final: the best offer of each node's dist.  Only listed edges, and rows relaxed
     // whole, can make one.
@@ -321,10 +325,11 @@ int plan_light(int32_t max_n, int32_t k, int kind, LightPlan* plan) {
                    2 * (plan->smem + kLightCtaStatic) <= static_cast<size_t>(ctx->max_smem_optin);
   plan->fn = kind == kJobsServe    ? reinterpret_cast<void*>(&k_light_cta<192, 1, ServeJobs>)
              : kind == kJobsSingle ? reinterpret_cast<void*>(&k_light_cta<512, 1, SingleJob>)
+             : kind == kJobsTrial  ? reinterpret_cast<void*>(&k_light_cta<512, 1, LightTrialJobs>)
              : two                 ? reinterpret_cast<void*>(&k_light_cta<512, 2, BatchJobs>)
                                    : reinterpret_cast<void*>(&k_light_cta<512, 1, BatchJobs>);
   if (int rc = prepare_function(ctx, plan->fn, plan->smem, false)) return rc;
-  plan->ctas = kind == kJobsSingle ? 1 : ctx->num_sms * (two ? 2 : 1);
+  plan->ctas = kind == kJobsSingle ? 1 : kind == kJobsTrial ? kMoreTrials : ctx->num_sms * (two ? 2 : 1);
   if (kind == kJobsBatch) plan->ctas = std::max(1, std::min(plan->ctas, static_cast<int>(k)));
   return DJ_OK;
 }
@@ -356,7 +361,7 @@ int run_light_batch(const LightPlan& plan, const SolveDesc* descs_dev, int32_t k
     cudaError_t e = cudaMemsetAsync(queue, 0, 2 * sizeof(uint32_t), st);
     if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync(queue)");
   }
-  LightCtaParams p{nullptr, plan.npad};
+  LightCtaParams p{plan.npad};
   BatchJobs jobs;
   jobs.descs = descs_dev;
   jobs.queue = queue;
@@ -365,9 +370,8 @@ int run_light_batch(const LightPlan& plan, const SolveDesc* descs_dev, int32_t k
   return launch_light(plan, args, st, false);
 }
 
-int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, uint32_t* heavy, bool early,
-                     cudaStream_t st) {
-  LightCtaParams p{heavy, plan.npad};
+int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, bool early, cudaStream_t st) {
+  LightCtaParams p{plan.npad};
   SingleJob job;
   job.d = d;
   job.phases_out = phases_out;
@@ -376,8 +380,17 @@ int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases
   return launch_light(plan, args, st, true);
 }
 
+int run_light_trials(const LightPlan& plan, const SolveDesc& d, uint32_t* light, cudaStream_t st) {
+  LightCtaParams p{plan.npad};
+  LightTrialJobs jobs;
+  jobs.d = d;
+  jobs.light = light;
+  void* args[] = {&p, &jobs};
+  return launch_light(plan, args, st, false);
+}
+
 int run_light_serve(const LightPlan& plan, const ServeRing& r, cudaStream_t st) {
-  LightCtaParams p{nullptr, plan.npad};
+  LightCtaParams p{plan.npad};
   ServeJobs jobs;
   jobs.ring = r.ring;
   jobs.tail = r.tail;

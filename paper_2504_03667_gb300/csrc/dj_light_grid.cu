@@ -46,13 +46,13 @@ struct LightGridParams {
   uint32_t* ctl;              // workspace control words (zero when a launch starts)
   unsigned long long* gkey;   // n keys
   uint32_t* words;            // per-device words: [0] error bits, [1] phases
-  uint32_t* heavy;            // optional: rows relaxed whole are counted here
-  uint32_t* guess;            // trial: the index's kLightGuess
+  uint32_t* heavy;            // trial: rows relaxed whole are counted here
+  uint32_t* guess;            // the first trial: the index's kLightGuess
   int64_t pitch;
   int64_t timeout_ns;
   int32_t n;
   int32_t swcap;
-  int32_t source;
+  int32_t source;             // trial: or kTrialFirst, kTrialFar
   uint32_t bits_u;
   uint32_t delta;     // compressed rows (dense graphs: from the index's statistics, light_window)
   int32_t gshift;     // the same: log2 of the lanes that share a row
@@ -180,12 +180,15 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
   if (!CSR) light_window(p.light, kGridDelta, &delta, &gshift);
   // a trial is of use to graphs whose solves may take this engine: some list cut, no weight of 0
   if (!CSR && p.trial && !light_needs_trial(hmin_min, ~__ldg(p.light + 8))) return;
+  const int source = p.source >= 0            ? p.source
+                     : p.source == kTrialFirst ? static_cast<int>(light_trial_source(__ldcg(p.light + 7), p.n))
+                                               : static_cast<int>(__ldcg(p.light + kLightFar));
   // offers above the guessed largest dist are dropped at first (see below); the trial makes the guess
   uint32_t guess = CSR || p.trial || hmin_min >= kInf ? kNone : light_guess(p.light, 8);
   for (int j = tid; j < sw; j += T0) {
     const int v = c0 + j;
-    p.gkey[v] = v == p.source ? 0ull : ~0ull;
-    rdist[j] = v == p.source ? 0u : kInf;
+    p.gkey[v] = v == source ? 0ull : ~0ull;
+    rdist[j] = v == source ? 0u : kInf;
     flags[j] = static_cast<uint32_t>(__ldg(p.minin + v)) < kInf ? 1 : 0;
     if (CSR) {
       const int64_t s0 = p.row_ptr[v];
@@ -199,14 +202,14 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
   // the source's listed edges that land in this slice (every CTA reads the list)
   uint32_t lmin = kNone;
   {
-    const int64_t s0 = CSR ? p.row_ptr[p.source] : static_cast<int64_t>(p.source) * kLightCap;
-    const int64_t len = CSR ? p.row_ptr[p.source + 1] - s0 : most;
+    const int64_t s0 = CSR ? p.row_ptr[source] : static_cast<int64_t>(source) * kLightCap;
+    const int64_t len = CSR ? p.row_ptr[source + 1] - s0 : most;
     for (int64_t i = tid; i < len; i += T0) {
       const uint32_t e = __ldg(p.edge + s0 + i + (!CSR && i >= kLightCap ? light_apart(p.n) : 0));
       if (e == kNoEdge) break;
       const uint32_t v = e & umask;
-      if (v - static_cast<uint32_t>(c0) >= static_cast<uint32_t>(sw) || static_cast<int>(v) == p.source) continue;
-      const uint64_t key = light_key(0u, e >> bits_u, static_cast<uint32_t>(p.source), bits_u);
+      if (v - static_cast<uint32_t>(c0) >= static_cast<uint32_t>(sw) || static_cast<int>(v) == source) continue;
+      const uint64_t key = light_key(0u, e >> bits_u, static_cast<uint32_t>(source), bits_u);
       p.gkey[v] = key;  // one edge per target
       lmin = min(lmin, e >> bits_u);
     }
@@ -365,20 +368,29 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
     // every row that was dirty has been relaxed, so the slice's dists (and D) only change through these rows
     if (!light_barrier(p, sh, nbar++, lmin, Dx, &m, &D)) return;
     ++phases;
+    // a further trial has its answer (every CTA reads the same count: the next one is added after a barrier)
+    if (p.trial && !p.guess && __ldcg(p.heavy) > kTrialRows) return;
   }
-  for (int j = p.trial ? sw : tid; j < sw; j += T0) {
+  if (p.trial) {
+    uint64_t far = 0;
+    for (int j = tid; j < sw; j += T0)
+      if (rdist[j] < kInf) far = max(far, (static_cast<uint64_t>(rdist[j]) << 32) | static_cast<uint32_t>(c0 + j));
+    const uint32_t hi = __reduce_max_sync(0xffffffffu, static_cast<uint32_t>(far >> 32));
+    const uint32_t lo = __reduce_max_sync(0xffffffffu, static_cast<uint32_t>(far >> 32) == hi ? static_cast<uint32_t>(far) : 0u);
+    if ((tid & 31) == 0)
+      atomicMax(reinterpret_cast<unsigned long long*>(const_cast<uint32_t*>(p.light) + kLightFar),
+                (static_cast<unsigned long long>(hi) << 32) | lo);
+    if (b == 0 && tid == 0 && p.guess && D < kInf) p.guess[0] = D + 1;
+    return;
+  }
+  for (int j = tid; j < sw; j += T0) {
     const uint64_t k = __ldcg(p.gkey + c0 + j);
     const uint32_t d = static_cast<uint32_t>(k >> 32);
     const bool reached = d < kInf;
     p.dist_out[c0 + j] = static_cast<int32_t>(reached ? d : kInf);
-    p.pred_out[c0 + j] = reached && c0 + j != p.source ? static_cast<int32_t>(static_cast<uint32_t>(k) & umask) : -1;
+    p.pred_out[c0 + j] = reached && c0 + j != source ? static_cast<int32_t>(static_cast<uint32_t>(k) & umask) : -1;
   }
-  if (b == 0 && tid == 0) {
-    if (!p.trial)
-      p.words[1] = phases;
-    else if (D < kInf)
-      p.guess[0] = D + 1;
-  }
+  if (b == 0 && tid == 0) p.words[1] = phases;
 }
 
 template <bool CSR>
@@ -411,8 +423,9 @@ __global__ void __launch_bounds__(kLightGridThreads, 1) k_light_grid(const Light
 
 namespace dj {
 
-int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
-                      uint32_t* heavy, cudaStream_t st) {
+// heavy: the launch is a trial.
+static int run_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
+                          uint32_t* heavy, cudaStream_t st) {
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   if (!ctx->coop) return set_error(DJ_EUNSUPPORTED, "device lacks cooperative launch");
@@ -447,7 +460,7 @@ int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t*
   p.gkey = reinterpret_cast<unsigned long long*>(ws + ctl_bytes);
   p.words = ctx->words;
   p.heavy = heavy;
-  p.guess = csr ? nullptr : g->light + kLightGuess;
+  p.guess = heavy && source == kTrialFirst ? g->light + kLightGuess : nullptr;
   p.pitch = g->pitch;
   p.timeout_ns = o.timeout_ns > 0 ? o.timeout_ns : 2000000000LL;
   p.n = g->n;
@@ -456,13 +469,24 @@ int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t*
   p.bits_u = host_bits_for(static_cast<uint32_t>(g->n));
   p.delta = static_cast<uint32_t>(std::min(1.0e9f, kGridDelta * g->light_spacing));
   p.gshift = g->light_gshift;
-  p.trial = dist ? 0 : 1;
+  p.trial = heavy ? 1 : 0;
   p.skip_cta = o.debug_skip_cta;
   void* args[] = {&p};
   e = launch_cooperative(fn, G, kLightGridThreads, args, smem, st, true);
   if (own_ws) cudaFreeAsync(ws, st);
   if (e != cudaSuccess) return cuda_error(e, "cooperative launch (light engine)");
   return DJ_OK;
+}
+
+int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
+                      cudaStream_t st) {
+  return run_light_grid(g, source, dist, pred, o, nullptr, st);
+}
+
+int launch_light_trial(const dj_graph* g, int32_t source, uint32_t* heavy, cudaStream_t st) {
+  dj_solve_opts o;
+  dj_solve_opts_init(&o);
+  return run_light_grid(g, source, nullptr, nullptr, o, heavy, st);
 }
 
 }  // namespace dj

@@ -33,6 +33,26 @@ DJ_RULE bool light_final(uint32_t dist, uint32_t hb) { return dist <= hb; }
 // engines then, and its lists may hold nothing but a few of a row's edges of weight 0).
 DJ_RULE bool light_needs_trial(uint32_t hmin_min, uint32_t wmin) { return hmin_min < kRuleInf && wmin > 0; }
 
+// The first trial's source: a row with edges, of those with the most edges listed, n / 2 if it is one of
+// them (a node that leads nowhere, or into a small part of the graph, says nothing about the others).  The
+// rows' words are combined by maximum; n is below 2^24 (the matrix has n^2 entries).
+DJ_RULE uint32_t light_trial_word(uint32_t u, uint32_t listed, bool has_edges, uint32_t n) {
+  const uint32_t back = (u + n - n / 2 - 1) % n;  // n - 1 for u = n / 2
+  return ((has_edges ? listed + 1 : 0u) << 24) | back;
+}
+DJ_RULE uint32_t light_trial_source(uint32_t word, uint32_t n) { return ((word & 0xFFFFFFu) + n / 2 + 1) % n; }
+
+// What the first trial says about a graph with cut lists.  kTrialNo: no.  kTrialAll: no source needs a whole
+// row -- on a symmetric matrix no largest dist is more than twice the trial's, and every unlisted edge is
+// heavier.  kTrialAsk: other sources have to be tried (a structured graph's, or one of few distinct weights,
+// may need many rows where this one needed none).
+enum { kTrialNo, kTrialAll, kTrialAsk };
+constexpr uint32_t kTrialRows = 4;  // whole rows a trial may need
+inline int light_trial_verdict(uint32_t rows, uint32_t guess, uint32_t hmin_min, bool symmetric) {
+  if (guess == 0 || rows > kTrialRows) return kTrialNo;  // guess 0: not every node that has an in-edge was reached
+  return symmetric && hmin_min > 2 * static_cast<uint64_t>(guess - 1) ? kTrialAll : kTrialAsk;
+}
+
 // Whether the device may read a caller's host array in place: 4-byte loads fault on other addresses.
 inline bool in_place(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
 inline bool edges_in_place(const void* src, const void* dst, const void* w) {

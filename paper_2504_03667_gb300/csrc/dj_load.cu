@@ -159,7 +159,7 @@ struct LightOut {
 };
 struct LightSums {
   unsigned long long last = 0, cnt = 0;
-  uint32_t hmin = 0xFFFFFFFFu, most = 0;
+  uint32_t hmin = 0xFFFFFFFFu, most = 0, trial = 0;
 };
 
 // The first threshold of light_select, in the middle of its window of counts: as if the weights were
@@ -209,6 +209,7 @@ __device__ __forceinline__ void light_row(const LightOut& o, const Scan& scan, u
   sums.cnt += r.cnt;
   sums.hmin = min(sums.hmin, r.hmin);
   sums.most = max(sums.most, r.cnt);
+  sums.trial = max(sums.trial, light_trial_word(u, r.cnt, r.first < kInf, static_cast<uint32_t>(o.n)));
 }
 
 __device__ __forceinline__ void light_sums_out(const LightOut& o, const LightSums& s) {
@@ -217,6 +218,7 @@ __device__ __forceinline__ void light_sums_out(const LightOut& o, const LightSum
   atomicAdd(reinterpret_cast<unsigned long long*>(o.light + 2), s.last);
   atomicAdd(reinterpret_cast<unsigned long long*>(o.light + 4), s.cnt);
   atomicMax(o.light + 6, s.most);
+  atomicMax(o.light + 7, s.trial);
 }
 
 // The rows of the resident matrix; with `stats` also the finite min / max and the number of finite
@@ -618,12 +620,38 @@ static void launch_minima(dj_graph* g, uint32_t* stats, cudaStream_t st, bool ha
 
 // The trial solve on the index, and the index's leading words on their way to the host.
 static bool launch_trial(dj_graph* g, uint32_t* idx, cudaStream_t st) {
-  dj_solve_opts o;
-  dj_solve_opts_init(&o);
-  const bool tried = launch_light_grid(g, g->n / 2, nullptr, nullptr, o, g->light + 1, st) == DJ_OK;
+  const bool tried = launch_light_trial(g, kTrialFirst, g->light + 1, st) == DJ_OK;
   clear_error();  // it cannot run here: the other engines
   cudaMemcpyAsync(idx, g->light, 16 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
   return tried;
+}
+
+// Whether a graph with cut lists is one whose solves hardly need a row whole, by its trial (idx) and, where
+// that leaves it open, by further ones: side by side, a CTA each, where the state fits one (n = 300, 1500
+// and 8192: about 35, 70 and 180 us), else one after another over every SM.
+static int judge_cut(dj_graph* g, const uint32_t* idx, cudaStream_t st, bool* good) {
+  const int verdict = light_trial_verdict(idx[1], idx[kLightGuess], ~idx[0], !g->directed);
+  *good = verdict == kTrialAll;
+  if (verdict != kTrialAsk) return DJ_OK;
+  uint32_t* more = g->light + kLightMore;
+  cudaMemsetAsync(more, 0, kMoreTrials * sizeof(uint32_t), st);
+  bool tried = true;
+  if (light_cta_fits(g->n)) {
+    LightPlan plan;
+    tried = plan_light(g->n, kMoreTrials, kJobsTrial, &plan) == DJ_OK &&
+            run_light_trials(plan, make_desc(g, 0, nullptr, nullptr, 0), g->light, st) == DJ_OK;
+  } else {
+    for (int i = 0; i < 6; ++i)  // the farthest node, the farthest from that, and four places
+      tried = tried && launch_light_trial(g, i < 2 ? kTrialFar : static_cast<int32_t>(static_cast<int64_t>(g->n) * (2 * i - 3) / 8),
+                                          more + i, st) == DJ_OK;
+  }
+  clear_error();
+  uint32_t rows[kMoreTrials] = {0};
+  cudaMemcpyAsync(rows, more, sizeof(rows), cudaMemcpyDeviceToHost, st);
+  const cudaError_t e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return cuda_error(e, "trial solves");
+  *good = tried && *std::max_element(rows, rows + kMoreTrials) <= kTrialRows;
+  return DJ_OK;
 }
 
 // Whether lists of kLightWide edges would hold every edge that matters: the source's row needs the most of
@@ -670,27 +698,36 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   g->light_deg = static_cast<float>(static_cast<double>(g->entries) / g->n);
   if (g->n > 1 && static_cast<int64_t>(g->n - 1) * g->wmax >= static_cast<int64_t>(DJ_INF))
     return set_error(DJ_EOVERFLOW, "(n-1) * max weight >= INT32_MAX: path lengths could overflow int32");
-  // Taken at once if every row's list is complete, else if a trial solve relaxed next to no row whole:
-  // where many are needed (nearly equal weights, distances long against what the lists reach) the other
-  // engines stream the matrix better (n = 8192, p = 0.5, weights 1..10: 410 rows whole, 112 us; grid
-  // engine 37).  One CTA or cluster relaxes many whole rows slowly (4500 in 7 ms, the grid form in 0.2),
-  // so these forms are for complete lists and symmetric matrices: no source's largest dist is then more
-  // than twice the trial's, while a directed graph's may be by any factor.
+  // Taken at once if every row's list is complete, else if trial solves relaxed next to no row whole:
+  // where many are needed (nearly equal weights, distances long against what the lists reach, parts that
+  // a source cannot reach) the other engines stream the matrix better (n = 8192, p = 0.5, weights 1..10: 410
+  // rows whole, 112 us; grid engine 37).  One CTA or cluster relaxes many whole rows slowly (4500 in 7 ms,
+  // the grid form in 0.2), so these forms are for complete lists and symmetric matrices.  Where the first
+  // trial does not settle it for every source (light_trial_verdict), more are made.  A graph whose
+  // trial did not reach every node that something leads to is left to the other engines: two parts of 4000
+  // nodes, p = 0.3, took a CTA 15.3 ms a solve, the cluster engine 0.7.
   // Lists of kLightWide edges are built instead (one more pass and trial) where these look enough: n = 6001,
   // p = 0.05, weights 1..10 needs 288 rows whole with 64 edges listed, none with 128, and takes 14.6 us a
   // solve (the streaming grid engine 51) for a load of 0.54 ms instead of 0.45 (before the index: 1.64).
-  if (tried && g->wmin >= 1 && ~idx[0] < kInf && idx[1] > 4 && wide_suffices(g, idx)) {
+  bool good = false;
+  tried = tried && g->wmin >= 1;
+  bool complete = tried && ~idx[0] >= kInf;
+  if (tried && !complete)
+    if (int rc = judge_cut(g, idx, st, &good)) return rc;
+  if (tried && !complete && !good && wide_suffices(g, idx)) {
     cudaMemsetAsync(g->light, 0, 8 * sizeof(uint32_t), st);
-    cudaMemsetAsync(g->light + kLightGuess, 0, sizeof(uint32_t), st);
+    cudaMemsetAsync(g->light + kLightGuess, 0, 3 * sizeof(uint32_t), st);  // and kLightFar
     k_light_rows<kLightWide><<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(g->W, g->pitch, light_out(g),
                                                                                         false);
     tried = launch_trial(g, idx, st);
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_error(e, "building the longer lists");
     g->light_wide = true;
+    complete = tried && ~idx[0] >= kInf;
+    if (tried && !complete)
+      if (int rc = judge_cut(g, idx, st, &good)) return rc;
   }
-  const bool complete = ~idx[0] >= kInf;
-  g->light_ok = tried && g->wmin >= 1 && (complete || idx[1] <= 4);
+  g->light_ok = complete || good;
   g->light_cta = g->light_ok && (complete || !g->directed);
   // graphs that are not dense keep in-lists for the grid engine's dynamic IN bound
   const uint64_t nn = static_cast<uint64_t>(g->n) * static_cast<uint64_t>(g->n);

@@ -326,3 +326,40 @@ def test_longer_lists_end_with_an_upload(dj, orc, n):
         del cg
         batch.free()
         G.free()
+
+
+def without(e, nodes):
+    """e with the given nodes isolated."""
+    keep = ~(np.isin(e.src, nodes) | np.isin(e.dst, nodes))
+    return graphgen.EdgeList(e.n, e.src[keep], e.dst[keep], e.w[keep], e.directed)
+
+
+def star(parts, size, bridge, seed):
+    """Dense parts whose first nodes hang on the middle part's: from that node the lists suffice."""
+    es = [graphgen.bernoulli(size, 0.5, 1, 1000, seed + i) for i in range(parts)]
+    hubs = np.arange(parts, dtype=np.int32) * size
+    mid = hubs[parts // 2]
+    src = np.concatenate([e.src + h for e, h in zip(es, hubs)] + [np.full(parts - 1, mid)])
+    dst = np.concatenate([e.dst + h for e, h in zip(es, hubs)] + [hubs[hubs != mid]])
+    w = np.concatenate([e.w for e in es] + [np.full(parts - 1, bridge)])
+    return graphgen.EdgeList(parts * size, src.astype(np.int32), dst.astype(np.int32), w.astype(np.int32), False)
+
+
+@pytest.mark.parametrize("n", [300, 1500, 5000])
+def test_one_source_says_nothing_about_the_others(dj, orc, n):
+    """Graphs whose middle node leads nowhere, into a small part, or is nearer to everything than any other."""
+    h = n // 2
+    for whi in (2, 10, 1000):
+        b = graphgen.bernoulli(n, 0.4, 1, whi, n)
+        check(dj, orc, without(b, [h]), [0, h, n - 1], f"n={n} isolated middle, w up to {whi}")
+    d = graphgen.EdgeList(n, np.concatenate([b.src, b.dst]), np.concatenate([b.dst, b.src]),
+                          np.concatenate([b.w, b.w]), True)
+    keep = d.src != h
+    check(dj, orc, graphgen.EdgeList(n, d.src[keep], d.dst[keep], d.w[keep], True), [1, h], f"n={n} sink in the middle")
+    two = without(b, [h, h + 1])
+    keep = (two.src < h) == (two.dst < h)
+    pair = graphgen.EdgeList(n, np.append(two.src[keep], h).astype(np.int32), np.append(two.dst[keep], h + 1).astype(np.int32),
+                             np.append(two.w[keep], 7).astype(np.int32), False)
+    check(dj, orc, pair, [0, h, n - 1], f"n={n} two parts and a pair")
+    for bridge in (20, 150):
+        check(dj, orc, star(3, n // 3, bridge, n), [0, n // 3 + 5, n // 3 * 3 - 1], f"n={n} star, bridge {bridge}")

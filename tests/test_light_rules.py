@@ -22,6 +22,13 @@ unsigned pending(unsigned dist, unsigned hmin, unsigned D) { return dj::light_pe
 int is_final(unsigned dist, unsigned hb) { return dj::light_final(dist, hb); }
 int in_place(size_t a, size_t b, size_t c) { return dj::edges_in_place((void*)a, (void*)b, (void*)c); }
 int upload_in_place(size_t a) { return dj::in_place((void*)a); }
+unsigned trial_word(unsigned u, unsigned listed, int has_edges, unsigned n) {
+  return dj::light_trial_word(u, listed, has_edges, n);
+}
+unsigned trial_source(unsigned word, unsigned n) { return dj::light_trial_source(word, n); }
+int verdict(unsigned rows, unsigned guess, unsigned hmin_min, int symmetric) {
+  return dj::light_trial_verdict(rows, guess, hmin_min, symmetric);
+}
 int needs_trial(unsigned hmin_min, unsigned wmin) { return dj::light_needs_trial(hmin_min, wmin); }
 }
 """
@@ -37,11 +44,13 @@ def rules(tmp_path_factory):
     src.write_text(PROG)
     subprocess.run([cxx, "-std=c++17", "-O1", "-fPIC", "-shared", "-I", CSRC, str(src), "-o", str(lib)], check=True)
     lib = ctypes.CDLL(str(lib))
-    for f, args in ((lib.pending, 3), (lib.is_final, 2), (lib.needs_trial, 2)):
+    for f, args in ((lib.pending, 3), (lib.is_final, 2), (lib.needs_trial, 2), (lib.trial_word, 4), (lib.trial_source, 2),
+                    (lib.verdict, 4)):
         f.argtypes = [ctypes.c_uint32] * args
     lib.upload_in_place.argtypes = [ctypes.c_size_t]
     lib.in_place.argtypes = [ctypes.c_size_t] * 3
-    lib.pending.restype = ctypes.c_uint32
+    for f in (lib.pending, lib.trial_word, lib.trial_source):
+        f.restype = ctypes.c_uint32
     return lib
 
 
@@ -110,3 +119,25 @@ def test_unaligned_edge_arrays_are_not_read_in_place(rules):
 
 def test_unaligned_matrix_is_not_read_in_place(rules):
     assert [rules.upload_in_place(4096 + i) for i in range(5)] == [1, 0, 0, 0, 1]
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 8, 9, 1000, 262145])
+def test_trial_source_has_edges(rules, n):
+    """n / 2 if it lists as many edges as any, else a row that does; never a row without edges while one has some."""
+    h = n // 2
+    best = lambda rows: rules.trial_source(max(rules.trial_word(u, c, e, n) for u, c, e in rows), n)
+    nodes = sorted({0, 1 % n, h, n - 1})
+    assert best([(u, 64, 1) for u in nodes]) == h
+    for u in nodes:
+        assert best([(v, 0, int(v == u)) for v in nodes]) == u  # only u has edges (all too heavy to list)
+        assert best([(v, 128 if v == u else 127, 1) for v in nodes]) == u
+        assert rules.trial_word(u, 128, 1, n) < 2**32
+
+
+def test_trial_verdict(rules):
+    no, every, ask = 0, 1, 2
+    assert rules.verdict(0, 0, 10**6, 1) == no  # did not reach every node that something leads to
+    assert rules.verdict(5, 10, 10**6, 1) == no and rules.verdict(4, 10, 10**6, 1) == every
+    assert rules.verdict(0, 10, 18, 1) == ask and rules.verdict(0, 10, 19, 1) == every  # largest dist 9
+    assert rules.verdict(0, 10, 10**6, 0) == ask  # directed: any other source may be farther from the rest
+    assert rules.verdict(0, 2**31 - 1, 2**31 - 2, 1) == ask
