@@ -205,18 +205,23 @@ static int default_cluster_size(int32_t n) {
   return 8;
 }
 
-static int solve_cluster_single(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred,
-                                const dj_solve_opts& o, cudaStream_t st) {
+// The cluster engine's plan for single solves of g (which also sets its kernel's launch attributes).
+static int plan_cluster_single(const dj_graph* g, const dj_solve_opts& o, ClusterPlan* plan) {
   ClusterLaunch cl;
   cl.cluster_size = o.cluster_size > 0 ? o.cluster_size : default_cluster_size(g->n);
   cl.clusters = 1;
+  return plan_cluster(g->pitch, cl, 1, plan, kJobsSingle);
+}
+
+static int solve_cluster_single(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred,
+                                const dj_solve_opts& o, cudaStream_t st) {
   SolveDesc d = make_desc(g, source, dist, pred, o.mode == DJ_MODE_PLAIN ? 1 : 0);
   if (o.settle == DJ_SETTLE_OUT) d.use_in = 0;
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   // one cluster, the descriptor in the kernel's parameters: a single launch, no device memory
   ClusterPlan plan;
-  if (int rc = plan_cluster(g->pitch, cl, 1, &plan, kJobsSingle)) return rc;
+  if (int rc = plan_cluster_single(g, o, &plan)) return rc;
   // right after an upload the solve waits for the kernels before it before reading the graph
   const bool early = g->upload_pending == 0;
   const_cast<dj_graph*>(g)->upload_pending = 0;
@@ -293,6 +298,12 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   return run_light_single(plan, d, ctx->words + 1, early, st);
 }
 
+// Whether solves of g behind others on their stream take the light engine.  A directed matrix with cut lists
+// has only its grid form, which takes them one after another; on the sizes of the cluster engine that one
+// runs them side by side (n = 1024, p = 0.3: 19 us a solve, 11 in a CUDA graph; the grid form 41 in either).
+// A lone solve is faster on the grid form (62 us from call to end, the cluster engine 147).
+static bool light_behind(const dj_graph* g) { return g->format == DJ_FORMAT_CSR || g->light_cta || auto_grid(g); }
+
 extern "C" int dj_sssp_ex(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts* opts,
                           uint64_t stream) {
   clear_error();
@@ -307,7 +318,14 @@ extern "C" int dj_sssp_ex(const dj_graph* g, int32_t source, int32_t* dist, int3
   if (o.rowsplit < -1) return set_error(DJ_EINVAL, "rowsplit must be -1, 0 or a candidate count");
   if (o.rowpush < -1) return set_error(DJ_EINVAL, "rowpush must be -1, 0 or a candidate count");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (light_auto(g, o)) return solve_light(g, source, dist, pred, o, st);
+  if (light_auto(g, o)) {
+    if (light_behind(g)) return solve_light(g, source, dist, pred, o, st);
+    if (stream_idle(st)) {
+      ClusterPlan later;  // the next call may be captured, and then takes the cluster engine
+      if (int rc = plan_cluster_single(g, o, &later)) return rc;
+      return solve_light(g, source, dist, pred, o, st);
+    }
+  }
   if (g->format == DJ_FORMAT_CSR) return launch_csr(g, source, dist, pred, o, st);
   int engine = o.engine;
   if (engine == DJ_ENGINE_AUTO) engine = auto_grid(g) ? DJ_ENGINE_GRID : DJ_ENGINE_CLUSTER;

@@ -363,3 +363,43 @@ def test_one_source_says_nothing_about_the_others(dj, orc, n):
     check(dj, orc, pair, [0, h, n - 1], f"n={n} two parts and a pair")
     for bridge in (20, 150):
         check(dj, orc, star(3, n // 3, bridge, n), [0, n // 3 + 5, n // 3 * 3 - 1], f"n={n} star, bridge {bridge}")
+
+
+@pytest.mark.parametrize("n,p", [(70, 0.95), (1024, 0.3), (2500, 0.1), (3000, 0.3)])
+def test_directed_matrices_with_cut_lists(dj, orc, n, p):
+    """Alone, behind one another, captured and after an upload: the answer is the same whichever engine takes them."""
+    import torch
+    b = [graphgen.bernoulli(n, p, 1, 1000, n + i) for i in range(2)]
+    e = graphgen.EdgeList(n, np.concatenate([b[0].src, b[1].dst]), np.concatenate([b[0].dst, b[1].src]),
+                          np.concatenate([b[0].w, b[1].w]), True)
+    W = orc.build_matrix(n, e.src, e.dst, e.w, True)
+    srcs = [0, n // 2, n - 1]
+    refs = [orc.dijkstra(W, s) for s in srcs]
+    for g in (dj.dj_load_edges(n, e.src, e.dst, e.w, True), dj.dj_load_dense(W)):
+        st = torch.cuda.Stream()
+        D = torch.empty((3, n), dtype=torch.int32, device="cuda")
+        P = torch.empty_like(D)
+
+        def solve(alone):
+            for i, s in enumerate(srcs):
+                dj.dj_sssp(g, s, D[i], P[i], st)
+                if alone:
+                    dj.dj_sync(st)
+
+        solve(True)
+        cg = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(cg, stream=st):
+            solve(False)
+        for how, again in (("alone", lambda: solve(True)), ("behind", lambda: solve(False)), ("captured", cg.replay),
+                           ("uploaded", lambda: (dj.dj_graph_upload(g, W, st), solve(False)))):
+            torch.cuda.synchronize()
+            D.fill_(-5)
+            P.fill_(-5)
+            torch.cuda.synchronize()
+            again()
+            torch.cuda.synchronize()
+            for i in range(3):
+                assert np.array_equal(D[i].cpu().numpy(), refs[i][0]), (how, i)
+                assert np.array_equal(P[i].cpu().numpy(), refs[i][1]), (how, i)
+        del cg
+        g.free()
