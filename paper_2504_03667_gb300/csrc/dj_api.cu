@@ -13,6 +13,7 @@
 
 #include "dj_common.cuh"
 #include "dj_internal.h"
+#include "dj_light_rules.h"
 
 namespace dj {
 
@@ -247,7 +248,6 @@ static bool light_auto(const dj_graph* g, const dj_solve_opts& o) {
 // the grid form gives one solve every SM.  So a large solve takes the grid form only when nothing is
 // ahead of it on its stream (someone is waiting for this one), and so it does when one CTA or cluster
 // would be slow with the whole rows its graph may need.
-static constexpr int32_t kLightClusterMinN = 2048;
 static constexpr int32_t kLightIdleGridMinN = 6144;
 static constexpr int32_t kLightIdleGridMinNComplete = 16384;  // compressed rows: fewer offers per phase
 static constexpr uint32_t kLightClusterMaxRow = 512;          // longer compressed rows: the grid form shares them out
@@ -277,7 +277,8 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   // Longer lists have ten times the edges to offer, which every SM takes faster than one CTA or cluster, at
   // any size: 6001 nodes alone 127 us on a cluster, 52 here (the streaming grid engine: 78), 1500 nodes
   // 82 and 44 (94); behind other solves the forms that run side by side stay (15 us a solve against 50).
-  if (g->light_wide && stream_idle(st)) return launch_light_grid(g, source, dist, pred, o, st);
+  // (Graphs of few phases come here only on an idle stream.)
+  if (g->light_few || (g->light_wide && stream_idle(st))) return launch_light_grid(g, source, dist, pred, o, st);
   if (!cta && (!cluster || o.debug_skip_cta >= 0 ||
                (g->n >= (csr ? kLightIdleGridMinNComplete : kLightIdleGridMinN) && stream_idle(st))))
     return launch_light_grid(g, source, dist, pred, o, st);
@@ -301,8 +302,11 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
 // Whether solves of g behind others on their stream take the light engine.  A directed matrix with cut lists
 // has only its grid form, which takes them one after another; on the sizes of the cluster engine that one
 // runs them side by side (n = 1024, p = 0.3: 19 us a solve, 11 in a CUDA graph; the grid form 41 in either).
-// A lone solve is faster on the grid form (62 us from call to end, the cluster engine 147).
-static bool light_behind(const dj_graph* g) { return g->format == DJ_FORMAT_CSR || g->light_cta || auto_grid(g); }
+// A lone solve is faster on the grid form (62 us from call to end, the cluster engine 147).  So it is with
+// graphs of few phases (light_few).
+static bool light_behind(const dj_graph* g) {
+  return g->format == DJ_FORMAT_CSR || (g->light_cta && !g->light_few) || auto_grid(g);
+}
 
 extern "C" int dj_sssp_ex(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts* opts,
                           uint64_t stream) {
@@ -596,11 +600,15 @@ static int batch_descs(const dj_graph* const* graphs, const int32_t* sources, in
                        int32_t* const* pred, int plain, int device, std::vector<SolveDesc>* h, int32_t* max_n,
                        int32_t* max_pitch);
 
-// Whether every solve's graph takes the light engine and its keys fit one CTA.
+// Whether every solve's graph takes the light engine and its keys fit one CTA, and not all are small graphs of
+// few phases (light_few).
 static bool light_batch_ok(const dj_graph* const* graphs, int32_t k, int32_t max_n) {
-  for (int32_t i = 0; i < k; ++i)
+  bool pays = false;
+  for (int32_t i = 0; i < k; ++i) {
     if (!graphs[i]->light_cta) return false;
-  return k > 0 && light_cta_fits(max_n);
+    pays = pays || !graphs[i]->light_few || graphs[i]->n >= kFewBatchMinN;
+  }
+  return pays && light_cta_fits(max_n);
 }
 
 // The one graph every solve of the batch uses, or nullptr.

@@ -38,6 +38,7 @@ struct dj_graph {
   uint64_t light_bytes = 0;
   bool light_ok = false;      // solves take the light engine unless the caller chose another
   bool light_cta = false;     // its CTA form too: hardly any source needs whole rows (slow in one CTA)
+  bool light_few = false;     // few phases (light_few): single solves behind others stay on the cluster engine
   bool light_wide = false;    // the lists are kLightWide long
   float light_deg = 0.f;      // dense: edges per row
   float light_spacing = 0.f;  // compressed rows: mean spacing of a row's lightest weights

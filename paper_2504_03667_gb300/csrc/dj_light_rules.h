@@ -53,6 +53,17 @@ inline int light_trial_verdict(uint32_t rows, uint32_t guess, uint32_t hmin_min,
   return symmetric && hmin_min > 2 * static_cast<uint64_t>(guess - 1) ? kTrialAll : kTrialAsk;
 }
 
+// Whether a graph whose lists of 64 edges are cut and that has less than kLightClusterMinN nodes is one of few phases: its largest dist
+// is at most three times its smallest weight, so the streaming engines need about three phases.  Single solves
+// that run behind others then stay on the cluster engine: captured alone, n = 550, p = 0.7, weights 1..10 takes
+// 35 us there and 50 on the light engine's CTA form, n = 1024 51 and 53; with a largest dist of 4 n = 1300,
+// p = 0.3 already takes 70 and 59.  So do batches if every graph is such and has less than kFewBatchMinN nodes
+// (16 solves, us: n = 300 39 and 47, n = 550 55 and 57, n = 700, p = 0.1 66 and 56, n = 1024 90 and 60).
+constexpr int kLightClusterMinN = 2048, kFewBatchMinN = 600;
+inline bool light_few(int32_t n, uint32_t guess, int32_t wmin) {
+  return guess != 0 && n < kLightClusterMinN && static_cast<int64_t>(guess) - 1 <= 3 * static_cast<int64_t>(wmin);
+}
+
 // Whether the device may read a caller's host array in place: 4-byte loads fault on other addresses.
 inline bool in_place(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3u) == 0; }
 inline bool edges_in_place(const void* src, const void* dst, const void* w) {

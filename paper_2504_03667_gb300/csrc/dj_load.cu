@@ -710,6 +710,7 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   // p = 0.05, weights 1..10 needs 288 rows whole with 64 edges listed, none with 128, and takes 14.6 us a
   // solve (the streaming grid engine 51) for a load of 0.54 ms instead of 0.45 (before the index: 1.64).
   bool good = false;
+  uint32_t guess = idx[kLightGuess];  // 0: lists of 64 hold every edge, or the trial missed some node
   tried = tried && g->wmin >= 1;
   bool complete = tried && ~idx[0] >= kInf;
   if (tried && !complete)
@@ -723,11 +724,13 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_error(e, "building the longer lists");
     g->light_wide = true;
-    complete = tried && ~idx[0] >= kInf;
+    complete = tried && ~idx[0] >= kInf;  // (then there was no trial on the longer ones)
+    if (idx[kLightGuess]) guess = idx[kLightGuess];
     if (tried && !complete)
       if (int rc = judge_cut(g, idx, st, &good)) return rc;
   }
   g->light_ok = complete || good;
+  g->light_few = g->light_ok && light_few(g->n, guess, g->wmin);
   g->light_cta = g->light_ok && (complete || !g->directed);
   // graphs that are not dense keep in-lists for the grid engine's dynamic IN bound
   const uint64_t nn = static_cast<uint64_t>(g->n) * static_cast<uint64_t>(g->n);
@@ -939,7 +942,7 @@ extern "C" int dj_graph_upload(dj_graph* g, const int32_t* W, int64_t ld, uint64
   g->upload_pending = 1;
   // The index follows the matrix (a captured solve may be replayed on it), but it was judged for the
   // loaded one: nothing tells here, without a wait, whether the new one suits it.
-  g->light_ok = g->light_cta = g->light_wide = false;
+  g->light_ok = g->light_cta = g->light_few = g->light_wide = false;
   launch_minima(g, nullptr, st, zero_copy);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_error(e, "row minima");

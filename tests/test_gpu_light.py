@@ -365,6 +365,26 @@ def test_one_source_says_nothing_about_the_others(dj, orc, n):
         check(dj, orc, star(3, n // 3, bridge, n), [0, n // 3 + 5, n // 3 * 3 - 1], f"n={n} star, bridge {bridge}")
 
 
+@pytest.mark.parametrize("n", [70, 300, 599, 600, 1500, 2047, 2048])
+def test_few_phases(dj, orc, n):
+    """Narrow weights: a largest dist of two or three, lists of 64 cut, alone, behind others and batched; and a
+    batch with another graph."""
+    import torch
+    for p, whi in ((min(0.95, 250 / n), 1), (min(0.95, 250 / n), 3), (min(0.95, 400 / n), 9)):
+        e = graphgen.bernoulli(n, p, 1, whi, n)
+        check(dj, orc, e, sorted({0, n // 2, n - 1}), f"n={n} p={p:.2f} w up to {whi}")
+    b = graphgen.bernoulli(900, 0.3, 1, 1000, n)
+    gs = [dj.dj_load_edges(x.n, x.src, x.dst, x.w, False) for x in (e, b)]
+    outs = [[torch.empty(x.n, dtype=torch.int32, device="cuda") for x in (e, b)] for _ in range(2)]
+    dj.dj_sssp_batch(gs, [1, 1], outs[0], outs[1])
+    dj.dj_sync()
+    for i, x in enumerate((e, b)):
+        ref = orc.dijkstra(orc.build_matrix(x.n, x.src, x.dst, x.w, False), 1)
+        assert np.array_equal(outs[0][i].cpu().numpy(), ref[0]) and np.array_equal(outs[1][i].cpu().numpy(), ref[1]), i
+    for g in gs:
+        g.free()
+
+
 @pytest.mark.parametrize("n,p", [(70, 0.95), (1024, 0.3), (2500, 0.1), (3000, 0.3)])
 def test_directed_matrices_with_cut_lists(dj, orc, n, p):
     """Alone, behind one another, captured and after an upload: the answer is the same whichever engine takes them."""

@@ -29,6 +29,7 @@ unsigned trial_source(unsigned word, unsigned n) { return dj::light_trial_source
 int verdict(unsigned rows, unsigned guess, unsigned hmin_min, int symmetric) {
   return dj::light_trial_verdict(rows, guess, hmin_min, symmetric);
 }
+int few(int n, unsigned guess, int wmin) { return dj::light_few(n, guess, wmin); }
 int needs_trial(unsigned hmin_min, unsigned wmin) { return dj::light_needs_trial(hmin_min, wmin); }
 }
 """
@@ -45,7 +46,7 @@ def rules(tmp_path_factory):
     subprocess.run([cxx, "-std=c++17", "-O1", "-fPIC", "-shared", "-I", CSRC, str(src), "-o", str(lib)], check=True)
     lib = ctypes.CDLL(str(lib))
     for f, args in ((lib.pending, 3), (lib.is_final, 2), (lib.needs_trial, 2), (lib.trial_word, 4), (lib.trial_source, 2),
-                    (lib.verdict, 4)):
+                    (lib.verdict, 4), (lib.few, 3)):
         f.argtypes = [ctypes.c_uint32] * args
     lib.upload_in_place.argtypes = [ctypes.c_size_t]
     lib.in_place.argtypes = [ctypes.c_size_t] * 3
@@ -141,3 +142,11 @@ def test_trial_verdict(rules):
     assert rules.verdict(0, 10, 18, 1) == ask and rules.verdict(0, 10, 19, 1) == every  # largest dist 9
     assert rules.verdict(0, 10, 10**6, 0) == ask  # directed: any other source may be farther from the rest
     assert rules.verdict(0, 2**31 - 1, 2**31 - 2, 1) == ask
+
+
+def test_few_phases(rules):
+    for wmin in (1, 7, 2**30):  # the largest dist is guess - 1
+        assert rules.few(2047, min(3 * wmin + 1, 2**31 - 1), wmin) == 1
+        assert rules.few(2048, 2, wmin) == 0
+    assert rules.few(100, 5, 1) == 0 and rules.few(100, 4, 1) == 1 and rules.few(100, 23, 7) == 0
+    assert rules.few(100, 0, 1) == 0  # no trial
