@@ -56,6 +56,15 @@ int get_ctx(DevCtx** out) {
     if (e != cudaSuccess) return cuda_error(e, "cudaMalloc(device words)");
     e = cudaMemset(c.words, 0, 64 * sizeof(uint32_t));
     if (e != cudaSuccess) return cuda_error(e, "cudaMemset(device words)");
+    const size_t solved = kMaxStreamSolves * kSolvedStride * sizeof(uint32_t);
+    if (cudaHostAlloc(&c.solved_h, solved, cudaHostAllocMapped) == cudaSuccess &&
+        cudaHostGetDevicePointer(&c.solved_d, c.solved_h, 0) == cudaSuccess) {
+      std::memset(c.solved_h, 0, solved);
+      c.solves.reserve(kMaxStreamSolves);
+    } else {
+      cudaGetLastError();
+      c.solved_h = nullptr;  // then by the stream's state (stream_idle)
+    }
     c.device = dev;
   }
   *out = &c;
@@ -215,7 +224,7 @@ static int plan_cluster_single(const dj_graph* g, const dj_solve_opts& o, Cluste
 }
 
 static int solve_cluster_single(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred,
-                                const dj_solve_opts& o, cudaStream_t st) {
+                                const dj_solve_opts& o, const SolveMark& mark, cudaStream_t st) {
   SolveDesc d = make_desc(g, source, dist, pred, o.mode == DJ_MODE_PLAIN ? 1 : 0);
   if (o.settle == DJ_SETTLE_OUT) d.use_in = 0;
   DevCtx* ctx = nullptr;
@@ -226,7 +235,7 @@ static int solve_cluster_single(const dj_graph* g, int32_t source, int32_t* dist
   // right after an upload the solve waits for the kernels before it before reading the graph
   const bool early = g->upload_pending == 0;
   const_cast<dj_graph*>(g)->upload_pending = 0;
-  return run_cluster_single(plan, d, ctx->words + 1, o.trace, o.trace ? o.trace_cap : 0, early, st);
+  return run_cluster_single(plan, d, ctx->words + 1, o.trace, o.trace ? o.trace_cap : 0, early, mark, st);
 }
 
 // The light engine's place: the caller left every choice of engine, bound and path to the library,
@@ -245,43 +254,116 @@ static bool light_auto(const dj_graph* g, const dj_solve_opts& o) {
 //   n = 16384, p = 0.5               35 / 255      16 / 117      31 /  41
 //   n = 32768, 8 edges per node                    20 / 142      81 /  91
 // CTA and cluster solves leave most SMs to the next solves on the stream, which then run side by side;
-// the grid form gives one solve every SM.  So a large solve takes the grid form only when nothing is
+// the grid form gives one solve every SM.  So a large solve takes the grid form only when none of them is
 // ahead of it on its stream (someone is waiting for this one), and so it does when one CTA or cluster
 // would be slow with the whole rows its graph may need.
 static constexpr int32_t kLightIdleGridMinN = 6144;
 static constexpr int32_t kLightIdleGridMinNComplete = 16384;  // compressed rows: fewer offers per phase
 static constexpr uint32_t kLightClusterMaxRow = 512;          // longer compressed rows: the grid form shares them out
 
+// Without a word for the stream (StreamSolves): whether anything at all is ahead on it.
 static bool stream_idle(cudaStream_t st) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  if (cap != cudaStreamCaptureStatusNone) return false;
   const cudaError_t e = cudaStreamQuery(st);
   if (e != cudaSuccess && e != cudaErrorNotReady) cudaGetLastError();  // the launch reports it
   return e == cudaSuccess;
 }
 
+// What a call finds on its stream, and what its kernel has to write.
+struct StreamState {
+  bool capturing = false;
+  bool ahead = true;  // one of this library's solves (those that leave a mark) is directly ahead, or still under way
+  SolveMark mark;
+};
+
+static std::mutex g_solves_mu;
+
+static StreamSolves* stream_solves(DevCtx* ctx, cudaStream_t st) {  // g_solves_mu held
+  for (auto& s : ctx->solves)
+    if (s.stream == st) return &s;
+  if (ctx->solves.size() < kMaxStreamSolves) {
+    ctx->solves.push_back(StreamSolves{});
+    ctx->solves.back().stream = st;
+    return &ctx->solves.back();
+  }
+  for (size_t i = 0; i < ctx->solves.size(); ++i) {  // a stream with nothing under way makes room
+    StreamSolves& s = ctx->solves[i];
+    if (s.issued != *const_cast<volatile uint32_t*>(ctx->solved_h + kSolvedStride * i)) continue;
+    s.stream = st;
+    s.capture = 0;
+    return &s;
+  }
+  return nullptr;
+}
+
+// The capture's number and the one node at its end on st; false: no such node.
+static bool capture_end(cudaStream_t st, unsigned long long* id, cudaGraphNode_t* node) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  const cudaGraphNode_t* nodes = nullptr;
+  const cudaGraphEdgeData* edges = nullptr;
+  size_t count = 0;
+  if (cudaStreamGetCaptureInfo(st, &status, id, nullptr, &nodes, &edges, &count) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (status != cudaStreamCaptureStatusActive || count != 1) return false;
+  *node = nodes[0];
+  return true;
+}
+
+// Only another solve of this library can run side by side with this one, so only that counts as ahead: after an
+// event record, a copy or a caller's kernel a solve is as alone as on an idle stream (n = 6001, weights 1..10:
+// 120 us on a cluster, 40 on the grid form).
+static StreamState stream_state(DevCtx* ctx, cudaStream_t st) {
+  StreamState x;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return x;
+  }
+  x.capturing = cap != cudaStreamCaptureStatusNone;
+  std::lock_guard<std::mutex> lk(g_solves_mu);
+  StreamSolves* s = ctx->solved_h ? stream_solves(ctx, st) : nullptr;
+  if (x.capturing) {
+    unsigned long long id = 0;
+    cudaGraphNode_t node = nullptr;
+    x.ahead = s && capture_end(st, &id, &node) && s->capture == id && s->last == node;
+  } else if (s) {
+    const size_t i = static_cast<size_t>(s - ctx->solves.data()) * kSolvedStride;
+    x.ahead = s->issued != *const_cast<volatile uint32_t*>(ctx->solved_h + i);
+    x.mark.done = ctx->solved_d + i;
+    x.mark.seq = s->issued + 1;
+  } else {
+    x.ahead = !stream_idle(st);
+  }
+  return x;
+}
+
+// After the solve's launch.
+static void solve_enqueued(DevCtx* ctx, cudaStream_t st, const StreamState& x) {
+  std::lock_guard<std::mutex> lk(g_solves_mu);
+  StreamSolves* s = ctx->solved_h ? stream_solves(ctx, st) : nullptr;
+  if (!s) return;
+  if (x.mark.done) s->issued = x.mark.seq;
+  if (x.capturing && !capture_end(st, &s->capture, &s->last)) s->capture = 0;
+}
+
+// lone: nothing is ahead that the solve could run side by side with.
 static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
-                       cudaStream_t st) {
+                       bool lone, const SolveMark& mark, cudaStream_t st) {
   const bool csr = g->format == DJ_FORMAT_CSR;
   const int C = g->n < 1024 ? 4 : g->n < 4096 ? 8 : 16;
   const bool cta = !csr && g->light_cta && g->n < kLightClusterMinN && light_cta_fits(g->n);
   const bool cluster = !cta && (csr ? g->light_longest <= kLightClusterMaxRow : g->light_cta) &&
                        light_cluster_fits(g->n, C, csr);
-  if (cluster) {  // whichever form this call takes: a later one may be captured
+  // whichever form this call takes: a later one may be captured
+  LightPlan plan;
+  if (cta) {
+    if (int rc = plan_light(g->n, 1, kJobsSingle, &plan)) return rc;
+  } else if (cluster) {
     if (int rc = prepare_light_cluster(csr, C)) return rc;
   }
-  // Longer lists have ten times the edges to offer, which every SM takes faster than one CTA or cluster, at
-  // any size: 6001 nodes alone 127 us on a cluster, 52 here (the streaming grid engine: 78), 1500 nodes
-  // 82 and 44 (94); behind other solves the forms that run side by side stay (15 us a solve against 50).
-  // (Graphs of few phases come here only on an idle stream.)
-  if (g->light_few || (g->light_wide && stream_idle(st))) return launch_light_grid(g, source, dist, pred, o, st);
-  if (!cta && (!cluster || o.debug_skip_cta >= 0 ||
-               (g->n >= (csr ? kLightIdleGridMinNComplete : kLightIdleGridMinN) && stream_idle(st))))
-    return launch_light_grid(g, source, dist, pred, o, st);
+  if (lone || (!cta && (!cluster || o.debug_skip_cta >= 0)))
+    return launch_light_grid(g, source, dist, pred, o, mark, st);
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   const SolveDesc d = make_desc(g, source, dist, pred, 0);
@@ -289,14 +371,12 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   const bool early = g->upload_pending == 0;
   const_cast<dj_graph*>(g)->upload_pending = 0;
   if (cluster) {
-    const int rc = run_light_cluster(g, C, d, ctx->words + 1, early, st);
+    const int rc = run_light_cluster(g, C, d, ctx->words + 1, early, mark, st);
     if (rc != DJ_ECUDA) return rc;
     clear_error();  // no such cluster here
-    return launch_light_grid(g, source, dist, pred, o, st);
+    return launch_light_grid(g, source, dist, pred, o, mark, st);
   }
-  LightPlan plan;
-  if (int rc = plan_light(g->n, 1, kJobsSingle, &plan)) return rc;
-  return run_light_single(plan, d, ctx->words + 1, early, st);
+  return run_light_single(plan, d, ctx->words + 1, early, mark, st);
 }
 
 // Whether solves of g behind others on their stream take the light engine.  A directed matrix with cut lists
@@ -306,6 +386,33 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
 // graphs of few phases (light_few).
 static bool light_behind(const dj_graph* g) {
   return g->format == DJ_FORMAT_CSR || (g->light_cta && !g->light_few) || auto_grid(g);
+}
+
+// Whether a lone solve of g takes the grid form and one behind others another: large graphs; graphs with lists of
+// kLightWide edges at any size (these have ten times the edges to offer, which every SM takes faster than one
+// CTA or cluster: 6001 nodes alone 127 us on a cluster, 52 here, the streaming grid engine 78; 1500 nodes 82, 44
+// and 94; behind others 15 us a solve against 50); and those of light_behind.
+static bool light_lone_grid(const dj_graph* g) {
+  if (g->format == DJ_FORMAT_CSR) return g->n >= kLightIdleGridMinNComplete;
+  return !light_behind(g) || (g->light_cta && (g->light_wide || g->n >= kLightIdleGridMinN));
+}
+
+// A single solve by the light engine, or on the cluster engine where that is the better one behind others.
+static int solve_small(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
+                       cudaStream_t st) {
+  if (!light_lone_grid(g)) return solve_light(g, source, dist, pred, o, false, SolveMark(), st);
+  DevCtx* ctx = nullptr;
+  if (int rc = get_ctx(&ctx)) return rc;
+  const StreamState x = stream_state(ctx, st);
+  // a captured solve of the grid form owns its workspace, which the cluster engine's sizes do without
+  const bool lone = !x.ahead && (!x.capturing || g->format == DJ_FORMAT_CSR || auto_grid(g));
+  ClusterPlan later;  // a later call behind this one, or captured, takes the cluster engine
+  int rc = light_behind(g) ? DJ_OK : plan_cluster_single(g, o, &later);
+  if (rc == DJ_OK)
+    rc = lone || light_behind(g) ? solve_light(g, source, dist, pred, o, lone, x.mark, st)
+                                 : solve_cluster_single(g, source, dist, pred, o, x.mark, st);
+  if (rc == DJ_OK) solve_enqueued(ctx, st, x);
+  return rc;
 }
 
 extern "C" int dj_sssp_ex(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts* opts,
@@ -322,19 +429,12 @@ extern "C" int dj_sssp_ex(const dj_graph* g, int32_t source, int32_t* dist, int3
   if (o.rowsplit < -1) return set_error(DJ_EINVAL, "rowsplit must be -1, 0 or a candidate count");
   if (o.rowpush < -1) return set_error(DJ_EINVAL, "rowpush must be -1, 0 or a candidate count");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (light_auto(g, o)) {
-    if (light_behind(g)) return solve_light(g, source, dist, pred, o, st);
-    if (stream_idle(st)) {
-      ClusterPlan later;  // the next call may be captured, and then takes the cluster engine
-      if (int rc = plan_cluster_single(g, o, &later)) return rc;
-      return solve_light(g, source, dist, pred, o, st);
-    }
-  }
+  if (light_auto(g, o)) return solve_small(g, source, dist, pred, o, st);
   if (g->format == DJ_FORMAT_CSR) return launch_csr(g, source, dist, pred, o, st);
   int engine = o.engine;
   if (engine == DJ_ENGINE_AUTO) engine = auto_grid(g) ? DJ_ENGINE_GRID : DJ_ENGINE_CLUSTER;
   if (engine == DJ_ENGINE_GRID) return launch_grid(g, source, dist, pred, o, st);
-  if (engine == DJ_ENGINE_CLUSTER) return solve_cluster_single(g, source, dist, pred, o, st);
+  if (engine == DJ_ENGINE_CLUSTER) return solve_cluster_single(g, source, dist, pred, o, SolveMark(), st);
   return set_error(DJ_EINVAL, "unknown engine");
 }
 

@@ -115,6 +115,24 @@ struct StreamWs {
   size_t bytes = 0;
 };
 
+// The single solves enqueued on a stream, as far as they count for the form of the next one (solve_ahead).
+// Each writes its number to the stream's word in host memory as it ends; in a capture the node that the last
+// one left at the end of the stream tells.
+struct StreamSolves {
+  cudaStream_t stream = nullptr;
+  uint32_t issued = 0;
+  unsigned long long capture = 0;
+  cudaGraphNode_t last = nullptr;
+};
+constexpr size_t kMaxStreamSolves = 64;  // streams; then the longest without a solve under way makes room
+constexpr size_t kSolvedStride = 16;     // 32-bit words: a cache line each
+
+// What a solve's kernel writes when it ends (nullptr: nothing).
+struct SolveMark {
+  uint32_t* done = nullptr;
+  uint32_t seq = 0;
+};
+
 // A kernel's launch set-up on one device, done once: its dynamic shared-memory
 // limit raised to all the device allows next to its static shared memory, the
 // non-portable cluster size allowance, and its resident CTAs per SM at the
@@ -138,6 +156,9 @@ struct DevCtx {
   uint32_t* words = nullptr;  // device: [0] error bits, [1] phases of the last single solve
   std::vector<StreamWs> ws;   // per-stream workspaces of the grid engine (see stream_workspace)
   std::vector<FnSetup> fns;   // see prepare_function
+  std::vector<StreamSolves> solves;  // see solve_ahead
+  uint32_t* solved_h = nullptr;      // their words: mapped host memory, and its device address
+  uint32_t* solved_d = nullptr;
 };
 
 // error reporting (thread-local message)
@@ -230,7 +251,7 @@ int run_cluster(const ClusterPlan& plan, const SolveDesc* descs_dev, int32_t k, 
 // that kernel ends and waits for it only before writing its outputs (and, unless `early`, before
 // reading the graph).
 int run_cluster_single(const ClusterPlan& plan, const SolveDesc& d, uint32_t* phases_out, uint64_t* trace,
-                       int32_t trace_cap, bool early, cudaStream_t st);
+                       int32_t trace_cap, bool early, const SolveMark& mark, cudaStream_t st);
 
 // The serving request ring as the persistent kernel sees it (device-usable
 // addresses of mapped pinned host memory, plus the device-side head).
@@ -281,7 +302,8 @@ int plan_light(int32_t max_n, int32_t k, int kind, LightPlan* plan);
 // as run_cluster, run_cluster_single and run_serve_kernel
 int run_light_batch(const LightPlan& plan, const SolveDesc* descs_dev, int32_t k, uint32_t* queue, bool zero_queue,
                     cudaStream_t st);
-int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, bool early, cudaStream_t st);
+int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, bool early,
+                     const SolveMark& mark, cudaStream_t st);
 // kMoreTrials trial solves of one graph side by side (LightTrialJobs): words [kLightMore..] count the rows
 // that each relaxed whole, up to the first count above kTrialRows.
 int run_light_trials(const LightPlan& plan, const SolveDesc& d, uint32_t* light, cudaStream_t st);
@@ -290,10 +312,10 @@ int run_light_serve(const LightPlan& plan, const ServeRing& r, cudaStream_t st);
 bool light_cluster_fits(int32_t n, int C, bool csr);
 int prepare_light_cluster(bool csr, int C);  // its launch attributes, before a capture may need them
 int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t* phases_out, bool early,
-                      cudaStream_t st);
+                      const SolveMark& mark, cudaStream_t st);
 // One solve over every SM (a graph with an index, or in compressed rows).
 int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
-                      cudaStream_t st);
+                      const SolveMark& mark, cudaStream_t st);
 // A trial solve, which writes nothing but the index's words.  From the source that the rows' words name
 // (kTrialFirst: it leaves kLightGuess), from the farthest node of the trials so far (kTrialFar), or from a
 // given one; those stop once more than kTrialRows rows were relaxed whole, counted in *heavy.

@@ -7,6 +7,11 @@
 
 namespace dj {
 
+// A single solve's last write (SolveMark): the host looks whether it has ended, nothing else hangs on it.
+__device__ __forceinline__ void mark_done(const SolveMark& m) {
+  if (m.done) *const_cast<volatile uint32_t*>(m.done) = m.seq;
+}
+
 // fetch() and complete() run on thread 0 of cluster rank 0 (of the CTA in the light engine) only.
 struct BatchJobs {
   const SolveDesc* descs;
@@ -50,6 +55,7 @@ struct SingleJob {
   SolveDesc d;
   uint32_t* phases_out;
   int32_t early_ok;
+  SolveMark mark;
   __device__ bool fetch(uint32_t* job, uint32_t iter) const {
     *job = 0;
     return iter == 0 && cluster_id_x() == 0;
@@ -57,6 +63,7 @@ struct SingleJob {
   __device__ SolveDesc desc(uint32_t) const { return d; }
   __device__ void complete(uint32_t, uint32_t phases) const {
     if (phases_out) *phases_out = phases;
+    mark_done(mark);
   }
   static constexpr uint32_t kGuessPart = 8;
   static constexpr bool kTrial = false;

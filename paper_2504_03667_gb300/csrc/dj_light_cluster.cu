@@ -16,6 +16,7 @@
 
 #include "dj_common.cuh"
 #include "dj_internal.h"
+#include "dj_jobs.cuh"
 #include "dj_light.cuh"
 
 namespace dj {
@@ -34,6 +35,7 @@ struct LightClusterParams {
   const uint32_t* edge;
   const int32_t* minin;
   uint32_t* phases_out;
+  SolveMark mark;
   uint32_t delta;          // compressed rows (dense: from the index)
   int32_t early;           // the graph may be read before the kernel ahead on the stream has completed
   int32_t cshift;          // log2 C
@@ -311,7 +313,10 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
     d.dist[v] = static_cast<int32_t>(dv == kNone ? kInf : dv);
     d.pred[v] = dv == kNone || v == d.source ? -1 : static_cast<int32_t>(tie[32 * lw + lane] & umask);
   }
-  if (rank == 0 && tid == 0 && p.phases_out) *p.phases_out = phase;
+  if (rank == 0 && tid == 0) {
+    if (p.phases_out) *p.phases_out = phase;
+    mark_done(p.mark);
+  }
 }
 
 // ============================================================ host
@@ -335,7 +340,7 @@ int prepare_light_cluster(bool csr, int C) {
 }
 
 int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t* phases_out, bool early,
-                      cudaStream_t st) {
+                      const SolveMark& mark, cudaStream_t st) {
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   const bool csr = g->format == DJ_FORMAT_CSR;
@@ -348,6 +353,7 @@ int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t*
   p.edge = g->edge;
   p.minin = g->minin;
   p.phases_out = phases_out;
+  p.mark = mark;
   p.delta = static_cast<uint32_t>(std::min(1.0e9f, kClDelta * g->light_spacing));
   p.early = early ? 1 : 0;
   p.cshift = 0;

@@ -370,12 +370,14 @@ int run_light_batch(const LightPlan& plan, const SolveDesc* descs_dev, int32_t k
   return launch_light(plan, args, st, false);
 }
 
-int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, bool early, cudaStream_t st) {
+int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, bool early,
+                     const SolveMark& mark, cudaStream_t st) {
   LightCtaParams p{plan.npad};
   SingleJob job;
   job.d = d;
   job.phases_out = phases_out;
   job.early_ok = early ? 1 : 0;
+  job.mark = mark;
   void* args[] = {&p, &job};
   return launch_light(plan, args, st, true);
 }

@@ -23,6 +23,7 @@
 
 #include "dj_common.cuh"
 #include "dj_internal.h"
+#include "dj_jobs.cuh"
 #include "dj_light.cuh"
 
 namespace dj {
@@ -47,6 +48,7 @@ struct LightGridParams {
   unsigned long long* gkey;   // n keys
   uint32_t* words;            // per-device words: [0] error bits, [1] phases
   uint32_t* heavy;            // trial: rows relaxed whole are counted here
+  SolveMark mark;
   uint32_t* guess;            // the first trial: the index's kLightGuess
   int64_t pitch;
   int64_t timeout_ns;
@@ -413,6 +415,7 @@ __global__ void __launch_bounds__(kLightGridThreads, 1) k_light_grid(const Light
       p.ctl[kLgAbort] = 0;
       p.ctl[kLgExit] = 0;
       for (int i = 0; i < 12; ++i) p.ctl[kLgSlots + i] = 0;
+      mark_done(p.mark);
     }
   }
 }
@@ -425,7 +428,7 @@ namespace dj {
 
 // heavy: the launch is a trial.
 static int run_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
-                          uint32_t* heavy, cudaStream_t st) {
+                          uint32_t* heavy, const SolveMark& mark, cudaStream_t st) {
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   if (!ctx->coop) return set_error(DJ_EUNSUPPORTED, "device lacks cooperative launch");
@@ -460,6 +463,7 @@ static int run_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int3
   p.gkey = reinterpret_cast<unsigned long long*>(ws + ctl_bytes);
   p.words = ctx->words;
   p.heavy = heavy;
+  p.mark = mark;
   p.guess = heavy && source == kTrialFirst ? g->light + kLightGuess : nullptr;
   p.pitch = g->pitch;
   p.timeout_ns = o.timeout_ns > 0 ? o.timeout_ns : 2000000000LL;
@@ -479,14 +483,14 @@ static int run_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int3
 }
 
 int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
-                      cudaStream_t st) {
-  return run_light_grid(g, source, dist, pred, o, nullptr, st);
+                      const SolveMark& mark, cudaStream_t st) {
+  return run_light_grid(g, source, dist, pred, o, nullptr, mark, st);
 }
 
 int launch_light_trial(const dj_graph* g, int32_t source, uint32_t* heavy, cudaStream_t st) {
   dj_solve_opts o;
   dj_solve_opts_init(&o);
-  return run_light_grid(g, source, nullptr, nullptr, o, heavy, st);
+  return run_light_grid(g, source, nullptr, nullptr, o, heavy, SolveMark(), st);
 }
 
 }  // namespace dj

@@ -1136,7 +1136,7 @@ int launch_cluster(const SolveDesc* descs_dev, int32_t k, int32_t /*max_n*/, int
 }
 
 int run_cluster_single(const ClusterPlan& plan, const SolveDesc& d, uint32_t* phases_out, uint64_t* trace,
-                       int32_t trace_cap, bool early, cudaStream_t st) {
+                       int32_t trace_cap, bool early, const SolveMark& mark, cudaStream_t st) {
   ClusterParams p = params_of(plan);
   p.trace = trace;
   p.trace_cap = trace ? trace_cap : 0;
@@ -1144,6 +1144,7 @@ int run_cluster_single(const ClusterPlan& plan, const SolveDesc& d, uint32_t* ph
   job.d = d;
   job.phases_out = phases_out;
   job.early_ok = early ? 1 : 0;
+  job.mark = mark;
   void* args[] = {&p, &job};
   return launch_plan(plan, args, st, true);
 }

@@ -423,3 +423,60 @@ def test_directed_matrices_with_cut_lists(dj, orc, n, p):
                 assert np.array_equal(P[i].cpu().numpy(), refs[i][1]), (how, i)
         del cg
         g.free()
+
+
+@pytest.mark.parametrize("kind", ["large", "longer lists", "few phases", "directed"])
+def test_solves_on_many_streams(dj, orc, kind):
+    """More streams than the library keeps a word for, several solves on each, some behind an event, a copy or
+    another kernel, some captured (alone and behind one another): every form gives the same answer."""
+    import torch
+    n = 6200 if kind == "large" else 1500
+    if kind == "directed":
+        b = graphgen.bernoulli(n, 0.2, 1, 1000, 1)
+        e = graphgen.EdgeList(n, np.concatenate([b.src, b.dst]), np.concatenate([b.dst, b.src]),
+                              np.concatenate([b.w, b.w[::-1]]), True)
+    else:
+        p, whi = {"large": (0.05, 1000), "longer lists": (0.2, 10), "few phases": (0.5, 9)}[kind]
+        e = graphgen.bernoulli(n, p, 1, whi, 1)
+    W = orc.build_matrix(n, e.src, e.dst, e.w, e.directed)
+    srcs = [0, 7, n - 1]
+    refs = [orc.dijkstra(W, s) for s in srcs]
+    g = dj.dj_load_edges(n, e.src, e.dst, e.w, e.directed)
+    streams = [torch.cuda.Stream() for _ in range(70)]
+    D = torch.empty((len(streams), 3, n), dtype=torch.int32, device="cuda")
+    P = torch.empty_like(D)
+
+    def run(j):
+        for i, s in enumerate(srcs):
+            with torch.cuda.stream(streams[j]):
+                if (i + j) % 4 == 1:
+                    torch.cuda.Event().record()
+                elif (i + j) % 4 == 2:
+                    D[j, i].fill_(-9)
+            dj.dj_sssp(g, s, D[j, i], P[j, i], streams[j])
+
+    graphs = []
+    run(0)
+    torch.cuda.synchronize()
+    for j in (0, 1):  # one solve a graph, and three
+        cg = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(cg, stream=streams[j]):
+            for i in range(1 if j == 0 else 3):
+                dj.dj_sssp(g, srcs[i], D[j, i], P[j, i], streams[j])
+        graphs.append(cg)
+    for turn in range(3):
+        D.fill_(-5)
+        P.fill_(-5)
+        torch.cuda.synchronize()
+        for j in range(len(streams)):
+            if turn == 2 and j < 2:
+                graphs[j].replay()
+            else:
+                run(j)
+        torch.cuda.synchronize()
+        d, p = D.cpu().numpy(), P.cpu().numpy()
+        for j in range(len(streams)):
+            for i in range(1 if turn == 2 and j == 0 else 3):
+                assert np.array_equal(d[j, i], refs[i][0]) and np.array_equal(p[j, i], refs[i][1]), (turn, j, i)
+    del graphs
+    g.free()
