@@ -258,7 +258,10 @@ static bool light_auto(const dj_graph* g, const dj_solve_opts& o) {
 // ahead of it on its stream (someone is waiting for this one), and so it does when one CTA or cluster
 // would be slow with the whole rows its graph may need.
 static constexpr int32_t kLightIdleGridMinN = 6144;
-static constexpr int32_t kLightIdleGridMinNComplete = 16384;  // compressed rows: fewer offers per phase
+// Compressed rows have fewer offers per phase: by nodes, or by edges (a lone solve of n = 3000, us on a cluster
+// and on the grid form: 64 edges per node 176 and 86, 300 edges 558 and 108; n = 8000, 16 edges 111 and about 90).
+static constexpr int32_t kLightIdleGridMinNComplete = 16384;
+static constexpr uint64_t kLightIdleGridMinEdges = 131072;
 static constexpr uint32_t kLightClusterMaxRow = 512;          // longer compressed rows: the grid form shares them out
 
 // Without a word for the stream (StreamSolves): whether anything at all is ahead on it.
@@ -393,8 +396,18 @@ static bool light_behind(const dj_graph* g) {
 // CTA or cluster: 6001 nodes alone 127 us on a cluster, 52 here, the streaming grid engine 78; 1500 nodes 82, 44
 // and 94; behind others 15 us a solve against 50); and those of light_behind.
 static bool light_lone_grid(const dj_graph* g) {
-  if (g->format == DJ_FORMAT_CSR) return g->n >= kLightIdleGridMinNComplete;
+  if (g->format == DJ_FORMAT_CSR) return g->n >= kLightIdleGridMinNComplete || g->entries >= kLightIdleGridMinEdges;
   return !light_behind(g) || (g->light_cta && (g->light_wide || g->n >= kLightIdleGridMinN));
+}
+
+// Whether so does the first of a captured chain: only where the form for solves behind others is slow alone, since
+// it holds up the chain (16 solves of n = 8000, 32 edges per node: 24 us each, 28 so), and not on the cluster
+// engine's sizes (its captured solves do without a workspace).  Captured alone n = 6001, weights 1..10 takes
+// 120 us on a cluster and 44 on the grid form; compressed rows, n = 900: 150 edges per node 184 and 60 (the engine
+// for chosen bounds 286), 250 edges 309 and 68 (262).
+static bool light_captured_grid(const dj_graph* g) {
+  if (g->format == DJ_FORMAT_CSR) return g->entries >= 192 * static_cast<uint64_t>(g->n);
+  return g->light_wide && auto_grid(g);
 }
 
 // A single solve by the light engine, or on the cluster engine where that is the better one behind others.
@@ -404,8 +417,7 @@ static int solve_small(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   const StreamState x = stream_state(ctx, st);
-  // a captured solve of the grid form owns its workspace, which the cluster engine's sizes do without
-  const bool lone = !x.ahead && (!x.capturing || g->format == DJ_FORMAT_CSR || auto_grid(g));
+  const bool lone = !x.ahead && (!x.capturing || light_captured_grid(g));
   ClusterPlan later;  // a later call behind this one, or captured, takes the cluster engine
   int rc = light_behind(g) ? DJ_OK : plan_cluster_single(g, o, &later);
   if (rc == DJ_OK)

@@ -96,3 +96,46 @@ def test_dense_only_calls_reject_compressed_rows(dj):
             call()
         assert ei.value.status == dj.DJ_EUNSUPPORTED
     G.free()
+
+
+@pytest.mark.parametrize("n,deg", [(400, 330), (900, 140), (900, 150), (700, 260), (3000, 60)])
+def test_long_rows_alone_behind_and_captured(dj, orc, n, deg):
+    """Edges around the counts from which a lone or captured solve takes another form than one behind others."""
+    import torch
+    b = [graphgen.bernoulli(n, deg / n, 1, 1000, n + i) for i in range(2)]
+    src, dst = np.concatenate([b[0].src, b[1].dst]), np.concatenate([b[0].dst, b[1].src])
+    w = np.concatenate([b[0].w, b[1].w])
+    G = dj.dj_load_edges_csr(n, src, dst, w, True)
+    W = orc.build_matrix(n, src, dst, w, True)
+    srcs = [0, n // 2, n - 1]
+    refs = [orc.dijkstra(W, s) for s in srcs]
+    st = torch.cuda.Stream()
+    D = torch.empty((3, n), dtype=torch.int32, device="cuda")
+    P = torch.empty_like(D)
+
+    def run(alone):
+        for i, s in enumerate(srcs):
+            dj.dj_sssp(G, s, D[i], P[i], st)
+            if alone:
+                dj.dj_sync(st)
+
+    run(True)
+    graphs = []
+    for k in (1, 3):
+        cg = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(cg, stream=st):
+            for i in range(k):
+                dj.dj_sssp(G, srcs[i], D[i], P[i], st)
+        graphs.append(cg)
+    for what, again, k in (("alone", lambda: run(True), 3), ("behind", lambda: run(False), 3),
+                           ("captured alone", graphs[0].replay, 1), ("captured", graphs[1].replay, 3)):
+        torch.cuda.synchronize()
+        D.fill_(-5)
+        P.fill_(-5)
+        torch.cuda.synchronize()
+        again()
+        torch.cuda.synchronize()
+        for i in range(k):
+            same((D[i].cpu().numpy(), P[i].cpu().numpy()), refs[i], f"n={n} deg={deg} {what} {i}")
+    del graphs
+    G.free()
