@@ -139,3 +139,18 @@ def test_long_rows_alone_behind_and_captured(dj, orc, n, deg):
             same((D[i].cpu().numpy(), P[i].cpu().numpy()), refs[i], f"n={n} deg={deg} {what} {i}")
     del graphs
     G.free()
+
+
+def test_long_rows_of_repeats(dj, orc):
+    """Rows longer than a list, with most targets repeated in any order of weights."""
+    for n, m, directed in ((40, 30000, True), (700, 300000, False)):
+        e = graphgen.random_edges(n, m, 1, 1000, seed=n, directed=directed)
+        G = dj.dj_load_edges_csr(n, e.src, e.dst, e.w, directed)
+        W = orc.build_matrix(n, e.src, e.dst, e.w, directed)
+        info = dj.dj_graph_get_info(G)
+        off = W[~np.eye(n, dtype=bool)]
+        assert info["entries"] == np.count_nonzero(off < 2**31 - 1) and info["min_weight"] == off.min()
+        for s in (0, n - 1):
+            same(solve(dj, G, s), orc.dijkstra(W, s), f"n={n} s={s}")
+            same(solve(dj, G, s, 2), orc.dijkstra(W, s), f"n={n} s={s} plain")
+        G.free()
