@@ -225,10 +225,10 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
           __syncthreads();
           hb = s_bound;
           if (hb == kNone) break;
-          // those up to it are final: relaxed whole, as many as the list holds now
+          // the final ones (light_final): relaxed whole, as many as the list holds now
           for (int wi = warp; wi < nwords; wi += NW) {
             const uint32_t dv = s.dist[32 * wi + lane];
-            const bool go = light_final(dv, hb) && pending(wi, dv) != kNone;
+            const bool go = pending(wi, dv) != kNone && light_final(dv, __ldg(hmin + 32 * wi + lane), hb);
             const uint32_t todo = __ballot_sync(0xffffffffu, go);
             if (todo == 0) continue;
             uint32_t pos = 0;

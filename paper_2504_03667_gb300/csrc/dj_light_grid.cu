@@ -12,9 +12,9 @@
 // relaxed once more.  Then the index's test (hmin) either proves the answer complete or names the rows to
 // relax whole from the matrix:
 //   pending = { u : dist[u] + hmin[u] <= D, not yet relaxed whole }, and
-//   those with dist[u] <= min over pending of (dist + hmin) are final -- a shorter path would use an
-//   unlisted edge of a pending row -- so each row is read from the matrix at most once, and every round
-//   takes at least the row that gives the minimum.
+//   those with dist[u] < min over pending of (dist + hmin) are final -- a shorter path would use an
+//   unlisted edge of a pending row -- so each row is read from the matrix at most once (light_final also
+//   sees to it that every round takes the row that gives the minimum).
 //
 // What bounds it: latency.  A phase is one grid barrier (which also carries m and D) and a chain of
 // three L2 round trips (own keys, edges, targets' keys) around a few hundred KB of list reads.
@@ -335,7 +335,7 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
     D = Dx;
     if (hb == kNone) break;
     for (int j = tid; j < sw; j += T0) {
-      if ((flags[j] & 2) || rdist[j] >= kInf || !light_final(rdist[j], hb) || light_pending(rdist[j], aux[j], Dx) == kNone)
+      if ((flags[j] & 2) || rdist[j] >= kInf || !light_final(rdist[j], aux[j], hb) || light_pending(rdist[j], aux[j], Dx) == kNone)
         continue;
       list[atomicAdd(&sh.cnt, 1u)] = make_uint2(static_cast<uint32_t>(j), rdist[j]);
       flags[j] |= 2;

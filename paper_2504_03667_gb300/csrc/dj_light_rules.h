@@ -25,9 +25,11 @@ DJ_RULE uint32_t light_pending(uint32_t dist, uint32_t hmin, uint32_t D) {
 
 // Whether a pending row is relaxed whole now, hb being the least of what the pending rows offer: a path
 // shorter than dist would have to use an unlisted edge of a pending row, which offers no less than hb.
-// So dist <= hb is final, and the row that gives hb is always among those taken, even with unlisted edges
-// of weight 0 (dist < hb took none then, and the solve never ended).
-DJ_RULE bool light_final(uint32_t dist, uint32_t hb) { return dist <= hb; }
+// So dist <= hb is final.  The row that gives hb is always among those taken: it has dist < hb, or dist == hb
+// and an unlisted edge of weight 0 (without the second clause no row was taken then, and the solve never ended).
+// Other rows of dist == hb wait: most need not be relaxed once those below are (n = 8192, p = 0.5, weights
+// 1..10: twice as many, and the trial at load 0.2 ms longer).
+DJ_RULE bool light_final(uint32_t dist, uint32_t hmin, uint32_t hb) { return dist < hb || (dist == hb && hmin == 0); }
 
 // Whether a graph's trial solve is run: some list is cut, and no weight is 0 (its solves take the other
 // engines then, and its lists may hold nothing but a few of a row's edges of weight 0).
