@@ -418,11 +418,13 @@ static int solve_small(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   if (int rc = get_ctx(&ctx)) return rc;
   const StreamState x = stream_state(ctx, st);
   const bool lone = !x.ahead && (!x.capturing || light_captured_grid(g));
-  ClusterPlan later;  // a later call behind this one, or captured, takes the cluster engine
-  int rc = light_behind(g) ? DJ_OK : plan_cluster_single(g, o, &later);
-  if (rc == DJ_OK)
-    rc = lone || light_behind(g) ? solve_light(g, source, dist, pred, o, lone, x.mark, st)
-                                 : solve_cluster_single(g, source, dist, pred, o, x.mark, st);
+  const bool light = lone || light_behind(g);
+  if (light && !light_behind(g)) {
+    ClusterPlan later;  // a call behind this one, or captured, takes the cluster engine
+    if (int rc = plan_cluster_single(g, o, &later)) return rc;
+  }
+  const int rc = light ? solve_light(g, source, dist, pred, o, lone, x.mark, st)
+                       : solve_cluster_single(g, source, dist, pred, o, x.mark, st);
   if (rc == DJ_OK) solve_enqueued(ctx, st, x);
   return rc;
 }
