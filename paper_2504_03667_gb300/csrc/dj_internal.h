@@ -41,6 +41,7 @@ struct dj_graph {
   bool light_few = false;     // few phases (light_few): single solves behind others stay on the cluster engine
   bool light_wide = false;    // the lists are kLightWide long
   float light_deg = 0.f;      // dense: edges per row
+  float light_first = 0.f;    // dense: first threshold of an upload's selection (LightOut)
   float light_spacing = 0.f;  // compressed rows: mean spacing of a row's lightest weights
   uint32_t light_longest = 0; // compressed rows: edges of the longest row
   int32_t light_gshift = 5;   // compressed rows: log2 of the lanes that share a row
@@ -72,9 +73,14 @@ constexpr int kLightStats = 64;  // leading words: [0] ~(smallest hmin), [1] row
                                  // (light_trial_word), [8..11] ~(finite min), finite max, finite entries
                                  // (at load), [12..14] the edge list's check (k_scatter),
                                  // [15] kLightGuess, [16..17] the trials' farthest node (dist, node),
-                                 // [24..] rows relaxed whole by each further trial
+                                 // [18..22] of the rows with cut lists (at load): sum of the edges up to their
+                                 // thresholds, of these, rows; [23] rows that some source may need whole
+                                 // (light_risky); [24..] rows relaxed whole by each further trial
+constexpr int kLightHost = 24;   // the words that the host reads
 constexpr int kLightGuess = 15;  // 1 + the trial solve's largest dist (0: unknown)
 constexpr int kLightFar = 16;
+constexpr int kLightSeen = 18;
+constexpr int kLightRisky = 23;
 constexpr int kLightMore = 24;
 constexpr int kMoreTrials = 16;  // from the farthest node and fifteen places (without the CTA form: fewer)
 inline

@@ -310,6 +310,10 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
       }
       if (!light_barrier(p, sh, nbar++, lmin, dmax, &m, &D)) return;
       ++phases;
+      if (p.trial && phases > kTrialPhases) {
+        if (b == 0 && tid == 0) atomicAdd(p.heavy, kTrialManyRows);
+        break;
+      }
       continue;
     }
     // nothing is dirty anywhere; with complete lists (no bound was set) that is all
@@ -342,7 +346,12 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
     }
     __syncthreads();
     const int cnt = static_cast<int>(sh.cnt);
-    if (p.heavy && tid == 0 && cnt) atomicAdd(p.heavy, static_cast<uint32_t>(cnt));
+    if (p.trial) {  // enough is known once these are too many; every CTA reads the same count between two barriers
+      if (tid == 0 && cnt) atomicAdd(p.heavy, static_cast<uint32_t>(cnt));
+      uint32_t unused;
+      if (!light_barrier(p, sh, nbar++, kNone, 0u, &m, &unused)) return;
+      if (__ldcg(p.heavy) > (p.guess ? kTrialManyRows : kTrialRows)) break;
+    }
     const int nv = static_cast<int>(p.pitch / 4);
     for (int i = 0; i < cnt; ++i) {
       const uint2 x = list[i];
@@ -370,8 +379,6 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
     // every row that was dirty has been relaxed, so the slice's dists (and D) only change through these rows
     if (!light_barrier(p, sh, nbar++, lmin, Dx, &m, &D)) return;
     ++phases;
-    // a further trial has its answer (every CTA reads the same count: the next one is added after a barrier)
-    if (p.trial && !p.guess && __ldcg(p.heavy) > kTrialRows) return;
   }
   if (p.trial) {
     uint64_t far = 0;
@@ -382,7 +389,13 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
     if ((tid & 31) == 0)
       atomicMax(reinterpret_cast<unsigned long long*>(const_cast<uint32_t*>(p.light) + kLightFar),
                 (static_cast<unsigned long long>(hi) << 32) | lo);
-    if (b == 0 && tid == 0 && p.guess && D < kInf) p.guess[0] = D + 1;
+    if (p.guess && D < kInf) {
+      if (b == 0 && tid == 0) p.guess[0] = D + 1;
+      uint32_t risky = 0;
+      for (int j = tid; j < sw; j += T0) risky += light_risky(rdist[j], aux[j], D) ? 1u : 0u;
+      risky = warp_sum_u32(risky);
+      if ((tid & 31) == 0 && risky) atomicAdd(const_cast<uint32_t*>(p.light) + kLightRisky, risky);
+    }
     return;
   }
   for (int j = tid; j < sw; j += T0) {

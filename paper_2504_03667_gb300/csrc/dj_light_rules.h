@@ -44,15 +44,24 @@ DJ_RULE uint32_t light_trial_word(uint32_t u, uint32_t listed, bool has_edges, u
 }
 DJ_RULE uint32_t light_trial_source(uint32_t word, uint32_t n) { return ((word & 0xFFFFFFu) + n / 2 + 1) % n; }
 
-// What the first trial says about a graph with cut lists.  kTrialNo: no.  kTrialAll: no source needs a whole
-// row -- on a symmetric matrix no largest dist is more than twice the trial's, and every unlisted edge is
-// heavier.  kTrialAsk: other sources have to be tried (a structured graph's, or one of few distinct weights,
-// may need many rows where this one needed none).
+// Whether a row may have to be relaxed whole for some source s of a symmetric matrix, by the trial from t with the
+// largest dist D: s's largest dist is at most D + d(t, s), and the row is pending only if d(s, u) + hmin does not
+// exceed that, where d(s, u) >= |d(t, s) - d(t, u)|; so only if hmin <= D + d(t, u).
+DJ_RULE bool light_risky(uint32_t dist, uint32_t hmin, uint32_t D) {
+  return dist < kRuleInf && hmin < kRuleInf && hmin <= D + dist;
+}
+
+// What the first trial says about a graph with cut lists.  kTrialNo: no.  kTrialAll: next to no row is ever
+// relaxed whole, whatever the source (on a directed matrix the bound is none, but a good sign, and only the grid
+// form is at stake).  kTrialAsk: other sources have to be tried (a structured graph's, or one of few distinct
+// weights, may need many rows where this one needed none).
 enum { kTrialNo, kTrialAll, kTrialAsk };
-constexpr uint32_t kTrialRows = 4;  // whole rows a trial may need
-inline int light_trial_verdict(uint32_t rows, uint32_t guess, uint32_t hmin_min, bool symmetric) {
+constexpr uint32_t kTrialRows = 4;         // whole rows a trial may need
+constexpr uint32_t kTrialManyRows = 1024;  // the first trial stops beyond: its D, on which the longer lists hang, is settled
+constexpr uint32_t kTrialPhases = 64;      // and here: dists reach far beyond the lists (a phase is an eighth of them)
+inline int light_trial_verdict(uint32_t rows, uint32_t guess, uint32_t risky) {
   if (guess == 0 || rows > kTrialRows) return kTrialNo;  // guess 0: not every node that has an in-edge was reached
-  return symmetric && hmin_min > 2 * static_cast<uint64_t>(guess - 1) ? kTrialAll : kTrialAsk;
+  return risky <= kTrialRows ? kTrialAll : kTrialAsk;
 }
 
 // Whether a graph whose lists of 64 edges are cut and that has less than kLightClusterMinN nodes is one of few phases: its largest dist

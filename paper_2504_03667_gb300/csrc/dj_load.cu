@@ -622,7 +622,7 @@ static void launch_minima(dj_graph* g, uint32_t* stats, cudaStream_t st, bool ha
 static bool launch_trial(dj_graph* g, uint32_t* idx, cudaStream_t st) {
   const bool tried = launch_light_trial(g, kTrialFirst, g->light + 1, st) == DJ_OK;
   clear_error();  // it cannot run here: the other engines
-  cudaMemcpyAsync(idx, g->light, 16 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
+  cudaMemcpyAsync(idx, g->light, kLightHost * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
   return tried;
 }
 
@@ -630,13 +630,15 @@ static bool launch_trial(dj_graph* g, uint32_t* idx, cudaStream_t st) {
 // that leaves it open, by further ones: side by side, a CTA each, where the state fits one (n = 300, 1500
 // and 8192: about 35, 70 and 180 us), else one after another over every SM.
 static int judge_cut(dj_graph* g, const uint32_t* idx, cudaStream_t st, bool* good) {
-  const int verdict = light_trial_verdict(idx[1], idx[kLightGuess], ~idx[0], !g->directed);
+  const int verdict = light_trial_verdict(idx[1], idx[kLightGuess], idx[kLightRisky]);
   *good = verdict == kTrialAll;
   if (verdict != kTrialAsk) return DJ_OK;
   uint32_t* more = g->light + kLightMore;
   cudaMemsetAsync(more, 0, kMoreTrials * sizeof(uint32_t), st);
   bool tried = true;
-  if (light_cta_fits(g->n)) {
+  if (g->directed) {  // for the grid form: one more
+    tried = launch_light_trial(g, kTrialFar, more, st) == DJ_OK;
+  } else if (light_cta_fits(g->n)) {
     LightPlan plan;
     tried = plan_light(g->n, kMoreTrials, kJobsTrial, &plan) == DJ_OK &&
             run_light_trials(plan, make_desc(g, 0, nullptr, nullptr, 0), g->light, st) == DJ_OK;
@@ -673,7 +675,7 @@ static bool wide_suffices(const dj_graph* g, const uint32_t* idx) {
 // the wait, the only one unless longer lists are worth a try.
 static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   uint32_t* stats = g->light ? g->light + 8 : nullptr;
-  uint32_t idx[16] = {0};
+  uint32_t idx[kLightHost] = {0};
   cudaError_t e = cudaSuccess;
   if (!g->light) {
     e = cudaMallocAsync(&stats, 4 * sizeof(uint32_t), st);
@@ -717,7 +719,7 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
     if (int rc = judge_cut(g, idx, st, &good)) return rc;
   if (tried && !complete && !good && wide_suffices(g, idx)) {
     cudaMemsetAsync(g->light, 0, 8 * sizeof(uint32_t), st);
-    cudaMemsetAsync(g->light + kLightGuess, 0, 3 * sizeof(uint32_t), st);  // and kLightFar
+    cudaMemsetAsync(g->light + kLightGuess, 0, 9 * sizeof(uint32_t), st);  // to kLightRisky
     k_light_rows<kLightWide><<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(g->W, g->pitch, light_out(g),
                                                                                         false);
     tried = launch_trial(g, idx, st);

@@ -26,9 +26,8 @@ unsigned trial_word(unsigned u, unsigned listed, int has_edges, unsigned n) {
   return dj::light_trial_word(u, listed, has_edges, n);
 }
 unsigned trial_source(unsigned word, unsigned n) { return dj::light_trial_source(word, n); }
-int verdict(unsigned rows, unsigned guess, unsigned hmin_min, int symmetric) {
-  return dj::light_trial_verdict(rows, guess, hmin_min, symmetric);
-}
+int verdict(unsigned rows, unsigned guess, unsigned risky) { return dj::light_trial_verdict(rows, guess, risky); }
+int risky(unsigned dist, unsigned hmin, unsigned D) { return dj::light_risky(dist, hmin, D); }
 int few(int n, unsigned guess, int wmin) { return dj::light_few(n, guess, wmin); }
 int needs_trial(unsigned hmin_min, unsigned wmin) { return dj::light_needs_trial(hmin_min, wmin); }
 }
@@ -46,7 +45,7 @@ def rules(tmp_path_factory):
     subprocess.run([cxx, "-std=c++17", "-O1", "-fPIC", "-shared", "-I", CSRC, str(src), "-o", str(lib)], check=True)
     lib = ctypes.CDLL(str(lib))
     for f, args in ((lib.pending, 3), (lib.is_final, 3), (lib.needs_trial, 2), (lib.trial_word, 4), (lib.trial_source, 2),
-                    (lib.verdict, 4), (lib.few, 3)):
+                    (lib.verdict, 3), (lib.risky, 3), (lib.few, 3)):
         f.argtypes = [ctypes.c_uint32] * args
     lib.upload_in_place.argtypes = [ctypes.c_size_t]
     lib.in_place.argtypes = [ctypes.c_size_t] * 3
@@ -137,11 +136,39 @@ def test_trial_source_has_edges(rules, n):
 
 def test_trial_verdict(rules):
     no, every, ask = 0, 1, 2
-    assert rules.verdict(0, 0, 10**6, 1) == no  # did not reach every node that something leads to
-    assert rules.verdict(5, 10, 10**6, 1) == no and rules.verdict(4, 10, 10**6, 1) == every
-    assert rules.verdict(0, 10, 18, 1) == ask and rules.verdict(0, 10, 19, 1) == every  # largest dist 9
-    assert rules.verdict(0, 10, 10**6, 0) == ask  # directed: any other source may be farther from the rest
-    assert rules.verdict(0, 2**31 - 1, 2**31 - 2, 1) == ask
+    assert rules.verdict(0, 0, 0) == no  # did not reach every node that something leads to
+    assert rules.verdict(5, 10, 0) == no and rules.verdict(4, 10, 4) == every
+    assert rules.verdict(0, 10, 5) == ask
+    assert not rules.risky(NONE, 1, 5) and not rules.risky(INF, 1, 5) and not rules.risky(3, INF, 5)
+    assert rules.risky(3, 8, 5) and not rules.risky(3, 9, 5)
+
+
+@pytest.mark.parametrize("cap", [2, 5, 12])
+def test_rows_not_at_risk_are_never_pending(orc, rules, cap):
+    """Symmetric matrices, random and in parts on a chain or a star: whatever the source, a row pending at the
+    end of its solve is one that the trial from any other source counts."""
+    rng = np.random.default_rng(cap)
+    for trial in range(25):
+        n = int(rng.integers(6, 40))
+        parts = int(rng.integers(1, 4))
+        part = np.arange(n) % parts
+        far = int(rng.choice([1, 20, 60]))
+        k = np.triu(rng.random((n, n)) < rng.choice([0.3, 0.9]), 1)
+        w = rng.integers(1, int(rng.choice([2, 5, 60])) + 1, (n, n)) + far * np.abs(part[:, None] - part[None, :])
+        k &= (np.abs(part[:, None] - part[None, :]) <= 1) | (rng.random((n, n)) < 0.1)
+        src, dst = (x.astype(np.int32) for x in np.nonzero(k))
+        W = orc.build_matrix(n, src, dst, w[src, dst].astype(np.int32), False)
+        _, hmin = build_index(W, cap, True)
+        dist = [orc.dijkstra(W, s)[0].astype(np.int64) for s in range(n)]
+        reached = [d < INF for d in dist]
+        if any(not r.all() for r in reached):
+            continue
+        pending = [{u for u in range(n) if rules.pending(int(d[u]), hmin[u], int(d.max())) != NONE} for d in dist]
+        for t in range(n):
+            D = int(dist[t].max())
+            risk = {u for u in range(n) if rules.risky(int(dist[t][u]), hmin[u], D)}
+            for s in range(n):
+                assert pending[s] <= risk, (trial, s, t)
 
 
 def test_few_phases(rules):
