@@ -66,13 +66,15 @@ __device__ __forceinline__ uint32_t light_guess(const uint32_t* light, uint32_t 
 }
 
 // Per-warp selection of a row's lightest edges.  scan(f, pass) must call f(c0, x) for every group of
-// four columns c0 .. c0 + 3 of the row, one group per lane, warp-uniformly often (a lane without a
-// group, and columns beyond n, pass INF).  `thr` is the warp's weight threshold, carried from row to
+// four columns c0 .. c0 + 3 of the row (or f(c0, x, step): c0 .. c0 + 3 * step), one group per lane,
+// warp-uniformly often (a lane without a group, and columns beyond n, pass INF).  `thr` is the warp's weight threshold, carried from row to
 // row: rows of one graph look alike, so one scan is the rule.
 //   A scan puts the edges of weight <= thr into buf (kLightBuf words of shared memory) and takes
 //   their count and the smallest weight above thr.  Too few (below Cap, and more exist) or too
 //   many (above kLightBuf): thr moves and the row (in L2 by now) is scanned again; thr is bracketed
-//   by [lo, hi], which shrinks with every scan.
+//   by [lo, hi], which shrinks with every scan.  After too many, buf holds a sample of them, and thr
+//   goes where the sample says that about Cap + 96 edges lie (light_sample): one scan more instead of up to
+//   ten by halving where weights are spread unevenly.
 // Then the Cap smallest packed words (weight, column) go out in ascending order, from the kLightCap-th on
 // at edge2: an entry's place is the number of smaller ones.
 constexpr int kLightBuf = 384;
@@ -83,7 +85,24 @@ struct LightRow {
   uint32_t cnt;    // listed edges
   uint32_t hmin;   // smallest weight not listed (INF: every edge is listed)
   uint32_t last;   // largest weight listed (0: none)
+  uint32_t seen;   // edges of weight <= thr
 };
+
+// The largest t in [lo, hi] that at most k of the warp's weights x do not exceed (lo if there is none).
+template <int N>
+__device__ __forceinline__ uint32_t light_sample(const uint32_t (&x)[N], uint32_t k, uint32_t lo, uint32_t hi) {
+  while (lo < hi) {
+    const uint32_t mid = hi - (hi - lo) / 2;
+    uint32_t c = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) c += x[i] <= mid ? 1u : 0u;
+    if (warp_sum_u32(c) <= k)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  return lo;
+}
 
 template <int Cap, class Scan>
 __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, uint32_t bits_u, uint32_t* buf,
@@ -92,20 +111,20 @@ __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, u
   const uint32_t lt = (1u << lane) - 1u;
   const uint32_t wcap = min(weight_field(bits_u), kInf - 1u);  // weights beyond it are never listed
   uint32_t lo = 0, hi = wcap;
-  uint32_t cnt = 0, rest = kInf;
+  uint32_t cnt = 0, rest = kInf, few = 1;  // few: the edges of weight < lo, as scanned
   thr = min(thr, wcap);
   for (int pass = 0;; ++pass) {
     cnt = 0;
     rest = kInf;
     const uint32_t t = thr;
     scan(
-        [&](uint32_t c0, int4 x) {
+        [&](uint32_t c0, int4 x, uint32_t step = 1) {
           uint32_t w[4] = {static_cast<uint32_t>(x.x), static_cast<uint32_t>(x.y), static_cast<uint32_t>(x.z),
                            static_cast<uint32_t>(x.w)};
           bool h[4];
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            if (c0 + q == u) w[q] = kInf;  // the diagonal is no edge
+            if (c0 + step * q == u) w[q] = kInf;  // the diagonal is no edge
             h[q] = w[q] <= t;
             rest = min(rest, h[q] ? kInf : w[q]);
           }
@@ -114,7 +133,7 @@ __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, u
             for (int q = 0; q < 4; ++q) {
               const uint32_t bal = __ballot_sync(0xffffffffu, h[q]);
               const uint32_t at = cnt + __popc(bal & lt);
-              if (h[q] && at < static_cast<uint32_t>(kLightBuf)) buf[at] = (w[q] << bits_u) | (c0 + q);
+              if (h[q] && at < static_cast<uint32_t>(kLightBuf)) buf[at] = (w[q] << bits_u) | (c0 + step * q);
               cnt += __popc(bal);
             }
           }
@@ -128,11 +147,20 @@ __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, u
         break;
       }
       hi = t - 1;
-      thr = hi > lo ? lo + (hi - lo) / 2 : hi;
+      if (hi < lo && few == 0) {  // weights below t: none, of weight t: too many
+        rest = t;
+        cnt = 0;
+        break;
+      }
+      __syncwarp();
+      uint32_t x[kLightBuf / 32];
+#pragma unroll
+      for (int i = 0; i < kLightBuf / 32; ++i) x[i] = buf[32 * i + lane] >> bits_u;
+      thr = hi > lo ? light_sample(x, max(1u, kLightBuf * (Cap + 96u) / cnt), lo, hi) : hi;
     } else if (cnt < static_cast<uint32_t>(Cap) && rest < kInf && t < hi) {  // too few, and more exist
       lo = t + 1;
-      // the next weight at least; fast growth while there is no upper bracket
-      thr = min(hi, max(hi == wcap ? 2 * t + 1 : lo + (hi - lo) / 2, rest));
+      few = cnt;
+      thr = min(hi, max(min(2 * t + 1, lo + (hi - lo) / 2), rest));  // the next weight at least
     } else {
       break;
     }
@@ -144,20 +172,35 @@ __device__ __forceinline__ LightRow light_select(const Scan& scan, uint32_t u, u
   for (uint32_t i = lane; i < cnt; i += 32) first = min(first, buf[i]);
   first = warp_min_u32(first);
   r.first = cnt ? first >> bits_u : rest;
+  r.seen = cnt;
+  const uint32_t r_first = r.first;
   uint32_t beyond = kNoEdge, ties = 0, last = 0;
-  for (uint32_t i = lane; i < cnt; i += 32) {
-    const uint32_t e = buf[i];
-    uint32_t rank = 0;
-    for (uint32_t j = 0; j < cnt; ++j) rank += buf[j] < e ? 1u : 0u;
-    if (rank < static_cast<uint32_t>(Cap)) {
-      if (Cap == kLightCap || rank < static_cast<uint32_t>(kLightCap))
-        edge[rank] = e;
-      else
-        edge2[rank - kLightCap] = e;
-      ties += (e >> bits_u) == r.first ? 1u : 0u;
-      last = max(last, e >> bits_u);
-    } else {
-      beyond = min(beyond, e);
+  if (lane < 4 && cnt + lane < static_cast<uint32_t>(kLightBuf)) buf[cnt + lane] = kNoEdge;
+  __syncwarp();
+  for (uint32_t i0 = lane; i0 - lane < cnt; i0 += 128) {
+    // four entries a lane against four of the buffer per 16-byte load
+    uint32_t e[4], rank[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int r = 0; r < 4; ++r) e[r] = i0 + 32 * r < cnt ? buf[i0 + 32 * r] : kNoEdge;
+    for (uint32_t j = 0; j < cnt; j += 4) {
+      const uint4 y = *reinterpret_cast<const uint4*>(buf + j);
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        rank[r] += (y.x < e[r] ? 1u : 0u) + (y.y < e[r] ? 1u : 0u) + (y.z < e[r] ? 1u : 0u) + (y.w < e[r] ? 1u : 0u);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (e[r] == kNoEdge) continue;
+      if (rank[r] < static_cast<uint32_t>(Cap)) {
+        if (Cap == kLightCap || rank[r] < static_cast<uint32_t>(kLightCap))
+          edge[rank[r]] = e[r];
+        else
+          edge2[rank[r] - kLightCap] = e[r];
+        ties += (e[r] >> bits_u) == r_first ? 1u : 0u;
+        last = max(last, e[r] >> bits_u);
+      } else {
+        beyond = min(beyond, e[r]);
+      }
     }
   }
   beyond = warp_min_u32(beyond);

@@ -155,38 +155,41 @@ struct LightOut {
   uint32_t bits_u;
   int32_t n;
   float deg;      // edges per row and largest weight if known (deg 0: not; wmax 0: word 14 of the index),
-  uint32_t wmax;  // for each warp's first threshold
+  uint32_t wmax;  // for each warp's first threshold (first_threshold)
+  float first;    // uploads: the first threshold itself
 };
 struct LightSums {
   unsigned long long last = 0, cnt = 0;
+  unsigned long long seen = 0, thr = 0;  // rows with cut lists: edges up to their thresholds, and these
+  uint32_t cut = 0;
   uint32_t hmin = 0xFFFFFFFFu, most = 0, trial = 0;
 };
 
-// The first threshold of light_select, in the middle of its window of counts: as if the weights were
-// uniform up to the largest (of the edge list: word 14), with deg edges per row.  A warp has only a few
-// rows, so a bad guess costs scans: 8192 rows of 4096 edges took 265 us from 0 and take 98 us, against
-// 125 us for the row minima and tie sources this pass replaces.
-// Where deg is not known (a matrix was loaded), the warp takes both from the first columns of its first row.
-__device__ __forceinline__ uint32_t first_threshold(const LightOut& o, const int32_t* row, float most) {
-  float deg = o.deg, wmax = static_cast<float>(o.wmax ? o.wmax : o.light[14]);
-  if (deg == 0.f && row) {
-    const int c1 = min(o.n, 1024);
-    float sum = 0.f;
-    uint32_t cnt = 0;
-    for (int c = static_cast<int>(threadIdx.x) & 31; c < c1; c += 32) {
-      const uint32_t w = static_cast<uint32_t>(row[c]);
-      if (w > 0 && w < kInf) {
-        sum += static_cast<float>(w);
-        ++cnt;
-      }
-    }
-    for (int k = 16; k > 0; k >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, k);
-    cnt = warp_sum_u32(cnt);
-    deg = static_cast<float>(cnt) / static_cast<float>(c1) * static_cast<float>(o.n);
-    wmax = cnt ? 2.f * sum / static_cast<float>(cnt) : 2.0e9f;
+// The first threshold of light_select, in the middle of its window of counts: an upload takes the mean of those
+// that served the loaded matrix, an edge list's load goes by deg edges per row, as if the weights were uniform up to
+// the largest (word 14), and a matrix's load takes the weight that about `want` edges of the warp's first row do not
+// exceed, by the row's first 512 columns.  A warp has only a few rows, so a bad guess costs scans: 8192 rows of 4096
+// edges took 265 us from 0 and take 98, against 125 us for the row minima and tie sources this pass replaces.
+__device__ __forceinline__ uint32_t first_threshold(const LightOut& o, const int32_t* row, uint32_t u, float want) {
+  if (!row) return static_cast<uint32_t>(o.first);
+  if (o.deg > 0.f) {
+    const float wmax = static_cast<float>(o.wmax ? o.wmax : o.light[14]);
+    return static_cast<uint32_t>(fminf(2.0e9f, o.deg <= want ? wmax : wmax * want / o.deg));
   }
-  const float want = 2.25f * most;
-  return static_cast<uint32_t>(fminf(2.0e9f, deg <= want ? wmax : wmax * want / deg));
+  const int c1 = min(o.n, 512);
+  uint32_t x[16], most = 0, cnt = 0;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int c = 32 * i + (static_cast<int>(threadIdx.x) & 31);
+    x[i] = c < c1 && static_cast<uint32_t>(c) != u ? static_cast<uint32_t>(row[c]) : kInf;
+    if (x[i] < kInf) {
+      most = max(most, x[i]);
+      ++cnt;
+    }
+  }
+  const uint32_t k = static_cast<uint32_t>(want * static_cast<float>(c1) / static_cast<float>(o.n));
+  if (warp_sum_u32(cnt) <= k) return kInf;
+  return light_sample(x, k, 0, __reduce_max_sync(0xffffffffu, most));
 }
 
 template <int Cap, class Scan>
@@ -205,6 +208,11 @@ __device__ __forceinline__ void light_row(const LightOut& o, const Scan& scan, u
   }
   if (o.tsrc && lane < o.cap && static_cast<uint32_t>(lane) < r.ties)
     o.tsrc[static_cast<int64_t>(u) * o.cap + lane] = static_cast<int32_t>(edge[lane] & ((1u << o.bits_u) - 1u));
+  if (r.hmin < kInf && r.seen > 0) {
+    sums.seen += r.seen;
+    sums.thr += thr;
+    ++sums.cut;
+  }
   sums.last += r.last;
   sums.cnt += r.cnt;
   sums.hmin = min(sums.hmin, r.hmin);
@@ -212,13 +220,39 @@ __device__ __forceinline__ void light_row(const LightOut& o, const Scan& scan, u
   sums.trial = max(sums.trial, light_trial_word(u, r.cnt, r.first < kInf, static_cast<uint32_t>(o.n)));
 }
 
-__device__ __forceinline__ void light_sums_out(const LightOut& o, const LightSums& s) {
-  if ((threadIdx.x & 31) != 0) return;
-  if (s.hmin < kInf) atomicMax(o.light, ~s.hmin);
-  atomicAdd(reinterpret_cast<unsigned long long*>(o.light + 2), s.last);
-  atomicAdd(reinterpret_cast<unsigned long long*>(o.light + 4), s.cnt);
-  atomicMax(o.light + 6, s.most);
-  atomicMax(o.light + 7, s.trial);
+// Every warp's sums into the index: the block's first, then one reduction per word and block (one per warp to the
+// same few words took 15 us for 8192 rows).
+struct LightBlockSums {
+  unsigned long long add[5];  // last, cnt, seen, thr, finite entries
+  uint32_t top[5];            // ~hmin, most, trial, ~finite min, finite max
+  uint32_t cut;
+};
+__device__ __forceinline__ void light_sums_out(const LightOut& o, const LightSums& s, bool stats = false,
+                                               uint32_t gmin = 0, uint32_t gmax = 0, unsigned long long entries = 0) {
+  __shared__ LightBlockSums t;
+  const int tid = static_cast<int>(threadIdx.x);
+  __syncthreads();
+  if (tid < 5) {
+    t.add[tid] = 0;
+    t.top[tid] = 0;
+  }
+  if (tid == 0) t.cut = 0;
+  __syncthreads();
+  if ((tid & 31) == 0) {
+    const unsigned long long add[5] = {s.last, s.cnt, s.seen, s.thr, entries};
+    const uint32_t top[5] = {s.hmin < kInf ? ~s.hmin : 0u, s.most, s.trial, ~gmin, gmax};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      atomicAdd(&t.add[i], add[i]);
+      atomicMax(&t.top[i], top[i]);
+    }
+    atomicAdd(&t.cut, s.cut);
+  }
+  __syncthreads();
+  constexpr int kAdd[5] = {2, 4, kLightSeen, kLightSeen + 2, 10}, kTop[5] = {0, 6, 7, 8, 9};
+  if (tid < (stats ? 5 : 4)) atomicAdd(reinterpret_cast<unsigned long long*>(o.light + kAdd[tid]), t.add[tid]);
+  if (tid < (stats ? 5 : 3) && t.top[tid]) atomicMax(o.light + kTop[tid], t.top[tid]);
+  if (tid == 0 && t.cut) atomicAdd(o.light + kLightSeen + 4, t.cut);
 }
 
 // The rows of the resident matrix; with `stats` also the finite min / max and the number of finite
@@ -226,12 +260,12 @@ __device__ __forceinline__ void light_sums_out(const LightOut& o, const LightSum
 template <int Cap>
 __global__ void __launch_bounds__(256) k_light_rows(const int32_t* __restrict__ W, int64_t pitch, const LightOut o,
                                                     bool stats) {
-  __shared__ uint32_t s_buf[8][kLightBuf];
+  __shared__ __align__(16) uint32_t s_buf[8][kLightBuf];
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
   const int64_t nq = pitch / 4;
-  uint32_t thr = first_threshold(o, warp < o.n ? W + warp * pitch : nullptr, Cap), gmin = kInf, gmax = 0;
+  uint32_t thr = warp < o.n ? first_threshold(o, W + warp * pitch, static_cast<uint32_t>(warp), 2.25f * Cap) : 0u, gmin = kInf, gmax = 0;
   unsigned long long cnt = 0;
   LightSums sums;
   for (int64_t u = warp; u < o.n; u += nwarps) {
@@ -268,42 +302,53 @@ __global__ void __launch_bounds__(256) k_light_rows(const int32_t* __restrict__ 
     gmax = max(gmax, mx);
     cnt += c;
   }
-  light_sums_out(o, sums);
-  if (stats) {
-    for (int k = 16; k > 0; k >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, k);
-    gmax = __reduce_max_sync(0xffffffffu, gmax);
-    if (lane == 0) {
-      atomicMax(o.light + 8, ~gmin);
-      atomicMax(o.light + 9, gmax);
-      atomicAdd(reinterpret_cast<unsigned long long*>(o.light + 10), cnt);
-    }
-  }
+  for (int k = 16; k > 0; k >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, k);
+  light_sums_out(o, sums, stats, gmin, __reduce_max_sync(0xffffffffu, gmax), cnt);
 }
 
 // Upload from pinned host memory (device-accessible through unified addressing): each warp copies one
 // row at a time from `src` (row stride ld) into the graph's row and selects its light edges on the
 // way (k_light_rows), so the matrix crosses the host link once and is not read from HBM again.  With
 // `vec` (ld a multiple of 4, src 16-byte aligned) the row moves in 16-byte pieces, four in flight per
-// lane; otherwise it is copied entry by entry and selected from the copy.  Padding columns are left
-// as they are (INF).
+// lane, otherwise in 4-byte pieces, sixteen in flight.  Padding columns are left as they are (INF).
 __global__ void __launch_bounds__(256) k_upload_rows(const int32_t* __restrict__ src, int64_t ld,
                                                      int32_t* __restrict__ W, int64_t pitch, const LightOut o,
                                                      int vec) {
-  __shared__ uint32_t s_buf[8][kLightBuf];
+  __shared__ __align__(16) uint32_t s_buf[8][kLightBuf];
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
   const int4 none = make_int4(int(kInf), int(kInf), int(kInf), int(kInf));
-  uint32_t thr = first_threshold(o, nullptr, kLightCap);
+  uint32_t thr = first_threshold(o, nullptr, 0, 0.f);
   LightSums sums;
   for (int64_t u = warp; u < o.n; u += nwarps) {
     const int32_t* s = src + u * ld;
     int32_t* d = W + u * pitch;
-    if (!vec) {
-      for (int64_t c = lane; c < o.n; c += 32) d[c] = s[c];
-      __syncwarp();  // the row as every lane wrote it
-    }
     auto scan = [&](const auto& f, int pass) {
+      if (!vec && pass == 0) {
+        for (int64_t b = 0; b < o.n; b += 4 * 128) {
+          int4 x[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const int64_t c = b + 128 * r + lane;
+            x[r].x = c < o.n ? s[c] : none.x;
+            x[r].y = c + 32 < o.n ? s[c + 32] : none.x;
+            x[r].z = c + 64 < o.n ? s[c + 64] : none.x;
+            x[r].w = c + 96 < o.n ? s[c + 96] : none.x;
+          }
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const int64_t c = b + 128 * r + lane;
+            if (c < o.n) d[c] = x[r].x;
+            if (c + 32 < o.n) d[c + 32] = x[r].y;
+            if (c + 64 < o.n) d[c + 64] = x[r].z;
+            if (c + 96 < o.n) d[c + 96] = x[r].w;
+            if (b + 128 * r < o.n) f(static_cast<uint32_t>(c), x[r], 32u);
+          }
+        }
+        __syncwarp();  // later scans read the row as every lane wrote it
+        return;
+      }
       const bool copy = vec && pass == 0;
       const int4* from = reinterpret_cast<const int4*>(copy ? s : d);
       const int64_t nq = copy ? o.n / 4 : pitch / 4;
@@ -591,7 +636,7 @@ static void launch_inlists(dj_graph* g, cudaStream_t st) {
 static LightOut light_out(const dj_graph* g) {
   return LightOut{g->light, g->minout, g->directed ? nullptr : g->tsrc, g->tcnt, g->tcap,
                   host_bits_for(static_cast<uint32_t>(g->n)), g->n, g->light_deg,
-                  static_cast<uint32_t>(g->wmax)};
+                  static_cast<uint32_t>(g->wmax), g->light_first};
 }
 
 // Row minima (with the index, on a symmetric matrix the tie sources too; unless `have_rows`: the upload kernel took
@@ -657,14 +702,17 @@ static int judge_cut(dj_graph* g, const uint32_t* idx, cudaStream_t st, bool* go
 }
 
 // Whether lists of kLightWide edges would hold every edge that matters: the source's row needs the most of
-// them, those of weight up to the largest dist (the trial's).  Their number is estimated from the lists, and as
-// if the weights were uniform between the smallest and the largest, whichever is more.
+// them, those of weight up to the largest dist (the trial's).  Their number is estimated from the lists, from the
+// edges up to the thresholds (a list cut among equal weights misses some of those), and as if the weights were uniform
+// between the smallest and the largest, whichever is most.
+static double sum_at(const uint32_t* words) { return words[0] + 4294967296.0 * words[1]; }
 static bool wide_suffices(const dj_graph* g, const uint32_t* idx) {
   if (idx[kLightGuess] == 0) return false;
   const double D = idx[kLightGuess] - 1.0;
-  const double last = idx[2] + 4294967296.0 * idx[3], cnt = idx[4] + 4294967296.0 * idx[5];
+  const double listed = sum_at(idx + 4), last = sum_at(idx + 2);  // edges per unit of weight, in the lists
+  const double seen = sum_at(idx + kLightSeen), thr = sum_at(idx + kLightSeen + 2);  // and up to the thresholds
   const double uniform = g->light_deg * (D - g->wmin + 1.0) / (static_cast<double>(g->wmax) - g->wmin + 1.0);
-  return std::max(last > 0 ? cnt / last * D : 0.0, uniform) <= 1.1 * kLightWide;
+  return std::max({last > 0 ? listed / last * D : 0.0, thr > 0 ? seen / thr * D : 0.0, uniform}) <= 1.1 * kLightWide;
 }
 
 // Row and column minima, index, global weight range, then the overflow rule (n-1) * wmax < INT32_MAX.
@@ -731,6 +779,9 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
     if (tried && !complete)
       if (int rc = judge_cut(g, idx, st, &good)) return rc;
   }
+  // an upload's first threshold: the mean of those that served this matrix (the new one is likely of its kind)
+  const uint32_t cut = idx[kLightSeen + 4];
+  g->light_first = cut ? static_cast<float>(sum_at(idx + kLightSeen + 2) / cut + 0.5) : ~idx[0] >= kInf ? 2.0e9f : 0.f;
   g->light_ok = complete || good;
   g->light_few = g->light_ok && light_few(g->n, guess, g->wmin);
   g->light_cta = g->light_ok && (complete || !g->directed);
@@ -931,7 +982,10 @@ extern "C" int dj_graph_upload(dj_graph* g, const int32_t* W, int64_t ld, uint64
   if (zero_copy) {
     const int32_t* src = static_cast<const int32_t*>(pa.devicePointer);
     const int vec = (ld % 4 == 0 && reinterpret_cast<uintptr_t>(src) % 16 == 0) ? 1 : 0;
-    k_upload_rows<<<grid_for(static_cast<int64_t>(g->n) * 32), 256, 0, st>>>(src, ld, g->W, g->pitch, light_out(g), vec);
+    // two blocks an SM keep the host link busy; with a warp for every row all would select their edges at the end,
+    // when nothing is left to copy (n = 8192, weights 1..10: 1358 us, 1323 so; n = 6001, unaligned: 827 and 797)
+    const int blocks = std::min((g->n + 7) / 8, 152 * 2);
+    k_upload_rows<<<blocks, 256, 0, st>>>(src, ld, g->W, g->pitch, light_out(g), vec);
     e = cudaGetLastError();
   } else if (ld == g->n && g->n == g->pitch) {  // no padding columns on either side: one contiguous copy
     e = cudaMemcpyAsync(g->W, W, static_cast<size_t>(g->n) * g->pitch * sizeof(int32_t), cudaMemcpyHostToDevice, st);
