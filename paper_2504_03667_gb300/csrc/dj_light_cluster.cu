@@ -306,6 +306,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
         [&](int lw, int i) { return make_uint2(static_cast<uint32_t>(32 * global_word(lw) + i), dist[32 * lw + i]); }, B);
   cluster_sync_all();  // every offer has arrived; nobody touches another CTA's memory from here on
   pdl_wait();          // results reach memory in stream order
+  if (rank == 0 && tid == 0) mark_done(p.mark);  // before them: it goes to host memory
   for (int lw = warp; lw < LW; lw += kClWarps) {
     const int v = 32 * global_word(lw) + lane;
     if (v >= n) continue;
@@ -313,10 +314,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
     d.dist[v] = static_cast<int32_t>(dv == kNone ? kInf : dv);
     d.pred[v] = dv == kNone || v == d.source ? -1 : static_cast<int32_t>(tie[32 * lw + lane] & umask);
   }
-  if (rank == 0 && tid == 0) {
-    if (p.phases_out) *p.phases_out = phase;
-    mark_done(p.mark);
-  }
+  if (rank == 0 && tid == 0 && p.phases_out) *p.phases_out = phase;
 }
 
 // ============================================================ host
