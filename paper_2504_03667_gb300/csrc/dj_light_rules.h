@@ -51,17 +51,18 @@ DJ_RULE bool light_risky(uint32_t dist, uint32_t hmin, uint32_t D) {
   return dist < kRuleInf && hmin < kRuleInf && hmin <= D + dist;
 }
 
-// What the first trial says about a graph with cut lists.  kTrialNo: no.  kTrialAll: next to no row is ever
+// What the first trial says about a graph with cut lists.  kTrialNo: no.  kTrialAll: few rows are ever
 // relaxed whole, whatever the source (on a directed matrix the bound is none, but a good sign, and only the grid
 // form is at stake).  kTrialAsk: other sources have to be tried (a structured graph's, or one of few distinct
 // weights, may need many rows where this one needed none).
 enum { kTrialNo, kTrialAll, kTrialAsk };
 constexpr uint32_t kTrialRows = 4;         // whole rows a trial may need
+constexpr uint32_t kTrialRisky = 32;       // rows at risk: one CTA reads as many in 50 us (n = 8192), and hardly ever must
 constexpr uint32_t kTrialManyRows = 1024;  // the first trial stops beyond: its D, on which the longer lists hang, is settled
 constexpr uint32_t kTrialPhases = 64;      // and here: dists reach far beyond the lists (a phase is an eighth of them)
 inline int light_trial_verdict(uint32_t rows, uint32_t guess, uint32_t risky) {
   if (guess == 0 || rows > kTrialRows) return kTrialNo;  // guess 0: not every node that has an in-edge was reached
-  return risky <= kTrialRows ? kTrialAll : kTrialAsk;
+  return risky <= kTrialRisky ? kTrialAll : kTrialAsk;
 }
 
 // Whether a graph whose lists of 64 edges are cut and that has less than kLightClusterMinN nodes is one of few phases: its largest dist

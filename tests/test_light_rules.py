@@ -137,8 +137,8 @@ def test_trial_source_has_edges(rules, n):
 def test_trial_verdict(rules):
     no, every, ask = 0, 1, 2
     assert rules.verdict(0, 0, 0) == no  # did not reach every node that something leads to
-    assert rules.verdict(5, 10, 0) == no and rules.verdict(4, 10, 4) == every
-    assert rules.verdict(0, 10, 5) == ask
+    assert rules.verdict(5, 10, 0) == no and rules.verdict(4, 10, 32) == every
+    assert rules.verdict(0, 10, 33) == ask
     assert not rules.risky(NONE, 1, 5) and not rules.risky(INF, 1, 5) and not rules.risky(3, INF, 5)
     assert rules.risky(3, 8, 5) and not rules.risky(3, 9, 5)
 
