@@ -75,13 +75,15 @@ constexpr int kLightStats = 64;  // leading words: [0] ~(smallest hmin), [1] row
                                  // [15] kLightGuess, [16..17] the trials' farthest node (dist, node),
                                  // [18..22] of the rows with cut lists (at load): sum of the edges up to their
                                  // thresholds, of these, rows; [23] rows that some source may need whole
-                                 // (light_risky); [24..] rows relaxed whole by each further trial
+                                 // (light_risky); [24..] rows relaxed whole by each further trial,
+                                 // [40] kLightError
 constexpr int kLightHost = 24;   // the words that the host reads
 constexpr int kLightGuess = 15;  // 1 + the trial solve's largest dist (0: unknown)
 constexpr int kLightFar = 16;
 constexpr int kLightSeen = 18;
 constexpr int kLightRisky = 23;
 constexpr int kLightMore = 24;
+constexpr int kLightError = 40;  // a trial's error bits
 constexpr int kMoreTrials = 16;  // from the farthest node and fifteen places (without the CTA form: fewer)
 inline
 #ifdef __CUDACC__

@@ -474,7 +474,7 @@ static int run_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int3
   p.pred_out = pred;
   p.ctl = reinterpret_cast<uint32_t*>(ws);
   p.gkey = reinterpret_cast<unsigned long long*>(ws + ctl_bytes);
-  p.words = ctx->words;
+  p.words = heavy ? g->light + kLightError : ctx->words;  // a trial that ran out of time is no caller's error
   p.heavy = heavy;
   p.mark = mark;
   p.guess = heavy && source == kTrialFirst ? g->light + kLightGuess : nullptr;

@@ -693,11 +693,12 @@ static int judge_cut(dj_graph* g, const uint32_t* idx, cudaStream_t st, bool* go
                                           more + i, st) == DJ_OK;
   }
   clear_error();
-  uint32_t rows[kMoreTrials] = {0};
+  static_assert(kLightMore + kMoreTrials == kLightError, "one copy takes both");
+  uint32_t rows[kMoreTrials + 1] = {0};  // and the error bits
   cudaMemcpyAsync(rows, more, sizeof(rows), cudaMemcpyDeviceToHost, st);
   const cudaError_t e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_error(e, "trial solves");
-  *good = tried && *std::max_element(rows, rows + kMoreTrials) <= kTrialRows;
+  *good = tried && rows[kMoreTrials] == 0 && *std::max_element(rows, rows + kMoreTrials) <= kTrialRows;
   return DJ_OK;
 }
 
