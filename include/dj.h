@@ -153,17 +153,23 @@ int dj_graph_free(dj_graph* g);
 
 /* The light engine.  A loaded graph keeps, beside its matrix, each row's up to
  * 64 lightest edges, or 128 where 64 are too few and these enough, and the
- * smallest weight not among them (516 bytes a node; dj_graph_upload rebuilds 64).  A solve relaxes those; then dist[u] + (u's
+ * smallest weight not among them (room for 516 bytes a node; dj_graph_upload
+ * rebuilds 64).  A solve relaxes those; then dist[u] + (u's
  * smallest unlisted weight) > max dist proves that no unlisted edge matters,
  * and rows that fail the test are relaxed whole from the matrix, so dist and
  * pred are Algorithm 1's on every graph.  One solve runs on one CTA, on one
- * cluster or on every SM, by size and by whether anything is ahead of it on
- * its stream (dj_sssp).  Taken by DJ_ENGINE_AUTO in phase
+ * cluster or on every SM, by size and by whether another solve is ahead of it
+ * on its stream (dj_sssp).  Taken by DJ_ENGINE_AUTO in phase
  * mode when every weight is >= 1, every other option below is left at its
- * default, and a trial solve at load needed next to no whole row; also for
- * graphs in compressed rows.  After dj_graph_upload a graph's solves take the
+ * default, and trial solves at load needed next to no whole row; also for
+ * graphs in compressed rows.  Two kinds of small matrices take it only for
+ * solves that are alone on their stream, and in batches: directed ones with
+ * more edges per row than are listed (these not in batches either), and such
+ * of fewer than 2048 nodes whose largest dist is at most three times their
+ * smallest weight.  After dj_graph_upload a graph's solves take the
  * other engines (the new matrix has not been tried); solves captured into a
- * CUDA graph before stay valid. */
+ * CUDA graph before stay valid (if the new matrix has weights of 0, their dist
+ * does; ties among nodes that such edges connect may be broken otherwise). */
 
 typedef struct dj_solve_opts {
   int32_t mode;           /* DJ_MODE_* */
@@ -230,10 +236,10 @@ void dj_solve_opts_init(dj_solve_opts* opts);
 
 /* One solve of Algorithm 1 from `source` on graph g.
  *   dist, pred  DEVICE pointers to n int32 each (caller-owned), written by the kernel.
- * Asynchronous on `stream`: one kernel launch.  Large solves on an idle stream
- * use every SM; small ones, and those behind other work on their stream, a CTA
- * or a cluster each, so that back-to-back solves run side by side (same
- * results).  The grid engine keeps a small
+ * Asynchronous on `stream`: one kernel launch.  Large solves use every SM unless
+ * another solve is directly ahead on their stream or still under way there;
+ * those, and small ones, take a CTA or a cluster each, so that back-to-back
+ * solves run side by side (same results).  The grid engine keeps a small
  * workspace per (device, stream) -- about 32 bytes per matrix column plus 16 *
  * pitch bytes with the row split, at least 1 MiB -- created on the first solve
  * on that stream (a cudaMalloc) and grown, after synchronising the stream,
@@ -421,7 +427,7 @@ typedef struct dj_serve_stats {
   uint64_t submitted, completed, rejected;
   double p50_us, p90_us, p99_us, max_us, mean_us; /* submit-to-completion latency */
   double solves_per_s;                            /* completed / (last completion - first submit) */
-  uint64_t resident_bytes;                        /* graphs + result pool held on the device */
+  uint64_t resident_bytes;                        /* graphs (without their light-edge index) + result pool */
   int32_t kernel_launches;                        /* persistent kernel (re)launches so far */
   int32_t reserved[7];
 } dj_serve_stats;

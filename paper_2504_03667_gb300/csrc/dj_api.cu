@@ -239,7 +239,7 @@ static int solve_cluster_single(const dj_graph* g, int32_t source, int32_t* dist
 }
 
 // The light engine's place: the caller left every choice of engine, bound and path to the library,
-// and the graph's index pays (judge_index; compressed rows of weights >= 1).
+// and the graph's index pays (finish_graph in dj_load.cu; compressed rows of weights >= 1).
 static bool light_auto(const dj_graph* g, const dj_solve_opts& o) {
   return g->light_ok && o.mode != DJ_MODE_PLAIN && o.engine == DJ_ENGINE_AUTO && o.settle == DJ_SETTLE_AUTO &&
          o.cluster_size == 0 && o.threads == 0 && o.ctas_per_sm == 0 && o.unroll == 0 && o.live == 0 &&
@@ -370,16 +370,13 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   const SolveDesc d = make_desc(g, source, dist, pred, 0);
-  // right after an upload the solve waits for the kernels before it before reading the graph
-  const bool early = g->upload_pending == 0;
-  const_cast<dj_graph*>(g)->upload_pending = 0;
   if (cluster) {
-    const int rc = run_light_cluster(g, C, d, ctx->words + 1, early, mark, st);
+    const int rc = run_light_cluster(g, C, d, ctx->words + 1, mark, st);
     if (rc != DJ_ECUDA) return rc;
     clear_error();  // no such cluster here
     return launch_light_grid(g, source, dist, pred, o, mark, st);
   }
-  return run_light_single(plan, d, ctx->words + 1, early, mark, st);
+  return run_light_single(plan, d, ctx->words + 1, mark, st);
 }
 
 // Whether solves of g behind others on their stream take the light engine.  A directed matrix with cut lists
@@ -726,7 +723,6 @@ static bool light_batch_ok(const dj_graph* const* graphs, int32_t k, int32_t max
 }
 
 // The one graph every solve of the batch uses, or nullptr.
-
 static dj_graph* shared_graph(const dj_graph* const* graphs, int32_t k) {
   if (k < 1) return nullptr;
   for (int32_t i = 1; i < k; ++i)

@@ -111,7 +111,7 @@ struct SolveDesc {
   int32_t plain;
   int32_t use_in;  // settle by the IN bound too (every off-diagonal weight >= 1); minin = minout + n
   const uint32_t* light;  // light engine: the graph's index
-  int64_t reserved;
+  int64_t reserved;       // five 16-byte loads (ServeJobs::desc)
 };
 static_assert(sizeof(SolveDesc) == 80, "descriptor layout");
 
@@ -310,8 +310,8 @@ int plan_light(int32_t max_n, int32_t k, int kind, LightPlan* plan);
 // as run_cluster, run_cluster_single and run_serve_kernel
 int run_light_batch(const LightPlan& plan, const SolveDesc* descs_dev, int32_t k, uint32_t* queue, bool zero_queue,
                     cudaStream_t st);
-int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, bool early,
-                     const SolveMark& mark, cudaStream_t st);
+int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, const SolveMark& mark,
+                     cudaStream_t st);
 // kMoreTrials trial solves of one graph side by side (LightTrialJobs): words [kLightMore..] count the rows
 // that each relaxed whole, up to the first count above kTrialRows.
 int run_light_trials(const LightPlan& plan, const SolveDesc& d, uint32_t* light, cudaStream_t st);
@@ -319,8 +319,8 @@ int run_light_serve(const LightPlan& plan, const ServeRing& r, cudaStream_t st);
 // One solve on one cluster of C CTAs (a power of two up to 16), as run_light_single.
 bool light_cluster_fits(int32_t n, int C, bool csr);
 int prepare_light_cluster(bool csr, int C);  // its launch attributes, before a capture may need them
-int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t* phases_out, bool early,
-                      const SolveMark& mark, cudaStream_t st);
+int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t* phases_out, const SolveMark& mark,
+                      cudaStream_t st);
 // One solve over every SM (a graph with an index, or in compressed rows).
 int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t* pred, const dj_solve_opts& o,
                       const SolveMark& mark, cudaStream_t st);

@@ -1,4 +1,5 @@
-// The light-edge index of a graph and the 64-bit keys of the light engine (dj_light.cu).
+// The light-edge index of a graph and the 64-bit keys of the light engine (dj_light_cta.cu, dj_light_cluster.cu,
+// dj_light_grid.cu).
 //
 // Most entries of a dense matrix can never matter to a solve: an entry W[u][v] offers v at least
 // dist[u] + W[u][v], so once every node holds some path length, only entries of at most (largest
@@ -9,7 +10,7 @@
 // first are too few and these are enough) and the smallest weight it does not list (hmin).  A solve runs on the listed edges, and then
 //   dist[u] + hmin[u] > max over v of dist[v]   for every u
 // proves that no unlisted entry can improve or tie any node: the answer is exact.  The rows that
-// fail the test are relaxed whole from the matrix (see dj_light.cu), so the answer is exact on
+// fail the test are relaxed whole from the matrix (see dj_light_grid.cu), so the answer is exact on
 // every graph; the test only decides how many rows are read.
 //
 // Keys.  With every weight >= 1, Algorithm 1's pred[v] is the u of smallest (dist[u], u) among

@@ -37,7 +37,6 @@ struct LightClusterParams {
   uint32_t* phases_out;
   SolveMark mark;
   uint32_t delta;          // compressed rows (dense: from the index)
-  int32_t early;           // the graph may be read before the kernel ahead on the stream has completed
   int32_t cshift;          // log2 C
   int32_t lw;              // words per CTA
 };
@@ -118,7 +117,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
   uint32_t* len = whole + LW;
   const LightClusterStore s{smem_u32(dist), smem_u32(tie), smem_u32(dirty), p.cshift};
   pdl_launch_dependents();
-  if (!p.early) pdl_wait();  // the kernel before may still be writing the graph
+  // the graph is read at once: no kernel ahead on the stream writes it (an upload takes a graph off this engine)
 
   const SolveDesc& d = p.d;
   const int n = d.n;
@@ -250,7 +249,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
         }
         if (cnt > 0) relax(cnt);
       } else {
-        // the index proves the answer, or some rows are relaxed whole, a warp per row
+        // the index proves the answer, or some rows are relaxed whole, in pieces by all warps
         if (hmin_min > D) break;
         B = D;
         auto pending = [&](int lw, uint32_t dv) {  // dist + hmin of this lane's node if its row is pending
@@ -337,8 +336,8 @@ int prepare_light_cluster(bool csr, int C) {
                           0, C > 8);
 }
 
-int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t* phases_out, bool early,
-                      const SolveMark& mark, cudaStream_t st) {
+int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t* phases_out, const SolveMark& mark,
+                      cudaStream_t st) {
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
   const bool csr = g->format == DJ_FORMAT_CSR;
@@ -353,7 +352,6 @@ int run_light_cluster(const dj_graph* g, int C, const SolveDesc& desc, uint32_t*
   p.phases_out = phases_out;
   p.mark = mark;
   p.delta = static_cast<uint32_t>(std::min(1.0e9f, kClDelta * g->light_spacing));
-  p.early = early ? 1 : 0;
   p.cshift = 0;
   while ((1 << p.cshift) < C) ++p.cshift;
   p.lw = light_cluster_words(g->n, C);

@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
           }
           if (cnt > 0) relax(cnt);
         } else {
-          // the index proves the answer, or some rows are relaxed whole, a warp per row
+          // the index proves the answer, or some rows are relaxed whole, in pieces by all warps
           if (hmin_min > D) break;
           B = D;
           __syncthreads();  // everyone has read s_bound
@@ -313,8 +313,10 @@ bool light_cta_fits(int32_t n) {
 // allows (256 sources of n = 8192: 298 us, 354 with one; 48 graphs, which have an SM each, 112 with the
 // registers of one, 129 with those of two).  The server's persistent CTAs have 192 threads, one per SM:
 // other kernels must find room beside them for as long as the server runs (two CTAs of 512 threads fill
-// every register of an SM, and a caller's own kernels waited until the server left).  Its rate is the
-// host's (1500 waiting requests: 3.4 ms with 192 threads, 3.3 with 256, 3.1 with 512).
+// every register of an SM, and a caller's own kernels waited until the server left); 192 leave 47 of an SM's 64 K
+// registers, 256 leave 41.  (The load's trial solves, 54 K, fit beside neither: loading a graph with cut lists
+// waits until the server's kernel has left, as it did beside the cluster engine's.)  Its rate is the host's (1500
+// waiting requests: 3.4 ms with 192 threads, 3.3 with 256, 3.1 with 512).
 int plan_light(int32_t max_n, int32_t k, int kind, LightPlan* plan) {
   DevCtx* ctx = nullptr;
   if (int rc = get_ctx(&ctx)) return rc;
@@ -370,13 +372,13 @@ int run_light_batch(const LightPlan& plan, const SolveDesc* descs_dev, int32_t k
   return launch_light(plan, args, st, false);
 }
 
-int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, bool early,
-                     const SolveMark& mark, cudaStream_t st) {
+int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, const SolveMark& mark,
+                     cudaStream_t st) {
   LightCtaParams p{plan.npad};
   SingleJob job;
   job.d = d;
   job.phases_out = phases_out;
-  job.early_ok = early ? 1 : 0;
+  job.early_ok = 1;  // no kernel ahead on the stream writes the graph: an upload takes it off this engine
   job.mark = mark;
   void* args[] = {&p, &job};
   return launch_light(plan, args, st, true);

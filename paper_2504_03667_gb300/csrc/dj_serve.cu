@@ -324,8 +324,9 @@ extern "C" int dj_serve_add_graph(dj_server* s, const dj_graph* g, int32_t* grap
   if (!s || !g || !graph_id) return set_error(DJ_EINVAL, "NULL argument");
   if (g->device != s->device) return set_error(DJ_EINVAL, "graph on another device");
   if (int rc = require_dense(g)) return rc;
-  // the budget counts the matrix and what was always kept beside it, not the light-edge index (256
-  // bytes a node): budgets chosen for the matrices keep admitting the same graphs
+  // the budget (and resident_bytes) counts the matrix and what was always kept beside it, not the light-edge
+  // index (516 bytes a node, which the server's device memory holds as well): budgets chosen for the matrices
+  // keep admitting the same graphs
   const uint64_t bytes = g->bytes - g->light_bytes;
   if (s->graph_bytes + s->pool_bytes + s->fixed_bytes + bytes > s->opts.hbm_budget)
     return set_error(DJ_ENOMEM, "graph does not fit the serving HBM budget");
