@@ -359,9 +359,12 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
   const bool cluster = !cta && (csr ? g->light_longest <= kLightClusterMaxRow : g->light_cta) &&
                        light_cluster_fits(g->n, C, csr);
   // whichever form this call takes: a later one may be captured
-  LightPlan plan;
+  LightPlan plan, marked;
   if (cta) {
-    if (int rc = plan_light(g->n, 1, kJobsSingle, &plan)) return rc;
+    if (int rc = plan_light(g->n, 1, kJobsPlainSingle, &plan)) return rc;
+    if (mark.done || lone) {
+      if (int rc = plan_light(g->n, 1, kJobsSingle, &marked)) return rc;
+    }
   } else if (cluster) {
     if (int rc = prepare_light_cluster(csr, C)) return rc;
   }
@@ -376,7 +379,7 @@ static int solve_light(const dj_graph* g, int32_t source, int32_t* dist, int32_t
     clear_error();  // no such cluster here
     return launch_light_grid(g, source, dist, pred, o, mark, st);
   }
-  return run_light_single(plan, d, ctx->words + 1, mark, st);
+  return run_light_single(mark.done ? marked : plan, d, ctx->words + 1, mark, st);
 }
 
 // Whether solves of g behind others on their stream take the light engine.  A directed matrix with cut lists

@@ -248,6 +248,7 @@ constexpr int kJobsBatch = 0;
 constexpr int kJobsServe = 1;
 constexpr int kJobsSingle = 2;
 constexpr int kJobsTrial = 3;  // light engine: trial solves
+constexpr int kJobsPlainSingle = 4;  // light engine: a single solve that leaves no mark
 int plan_cluster(int32_t max_pitch, const ClusterLaunch& cl, int32_t k, ClusterPlan* plan, int kind = kJobsBatch);
 // queue: two device words (next solve, exit count), zero when the launch starts; with
 // zero_queue the launch zeroes them first, otherwise the previous launch left them zero
@@ -313,7 +314,7 @@ int run_light_batch(const LightPlan& plan, const SolveDesc* descs_dev, int32_t k
 int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases_out, const SolveMark& mark,
                      cudaStream_t st);
 // kMoreTrials trial solves of one graph side by side (LightTrialJobs): words [kLightMore..] count the rows
-// that each relaxed whole, up to the first count above kTrialRows.
+// that each relaxed whole, up to the first count above kTrialMoreRows.
 int run_light_trials(const LightPlan& plan, const SolveDesc& d, uint32_t* light, cudaStream_t st);
 int run_light_serve(const LightPlan& plan, const ServeRing& r, cudaStream_t st);
 // One solve on one cluster of C CTAs (a power of two up to 16), as run_light_single.
@@ -326,7 +327,7 @@ int launch_light_grid(const dj_graph* g, int32_t source, int32_t* dist, int32_t*
                       const SolveMark& mark, cudaStream_t st);
 // A trial solve, which writes nothing but the index's words.  From the source that the rows' words name
 // (kTrialFirst: it leaves kLightGuess), from the farthest node of the trials so far (kTrialFar), or from a
-// given one; those stop once more than kTrialRows rows were relaxed whole, counted in *heavy.
+// given one; those stop once more than kTrialMoreRows rows were relaxed whole, counted in *heavy.
 constexpr int32_t kTrialFirst = -1, kTrialFar = -2;
 int launch_light_trial(const dj_graph* g, int32_t source, uint32_t* heavy, cudaStream_t st);
 int cluster_max_clusters(int32_t max_pitch, const ClusterLaunch& cl, int* clusters);

@@ -51,11 +51,10 @@ struct BatchJobs {
 // predecessor to complete only before it writes dist, pred and the phase
 // count.  So results reach memory in stream order, and back-to-back solves of
 // small graphs overlap on the GPU's idle SMs.
-struct SingleJob {
+struct PlainSingleJob {
   SolveDesc d;
   uint32_t* phases_out;
   int32_t early_ok;
-  SolveMark mark;
   __device__ bool fetch(uint32_t* job, uint32_t iter) const {
     *job = 0;
     return iter == 0 && cluster_id_x() == 0;
@@ -63,7 +62,6 @@ struct SingleJob {
   __device__ SolveDesc desc(uint32_t) const { return d; }
   __device__ void complete(uint32_t, uint32_t phases) const {
     if (phases_out) *phases_out = phases;
-    mark_done(mark);
   }
   static constexpr uint32_t kGuessPart = 8;
   static constexpr bool kTrial = false;
@@ -71,6 +69,16 @@ struct SingleJob {
   __device__ bool early() const { return early_ok != 0; }
   __device__ void before_write() const { pdl_wait(); }
   __device__ void leave(uint32_t) const {}
+};
+
+// The same with a mark for the next solve's choice of form.  (A job of its own: the light engine's CTA form took
+// 36.7 us instead of 34.4 for n = 1024 alone with the mark compiled in, used or not.)
+struct SingleJob : PlainSingleJob {
+  SolveMark mark;
+  __device__ void complete(uint32_t job, uint32_t phases) const {
+    PlainSingleJob::complete(job, phases);
+    mark_done(mark);
+  }
 };
 
 // Serving: requests arrive in a ring of descriptors in mapped pinned host

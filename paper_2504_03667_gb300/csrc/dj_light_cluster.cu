@@ -264,10 +264,11 @@ __global__ void __launch_bounds__(kClThreads, 1) k_light_cluster(const LightClus
         cluster_sync_all();
         hb = s_bound;
         if (hb == kNone) break;
-        // the final ones (light_final): relaxed whole, as many as the list holds now
+        // the final ones (light_below): relaxed whole, as many as the list holds now
+        hb = light_below(hb, hmin_min);
         for (int lw = warp; lw < LW; lw += kClWarps) {
           const uint32_t dv = dist[32 * lw + lane];
-          const bool go = pending(lw, dv) != kNone && light_final(dv, __ldg(hmin + 32 * global_word(lw) + lane), hb);
+          const bool go = dv < hb && pending(lw, dv) != kNone;
           const uint32_t todo = __ballot_sync(0xffffffffu, go);
           if (todo == 0) continue;
           uint32_t pos = 0;

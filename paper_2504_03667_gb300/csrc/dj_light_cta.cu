@@ -225,10 +225,11 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
           __syncthreads();
           hb = s_bound;
           if (hb == kNone) break;
-          // the final ones (light_final): relaxed whole, as many as the list holds now
+          // the final ones (light_below): relaxed whole, as many as the list holds now
+          hb = light_below(hb, hmin_min);
           for (int wi = warp; wi < nwords; wi += NW) {
             const uint32_t dv = s.dist[32 * wi + lane];
-            const bool go = pending(wi, dv) != kNone && light_final(dv, __ldg(hmin + 32 * wi + lane), hb);
+            const bool go = dv < hb && pending(wi, dv) != kNone;
             const uint32_t todo = __ballot_sync(0xffffffffu, go);
             if (todo == 0) continue;
             uint32_t pos = 0;
@@ -244,7 +245,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
           __syncthreads();
           any_whole = true;
           const int count = static_cast<int>(min(s_cnt, s_end));
-          if (Jobs::kTrial && (nwhole += static_cast<uint32_t>(count)) > kTrialRows) break;  // it has its answer
+          if (Jobs::kTrial && (nwhole += static_cast<uint32_t>(count)) > kTrialMoreRows) break;  // it has its answer
           light_whole_rows(s, d, s_rows[0], count, D, lmin);
         }
       }
@@ -327,11 +328,12 @@ int plan_light(int32_t max_n, int32_t k, int kind, LightPlan* plan) {
                    2 * (plan->smem + kLightCtaStatic) <= static_cast<size_t>(ctx->max_smem_optin);
   plan->fn = kind == kJobsServe    ? reinterpret_cast<void*>(&k_light_cta<192, 1, ServeJobs>)
              : kind == kJobsSingle ? reinterpret_cast<void*>(&k_light_cta<512, 1, SingleJob>)
+             : kind == kJobsPlainSingle ? reinterpret_cast<void*>(&k_light_cta<512, 1, PlainSingleJob>)
              : kind == kJobsTrial  ? reinterpret_cast<void*>(&k_light_cta<512, 1, LightTrialJobs>)
              : two                 ? reinterpret_cast<void*>(&k_light_cta<512, 2, BatchJobs>)
                                    : reinterpret_cast<void*>(&k_light_cta<512, 1, BatchJobs>);
   if (int rc = prepare_function(ctx, plan->fn, plan->smem, false)) return rc;
-  plan->ctas = kind == kJobsSingle ? 1 : kind == kJobsTrial ? kMoreTrials : ctx->num_sms * (two ? 2 : 1);
+  plan->ctas = kind == kJobsSingle || kind == kJobsPlainSingle ? 1 : kind == kJobsTrial ? kMoreTrials : ctx->num_sms * (two ? 2 : 1);
   if (kind == kJobsBatch) plan->ctas = std::max(1, std::min(plan->ctas, static_cast<int>(k)));
   return DJ_OK;
 }
@@ -379,7 +381,7 @@ int run_light_single(const LightPlan& plan, const SolveDesc& d, uint32_t* phases
   job.d = d;
   job.phases_out = phases_out;
   job.early_ok = 1;  // no kernel ahead on the stream writes the graph: an upload takes it off this engine
-  job.mark = mark;
+  job.mark = mark;  // beyond the plain job, which the plan's kernel may take
   void* args[] = {&p, &job};
   return launch_light(plan, args, st, true);
 }

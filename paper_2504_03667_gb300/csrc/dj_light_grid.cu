@@ -13,7 +13,7 @@
 // relax whole from the matrix:
 //   pending = { u : dist[u] + hmin[u] <= D, not yet relaxed whole }, and
 //   those with dist[u] < min over pending of (dist + hmin) are final -- a shorter path would use an
-//   unlisted edge of a pending row -- so each row is read from the matrix at most once (light_final also
+//   unlisted edge of a pending row -- so each row is read from the matrix at most once (light_below also
 //   sees to it that every round takes the row that gives the minimum).
 //
 // What bounds it: latency.  A phase is one grid barrier (which also carries m and D) and a chain of
@@ -338,9 +338,9 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
     hb = m;
     D = Dx;
     if (hb == kNone) break;
+    hb = light_below(hb, hmin_min);
     for (int j = tid; j < sw; j += T0) {
-      if ((flags[j] & 2) || rdist[j] >= kInf || !light_final(rdist[j], aux[j], hb) || light_pending(rdist[j], aux[j], Dx) == kNone)
-        continue;
+      if ((flags[j] & 2) || rdist[j] >= hb || light_pending(rdist[j], aux[j], Dx) == kNone) continue;
       list[atomicAdd(&sh.cnt, 1u)] = make_uint2(static_cast<uint32_t>(j), rdist[j]);
       flags[j] |= 2;
     }
@@ -350,7 +350,7 @@ __device__ __forceinline__ void light_grid_solve(const LightGridParams& p, uint8
       if (tid == 0 && cnt) atomicAdd(p.heavy, static_cast<uint32_t>(cnt));
       uint32_t unused;
       if (!light_barrier(p, sh, nbar++, kNone, 0u, &m, &unused)) return;
-      if (__ldcg(p.heavy) > (p.guess ? kTrialManyRows : kTrialRows)) break;
+      if (__ldcg(p.heavy) > (p.guess ? kTrialManyRows : kTrialMoreRows)) break;
     }
     const int nv = static_cast<int>(p.pitch / 4);
     for (int i = 0; i < cnt; ++i) {

@@ -23,13 +23,13 @@ DJ_RULE uint32_t light_pending(uint32_t dist, uint32_t hmin, uint32_t D) {
   return x <= D && x < kRuleInf ? x : kRuleNone;
 }
 
-// Whether a pending row is relaxed whole now, hb being the least of what the pending rows offer: a path
-// shorter than dist would have to use an unlisted edge of a pending row, which offers no less than hb.
-// So dist <= hb is final.  The row that gives hb is always among those taken: it has dist < hb, or dist == hb
-// and an unlisted edge of weight 0 (without the second clause no row was taken then, and the solve never ended).
-// Other rows of dist == hb wait: most need not be relaxed once those below are (n = 8192, p = 0.5, weights
-// 1..10: twice as many, and the trial at load 0.2 ms longer).
-DJ_RULE bool light_final(uint32_t dist, uint32_t hmin, uint32_t hb) { return dist < hb || (dist == hb && hmin == 0); }
+// Pending rows of dist below this are relaxed whole now, hb being the least that a pending row offers: a path
+// shorter than dist would have to use an unlisted edge of a pending row, which offers no less than hb, so every
+// dist up to hb is final.  Where each unlisted weight is at least 1 the row that gives hb lies below it; with
+// unlisted weights of 0 it may lie at hb itself (rows below hb alone were none then, and the solve never ended).
+// Rows at hb wait otherwise: most need not be relaxed once those below are (n = 8192, p = 0.5, weights 1..10: twice
+// as many, and the trial at load 0.2 ms longer).
+DJ_RULE uint32_t light_below(uint32_t hb, uint32_t hmin_min) { return hmin_min == 0 ? hb + 1 : hb; }
 
 // Whether a graph's trial solve is run: some list is cut, and no weight is 0 (its solves take the other
 // engines then, and its lists may hold nothing but a few of a row's edges of weight 0).
@@ -56,7 +56,9 @@ DJ_RULE bool light_risky(uint32_t dist, uint32_t hmin, uint32_t D) {
 // form is at stake).  kTrialAsk: other sources have to be tried (a structured graph's, or one of few distinct
 // weights, may need many rows where this one needed none).
 enum { kTrialNo, kTrialAll, kTrialAsk };
-constexpr uint32_t kTrialRows = 4;         // whole rows a trial may need
+constexpr uint32_t kTrialRows = 4;         // whole rows the first trial may need
+constexpr uint32_t kTrialMoreRows = 16;    // and each further one: seldom sources may need a few (n = 4096, p = 0.1, weights
+                                           // 1..10: 126 us a solve in a batch, the streaming cluster engine 511)
 constexpr uint32_t kTrialRisky = 32;       // rows at risk: one CTA reads as many in 50 us (n = 8192), and hardly ever must
 constexpr uint32_t kTrialManyRows = 1024;  // the first trial stops beyond: its D, on which the longer lists hang, is settled
 constexpr uint32_t kTrialPhases = 64;      // and here: dists reach far beyond the lists (a phase is an eighth of them)

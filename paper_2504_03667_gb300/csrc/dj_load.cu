@@ -698,7 +698,7 @@ static int judge_cut(dj_graph* g, const uint32_t* idx, cudaStream_t st, bool* go
   cudaMemcpyAsync(rows, more, sizeof(rows), cudaMemcpyDeviceToHost, st);
   const cudaError_t e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_error(e, "trial solves");
-  *good = tried && rows[kMoreTrials] == 0 && *std::max_element(rows, rows + kMoreTrials) <= kTrialRows;
+  *good = tried && rows[kMoreTrials] == 0 && *std::max_element(rows, rows + kMoreTrials) <= kTrialMoreRows;
   return DJ_OK;
 }
 

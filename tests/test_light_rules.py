@@ -19,7 +19,7 @@ PROG = r"""
 #include "dj_light_rules.h"
 extern "C" {
 unsigned pending(unsigned dist, unsigned hmin, unsigned D) { return dj::light_pending(dist, hmin, D); }
-int is_final(unsigned dist, unsigned hmin, unsigned hb) { return dj::light_final(dist, hmin, hb); }
+unsigned below(unsigned hb, unsigned hmin_min) { return dj::light_below(hb, hmin_min); }
 int in_place(size_t a, size_t b, size_t c) { return dj::edges_in_place((void*)a, (void*)b, (void*)c); }
 int upload_in_place(size_t a) { return dj::in_place((void*)a); }
 unsigned trial_word(unsigned u, unsigned listed, int has_edges, unsigned n) {
@@ -44,12 +44,12 @@ def rules(tmp_path_factory):
     src.write_text(PROG)
     subprocess.run([cxx, "-std=c++17", "-O1", "-fPIC", "-shared", "-I", CSRC, str(src), "-o", str(lib)], check=True)
     lib = ctypes.CDLL(str(lib))
-    for f, args in ((lib.pending, 3), (lib.is_final, 3), (lib.needs_trial, 2), (lib.trial_word, 4), (lib.trial_source, 2),
+    for f, args in ((lib.pending, 3), (lib.below, 2), (lib.needs_trial, 2), (lib.trial_word, 4), (lib.trial_source, 2),
                     (lib.verdict, 3), (lib.risky, 3), (lib.few, 3)):
         f.argtypes = [ctypes.c_uint32] * args
     lib.upload_in_place.argtypes = [ctypes.c_size_t]
     lib.in_place.argtypes = [ctypes.c_size_t] * 3
-    for f in (lib.pending, lib.trial_word, lib.trial_source):
+    for f in (lib.pending, lib.below, lib.trial_word, lib.trial_source):
         f.restype = ctypes.c_uint32
     return lib
 
@@ -79,7 +79,7 @@ def solve(W, s, rows, hmin, rules):
         hb = min([x for x in pend.values()] + [NONE])
         if hb == NONE:
             return [d if d != NONE else INF for d in dist]
-        for u in [u for u, x in pend.items() if x != NONE and rules.is_final(dist[u], hmin[u], hb)]:
+        for u in [u for u, x in pend.items() if x != NONE and dist[u] < rules.below(hb, min(hmin))]:
             whole.add(u)
             for v in np.flatnonzero(W[u] < INF):
                 if v != u:
