@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(256) k_light_rows(const int32_t* __restrict__ 
 // row at a time from `src` (row stride ld) into the graph's row and selects its light edges on the
 // way (k_light_rows), so the matrix crosses the host link once and is not read from HBM again.  With
 // `vec` (ld a multiple of 4, src 16-byte aligned) the row moves in 16-byte pieces, four in flight per
-// lane, otherwise in 4-byte pieces, sixteen in flight.  Padding columns are left as they are (INF).
+// lane, otherwise in 4-byte pieces, eight in flight (sixteen: n = 6001 796 us, not 773).  Padding columns are left as they are (INF).
 __global__ void __launch_bounds__(256) k_upload_rows(const int32_t* __restrict__ src, int64_t ld,
                                                      int32_t* __restrict__ W, int64_t pitch, const LightOut o,
                                                      int vec) {
@@ -326,10 +326,10 @@ __global__ void __launch_bounds__(256) k_upload_rows(const int32_t* __restrict__
     int32_t* d = W + u * pitch;
     auto scan = [&](const auto& f, int pass) {
       if (!vec && pass == 0) {
-        for (int64_t b = 0; b < o.n; b += 4 * 128) {
-          int4 x[4];
+        for (int64_t b = 0; b < o.n; b += 2 * 128) {
+          int4 x[2];
 #pragma unroll
-          for (int r = 0; r < 4; ++r) {
+          for (int r = 0; r < 2; ++r) {
             const int64_t c = b + 128 * r + lane;
             x[r].x = c < o.n ? s[c] : none.x;
             x[r].y = c + 32 < o.n ? s[c + 32] : none.x;
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(256) k_upload_rows(const int32_t* __restrict__
             x[r].w = c + 96 < o.n ? s[c + 96] : none.x;
           }
 #pragma unroll
-          for (int r = 0; r < 4; ++r) {
+          for (int r = 0; r < 2; ++r) {
             const int64_t c = b + 128 * r + lane;
             if (c < o.n) d[c] = x[r].x;
             if (c + 32 < o.n) d[c + 32] = x[r].y;
@@ -984,7 +984,7 @@ extern "C" int dj_graph_upload(dj_graph* g, const int32_t* W, int64_t ld, uint64
     const int32_t* src = static_cast<const int32_t*>(pa.devicePointer);
     const int vec = (ld % 4 == 0 && reinterpret_cast<uintptr_t>(src) % 16 == 0) ? 1 : 0;
     // two blocks an SM keep the host link busy; with a warp for every row all would select their edges at the end,
-    // when nothing is left to copy (n = 8192, weights 1..10: 1358 us, 1323 so; n = 6001, unaligned: 827 and 797)
+    // when nothing is left to copy (n = 8192, weights 1..10: 1358 us, 1323 so; n = 6001, unaligned: 792 and 773)
     const int blocks = std::min((g->n + 7) / 8, 152 * 2);
     k_upload_rows<<<blocks, 256, 0, st>>>(src, ld, g->W, g->pitch, light_out(g), vec);
     e = cudaGetLastError();
