@@ -292,7 +292,7 @@ def main():
                 "kernel": "k_sssp_grid (DJ_ENGINE_GRID, not the default)", "us_per_solve": 1e6 * per_launch_s,
                 "traffic_note": traffic_note,
                 "dram_gbs_from_traffic": (traffic / per_launch_s / 1e9) if traffic else None}
-    light = {"bound": "latency", "kernels": "k_light_cluster (back to back), k_light_grid (idle stream)",
+    light = {"bound": "latency", "kernels": "k_light_cluster (back to back), k_light_grid (alone)",
              "index_bytes": index_bytes, "alone_l2_flushed_us": cold_us,
              "what": "the default path: exact dist and pred from each row's 64 (or 128) lightest edges and the proof that "
                      "no other entry of the matrix matters"}

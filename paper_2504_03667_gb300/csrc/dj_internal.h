@@ -132,7 +132,7 @@ struct StreamSolves {
   unsigned long long capture = 0;
   cudaGraphNode_t last = nullptr;
 };
-constexpr size_t kMaxStreamSolves = 64;  // streams; then the longest without a solve under way makes room
+constexpr size_t kMaxStreamSolves = 64;  // streams; then one without a solve under way makes room
 constexpr size_t kSolvedStride = 16;     // 32-bit words: a cache line each
 
 // What a solve's kernel writes when it ends (nullptr: nothing).

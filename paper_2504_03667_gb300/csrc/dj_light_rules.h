@@ -67,7 +67,7 @@ inline int light_trial_verdict(uint32_t rows, uint32_t guess, uint32_t risky) {
   return risky <= kTrialRisky ? kTrialAll : kTrialAsk;
 }
 
-// Whether a graph whose lists of 64 edges are cut and that has less than kLightClusterMinN nodes is one of few phases: its largest dist
+// Whether a graph of less than kLightClusterMinN nodes whose lists of 64 edges are cut is one of few phases: its largest dist
 // is at most three times its smallest weight, so the streaming engines need about three phases.  Single solves
 // that run behind others then stay on the cluster engine: captured alone, n = 550, p = 0.7, weights 1..10 takes
 // 35 us there and 50 on the light engine's CTA form, n = 1024 51 and 53; with a largest dist of 4 n = 1300,

@@ -757,9 +757,9 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   // trial does not settle it for every source (light_trial_verdict), more are made.  A graph whose
   // trial did not reach every node that something leads to is left to the other engines: two parts of 4000
   // nodes, p = 0.3, took a CTA 15.3 ms a solve, the cluster engine 0.7.
-  // Lists of kLightWide edges are built instead (one more pass and trial) where these look enough: n = 6001,
+  // Lists of kLightWide edges are built instead (one more pass and its trials) where these look enough: n = 6001,
   // p = 0.05, weights 1..10 needs 288 rows whole with 64 edges listed, none with 128, and takes 14.6 us a
-  // solve (the streaming grid engine 51) for a load of 0.54 ms instead of 0.45 (before the index: 1.64).
+  // solve (the streaming grid engine 51) for a load of 0.69 ms instead of 0.45 (before the index: 1.60).
   bool good = false;
   uint32_t guess = idx[kLightGuess];  // 0: lists of 64 hold every edge, or the trial missed some node
   tried = tried && g->wmin >= 1;
