@@ -274,7 +274,8 @@ static bool stream_idle(cudaStream_t st) {
 // What a call finds on its stream, and what its kernel has to write.
 struct StreamState {
   bool capturing = false;
-  bool ahead = true;  // one of this library's solves (those that leave a mark) is directly ahead, or still under way
+  bool ahead = true;  // one of this library's solves (StreamSolves) is directly ahead, or still under way
+  uint32_t seq = 0;   // the number of this one
   SolveMark mark;
 };
 
@@ -290,7 +291,7 @@ static StreamSolves* stream_solves(DevCtx* ctx, cudaStream_t st) {  // g_solves_
   }
   for (size_t i = 0; i < ctx->solves.size(); ++i) {  // a stream with nothing under way makes room
     StreamSolves& s = ctx->solves[i];
-    if (s.issued != *const_cast<volatile uint32_t*>(ctx->solved_h + kSolvedStride * i)) continue;
+    if (s.issued != s.marked || s.marked != *const_cast<volatile uint32_t*>(ctx->solved_h + kSolvedStride * i)) continue;
     s.stream = st;
     s.capture = 0;
     return &s;
@@ -332,9 +333,14 @@ static StreamState stream_state(DevCtx* ctx, cudaStream_t st) {
     x.ahead = s && capture_end(st, &id, &node) && s->capture == id && s->last == node;
   } else if (s) {
     const size_t i = static_cast<size_t>(s - ctx->solves.data()) * kSolvedStride;
-    x.ahead = s->issued != *const_cast<volatile uint32_t*>(ctx->solved_h + i);
-    x.mark.done = ctx->solved_d + i;
-    x.mark.seq = s->issued + 1;
+    // the last marked one has ended; whether those behind it have, an idle stream tells
+    const bool ended = s->marked == *const_cast<volatile uint32_t*>(ctx->solved_h + i);
+    x.ahead = !ended || (s->issued != s->marked && !stream_idle(st));
+    x.seq = s->issued + 1;
+    if (!x.ahead || x.seq % kMarkEvery == 0) {
+      x.mark.done = ctx->solved_d + i;
+      x.mark.seq = x.seq;
+    }
   } else {
     x.ahead = !stream_idle(st);
   }
@@ -346,7 +352,8 @@ static void solve_enqueued(DevCtx* ctx, cudaStream_t st, const StreamState& x) {
   std::lock_guard<std::mutex> lk(g_solves_mu);
   StreamSolves* s = ctx->solved_h ? stream_solves(ctx, st) : nullptr;
   if (!s) return;
-  if (x.mark.done) s->issued = x.mark.seq;
+  if (!x.capturing) s->issued = x.seq;
+  if (x.mark.done) s->marked = x.seq;
   if (x.capturing && !capture_end(st, &s->capture, &s->last)) s->capture = 0;
 }
 

@@ -123,15 +123,18 @@ struct StreamWs {
   size_t bytes = 0;
 };
 
-// The single solves enqueued on a stream, as far as they count for the form of the next one (solve_ahead).
-// Each writes its number to the stream's word in host memory as it ends; in a capture the node that the last
-// one left at the end of the stream tells.
+// The single solves enqueued on a stream, as far as they count for the form of the next one (stream_state).
+// Those that found nothing ahead, and every kMarkEvery-th other, write their number to the stream's word in host
+// memory as they end (each of a chain doing so cost it 2 %: n = 16384 14.9 -> 15.3 us a solve); in a capture the
+// node that the last one left at the end of the stream tells.
 struct StreamSolves {
   cudaStream_t stream = nullptr;
-  uint32_t issued = 0;
+  uint32_t issued = 0;  // the last solve's number
+  uint32_t marked = 0;  // and that of the last one that writes it
   unsigned long long capture = 0;
   cudaGraphNode_t last = nullptr;
 };
+constexpr uint32_t kMarkEvery = 8;
 constexpr size_t kMaxStreamSolves = 64;  // streams; then one without a solve under way makes room
 constexpr size_t kSolvedStride = 16;     // 32-bit words: a cache line each
 
@@ -164,7 +167,7 @@ struct DevCtx {
   uint32_t* words = nullptr;  // device: [0] error bits, [1] phases of the last single solve
   std::vector<StreamWs> ws;   // per-stream workspaces of the grid engine (see stream_workspace)
   std::vector<FnSetup> fns;   // see prepare_function
-  std::vector<StreamSolves> solves;  // see solve_ahead
+  std::vector<StreamSolves> solves;  // see stream_state
   uint32_t* solved_h = nullptr;      // their words: mapped host memory, and its device address
   uint32_t* solved_d = nullptr;
 };
