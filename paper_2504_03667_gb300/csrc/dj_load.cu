@@ -310,7 +310,8 @@ __global__ void __launch_bounds__(256) k_light_rows(const int32_t* __restrict__ 
 // row at a time from `src` (row stride ld) into the graph's row and selects its light edges on the
 // way (k_light_rows), so the matrix crosses the host link once and is not read from HBM again.  With
 // `vec` (ld a multiple of 4, src 16-byte aligned) the row moves in 16-byte pieces, four in flight per
-// lane, otherwise in 4-byte pieces, eight in flight (sixteen: n = 6001 796 us, not 773).  Padding columns are left as they are (INF).
+// lane, otherwise in 4-byte pieces, eight in flight (sixteen: n = 6001 796 us, not 773).  Padding columns are left
+// as they are (INF).
 __global__ void __launch_bounds__(256) k_upload_rows(const int32_t* __restrict__ src, int64_t ld,
                                                      int32_t* __restrict__ W, int64_t pitch, const LightOut o,
                                                      int vec) {
@@ -672,9 +673,9 @@ static bool launch_trial(dj_graph* g, uint32_t* idx, cudaStream_t st) {
 }
 
 // Whether a graph with cut lists is one whose solves hardly need a row whole, by its trial (idx) and, where
-// that leaves it open, by further ones: side by side, a CTA each, where the state fits one (n = 300, 1500
-// and 8192: about 35, 70 and 180 us), else one after another over every SM.
-static int judge_cut(dj_graph* g, const uint32_t* idx, cudaStream_t st, bool* good) {
+// that leaves it open, by further ones: side by side, a CTA each, where the state fits one (n = 4099 and 8192
+// 78 and 96 us, n = 6001 on lists of 128 133; one over every SM takes 34-52), else one after another.
+static int cut_lists_serve(dj_graph* g, const uint32_t* idx, cudaStream_t st, bool* good) {
   const int verdict = light_trial_verdict(idx[1], idx[kLightGuess], idx[kLightRisky]);
   *good = verdict == kTrialAll;
   if (verdict != kTrialAsk) return DJ_OK;
@@ -720,8 +721,8 @@ static bool wide_suffices(const dj_graph* g, const uint32_t* idx) {
 // The index's leading words are zero before, but for the edge list's check (words 12..14), whose
 // verdict *list gets (nullptr: there was no list).
 //
-// Whether solves take the light engine is judged here, by a trial solve: one more kernel in front of
-// the wait, the only one unless longer lists are worth a try.
+// Whether solves take the light engine is decided here, by a trial solve: one more kernel in front of
+// the wait, the only one unless that leaves it open or longer lists are worth a try.
 static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   uint32_t* stats = g->light ? g->light + 8 : nullptr;
   uint32_t idx[kLightHost] = {0};
@@ -765,7 +766,7 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
   tried = tried && g->wmin >= 1;
   bool complete = tried && ~idx[0] >= kInf;
   if (tried && !complete)
-    if (int rc = judge_cut(g, idx, st, &good)) return rc;
+    if (int rc = cut_lists_serve(g, idx, st, &good)) return rc;
   if (tried && !complete && !good && wide_suffices(g, idx)) {
     cudaMemsetAsync(g->light, 0, 8 * sizeof(uint32_t), st);
     cudaMemsetAsync(g->light + kLightGuess, 0, 9 * sizeof(uint32_t), st);  // to kLightRisky
@@ -778,7 +779,7 @@ static int finish_graph(dj_graph* g, cudaStream_t st, uint32_t* list) {
     complete = tried && ~idx[0] >= kInf;  // (then there was no trial on the longer ones)
     if (idx[kLightGuess]) guess = idx[kLightGuess];
     if (tried && !complete)
-      if (int rc = judge_cut(g, idx, st, &good)) return rc;
+      if (int rc = cut_lists_serve(g, idx, st, &good)) return rc;
   }
   // an upload's first threshold: the mean of those that served this matrix (the new one is likely of its kind)
   const uint32_t cut = idx[kLightSeen + 4];
@@ -997,8 +998,8 @@ extern "C" int dj_graph_upload(dj_graph* g, const int32_t* W, int64_t ld, uint64
   }
   if (e != cudaSuccess) return cuda_error(e, "host-to-device matrix copy (upload)");
   g->upload_pending = 1;
-  // The index follows the matrix (a captured solve may be replayed on it), but it was judged for the
-  // loaded one: nothing tells here, without a wait, whether the new one suits it.
+  // The index follows the matrix (a captured solve may be replayed on it), but it was tried on the
+  // loaded one: nothing tells here, without a wait, whether it suits the new one.
   g->light_ok = g->light_cta = g->light_few = g->light_wide = false;
   launch_minima(g, nullptr, st, zero_copy);
   e = cudaGetLastError();
